@@ -73,15 +73,18 @@ constexpr int kRedBlock = 256;
 
 // One block per (x plane, 8 y rows); 32 lanes stride along z.  Block b writes
 // its partial sums to slot b, so the reduction order is fixed.
-// With r32 != nullptr the float64 residual of every uncovered interior cell is also
-// stored, rounded to float32, as the source of the correction equation (mixed
-// precision); covered cells are skipped for both.
-template <int ORDER>
+// MIXED: the float64 residual of every uncovered interior cell is also stored in r32,
+// rounded to float32, as the source of the correction equation; covered cells are skipped
+// for both.  The stencil sums run on the integer pipe (mg_fixed.cuh) except in MIXED, where
+// the last bits of r decide float32 roundings of the whole correction cycle: with them
+// changed, displacements of the deepest nest of a 5-level hierarchy moved by 1.1e-9
+// relative, so that mode keeps the FP64 operations one by one.
+template <int ORDER, bool MIXED>
 __global__ void __launch_bounds__(kRedBlock)
     k_norm_partial(Grid G, const double* __restrict__ u, const double* __restrict__ f,
                    double invh2, double vol, Int3 clo, Int3 chi, double* __restrict__ partial,
                    float* __restrict__ r32) {
-  const long long sy = G.Zp, sx = (long long)G.Y * G.Zp;
+  const int sy = G.Zp, sx = G.Y * G.Zp;
   const int i = blockIdx.y;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -89,6 +92,7 @@ __global__ void __launch_bounds__(kRedBlock)
   if (j < G.n1) {
     const bool row_cov = i >= clo.x && i < chi.x && j >= clo.y && j < chi.y;
     const long long row = gidx(G, i, j, 0);
+#pragma unroll 1
     for (int k = lane; k < G.n2; k += 32) {
       // covered cells: no norm term, and no correction source either (the FAS
       // restriction overwrites a covered parent cell's source before the parent uses it)
@@ -96,8 +100,10 @@ __global__ void __launch_bounds__(kRedBlock)
       if (cov) continue;
       const long long p = row + k;
       const double fv = __ldg(f + p);
-      const double r = u ? fma(-invh2, lap_h2<ORDER, double>(u, p, sy, sx), fv) : fv;
-      if (r32) r32[p] = (float)r;
+      const double r = u ? add_lap_h2<ORDER, double, Ldg, !MIXED>(u, p, sy, sx, __ldg(u + p),
+                                                                 -invh2, fv)
+                         : fv;
+      if (MIXED) r32[p] = (float)r;
       rr = fma(r, r, rr);
       ff = fma(fv, fv, ff);
     }
@@ -392,9 +398,18 @@ cudaError_t launch_norm_partial(int order, const Grid& G, const double* u, const
   const dim3 grid((G.n1 + 7) / 8, G.n0);
   if ((int)(grid.x * grid.y) != blocks) return cudaErrorInvalidValue;
   switch (order) {
-    case 2: k_norm_partial<2><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32); break;
-    case 4: k_norm_partial<4><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32); break;
-    case 6: k_norm_partial<6><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32); break;
+    case 2:
+      if (r32) k_norm_partial<2, true><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
+      else k_norm_partial<2, false><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
+      break;
+    case 4:
+      if (r32) k_norm_partial<4, true><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
+      else k_norm_partial<4, false><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
+      break;
+    case 6:
+      if (r32) k_norm_partial<6, true><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
+      else k_norm_partial<6, false><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
+      break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -19,14 +19,15 @@ namespace {
 constexpr int kPairX = kVPairX;  // z-pairs per block row; blockDim.y = rows (1..8)
 // At least 5 blocks of up to 256 threads per SM: caps the smoother at 48 registers
 // (80 unbounded).  Measured on GB300 in CUDA graphs: float32 half-sweeps 15-20%
-// faster at 128^3 (more warps in flight for the L1-bound loads), float64 unchanged
-// (bound by the FP64 pipe).
-#ifndef MG_SMOOTH_MIN_BLOCKS
-#define MG_SMOOTH_MIN_BLOCKS 5
-#endif
+// faster at 128^3 (more warps in flight for the L1-bound loads).  float64 at order 6 holds
+// its 18 neighbours while their largest exponent is found (mg_fixed.cuh) and spills at 48
+// registers: 4 blocks give 17.6 us per 128^3 half-sweep, 5 blocks 21.9, 3 blocks 19.1; at
+// order 4, 5 blocks give 12.8, 4 blocks 13.6.
+template <int ORDER, typename T>
+constexpr int smooth_min_blocks = sizeof(T) == 8 && ORDER == 6 ? 4 : 5;
 
 template <int ORDER, typename T>
-__global__ void __launch_bounds__(kPairX * 8, MG_SMOOTH_MIN_BLOCKS)
+__global__ void __launch_bounds__(kPairX * 8, (smooth_min_blocks<ORDER, T>))
     k_smooth_half(Grid G, const T* __restrict__ uin, T* __restrict__ uout,
                   const T* __restrict__ f, T a_f, int colour, int periodic) {
   smooth_half_body<ORDER, T, Ldg>(G, uin, uout, f, a_f, colour, periodic, (int)blockDim.y,

@@ -229,17 +229,26 @@ __global__ void __launch_bounds__(32 * kTY)
           }
           const T* Cu = C + upd;
           auto comp = [&](const V2& v) { return upd ? v.y : v.x; };  // the updated cell's value
-          T s1 = (zm1 + zp1) + (Cu[-kBZ] + Cu[kBZ]) + (comp(q[tc - 1]) + comp(q[tc + 1]));
-          T s2 = T(0), s3 = T(0);
-          if constexpr (ORDER >= 4)
-            s2 = (zm2 + zp2) + (Cu[-2 * kBZ] + Cu[2 * kBZ]) + (comp(q[tc - 2]) + comp(q[tc + 2]));
-          if constexpr (ORDER >= 6)
-            s3 = (zm3 + zp3) + (Cu[-3 * kBZ] + Cu[3 * kBZ]) + (comp(q[tc - 3]) + comp(q[tc + 3]));
-          constexpr double wc = 3.0 * Lap<ORDER>::w0;
-          T v = a_f * tiles[(tc % kSlots) * TL::stride + fown + upd];
-          v = fma(T(-Lap<ORDER>::w1 / wc), s1, v);
-          if constexpr (ORDER >= 4) v = fma(T(-Lap<ORDER>::w2 / wc), s2, v);
-          if constexpr (ORDER >= 6) v = fma(T(-Lap<ORDER>::w3 / wc), s3, v);
+          T nb[3 * ORDER];
+          nb[0] = zm1;
+          nb[1] = zp1;
+          if constexpr (ORDER >= 4) {
+            nb[6] = zm2;
+            nb[7] = zp2;
+          }
+          if constexpr (ORDER >= 6) {
+            nb[12] = zm3;
+            nb[13] = zp3;
+          }
+#pragma unroll
+          for (int d = 1; d <= H; ++d) {
+            nb[6 * d - 4] = Cu[-d * kBZ];
+            nb[6 * d - 3] = Cu[d * kBZ];
+            nb[6 * d - 2] = comp(q[tc - d]);
+            nb[6 * d - 1] = comp(q[tc + d]);
+          }
+          const T v =
+              relax<ORDER, T>(nb, a_f * tiles[(tc % kSlots) * TL::stride + fown + upd]);
           T* o = orow + s * sx;
           const int i = i0 + s;
           const bool img = periodic && (yz_face || i < G.g || i >= G.n0 - G.g);

@@ -36,8 +36,8 @@ __device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restr
   const int i = b.bz;
   const int k0 = 2 * t;
   if (j >= G.n1 || k0 >= G.n2) return;
-  const long long sy = G.Zp;
-  const long long sx = (long long)G.Y * G.Zp;
+  const int sy = G.Zp;
+  const int sx = G.Y * G.Zp;
   const long long p0 = gidx(G, i, j, k0);
   const int upd = (((i + j + k0) & 1) == colour) ? 0 : 1;
   const bool pair = (k0 + 1) < G.n2;
@@ -48,14 +48,10 @@ __device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restr
     return;
   }
   const long long p = p0 + upd;
-  T s1, s2, s3;
-  neighbour_sums<ORDER, T, LD>(uin, p, sy, sx, s1, s2, s3);
   // u = (h^2 f - sum_off w u_nb) / w_centre
-  constexpr double wc = 3.0 * Lap<ORDER>::w0;
-  T v = a_f * LD::ld(f + p);
-  v = fma(T(-Lap<ORDER>::w1 / wc), s1, v);
-  if (ORDER >= 4) v = fma(T(-Lap<ORDER>::w2 / wc), s2, v);
-  if (ORDER >= 6) v = fma(T(-Lap<ORDER>::w3 / wc), s3, v);
+  T nb[3 * ORDER];
+  load_neighbours<ORDER, T, LD>(uin, p, sy, sx, nb);
+  const T v = relax<ORDER, T>(nb, a_f * LD::ld(f + p));
   if (pair) {
     typedef typename Vec2<T>::type V2;
     V2 out;
@@ -88,8 +84,8 @@ __device__ __forceinline__ void residual_restrict_body(const Grid& F, const T* _
   const int jc = b.by * 4 + b.ty;
   const int ic = b.bz;
   if (kc >= cn.z || jc >= cn.y) return;
-  const long long sy = F.Zp;
-  const long long sx = (long long)F.Y * F.Zp;
+  const int sy = F.Zp;
+  const int sx = F.Y * F.Zp;
   T su = T(0), sr = T(0);
 #pragma unroll
   for (int di = 0; di < 2; ++di) {
@@ -98,9 +94,9 @@ __device__ __forceinline__ void residual_restrict_body(const Grid& F, const T* _
 #pragma unroll
       for (int dk = 0; dk < 2; ++dk) {
         const long long p = gidx(F, 2 * ic + di, 2 * jc + dj, 2 * kc + dk);
-        const T lu = lap_h2<ORDER, T, LD>(u, p, sy, sx);
-        su += LD::ld(u + p);
-        sr += fma(-invh2, lu, LD::ld(f + p));
+        const T c = LD::ld(u + p);
+        su += c;
+        sr += add_lap_h2<ORDER, T, LD>(u, p, sy, sx, c, -invh2, LD::ld(f + p));
       }
     }
   }
@@ -121,10 +117,8 @@ __device__ __forceinline__ void fas_source_body(const Grid& P, const T* __restri
   const int jc = b.by * 4 + b.ty;
   const int ic = b.bz;
   if (kc >= cn.z || jc >= cn.y) return;
-  const long long sy = P.Zp;
-  const long long sx = (long long)P.Y * P.Zp;
   const long long q = gidx(P, off.x + ic, off.y + jc, off.z + kc);
-  pfas[q] = fma(invH2, lap_h2<ORDER, T, LD>(pu, q, sy, sx), pfas[q]);
+  pfas[q] = add_lap_h2<ORDER, T, LD>(pu, q, P.Zp, P.Y * P.Zp, LD::ld(pu + q), invH2, pfas[q]);
 }
 
 // ---- prolongation-correction: u += inject(parent u - ubar), one thread per z-pair ----
