@@ -2470,6 +2470,8 @@ mg_status mg_hierarchy_create(const mg_config* cfg, void* cuda_stream, mg_hierar
   cudaError_t e = cudaMallocHost(&h->host_red, kRedDoubles * sizeof(double));
   if (e == cudaSuccess) e = cudaMemsetAsync(h->red, 0, kRedDoubles * sizeof(double), h->s);
   if (e == cudaSuccess) e = setup_tma(h);
+  if (e == cudaSuccess) e = prepare_restrict_tile();
+  if (e == cudaSuccess) e = prepare_norm_tile();
   if (e != cudaSuccess) {
     mg_hierarchy_destroy(h);
     return MG_ECUDA;

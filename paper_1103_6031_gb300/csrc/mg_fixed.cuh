@@ -50,9 +50,12 @@ __device__ __forceinline__ bool fx_in_range(unsigned key) {
 __device__ __forceinline__ long long fx_align(double v, unsigned key) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
   const unsigned sh = (key - (hi << 1)) >> 21;
-  unsigned long long x = ((((unsigned long long)((hi & 0xfffffu) | 0x100000u)) << 32) | lo) << 6;
+  const unsigned xh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 6);
+  unsigned long long x = ((unsigned long long)xh << 32) | (lo << 6);
   asm("shr.u64 %0, %0, %1;" : "+l"(x) : "r"(sh));
-  return (long long)x ^ ((long long)(int)hi >> 63);
+  unsigned s;  // the sign in every bit (prmt's sign replication: 5% of a half-sweep)
+  asm("prmt.b32 %0, %1, 0, 0xbbbb;" : "=r"(s) : "r"(hi));
+  return (long long)(x ^ (((unsigned long long)s << 32) | s));
 }
 
 // c * 2^(e - kFxBias) by an addition to the exponent field; c a normal constant whose
@@ -86,8 +89,16 @@ struct FxUnit<6> {
   static constexpr double v = 256.0 / 180.0;
 };
 
-// The weighted sum of the 6 neighbours at each distance (nb[6 d .. 6 d + 5] at distance
-// d + 1) as an integer T; key as for fx_align.
+// The neighbours' part of T from their sums at distance 1, 2, 3.
+template <int ORDER>
+__device__ __forceinline__ long long fx_weighted(const long long (&s)[3]) {
+  if (ORDER == 2) return s[0];
+  if (ORDER == 4) return s[0] - (s[1] >> 4);
+  // 270/256 = 1 + 1/16 - 1/128, 27/256 = 1/8 - 1/64 - 1/256, 2/256 = 1/128
+  return s[0] + (s[0] >> 4) - (s[1] >> 3) + ((s[1] + (s[1] >> 2)) >> 6) + ((s[2] - s[0]) >> 7);
+}
+
+// The same from the neighbours (nb[6 d .. 6 d + 5] at distance d + 1); key as for fx_align.
 template <int ORDER>
 __device__ __forceinline__ long long fx_neighbours(const double (&nb)[3 * ORDER], unsigned key) {
   long long s[3] = {0, 0, 0};
@@ -95,10 +106,7 @@ __device__ __forceinline__ long long fx_neighbours(const double (&nb)[3 * ORDER]
   for (int d = 0; d < ORDER / 2; ++d)
 #pragma unroll
     for (int q = 0; q < 6; ++q) s[d] += fx_align(nb[6 * d + q], key);
-  if (ORDER == 2) return s[0];
-  if (ORDER == 4) return s[0] - (s[1] >> 4);
-  // 270/256 = 1 + 1/16 - 1/128, 27/256 = 1/8 - 1/64 - 1/256, 2/256 = 1/128
-  return s[0] + (s[0] >> 4) - (s[1] >> 3) + ((s[1] + (s[1] >> 2)) >> 6) + ((s[2] - s[0]) >> 7);
+  return fx_weighted<ORDER>(s);
 }
 
 // The centre's term of T (weight 3 w0), c its aligned integer.

@@ -86,6 +86,10 @@ template <typename T>
 cudaError_t launch_restrict_u(const Grid& F, const T* u, const Grid& P, T* pu, Int3 off,
                               Int3 cn, cudaStream_t s);
 
+// Opt the tile kernels in to their shared-memory size on the current device.
+cudaError_t prepare_restrict_tile();
+cudaError_t prepare_norm_tile();
+
 // ---- TMA-staged smoother (mg_smooth_tma.cu) ----
 // Same update and result as launch_smooth_half; the input buffer u is read through
 // tin, the source f through tf (both made by make_plane_tmap, with halo = true for

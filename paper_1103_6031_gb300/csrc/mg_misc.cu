@@ -3,6 +3,7 @@
 // displacement gradient (Hahn & Abel 2011, Sec. 3.1, 3.2).
 #include "mg_internal.h"
 #include "mg_stencil.cuh"
+#include "mg_tile.cuh"
 #include "mg_vbody.cuh"
 
 namespace mgk {
@@ -111,6 +112,68 @@ __global__ void __launch_bounds__(kRedBlock)
   block_sum2<kRedBlock>(rr, ff);
   if (threadIdx.x == 0) {
     const int b = blockIdx.y * gridDim.x + blockIdx.x;
+    partial[2 * b] = rr * vol;
+    partial[2 * b + 1] = ff * vol;
+  }
+}
+
+// The norm sums of float64 levels on tiles of aligned integers (mg_tile.cuh): 4 FP64
+// instructions per cell (the conversion, the residual, two squares).  Block b writes slot b,
+// the first block zeros the slots that k_norm_partial would use beyond.
+template <int ORDER>
+__global__ void __launch_bounds__(kTileThreads, 3)
+    k_norm_tile(Grid G, const double* __restrict__ u, const double* __restrict__ f, double invh2,
+                double vol, Int3 clo, Int3 chi, double* __restrict__ partial, int slots) {
+  extern __shared__ __align__(16) long long norm_smem[];
+  const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
+  const int b = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  const int blocks = gridDim.x * gridDim.y * gridDim.z;
+  if (b == 0)
+    for (int q = blocks + threadIdx.x; q < slots; q += kTileThreads)
+      partial[2 * q] = partial[2 * q + 1] = 0.0;
+  double rr = 0.0, ff = 0.0;
+  // a block inside the covered region has no leaf cell
+  const bool covered = i0 >= clo.x && min(i0 + kTileX, G.n0) <= chi.x && j0 >= clo.y &&
+                       min(j0 + kTileY, G.n1) <= chi.y && k0 >= clo.z &&
+                       min(k0 + kTileZ, G.n2) <= chi.z;
+  if (!covered) {
+    const unsigned key = tile_load<ORDER>(G, u, i0, j0, k0, norm_smem);
+    const TilePos t = tile_pos();
+    const int i = i0 + 4 * t.xh, j = j0 + t.y, k = k0 + 2 * t.zz;
+    const long long p = gidx(G, i, j, k);
+    const int sx = G.Y * G.Zp;
+    const double kr = -invh2 * FxUnit<ORDER>::v;
+    const bool fx = fx_in_range(key) && fx_scalable(kr, key);
+    const double ks = fx_scale(kr, key);
+    auto leaf = [&](int q, int dk) {
+      return i + q < G.n0 && j < G.n1 && k + dk < G.n2 &&
+             !(i + q >= clo.x && i + q < chi.x && j >= clo.y && j < chi.y && k + dk >= clo.z &&
+               k + dk < chi.z);
+    };
+    auto add = [&](double r, double fv) {
+      rr = fma(r, r, rr);
+      ff = fma(fv, fv, ff);
+    };
+    if (fx) {
+      tile_laplacians<ORDER>(norm_smem, [&](int q, longlong2 T, longlong2) {
+        const bool l0 = leaf(q, 0), l1 = leaf(q, 1);
+        if (!(l0 || l1)) return;
+        const double2 fv = __ldg(reinterpret_cast<const double2*>(f + p + q * sx));
+        if (l0) add(fma(ks, (double)T.x, fv.x), fv.x);
+        if (l1) add(fma(ks, (double)T.y, fv.y), fv.y);
+      });
+    } else {
+#pragma unroll 1
+      for (int q = 0; q < 8; ++q) {
+        if (!leaf(q >> 1, q & 1)) continue;
+        const long long e = p + (q >> 1) * sx + (q & 1);
+        const double fv = __ldg(f + e);
+        add(add_lap_h2<ORDER, double, Ldg, false>(u, e, G.Zp, sx, __ldg(u + e), -invh2, fv), fv);
+      }
+    }
+  }
+  block_sum2<kTileThreads>(rr, ff);
+  if (threadIdx.x == 0) {
     partial[2 * b] = rr * vol;
     partial[2 * b + 1] = ff * vol;
   }
@@ -397,6 +460,16 @@ cudaError_t launch_norm_partial(int order, const Grid& G, const double* u, const
                                 int blocks, float* r32, cudaStream_t s) {
   const dim3 grid((G.n1 + 7) / 8, G.n0);
   if ((int)(grid.x * grid.y) != blocks) return cudaErrorInvalidValue;
+  const dim3 tg = tile_grid(G);
+  if (!r32 && u && tile_pays(G) && (long long)tg.x * tg.y * tg.z <= blocks) {
+    switch (order) {
+      case 2: k_norm_tile<2><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(G, u, f, invh2, vol, clo, chi, partial, blocks); break;
+      case 4: k_norm_tile<4><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(G, u, f, invh2, vol, clo, chi, partial, blocks); break;
+      case 6: k_norm_tile<6><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(G, u, f, invh2, vol, clo, chi, partial, blocks); break;
+      default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+  }
   switch (order) {
     case 2:
       if (r32) k_norm_partial<2, true><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
@@ -413,6 +486,11 @@ cudaError_t launch_norm_partial(int order, const Grid& G, const double* u, const
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
+}
+
+cudaError_t prepare_norm_tile() {
+  return cudaFuncSetAttribute(k_norm_tile<6>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              FxTile<6>::bytes);
 }
 
 cudaError_t launch_sum_partial(const Grid& G, const double* f, double vol, Int3 clo, Int3 chi,

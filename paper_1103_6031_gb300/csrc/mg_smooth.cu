@@ -10,6 +10,7 @@
 // thread ever reads a value another thread of the same launch writes.
 #include "mg_internal.h"
 #include "mg_stencil.cuh"
+#include "mg_tile.cuh"
 #include "mg_vbody.cuh"
 
 namespace mgk {
@@ -131,6 +132,82 @@ __global__ void __launch_bounds__(128)
                                             (int)threadIdx.x, (int)threadIdx.y});
 }
 
+// The same on tiles of aligned integers (mg_tile.cuh), float64: the mean of a parent's 8
+// children and of their T are integer sums (T shifted by 3 first, so that the sum cannot
+// overflow: 2^-56 of the tile's largest value), leaving about 12 FP64 instructions per
+// parent cell, 7 of them the sum of f.  A thread holds 2 x 1 x 2 children of two parents;
+// the row above or below is in the other half of its warp.
+template <int ORDER>
+__global__ void __launch_bounds__(kTileThreads, 3)
+    k_residual_restrict_tile(Grid F, const double* __restrict__ u, const double* __restrict__ f,
+                             double invh2, Grid P, double* __restrict__ pu,
+                             double* __restrict__ pfas, double* __restrict__ ubar, Int3 off, Int3 cn,
+                             int parent_periodic) {
+  extern __shared__ __align__(16) long long tile_smem[];
+  const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
+  const unsigned key = tile_load<ORDER>(F, u, i0, j0, k0, tile_smem);
+  const TilePos t = tile_pos();
+  const int i = i0 + 4 * t.xh, j = j0 + t.y, k = k0 + 2 * t.zz;
+  const long long p = gidx(F, i, j, k);
+  const int sx = F.Y * F.Zp;
+  const bool row = j < F.n1 && k < F.n2;
+  const double kr = -invh2 * FxUnit<ORDER>::v;
+  double mu[2] = {0.0, 0.0}, mr[2] = {0.0, 0.0};  // sums over the two planes of a parent
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (!(row && i + q < F.n0)) continue;
+    const double2 fv = __ldg(reinterpret_cast<const double2*>(f + p + q * sx));
+    mr[q >> 1] += fv.x + fv.y;
+  }
+  if (fx_in_range(key) && fx_scalable(kr, key)) {
+    long long su[2] = {0, 0}, st[2] = {0, 0};
+    tile_laplacians<ORDER>(tile_smem, [&](int q, longlong2 T, longlong2 c) {
+      su[q >> 1] += c.x + c.y;
+      st[q >> 1] += (T.x >> 3) + (T.y >> 3);
+    });
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      mr[a] += __shfl_xor_sync(~0u, mr[a], 16);
+      su[a] += __shfl_xor_sync(~0u, su[a], 16);
+      st[a] += __shfl_xor_sync(~0u, st[a], 16);
+      mr[a] = fma(fx_scale(kr, key), (double)st[a], 0.125 * mr[a]);
+      mu[a] = fx_scale(0.125, key) * (double)su[a];
+    }
+  } else {
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+      if (!(row && i + q < F.n0)) continue;
+      for (int dk = 0; dk < 2; ++dk) {
+        const double c = __ldg(u + p + q * sx + dk);
+        const double r =
+            add_lap_h2<ORDER, double, Ldg, false>(u, p + q * sx + dk, F.Zp, sx, c, -invh2, 0.0);
+        if (q < 2) {
+          mu[0] += c;
+          mr[0] += r;
+        } else {
+          mu[1] += c;
+          mr[1] += r;
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      mr[a] = 0.125 * (mr[a] + __shfl_xor_sync(~0u, mr[a], 16));
+      mu[a] = 0.125 * (mu[a] + __shfl_xor_sync(~0u, mu[a], 16));
+    }
+  }
+  // the lower row's thread writes the first parent, the upper row's the second
+  const int a = t.y & 1;
+  const int ic = (i >> 1) + a, jc = j >> 1, kc = k >> 1;
+  if (!row || i + 2 * a >= F.n0) return;
+  const double vu = a ? mu[1] : mu[0];
+  const long long q = gidx(P, off.x + ic, off.y + jc, off.z + kc);
+  pu[q] = vu;
+  if (parent_periodic) write_images<double>(P, pu, off.x + ic, off.y + jc, off.z + kc, vu);
+  pfas[q] = a ? mr[1] : mr[0];
+  ubar[((long long)ic * cn.y + jc) * cn.z + kc] = vu;
+}
+
 // Covered parent cells: f_fas += L u (u = restricted fine solution there).
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
@@ -222,6 +299,18 @@ template <typename T>
 cudaError_t launch_residual_restrict(int order, const Grid& F, const T* u, const T* f,
                                      double invh2, const Grid& P, T* pu, T* pfas, T* ubar,
                                      Int3 off, Int3 cn, int parent_periodic, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (tile_pays(F)) {
+      const dim3 tg = tile_grid(F);
+      switch (order) {
+        case 2: k_residual_restrict_tile<2><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic); break;
+        case 4: k_residual_restrict_tile<4><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic); break;
+        case 6: k_residual_restrict_tile<6><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic); break;
+        default: return cudaErrorInvalidValue;
+      }
+      return cudaGetLastError();
+    }
+  }
   dim3 block(32, 4, 1);
   dim3 grid = coarse_grid(cn, block);
   switch (order) {
@@ -264,6 +353,11 @@ cudaError_t launch_restrict_u(const Grid& F, const T* u, const Grid& P, T* pu, I
   dim3 grid = coarse_grid(cn, block);
   k_restrict_u<T><<<grid, block, 0, s>>>(F, u, P, pu, off, cn);
   return cudaGetLastError();
+}
+
+cudaError_t prepare_restrict_tile() {
+  return cudaFuncSetAttribute(k_residual_restrict_tile<6>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, FxTile<6>::bytes);
 }
 
 #define MGK_INSTANTIATE(T)                                                                     \

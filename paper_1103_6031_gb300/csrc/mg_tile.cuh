@@ -1,0 +1,197 @@
+// Tiles of aligned integers in shared memory for the float64 stencils that need every
+// cell (mg_fixed.cuh): a block of 256 threads loads 8 x 8 x 32 cells with the halo of the
+// star-shaped stencil, aligns every value once to the block's largest exponent, and the
+// cells' sums read shared memory.  A value is aligned 2.7 times on average (halos) instead
+// of once for each of the 19 cells whose stencil it is in.
+//
+// What it is bounded by: the alignment and the sums, about 140 integer and shared-memory
+// instructions per cell; 63 KB of shared memory at order 6 let three blocks share an SM,
+// so that one block's loads overlap the others' sums.  A half-sweep, which needs only
+// every second cell's sum, gains nothing from it (17.8 against 17.6 us at 128^3).
+#pragma once
+
+#include "mg_fixed.cuh"
+#include "mg_internal.h"
+#include "mg_stencil.cuh"
+
+namespace mgk {
+
+constexpr int kTileX = 8, kTileY = 8, kTileZ = 32;
+constexpr int kTileThreads = 256;
+
+template <int ORDER>
+struct FxTile {
+  static constexpr int R = ORDER / 2;
+  static constexpr int RZ = (R + 1) / 2 * 2;  // z halo rounded up to pairs
+  static constexpr int SY = kTileY + 2 * R, SZ = kTileZ + 2 * RZ;
+  static constexpr int px = SY * SZ, py = SZ;  // element strides along x and y
+  static constexpr int elems = (kTileX + 2 * R) * px;
+  static constexpr int bytes = elems * 8;
+  // element of tile cell (x, y, z)
+  static __device__ __forceinline__ int at(int x, int y, int z) {
+    return (x + R) * px + (y + R) * py + z + RZ;
+  }
+};
+
+inline dim3 tile_grid(const Grid& G) {
+  return dim3((G.n2 + kTileZ - 1) / kTileZ, (G.n1 + kTileY - 1) / kTileY,
+              (G.n0 + kTileX - 1) / kTileX);
+}
+
+// Levels that the tile kernels take: below, their blocks are too few to hide a block's load
+// phase.
+constexpr long long kTileMinCells = 1ll << 17;
+
+inline bool tile_pays(const Grid& G) {
+  return (long long)G.n0 * G.n1 * G.n2 >= kTileMinCells;
+}
+
+// Which cells of the tile a thread works on: the z-pair 2 zz, 2 zz + 1 of row y in the
+// planes 4 xh .. 4 xh + 3 (lanes 0-15 and 16-31 of a warp: two neighbouring rows).
+struct TilePos {
+  int zz, y, xh;
+};
+
+__device__ __forceinline__ TilePos tile_pos() {
+  const int t = threadIdx.x;
+  return TilePos{t & 15, (t >> 4) & 7, t >> 7};
+}
+
+__device__ __forceinline__ unsigned block_max(unsigned m) {
+  __shared__ unsigned red[kTileThreads / 32];
+  m = __reduce_max_sync(~0u, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kTileThreads / 32; ++w) m = max(m, red[w]);
+  return m;
+}
+
+// Loads the tile at cell (i0, j0, k0) of u with its star halo into S, aligned to the
+// returned key (low bits set).  Values outside the stencils' reach (beyond the ghosts,
+// row padding, edge and corner ghosts) count as 0.  If the key is out of range
+// (fx_in_range), S is not written.
+template <int ORDER>
+__device__ __forceinline__ unsigned tile_load(const Grid& G, const double* __restrict__ u, int i0,
+                                              int j0, int k0, long long* S) {
+  typedef FxTile<ORDER> L;
+  constexpr int R = L::R, RZ = L::RZ;
+  const TilePos t = tile_pos();
+  const int sy = G.Zp, sx = G.Y * G.Zp;
+  const double* base = u + gidx(G, i0, j0, k0);
+  const int ex = min(kTileX, G.n0 - i0), ey = min(kTileY, G.n1 - j0), ez = min(kTileZ, G.n2 - k0);
+  const int z = 2 * t.zz;
+  // a pair at z >= ez is out along z; the first R cells there are ghosts
+  const bool in0 = z < ez, in1 = z + 1 < ez;
+  auto pair = [&](int x, int y, bool a, bool b) {
+    double2 v = make_double2(0.0, 0.0);
+    if (a || b) {
+      v = __ldg(reinterpret_cast<const double2*>(base + (x * sx + y * sy + z)));
+      if (!a) v.x = 0.0;
+      if (!b) v.y = 0.0;
+    }
+    return v;
+  };
+  double2 c[4], vx[R], vy[R], vz = make_double2(0.0, 0.0);
+  int xs[R], ys[R];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int x = 4 * t.xh + q;
+    const bool row = x < ex && t.y < ey;
+    // a row that is out along one axis, by at most R, is a halo row for its interior z
+    const bool halo = (x < ex && t.y < ey + R) || (x < ex + R && t.y < ey);
+    c[q] = pair(x, t.y, row ? z < ez + R : halo && in0, row ? z + 1 < ez + R : halo && in1);
+  }
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int s = t.xh + 2 * q;  // 0 .. 2 R - 1: the halo's layers
+    xs[q] = s < R ? s - R : kTileX + s - R;
+    ys[q] = s < R ? s - R : kTileY + s - R;
+    const bool ox = xs[q] < ex + R && t.y < ey;
+    vx[q] = pair(xs[q], t.y, ox && in0, ox && in1);
+    // y layers: the thread's row index runs along x
+    const bool oy = ys[q] < ey + R && t.y < ex;
+    vy[q] = pair(t.y, ys[q], oy && in0, oy && in1);
+  }
+  // z halo: RZ pairs per row, half of them on either side, 64 rows
+  const int zr = (int)threadIdx.x / RZ, ze = (int)threadIdx.x % RZ;
+  const int zx = zr >> 3, zy = zr & 7;
+  const int zo = ze < RZ / 2 ? 2 * ze - RZ : kTileZ + 2 * (ze - RZ / 2);
+  const bool zact = zr < 64;
+  if (zact && zx < ex && zy < ey) {
+    const bool a = zo >= -R && zo < ez + R, b = zo + 1 < ez + R;
+    if (a || b) {
+      vz = __ldg(reinterpret_cast<const double2*>(base + (zx * sx + zy * sy + zo)));
+      if (!a) vz.x = 0.0;
+      if (!b) vz.y = 0.0;
+    }
+  }
+  unsigned m = max(fx_key(vz.x), fx_key(vz.y));
+#pragma unroll
+  for (int q = 0; q < 4; ++q) m = max(m, max(fx_key(c[q].x), fx_key(c[q].y)));
+#pragma unroll
+  for (int q = 0; q < R; ++q)
+    m = max(m, max(max(fx_key(vx[q].x), fx_key(vx[q].y)), max(fx_key(vy[q].x), fx_key(vy[q].y))));
+  m = block_max(m) | 0x1fffffu;
+  if (fx_in_range(m)) {
+    auto put = [&](int x, int y, int zq, double2 v) {
+      longlong2 a;
+      a.x = fx_align(v.x, m);
+      a.y = fx_align(v.y, m);
+      *reinterpret_cast<longlong2*>(S + L::at(x, y, zq)) = a;
+    };
+#pragma unroll
+    for (int q = 0; q < 4; ++q) put(4 * t.xh + q, t.y, z, c[q]);
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      put(xs[q], t.y, z, vx[q]);
+      put(t.y, ys[q], z, vy[q]);
+    }
+    if (zact) put(zx, zy, zo, vz);
+  }
+  __syncthreads();
+  return m;
+}
+
+// T (mg_fixed.cuh: h^2 L u = T FxUnit 2^(e - kFxBias)) of the thread's 8 cells and their
+// aligned values: do_cell(q, T of the pair, values of the pair) for plane 4 xh + q.
+template <int ORDER, typename F>
+__device__ __forceinline__ void tile_laplacians(const long long* S, F do_pair) {
+  typedef FxTile<ORDER> L;
+  constexpr int R = L::R;
+  const TilePos t = tile_pos();
+  const long long* C = S + L::at(4 * t.xh, t.y, 2 * t.zz);
+  longlong2 w[4 + 2 * R];
+#pragma unroll
+  for (int q = 0; q < 4 + 2 * R; ++q)
+    w[q] = *reinterpret_cast<const longlong2*>(C + (q - R) * L::px);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const long long* c = C + q * L::px;
+    const longlong2 own = w[q + R];
+    // z window: elements -RZ .. RZ + 1
+    long long z[2 * L::RZ + 2];
+#pragma unroll
+    for (int a = 0; a < L::RZ + 1; ++a) {
+      const longlong2 v = 2 * a == L::RZ ? own
+                                         : *reinterpret_cast<const longlong2*>(c + 2 * a - L::RZ);
+      z[2 * a] = v.x;
+      z[2 * a + 1] = v.y;
+    }
+    long long s0[3] = {0, 0, 0}, s1[3] = {0, 0, 0};
+#pragma unroll
+    for (int d = 1; d <= R; ++d) {
+      const longlong2 ym = *reinterpret_cast<const longlong2*>(c - d * L::py);
+      const longlong2 yp = *reinterpret_cast<const longlong2*>(c + d * L::py);
+      s0[d - 1] = (z[L::RZ - d] + z[L::RZ + d]) + (ym.x + yp.x) + (w[q + R - d].x + w[q + R + d].x);
+      s1[d - 1] =
+          (z[L::RZ + 1 - d] + z[L::RZ + 1 + d]) + (ym.y + yp.y) + (w[q + R - d].y + w[q + R + d].y);
+    }
+    longlong2 T;
+    T.x = fx_weighted<ORDER>(s0) + fx_centre<ORDER>(own.x);
+    T.y = fx_weighted<ORDER>(s1) + fx_centre<ORDER>(own.y);
+    do_pair(q, T, own);
+  }
+}
+
+}  // namespace mgk
