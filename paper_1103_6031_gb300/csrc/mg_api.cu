@@ -604,6 +604,14 @@ int n_leaf(const mg_hierarchy* h) { return (int)h->L.size() - h->base; }
 
 // ---- level operations, templated on the V-cycle precision --------------------
 
+// MG_FP64 folds the coarse-fine flux step (mg_ghost.cu).  MG_MIXED keeps it operation by
+// operation in both precisions: its results depend on the last bits of the residual at the
+// 1e-9 level.
+template <typename T>
+bool fold_ghosts(const mg_hierarchy* h) {
+  return std::is_same<T, double>::value && !h->mixed;
+}
+
 template <typename T>
 mg_status tangential(mg_hierarchy* h, int l) {
   DevLevel& L = h->L[l];
@@ -625,7 +633,7 @@ mg_status tangential(mg_hierarchy* h, int l) {
   }
   KL(MG_K_GHOST, L.fs.base[6],
      launch_cf_tangential<T>(h->cfg.order, L.G, P.G, pb.u[pb.cur], L.off, L.fs, h->w,
-                             1.0 / P.geo.h, b.inter, b.fc_unc, h->s));
+                             L.geo.h, 1.0 / P.geo.h, fold_ghosts<T>(h), b.inter, b.fc_unc, h->s));
   return MG_OK;
 }
 
@@ -665,6 +673,17 @@ mg_status ghost_fill(mg_hierarchy* h, int l, bool edges) {
     o.s[4] = float(0.25 * invh * hh / h->w.ghost_coef[1]);
     rec_push(h, o, ceil_div(4 * L.fs.ebase[6], kPersistThreads));
     return MG_OK;
+  }
+  if constexpr (std::is_same<T, double>::value) {
+    if (fold_ghosts<T>(h)) {
+      KL(MG_K_GHOST, 4 * L.fs.ebase[6] * L.G.g,
+         launch_cf_flux_fold(h->cfg.order, L.G, b.u[b.cur], L.fs, h->w, b.inter, b.fc_unc,
+                             L.geo.h, 1.0 / P.geo.h, h->s));
+      if (edges)
+        KL(MG_K_GHOST, shell_of(L.G),
+           launch_cf_edges<T>(h->cfg.order, L.G, b.u[b.cur], P.G, pb.u[pb.cur], L.off, h->w, h->s));
+      return MG_OK;
+    }
   }
   KL(MG_K_GHOST, 4 * L.fs.ebase[6] * L.G.g,
      launch_cf_flux<T>(h->cfg.order, L.G, b.u[b.cur], L.fs, h->w, b.inter, b.fc_unc, L.geo.h,

@@ -114,12 +114,17 @@ template <typename T>
 cudaError_t launch_ghost_periodic(const Grid& G, T* u, cudaStream_t s);
 template <typename T>
 cudaError_t launch_cf_tangential(int order, const Grid& F, const Grid& P, const T* pu, Int3 off,
-                                 const FaceSet& fs, const CfWeights& w, double invH, T* inter,
-                                 T* fc_unc, cudaStream_t s);
+                                 const FaceSet& fs, const CfWeights& w, double h, double invH,
+                                 bool fold, T* inter, T* fc_unc, cudaStream_t s);
 template <typename T>
 cudaError_t launch_cf_flux(int order, const Grid& F, T* u, const FaceSet& fs, const CfWeights& w,
                            const T* inter, const T* fc_unc, double h, double invh, double invH,
                            int flux_fix, cudaStream_t s);
+// float64 after launch_cf_tangential with fold = true (which leaves the parent values'
+// parts of the ghosts and of their shift in inter and fc_unc)
+cudaError_t launch_cf_flux_fold(int order, const Grid& F, double* u, const FaceSet& fs,
+                                const CfWeights& w, const double* inter, const double* fc_unc,
+                                double h, double invH, cudaStream_t s);
 template <typename T>
 cudaError_t launch_cf_edges(int order, const Grid& F, T* u, const Grid& P, const T* pu, Int3 off,
                             const CfWeights& w, cudaStream_t s);

@@ -320,13 +320,12 @@ __device__ __forceinline__ void cf_flux_body(const Grid& F, T* __restrict__ u, c
   constexpr int half = ORDER / 2;
   if (t >= 4 * fs.ebase[6]) return;
   const unsigned quad = __activemask();
-  const long long e = t >> 2;
-  const int col = (int)(t & 3);
+  const int e = (int)(t >> 2), col = (int)(t & 3);
   const int f = face_of(fs, e, fs.ebase);
   const int a = f >> 1, side = f & 1;
   const int nt0 = fs.nt[f][0], nt1 = fs.nt[f][1];
-  const long long loc = e - fs.ebase[f];
-  const int jc = (int)(loc / (nt1 / 2)), kc = (int)(loc % (nt1 / 2));
+  const unsigned loc = (unsigned)(e - (int)fs.ebase[f]), ne1 = nt1 / 2;
+  const int jc = (int)(loc / ne1), kc = (int)(loc % ne1);
   const int tj = 2 * jc + (col >> 1), tk = 2 * kc + (col & 1);
   const long long sx = (long long)F.Y * F.Zp, sy = F.Zp;
   // strides along the normal (a) and the tangential axes (b, c) of this face
