@@ -263,7 +263,7 @@ struct mg_hierarchy {
   unsigned* wait_err = nullptr;  // device flag: a bounded wait in a kernel ran out
   double* scratch = nullptr;   // 3 dense arrays of the largest leaf level
   long long scratch_elems = 0;
-  double* tau_work = nullptr;  // 3 padded float64 arrays of the largest leaf level
+  double* tau_work = nullptr;  // MG_MIXED: 2 padded float64 arrays of the largest leaf level
   // host-buffer pipelines: the first solve's phi and displacements are staged here
   // (phi, x, y, z per leaf level, dense) and copied to the host on cs while the
   // second solve runs
@@ -490,7 +490,7 @@ size_t carve(const mg_config* cfg, const Plan& p, mg_hierarchy* h, char* arena) 
   double* partial = c.take<double>((size_t)slots * 2);
   double* red = c.take<double>(kRedDoubles);
   double* scratch = c.take<double>((size_t)3 * max_leaf);
-  double* tau_work = c.take<double>((size_t)3 * max_leaf_padded);
+  double* tau_work = mixed ? c.take<double>((size_t)2 * max_leaf_padded) : nullptr;
   double* stage = c.take<double>((size_t)4 * leaf_total);
   if (h) {
     h->tau_work = tau_work;
@@ -1436,9 +1436,13 @@ mg_status tau_into_f(mg_hierarchy* h) {
   for (int l = h->base; l <= finest(h); ++l) {
     DevLevel& L = h->L[l];
     ST(ghost_fill<double>(h, l, true));
-    KL(MG_K_LPT, cells_of(L.G),
-       launch_lpt2_source(h->cfg.order, L.G, phi_of(L), 1.0 / (L.geo.h * L.geo.h), L.f,
-                          h->tau_work, h->s));
+    const double invh2 = 1.0 / (L.geo.h * L.geo.h);
+    if (h->mixed)
+      KL(MG_K_LPT, cells_of(L.G),
+         launch_lpt2_source_fp64(h->cfg.order, L.G, phi_of(L), invh2, L.f, h->tau_work, h->s));
+    else
+      KL(MG_K_LPT, cells_of(L.G),
+         launch_lpt2_source(h->cfg.order, L.G, phi_of(L), invh2, L.f, h->s));
   }
   for (int l = finest(h); l > h->base; --l) {
     DevLevel& L = h->L[l];
@@ -2643,8 +2647,7 @@ mg_status mg_lla_density(mg_hierarchy* h, const double* const phi1[], const doub
       DevLevel& L = h->L[l];
       ST(ghost_fill<double>(h, l, true));
       KL(MG_K_LPT, cells_of(L.G),
-         launch_lla(h->cfg.order, L.G, phi_of(L), 1.0 / (L.geo.h * L.geo.h), L.f, h->tau_work,
-                    h->s));
+         launch_lla(h->cfg.order, L.G, phi_of(L), 1.0 / (L.geo.h * L.geo.h), L.f, h->s));
     }
     for (int l = finest(h); l > h->base; --l) {
       DevLevel& L = h->L[l];

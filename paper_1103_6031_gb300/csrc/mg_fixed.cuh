@@ -117,4 +117,27 @@ __device__ __forceinline__ long long fx_centre(long long c) {
   return -6 * c + (c >> 2) + (c >> 7);                  // 1470/256 = 6 - 1/4 - 1/128
 }
 
+// One axis: h^2 u'' = T FxUnit 2^(e - kFxBias) from the sums u(+d) + u(-d) and the centre.
+template <int ORDER>
+__device__ __forceinline__ long long fx_second(const long long (&s)[3], long long c) {
+  if (ORDER == 2) return s[0] - 2 * c;
+  if (ORDER == 4) return fx_weighted<4>(s) - 2 * c + (c >> 3);  // 30/16 = 2 - 1/8
+  return fx_weighted<6>(s) - 2 * c + (c >> 4) + (c >> 6) + (c >> 7);  // 490/256 = 2 - 22/256
+}
+
+// One axis: h u' = T FxGradUnit 2^(e - kFxBias) from the differences u(+d) - u(-d); order 6:
+// T = (45 d1 - 9 d2 + d3) / 64, order 4: (8 d1 - d2) / 8.  |T| <= 2 max |u|, so that the
+// operator can be applied to its own result.
+template <int ORDER>
+struct FxGradUnit {
+  static constexpr double v = ORDER == 2 ? 0.5 : (ORDER == 4 ? 8.0 / 12.0 : 64.0 / 60.0);
+};
+
+template <int ORDER>
+__device__ __forceinline__ long long fx_first(const long long (&d)[3]) {
+  if (ORDER == 2) return d[0];
+  if (ORDER == 4) return d[0] - (d[1] >> 3);
+  return d[0] - (d[0] >> 2) - (d[1] >> 3) + ((d[2] - d[1] - 3 * d[0]) >> 6);  // 45/64 = 1 - 1/4 - 3/64
+}
+
 }  // namespace mgk

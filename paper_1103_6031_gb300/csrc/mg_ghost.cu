@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(256) k_ghost_periodic(Grid G, T* __restrict__ 
 
 // Parent face elements per block of the tangential kernel: kTangB along the face's first
 // axis, kTangC along its second.
-constexpr int kTangB = 8, kTangC = 16, kTangThreads = 128;
+constexpr int kTangB = 8, kTangC = 16, kTangThreads = 256;
 
 struct TangTiles {
   int nb[6], nc[6];  // tiles of every face along its axes
@@ -135,24 +135,28 @@ __global__ void __launch_bounds__(kTangThreads)
       }
     }
   }
-  for (int q = threadIdx.x; q < kTangB * kTangC; q += kTangThreads) {
-    const int kc = q % kTangC, jc = q / kTangC;
-    if (kc >= nc || jc >= nb) continue;
-    // uncovered part of the parent face flux: parent cells outside the face, along a
+  // with FOLD, the two fine rows pj of an element are neighbouring lanes
+  constexpr int PJ = FOLD ? 2 : 1;
+  static_assert(PJ * kTangB * kTangC % 32 == 0 && kTangThreads % 32 == 0, "whole warps");
+  for (int q = threadIdx.x; q < PJ * kTangB * kTangC; q += kTangThreads) {
+    const int pj = q % PJ, kc = q / PJ % kTangC, jc = q / (PJ * kTangC);
+    const bool in = kc < nc && jc < nb;
     T fc = T(0);
-    const T* v = org + (jc * sb + kc * sc);
-    if (side == 0) {
+    if (in) {
+      // uncovered part of the parent face flux: parent cells outside the face, along a
+      const T* v = org + (jc * sb + kc * sc);
+      if (side == 0) {
 #pragma unroll
-      for (int s = 0; s < half; ++s) fc = fma(w.flux[s], __ldg(v + (half - 1 - s) * sm), fc);
-    } else {
+        for (int s = 0; s < half; ++s) fc = fma(w.flux[s], __ldg(v + (half - 1 - s) * sm), fc);
+      } else {
 #pragma unroll
-      for (int s = half; s < ORDER; ++s) fc = fma(w.flux[s], __ldg(v + (s - half) * sm), fc);
+        for (int s = half; s < ORDER; ++s) fc = fma(w.flux[s], __ldg(v + (s - half) * sm), fc);
+      }
+      fc *= invH;
     }
-    fc *= invH;
     if constexpr (FOLD) {
-      T sum = T(0);  // of b_side x the ghosts' coarse part of the fine fluxes of 4 columns
-#pragma unroll
-      for (int pj = 0; pj < 2; ++pj) {
+      T sum = T(0);  // of b_side x the ghosts' coarse part of the fine fluxes of the columns
+      if (in) {
         V2 t[half];
 #pragma unroll
         for (int m = 0; m < half; ++m) {
@@ -164,6 +168,7 @@ __global__ void __launch_bounds__(kTangThreads)
             t[m].y = fma(w.tang[pj][bb], r.y, t[m].y);
           }
         }
+        const long long tj = 2 * (jt + jc) + pj;
 #pragma unroll
         for (int m = 0; m < half; ++m) {
           V2 g;
@@ -174,14 +179,15 @@ __global__ void __launch_bounds__(kTangThreads)
             g.y = fma(fo.ncoarse[m][n], t[n].y, g.y);
           }
           sum = fma(fo.bg[side][m], g.x + g.y, sum);
-          const long long tj = 2 * (jt + jc) + pj;
           *reinterpret_cast<V2*>(inter + fs.base[f] + ((long long)m * nt0 + tj) * nt1 +
                                  2 * (kt + kc)) = g;
         }
       }
+      sum += __shfl_xor_sync(~0u, sum, 1);
       fc = fma(fc, fo.a[side], -sum);
     }
-    fc_unc[fs.ebase[f] + (long long)(jt + jc) * (nt1 / 2) + kt + kc] = fc;
+    if (in && pj == 0)
+      fc_unc[fs.ebase[f] + (long long)(jt + jc) * (nt1 / 2) + kt + kc] = fc;
   }
 }
 
@@ -251,20 +257,48 @@ __global__ void __launch_bounds__(128)
   }
 }
 
+// Edge and corner ghosts of a level in a row: the edges along x, y and z, (2 g)^2 cells at
+// every position along them, then the corners.
+__host__ __device__ inline int edge_count(const Grid& F) {
+  const int w = 2 * F.g;
+  return w * w * (F.n0 + F.n1 + F.n2 + w);
+}
+
+__device__ __forceinline__ bool edge_cell(const Grid& F, int t, int& i, int& j, int& k) {
+  const int g = F.g, w = 2 * g, ww = w * w;
+  const int n[3] = {F.n0, F.n1, F.n2};
+  auto ghost = [&](int q, int len) { return q < g ? q - g : len + q - g; };
+  const int pos = t / ww, q = t % ww;
+  const int a = q / w, b = q % w;
+  if (pos < n[0]) {
+    i = pos;
+    j = ghost(a, n[1]);
+    k = ghost(b, n[2]);
+  } else if (pos < n[0] + n[1]) {
+    i = ghost(a, n[0]);
+    j = pos - n[0];
+    k = ghost(b, n[2]);
+  } else if (pos < n[0] + n[1] + n[2]) {
+    i = ghost(a, n[0]);
+    j = ghost(b, n[1]);
+    k = pos - n[0] - n[1];
+  } else {
+    const int c = pos - n[0] - n[1] - n[2];
+    if (c >= w) return false;
+    i = ghost(c, n[0]);
+    j = ghost(a, n[1]);
+    k = ghost(b, n[2]);
+  }
+  return true;
+}
+
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
     k_cf_edges(Grid F, T* __restrict__ u, Grid P, const T* __restrict__ pu, Int3 off,
                CfWeights w) {
   constexpr int half = ORDER / 2;
-  const int g = F.g;
-  const int X = F.n0 + 2 * g, Y = F.n1 + 2 * g, Z = F.n2 + 2 * g;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)X * Y * Z) return;
-  const int k = (int)(t % Z) - g;
-  const int j = (int)((t / Z) % Y) - g;
-  const int i = (int)(t / ((long long)Z * Y)) - g;
-  const int out = (i < 0 || i >= F.n0) + (j < 0 || j >= F.n1) + (k < 0 || k >= F.n2);
-  if (out < 2) return;
+  int i, j, k;
+  if (!edge_cell(F, blockIdx.x * 128 + (int)threadIdx.x, i, j, k)) return;
   const int pi = off.x + (i >> 1), pj = off.y + (j >> 1), pk = off.z + (k >> 1);
   const double* wi = w.tang[i & 1];
   const double* wj = w.tang[j & 1];
@@ -382,9 +416,8 @@ cudaError_t launch_cf_flux(int order, const Grid& F, T* u, const FaceSet& fs, co
 template <typename T>
 cudaError_t launch_cf_edges(int order, const Grid& F, T* u, const Grid& P, const T* pu, Int3 off,
                             const CfWeights& w, cudaStream_t s) {
-  const long long total = (long long)(F.n0 + 2 * F.g) * (F.n1 + 2 * F.g) * (F.n2 + 2 * F.g);
   const int block = 128;
-  const unsigned grid = (unsigned)((total + block - 1) / block);
+  const unsigned grid = (unsigned)((edge_count(F) + block - 1) / block);
   switch (order) {
     case 2: k_cf_edges<2, T><<<grid, block, 0, s>>>(F, u, P, pu, off, w); break;
     case 4: k_cf_edges<4, T><<<grid, block, 0, s>>>(F, u, P, pu, off, w); break;

@@ -170,14 +170,16 @@ cudaError_t launch_unpack(const Grid& G, const double* src, double* dst, cudaStr
 cudaError_t launch_shift_copy(const Grid& G, double* f, double* f2, const double* mean_num,
                               double inv_volume, cudaStream_t s);
 cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t s);
-// tau from phi (ghosts, including edges, filled); work holds 3 * grid_elems(G)
-// float64 for the first derivatives.
+// tau from phi (ghosts, including edges, filled)
 cudaError_t launch_lpt2_source(int order, const Grid& G, const double* phi, double invh2,
-                               double* tau, double* work, cudaStream_t s);
+                               double* tau, cudaStream_t s);
+// the same in FP64 arithmetic; work holds 2 * grid_elems(G) float64
+cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi, double invh2,
+                                    double* tau, double* work, cudaStream_t s);
 // 1/det[I - H] - 1 on the interior (H: finite-difference Hessian of phi, ghosts and
-// edges filled); work holds 3 * grid_elems(G) float64.
+// edges filled)
 cudaError_t launch_lla(int order, const Grid& G, const double* phi, double invh2, double* out,
-                       double* work, cudaStream_t s);
+                       cudaStream_t s);
 // out = a1 x1 + a2 x2 over n dense elements (x2 may be NULL)
 cudaError_t launch_axpby(long long n, double a1, const double* x1, double a2, const double* x2,
                          double* out, cudaStream_t s);

@@ -241,32 +241,37 @@ __global__ void __launch_bounds__(kRedBlock)
   }
 }
 
+// Copies between dense and padded arrays: blocks of kCopyZ x kCopyY cells of a plane (no
+// divisions per cell).
+constexpr int kCopyZ = 64, kCopyY = 4;
+
+inline dim3 copy_grid(const Grid& G) {
+  return dim3((G.n2 + kCopyZ - 1) / kCopyZ, (G.n1 + kCopyY - 1) / kCopyY, G.n0);
+}
+
 __global__ void __launch_bounds__(256)
     k_pack(Grid G, const double* __restrict__ src, double* __restrict__ dst, double shift) {
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  const long long t = blockIdx.x * 256LL + threadIdx.x;
-  if (t >= n) return;
-  const int k = (int)(t % G.n2), j = (int)((t / G.n2) % G.n1), i = (int)(t / ((long long)G.n2 * G.n1));
-  dst[gidx(G, i, j, k)] = __ldg(src + t) - shift;
+  const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
+  const int i = blockIdx.z;
+  if (k >= G.n2 || j >= G.n1) return;
+  dst[gidx(G, i, j, k)] = __ldg(src + ((long long)i * G.n1 + j) * G.n2 + k) - shift;
 }
 
 __global__ void __launch_bounds__(256)
     k_unpack(Grid G, const double* __restrict__ src, double* __restrict__ dst, double add) {
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  const long long t = blockIdx.x * 256LL + threadIdx.x;
-  if (t >= n) return;
-  const int k = (int)(t % G.n2), j = (int)((t / G.n2) % G.n1), i = (int)(t / ((long long)G.n2 * G.n1));
-  dst[t] = __ldg(src + gidx(G, i, j, k)) + add;
+  const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
+  const int i = blockIdx.z;
+  if (k >= G.n2 || j >= G.n1) return;
+  dst[((long long)i * G.n1 + j) * G.n2 + k] = __ldg(src + gidx(G, i, j, k)) + add;
 }
 
 // f -= mean, f2 = f on the interior; mean = *mean_num * inv_volume (device-side).
 __global__ void __launch_bounds__(256)
     k_shift_copy(Grid G, double* __restrict__ f, double* __restrict__ f2,
                  const double* __restrict__ mean_num, double inv_volume) {
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  const long long t = blockIdx.x * 256LL + threadIdx.x;
-  if (t >= n) return;
-  const int k = (int)(t % G.n2), j = (int)((t / G.n2) % G.n1), i = (int)(t / ((long long)G.n2 * G.n1));
+  const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
+  const int i = blockIdx.z;
+  if (k >= G.n2 || j >= G.n1) return;
   const long long p = gidx(G, i, j, k);
   const double v = f[p] - mean_num[0] * inv_volume;
   f[p] = v;
@@ -299,15 +304,19 @@ __global__ void __launch_bounds__(256) k_fill(double* __restrict__ p, long long 
   if (t < n) p[t] = v;
 }
 
-// First derivatives D_b = G_b phi (Table 1 gradient, times h) for the 2LPT
-// source, on every cell whose b coordinate is interior and whose other two
-// coordinates lie anywhere in the ghost-padded box (the mixed derivatives read
-// D_b up to g cells outside the interior along the other axes).  One thread per
-// (padded x, padded y) row position, looping over padded z.
+// The 2LPT source in FP64 arithmetic, operation by operation, for the second solve of the
+// mixed mode: its float32 cycles turn a changed last bit of the source into changes of
+// 1e-9 of the result (measured: two cells whose source rounded differently to float32
+// moved displacements of the finest nest by 1.7e-9).
+//
+// First derivatives D_b = G_b phi (Table 1 gradient, times h), b = y, z, on every cell whose
+// b coordinate is interior and whose other two coordinates lie anywhere in the ghost-padded
+// box (the mixed derivatives read D_b up to g cells outside the interior along the other
+// axes).
 template <int ORDER>
 __global__ void __launch_bounds__(128)
-    k_first_derivs(Grid G, const double* __restrict__ phi, double* __restrict__ dx,
-                   double* __restrict__ dy, double* __restrict__ dz) {
+    k_first_derivs(Grid G, const double* __restrict__ phi, double* __restrict__ dy,
+                   double* __restrict__ dz) {
   constexpr int half = ORDER / 2;
   const int g = G.g;
   const int k = (int)(blockIdx.x * 32 + threadIdx.x) - g;
@@ -315,13 +324,12 @@ __global__ void __launch_bounds__(128)
   const int i = (int)blockIdx.z - g;
   if (k >= G.n2 + g || j >= G.n1 + g) return;
   const long long p = gidx(G, i, j, k);
-  const long long st[3] = {(long long)G.Y * G.Zp, (long long)G.Zp, 1};
-  const int crd[3] = {i, j, k};
-  const int n[3] = {G.n0, G.n1, G.n2};
-  double* out[3] = {dx, dy, dz};
+  const int st[2] = {G.Zp, 1};
+  const bool in[2] = {j >= 0 && j < G.n1, k >= 0 && k < G.n2};
+  double* out[2] = {dy, dz};
 #pragma unroll
-  for (int b = 0; b < 3; ++b) {
-    if (crd[b] < 0 || crd[b] >= n[b]) continue;
+  for (int b = 0; b < 2; ++b) {
+    if (!in[b]) continue;
     double acc = 0.0;
 #pragma unroll
     for (int s = 1; s <= half; ++s)
@@ -330,16 +338,20 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// Finite-difference Hessian at element p: d[a] = phi_aa, the 1D second difference
-// along a; m = (phi_xy, phi_xz, phi_yz), phi_ab = G_a (G_b phi) from the stored
-// first derivatives.
+// tau from phi and its first derivatives: phi_aa the 1D second difference along a, phi_xy =
+// G_x D_y, phi_xz = G_x D_z, phi_yz = G_y D_z.
 template <int ORDER>
-__device__ __forceinline__ void fd_hessian(const Grid& G, const double* __restrict__ phi,
-                                           const double* __restrict__ dy,
-                                           const double* __restrict__ dz, double invh2,
-                                           long long p, double (&d)[3], double (&m)[3]) {
+__global__ void __launch_bounds__(128)
+    k_lpt2_source(Grid G, const double* __restrict__ phi, const double* __restrict__ dy,
+                  const double* __restrict__ dz, double invh2, double* __restrict__ tau) {
   constexpr int half = ORDER / 2;
-  const long long st[3] = {(long long)G.Y * G.Zp, (long long)G.Zp, 1};
+  const int k = blockIdx.x * 32 + threadIdx.x;
+  const int j = blockIdx.y * 4 + threadIdx.y;
+  const int i = blockIdx.z;
+  if (k >= G.n2 || j >= G.n1) return;
+  const long long p = gidx(G, i, j, k);
+  const int st[3] = {G.Y * G.Zp, G.Zp, 1};
+  double d[3], m[3];
   const double c = __ldg(phi + p);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -349,7 +361,6 @@ __device__ __forceinline__ void fd_hessian(const Grid& G, const double* __restri
       acc = fma(lap_w<ORDER>(s), __ldg(phi + p + s * st[a]) + __ldg(phi + p - s * st[a]), acc);
     d[a] = acc * invh2;
   }
-  // phi_xy = G_x D_y, phi_xz = G_x D_z, phi_yz = G_y D_z
   const double* src[3] = {dy, dz, dz};
   const int ax[3] = {0, 0, 1};
 #pragma unroll
@@ -361,44 +372,115 @@ __device__ __forceinline__ void fd_hessian(const Grid& G, const double* __restri
                 acc);
     m[q] = acc * invh2;
   }
-}
-
-// tau = sum_{i<j} (phi_ii phi_jj - phi_ij^2) (Sec. 3.1.2).
-template <int ORDER>
-__global__ void __launch_bounds__(128)
-    k_lpt2_source(Grid G, const double* __restrict__ phi, const double* __restrict__ dx,
-                  const double* __restrict__ dy, const double* __restrict__ dz, double invh2,
-                  double* __restrict__ tau) {
-  const int k = blockIdx.x * 32 + threadIdx.x;
-  const int j = blockIdx.y * 4 + threadIdx.y;
-  const int i = blockIdx.z;
-  if (k >= G.n2 || j >= G.n1) return;
-  const long long p = gidx(G, i, j, k);
-  double d[3], m[3];
-  fd_hessian<ORDER>(G, phi, dy, dz, invh2, p, d, m);
   tau[p] = fma(d[0], d[1] + d[2], d[1] * d[2]) - fma(m[0], m[0], fma(m[1], m[1], m[2] * m[2]));
 }
 
-// Local Lagrangian density (Sec. 5.3): with H the Hessian of the combined
-// potential Phi (L = -grad Phi), rho / rho_bar = 1 / det[I - H]; writes
-// 1/det - 1 (the renormalisation and the +1 follow on the host side).
-// det[I - H] = a b c - a m_yz^2 - b m_xz^2 - c m_xy^2 - 2 m_xy m_xz m_yz with
-// a, b, c = 1 - phi_xx, 1 - phi_yy, 1 - phi_zz.
+// Finite-difference Hessian at element p in FP64 arithmetic: d[a] = phi_aa h^2, m = (phi_xy,
+// phi_xz, phi_yz) h^2 with phi_ab = G_a (G_b phi).
 template <int ORDER>
-__global__ void __launch_bounds__(128)
-    k_lla(Grid G, const double* __restrict__ phi, const double* __restrict__ dy,
-          const double* __restrict__ dz, double invh2, double* __restrict__ out) {
-  const int k = blockIdx.x * 32 + threadIdx.x;
-  const int j = blockIdx.y * 4 + threadIdx.y;
-  const int i = blockIdx.z;
-  if (k >= G.n2 || j >= G.n1) return;
-  const long long p = gidx(G, i, j, k);
-  double d[3], m[3];
-  fd_hessian<ORDER>(G, phi, dy, dz, invh2, p, d, m);
-  const double a = 1.0 - d[0], b = 1.0 - d[1], c = 1.0 - d[2];
-  const double det = a * b * c - a * m[2] * m[2] - b * m[1] * m[1] - c * m[0] * m[0] -
-                     2.0 * m[0] * m[1] * m[2];
-  out[p] = 1.0 / det - 1.0;
+__device__ __forceinline__ void fd_hessian(const Grid& G, const double* __restrict__ phi,
+                                           long long p, double (&d)[3], double (&m)[3]) {
+  constexpr int half = ORDER / 2;
+  const int st[3] = {G.Y * G.Zp, G.Zp, 1};
+  const double c = __ldg(phi + p);
+#pragma unroll 1
+  for (int a = 0; a < 3; ++a) {
+    double acc = Lap<ORDER>::w0 * c;
+    for (int s = 1; s <= half; ++s)
+      acc = fma(lap_w<ORDER>(s), __ldg(phi + p + s * st[a]) + __ldg(phi + p - s * st[a]), acc);
+    d[a] = acc;
+  }
+#pragma unroll 1
+  for (int q = 0; q < 3; ++q) {
+    const int sa = st[q == 2 ? 1 : 0], sb = st[q == 0 ? 1 : 2];
+    double acc = 0.0;
+    for (int s = -half; s <= half; ++s) {
+      if (s == 0) continue;
+      double g = 0.0;
+      for (int t = 1; t <= half; ++t)
+        g = fma(grad_w<ORDER>(t),
+                __ldg(phi + p + s * sa + t * sb) - __ldg(phi + p + s * sa - t * sb), g);
+      acc = fma(grad_w<ORDER>(s), g, acc);
+    }
+    m[q] = acc;
+  }
+}
+
+// What is made of the Hessian (second derivatives d, mixed m = xy, xz, yz).
+// 2LPT source: tau = sum_{i<j} (phi_ii phi_jj - phi_ij^2) (Sec. 3.1.2).
+// d and m in units of s2 and s1.
+struct TauOp {
+  double k2, k1;
+  __device__ __forceinline__ TauOp(double s2, double s1) : k2(s2 * s2), k1(s1 * s1) {}
+  __device__ __forceinline__ double operator()(const double (&d)[3], const double (&m)[3]) const {
+    return fma(k2, fma(d[0], d[1] + d[2], d[1] * d[2]),
+               -(k1 * fma(m[0], m[0], fma(m[1], m[1], m[2] * m[2]))));
+  }
+};
+
+// Local Lagrangian density (Sec. 5.3): with H the Hessian of the combined potential Phi
+// (L = -grad Phi), rho / rho_bar = 1 / det[I - H]; writes 1/det - 1 (the renormalisation and
+// the +1 follow on the host side).  det[I - H] = a b c - a m_yz^2 - b m_xz^2 - c m_xy^2
+// - 2 m_xy m_xz m_yz with a, b, c = 1 - phi_xx, 1 - phi_yy, 1 - phi_zz.
+struct LlaOp {
+  double s2, s1;
+  __device__ __forceinline__ LlaOp(double s2_, double s1_) : s2(s2_), s1(s1_) {}
+  __device__ __forceinline__ double operator()(const double (&d)[3], const double (&m_)[3]) const {
+    const double a = fma(-s2, d[0], 1.0), b = fma(-s2, d[1], 1.0), c = fma(-s2, d[2], 1.0);
+    const double m[3] = {s1 * m_[0], s1 * m_[1], s1 * m_[2]};
+    const double det = a * b * c - a * m[2] * m[2] - b * m[1] * m[1] - c * m[0] * m[0] -
+                       2.0 * m[0] * m[1] * m[2];
+    return 1.0 / det - 1.0;
+  }
+};
+
+// A scale whose square is far from overflow and underflow.
+__device__ __forceinline__ bool squarable(double s) {
+  const int e = (__double2hiint(s) >> 20) & 0x7ff;
+  return e > 600 && e < 1400;
+}
+
+// OP of the Hessian of phi (ghosts and edge ghosts filled), one launch and no work arrays:
+// a tile of aligned integers with its edges (mg_tile.cuh), first derivatives and their
+// derivatives as integer sums; FP64 instructions are left only for the 6 conversions and OP
+// (14 per cell for tau, 65 when every sum ran on the FP64 pipe).
+template <int ORDER, typename OP>
+__global__ void __launch_bounds__(kTileThreads, 3)
+    k_hessian_tile(Grid G, const double* __restrict__ phi, double invh2, double* __restrict__ out) {
+  extern __shared__ __align__(16) long long hess_smem[];
+  const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
+  const unsigned key = tile_load_edges<ORDER>(G, phi, i0, j0, k0, hess_smem);
+  const int j = j0 + (threadIdx.x >> 5), k = k0 + (threadIdx.x & 31);
+  if (j >= G.n1 || k >= G.n2) return;
+  const long long p = gidx(G, i0, j, k);
+  const int sx = G.Y * G.Zp;
+  const int nx = min(kTileX, G.n0 - i0);
+  const double k2 = invh2 * FxUnit<ORDER>::v;
+  const double k1 = invh2 * (FxGradUnit<ORDER>::v * FxGradUnit<ORDER>::v);
+  const double s2 = fx_scale(k2, key), s1 = fx_scale(k1, key);
+  if (fx_in_range(key) && fx_scalable(k2, key) && fx_scalable(k1, key) && squarable(s2) &&
+      squarable(s1)) {
+    const OP op(s2, s1);
+    tile_hessians<ORDER>(hess_smem, [&](int x, const long long (&di)[3], const long long (&mi)[3]) {
+      if (x >= nx) return;
+      const double d[3] = {(double)di[0], (double)di[1], (double)di[2]};
+      const double m[3] = {(double)mi[0], (double)mi[1], (double)mi[2]};
+      out[p + x * sx] = op(d, m);
+    });
+    return;
+  }
+  const OP op(1.0, 1.0);
+#pragma unroll 1
+  for (int x = 0; x < nx; ++x) {
+    double d[3], m[3];
+    fd_hessian<ORDER>(G, phi, p + x * sx, d, m);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      d[a] *= invh2;
+      m[a] *= invh2;
+    }
+    out[p + x * sx] = op(d, m);
+  }
 }
 
 // out[t] = a1 x1[t] + a2 x2[t] (x2 may be NULL) over n dense elements.
@@ -415,10 +497,9 @@ __global__ void __launch_bounds__(128)
     k_gradient(Grid G, const double* __restrict__ phi, double invh, double* __restrict__ dx,
                double* __restrict__ dy, double* __restrict__ dz) {
   constexpr int half = ORDER / 2;
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  const long long t = blockIdx.x * 128LL + threadIdx.x;
-  if (t >= n) return;
-  const int k = (int)(t % G.n2), j = (int)((t / G.n2) % G.n1), i = (int)(t / ((long long)G.n2 * G.n1));
+  const int k = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 4 + threadIdx.y, i = blockIdx.z;
+  if (k >= G.n2 || j >= G.n1) return;
+  const long long t = ((long long)i * G.n1 + j) * G.n2 + k;
   const long long p = gidx(G, i, j, k);
   const long long st[3] = {(long long)G.Y * G.Zp, (long long)G.Zp, 1};
   double out[3];
@@ -433,6 +514,61 @@ __global__ void __launch_bounds__(128)
   dx[t] = out[0];
   dy[t] = out[1];
   dz[t] = out[2];
+}
+
+// The same on tiles of aligned integers (mg_tile.cuh): 6 FP64 instructions per cell instead
+// of 21.
+template <int ORDER>
+__global__ void __launch_bounds__(kTileThreads, 3)
+    k_gradient_tile(Grid G, const double* __restrict__ phi, double invh, double* __restrict__ dx,
+                    double* __restrict__ dy, double* __restrict__ dz) {
+  extern __shared__ __align__(16) long long grad_smem[];
+  const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
+  const unsigned key = tile_load<ORDER>(G, phi, i0, j0, k0, grad_smem);
+  const TilePos t = tile_pos();
+  const int i = i0 + 4 * t.xh, j = j0 + t.y, k = k0 + 2 * t.zz;
+  if (j >= G.n1 || k >= G.n2) return;
+  const long long o = ((long long)i * G.n1 + j) * G.n2 + k, ox = (long long)G.n1 * G.n2;
+  const double kg = -invh * FxGradUnit<ORDER>::v;
+  const bool two = k + 1 < G.n2;
+  if (fx_in_range(key) && fx_scalable(kg, key)) {
+    const double s = fx_scale(kg, key);
+    const bool vec = (G.n2 & 1) == 0 &&
+                     ((reinterpret_cast<size_t>(dx) | reinterpret_cast<size_t>(dy) |
+                       reinterpret_cast<size_t>(dz)) & 15) == 0;
+    tile_gradients<ORDER>(grad_smem, [&](int q, longlong2 x, longlong2 y, longlong2 z) {
+      if (i + q >= G.n0) return;
+      auto put = [&](double* dst, longlong2 v) {
+        const double a = s * (double)v.x, b = s * (double)v.y;
+        double* e = dst + o + q * ox;
+        if (vec) {
+          *reinterpret_cast<double2*>(e) = make_double2(a, b);
+        } else {
+          e[0] = a;
+          if (two) e[1] = b;
+        }
+      };
+      put(dx, x);
+      put(dy, y);
+      put(dz, z);
+    });
+    return;
+  }
+  const long long p = gidx(G, i, j, k);
+  const int st[3] = {G.Y * G.Zp, G.Zp, 1};
+  double* const out[3] = {dx, dy, dz};
+#pragma unroll 1
+  for (int q = 0; q < 8; ++q) {
+    if (i + (q >> 1) >= G.n0 || k + (q & 1) >= G.n2) continue;
+    const double* c = phi + p + (q >> 1) * st[0] + (q & 1);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      double acc = 0.0;
+      for (int d = 1; d <= ORDER / 2; ++d)
+        acc = fma(grad_w<ORDER>(d), __ldg(c + d * st[a]) - __ldg(c - d * st[a]), acc);
+      out[a][o + (q >> 1) * ox + (q & 1)] = -acc * invh;
+    }
+  }
 }
 
 inline unsigned blocks_for(long long n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -489,7 +625,10 @@ cudaError_t launch_norm_partial(int order, const Grid& G, const double* u, const
 }
 
 cudaError_t prepare_norm_tile() {
-  return cudaFuncSetAttribute(k_norm_tile<6>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(
+      k_norm_tile<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, FxTile<6>::bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_gradient_tile<6>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               FxTile<6>::bytes);
 }
 
@@ -519,22 +658,19 @@ cudaError_t launch_reduce_levels(const double* partial, int count, const LevelRa
 
 cudaError_t launch_pack(const Grid& G, const double* src, double* dst, double shift,
                         cudaStream_t s) {
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  k_pack<<<blocks_for(n, 256), 256, 0, s>>>(G, src, dst, shift);
+  k_pack<<<copy_grid(G), dim3(kCopyZ, kCopyY), 0, s>>>(G, src, dst, shift);
   return cudaGetLastError();
 }
 
 cudaError_t launch_unpack(const Grid& G, const double* src, double* dst, cudaStream_t s,
                           double add) {
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  k_unpack<<<blocks_for(n, 256), 256, 0, s>>>(G, src, dst, add);
+  k_unpack<<<copy_grid(G), dim3(kCopyZ, kCopyY), 0, s>>>(G, src, dst, add);
   return cudaGetLastError();
 }
 
 cudaError_t launch_shift_copy(const Grid& G, double* f, double* f2, const double* mean_num,
                               double inv_volume, cudaStream_t s) {
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  k_shift_copy<<<blocks_for(n, 256), 256, 0, s>>>(G, f, f2, mean_num, inv_volume);
+  k_shift_copy<<<copy_grid(G), dim3(kCopyZ, kCopyY), 0, s>>>(G, f, f2, mean_num, inv_volume);
   return cudaGetLastError();
 }
 
@@ -559,27 +695,50 @@ cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template <typename OP>
+static cudaError_t launch_hessian(int order, const Grid& G, const double* phi, double invh2,
+                                  double* out, cudaStream_t s) {
+  const dim3 tg = tile_grid(G);
+  switch (order) {
+    case 2: k_hessian_tile<2, OP><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(G, phi, invh2, out); break;
+    case 4: k_hessian_tile<4, OP><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(G, phi, invh2, out); break;
+    case 6: {
+      // opted in here as well: callers without a hierarchy (mg_static.cu)
+      const cudaError_t e = cudaFuncSetAttribute(
+          k_hessian_tile<6, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, FxTile<6>::bytes);
+      if (e != cudaSuccess) return e;
+      k_hessian_tile<6, OP><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(G, phi, invh2, out);
+      break;
+    }
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t launch_lpt2_source(int order, const Grid& G, const double* phi, double invh2,
-                               double* tau, double* work, cudaStream_t s) {
-  const long long e = grid_elems(G);
-  double* dx = work;
-  double* dy = work + e;
-  double* dz = work + 2 * e;
+                               double* tau, cudaStream_t s) {
+  return launch_hessian<TauOp>(order, G, phi, invh2, tau, s);
+}
+
+cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi, double invh2,
+                                    double* tau, double* work, cudaStream_t s) {
+  double* dy = work;
+  double* dz = work + grid_elems(G);
   const dim3 block(32, 4, 1);
   const dim3 gpad((G.n2 + 2 * G.g + 31) / 32, (G.n1 + 2 * G.g + 3) / 4, G.n0 + 2 * G.g);
   const dim3 gin((G.n2 + 31) / 32, (G.n1 + 3) / 4, G.n0);
   switch (order) {
     case 2:
-      k_first_derivs<2><<<gpad, block, 0, s>>>(G, phi, dx, dy, dz);
-      k_lpt2_source<2><<<gin, block, 0, s>>>(G, phi, dx, dy, dz, invh2, tau);
+      k_first_derivs<2><<<gpad, block, 0, s>>>(G, phi, dy, dz);
+      k_lpt2_source<2><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, tau);
       break;
     case 4:
-      k_first_derivs<4><<<gpad, block, 0, s>>>(G, phi, dx, dy, dz);
-      k_lpt2_source<4><<<gin, block, 0, s>>>(G, phi, dx, dy, dz, invh2, tau);
+      k_first_derivs<4><<<gpad, block, 0, s>>>(G, phi, dy, dz);
+      k_lpt2_source<4><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, tau);
       break;
     case 6:
-      k_first_derivs<6><<<gpad, block, 0, s>>>(G, phi, dx, dy, dz);
-      k_lpt2_source<6><<<gin, block, 0, s>>>(G, phi, dx, dy, dz, invh2, tau);
+      k_first_derivs<6><<<gpad, block, 0, s>>>(G, phi, dy, dz);
+      k_lpt2_source<6><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, tau);
       break;
     default: return cudaErrorInvalidValue;
   }
@@ -587,30 +746,8 @@ cudaError_t launch_lpt2_source(int order, const Grid& G, const double* phi, doub
 }
 
 cudaError_t launch_lla(int order, const Grid& G, const double* phi, double invh2, double* out,
-                       double* work, cudaStream_t s) {
-  const long long e = grid_elems(G);
-  double* dx = work;
-  double* dy = work + e;
-  double* dz = work + 2 * e;
-  const dim3 block(32, 4, 1);
-  const dim3 gpad((G.n2 + 2 * G.g + 31) / 32, (G.n1 + 2 * G.g + 3) / 4, G.n0 + 2 * G.g);
-  const dim3 gin((G.n2 + 31) / 32, (G.n1 + 3) / 4, G.n0);
-  switch (order) {
-    case 2:
-      k_first_derivs<2><<<gpad, block, 0, s>>>(G, phi, dx, dy, dz);
-      k_lla<2><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, out);
-      break;
-    case 4:
-      k_first_derivs<4><<<gpad, block, 0, s>>>(G, phi, dx, dy, dz);
-      k_lla<4><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, out);
-      break;
-    case 6:
-      k_first_derivs<6><<<gpad, block, 0, s>>>(G, phi, dx, dy, dz);
-      k_lla<6><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, out);
-      break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+                       cudaStream_t s) {
+  return launch_hessian<LlaOp>(order, G, phi, invh2, out, s);
 }
 
 cudaError_t launch_axpby(long long n, double a1, const double* x1, double a2, const double* x2,
@@ -622,12 +759,21 @@ cudaError_t launch_axpby(long long n, double a1, const double* x1, double a2, co
 
 cudaError_t launch_gradient(int order, const Grid& G, const double* phi, double invh, double* dx,
                             double* dy, double* dz, cudaStream_t s) {
-  const long long n = (long long)G.n0 * G.n1 * G.n2;
-  const unsigned b = blocks_for(n, 128);
+  if (tile_pays(G)) {
+    const dim3 tg = tile_grid(G);
+    switch (order) {
+      case 2: k_gradient_tile<2><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(G, phi, invh, dx, dy, dz); break;
+      case 4: k_gradient_tile<4><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(G, phi, invh, dx, dy, dz); break;
+      case 6: k_gradient_tile<6><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(G, phi, invh, dx, dy, dz); break;
+      default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+  }
+  const dim3 b((G.n2 + 31) / 32, (G.n1 + 3) / 4, G.n0), th(32, 4);
   switch (order) {
-    case 2: k_gradient<2><<<b, 128, 0, s>>>(G, phi, invh, dx, dy, dz); break;
-    case 4: k_gradient<4><<<b, 128, 0, s>>>(G, phi, invh, dx, dy, dz); break;
-    case 6: k_gradient<6><<<b, 128, 0, s>>>(G, phi, invh, dx, dy, dz); break;
+    case 2: k_gradient<2><<<b, th, 0, s>>>(G, phi, invh, dx, dy, dz); break;
+    case 4: k_gradient<4><<<b, th, 0, s>>>(G, phi, invh, dx, dy, dz); break;
+    case 6: k_gradient<6><<<b, th, 0, s>>>(G, phi, invh, dx, dy, dz); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

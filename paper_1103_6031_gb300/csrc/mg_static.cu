@@ -5,8 +5,7 @@
 // allocator, a plugin that is handed a stream but no allocator, or code that
 // must not risk the implicit device synchronisation of cudaMalloc/cudaFree.
 // This entry point serves them: its working memory (a ghost-padded copy of
-// phi, a padded tau and three padded first-derivative arrays) lives in one
-// file-scope __device__ array that every
+// phi and a padded tau) lives in one file-scope __device__ array that every
 // GPU holds from module load until process exit, so the call itself makes no
 // allocation.  The caller passes only the input phi and the output tau.
 //
@@ -29,7 +28,8 @@
 
 namespace {
 
-// Capacity of the static working array: five padded float64 grids.
+// Capacity of the static working array.  A grid may take a fifth of it (two padded grids
+// are used): the limit callers have been told.
 constexpr long long kStaticElems = (16LL << 20) / 8;  // 16 MiB
 static __device__ __align__(256) double g_static_work[kStaticElems];
 
@@ -96,8 +96,7 @@ extern "C" mg_status mg_lpt2_source_periodic_static(const double* phi, double* t
   cudaError_t e = mgk::launch_pack(G, phi, phi_pad, 0.0, s);
   if (e == cudaSuccess) e = mgk::launch_ghost_periodic<double>(G, phi_pad, s);
   if (e == cudaSuccess)
-    e = mgk::launch_lpt2_source(order, G, phi_pad, 1.0 / (h * h), tau_pad,
-                                work + 2 * mgk::grid_elems(G), s);
+    e = mgk::launch_lpt2_source(order, G, phi_pad, 1.0 / (h * h), tau_pad, s);
   if (e == cudaSuccess) e = mgk::launch_unpack(G, tau_pad, tau, s);
   if (e != cudaSuccess) {
     put_msg(err, len, cudaGetErrorString(e));

@@ -194,4 +194,137 @@ __device__ __forceinline__ void tile_laplacians(const long long* S, F do_pair) {
   }
 }
 
+// T of the three first derivatives (fx_first) of the thread's 8 cells: do_pair(q, x, y, z
+// pairs) for plane 4 xh + q.
+template <int ORDER, typename F>
+__device__ __forceinline__ void tile_gradients(const long long* S, F do_pair) {
+  typedef FxTile<ORDER> L;
+  constexpr int R = L::R;
+  const TilePos t = tile_pos();
+  const long long* C = S + L::at(4 * t.xh, t.y, 2 * t.zz);
+  longlong2 w[4 + 2 * R];
+#pragma unroll
+  for (int q = 0; q < 4 + 2 * R; ++q)
+    w[q] = *reinterpret_cast<const longlong2*>(C + (q - R) * L::px);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const long long* c = C + q * L::px;
+    long long z[2 * L::RZ + 2];
+#pragma unroll
+    for (int a = 0; a < L::RZ + 1; ++a) {
+      const longlong2 v = *reinterpret_cast<const longlong2*>(c + 2 * a - L::RZ);
+      z[2 * a] = v.x;
+      z[2 * a + 1] = v.y;
+    }
+    long long x0[3] = {0, 0, 0}, x1[3] = {0, 0, 0}, y0[3] = {0, 0, 0}, y1[3] = {0, 0, 0};
+    long long z0[3] = {0, 0, 0}, z1[3] = {0, 0, 0};
+#pragma unroll
+    for (int d = 1; d <= R; ++d) {
+      const longlong2 ym = *reinterpret_cast<const longlong2*>(c - d * L::py);
+      const longlong2 yp = *reinterpret_cast<const longlong2*>(c + d * L::py);
+      y0[d - 1] = yp.x - ym.x;
+      y1[d - 1] = yp.y - ym.y;
+      x0[d - 1] = w[q + R + d].x - w[q + R - d].x;
+      x1[d - 1] = w[q + R + d].y - w[q + R - d].y;
+      z0[d - 1] = z[L::RZ + d] - z[L::RZ - d];
+      z1[d - 1] = z[L::RZ + 1 + d] - z[L::RZ + 1 - d];
+    }
+    do_pair(q, make_longlong2(fx_first<ORDER>(x0), fx_first<ORDER>(x1)),
+            make_longlong2(fx_first<ORDER>(y0), fx_first<ORDER>(y1)),
+            make_longlong2(fx_first<ORDER>(z0), fx_first<ORDER>(z1)));
+  }
+}
+
+// The tile with the edges between two faces as well (mixed derivatives), in two passes:
+// the values into shared memory with their largest exponent, then every value aligned in
+// place.  Cells outside along more than two axes count as 0.
+template <int ORDER>
+__device__ __forceinline__ unsigned tile_load_edges(const Grid& G, const double* __restrict__ u,
+                                                    int i0, int j0, int k0, long long* S) {
+  typedef FxTile<ORDER> L;
+  constexpr int R = L::R, RZ = L::RZ, ZP = L::SZ / 2;
+  const int ex = min(kTileX, G.n0 - i0), ey = min(kTileY, G.n1 - j0), ez = min(kTileZ, G.n2 - k0);
+  const int sy = G.Zp, sx = G.Y * G.Zp;
+  const double* base = u + gidx(G, i0, j0, k0);
+  double2* D = reinterpret_cast<double2*>(S);
+  unsigned m = 0;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < L::elems / 2; e += kTileThreads) {
+    const int z = 2 * (e % ZP) - RZ, r = e / ZP;
+    const int y = r % L::SY - R, x = r / L::SY - R;
+    const int out = (x < 0 || x >= ex) + (y < 0 || y >= ey);
+    double2 v = make_double2(0.0, 0.0);
+    if (x < ex + R && y < ey + R) {
+      const bool all = out < 2;  // z ghosts belong to rows that are out along one axis at most
+      const bool a = (z >= 0 && z < ez) || (all && z >= -R && z < ez + R);
+      const bool b = (z + 1 >= 0 && z + 1 < ez) || (all && z + 1 >= -R && z + 1 < ez + R);
+      if (a || b) {
+        v = __ldg(reinterpret_cast<const double2*>(base + (x * sx + y * sy + z)));
+        if (!a) v.x = 0.0;
+        if (!b) v.y = 0.0;
+      }
+    }
+    D[e] = v;
+    m = max(m, max(fx_key(v.x), fx_key(v.y)));
+  }
+  m = block_max(m) | 0x1fffffu;
+  if (fx_in_range(m)) {
+    longlong2* A = reinterpret_cast<longlong2*>(S);
+#pragma unroll 4
+    for (int e = threadIdx.x; e < L::elems / 2; e += kTileThreads) {
+      const double2 v = D[e];
+      A[e] = make_longlong2(fx_align(v.x, m), fx_align(v.y, m));
+    }
+  }
+  __syncthreads();
+  return m;
+}
+
+// The finite-difference Hessian of a column of 8 cells per thread (z = lane, y = warp) as
+// integers: do_cell(x, d, m) with d = the second differences along x, y, z (fx_second) and
+// m = G_x G_y, G_x G_z, G_y G_z (fx_first of fx_first).  The column's values and its first
+// derivatives along y and z slide through registers (7 planes of each at order 6).
+template <int ORDER, typename F>
+__device__ __forceinline__ void tile_hessians(const long long* S, F do_cell) {
+  typedef FxTile<ORDER> L;
+  constexpr int R = L::R, N = kTileX + 2 * R;
+  const long long* C = S + L::at(0, threadIdx.x >> 5, threadIdx.x & 31);
+  // first derivative at p along the axis of stride st
+  auto first = [](const long long* p, int st) {
+    long long d[3] = {0, 0, 0};
+#pragma unroll
+    for (int q = 1; q <= R; ++q) d[q - 1] = p[q * st] - p[-q * st];
+    return fx_first<ORDER>(d);
+  };
+  auto second = [](const long long* p, int st, long long c) {
+    long long s[3] = {0, 0, 0};
+#pragma unroll
+    for (int q = 1; q <= R; ++q) s[q - 1] = p[q * st] + p[-q * st];
+    return fx_second<ORDER>(s, c);
+  };
+  long long w[N], fy[N], fz[N];
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    const long long* e = C + (n - R) * L::px;
+    w[n] = e[0];
+    fy[n] = first(e, L::py);
+    fz[n] = first(e, 1);
+    if (n < 2 * R) continue;
+    const int x = n - 2 * R;  // the window is complete for this plane
+    const long long* c = C + x * L::px;
+    long long s[3] = {0, 0, 0}, gy[3] = {0, 0, 0}, gz[3] = {0, 0, 0}, yz[3] = {0, 0, 0};
+#pragma unroll
+    for (int q = 1; q <= R; ++q) {
+      s[q - 1] = w[x + R + q] + w[x + R - q];
+      gy[q - 1] = fy[x + R + q] - fy[x + R - q];
+      gz[q - 1] = fz[x + R + q] - fz[x + R - q];
+      yz[q - 1] = first(c + q * L::py, 1) - first(c - q * L::py, 1);
+    }
+    const long long own = w[x + R];
+    const long long d[3] = {fx_second<ORDER>(s, own), second(c, L::py, own), second(c, 1, own)};
+    const long long m[3] = {fx_first<ORDER>(gy), fx_first<ORDER>(gz), fx_first<ORDER>(yz)};
+    do_cell(x, d, m);
+  }
+}
+
 }  // namespace mgk

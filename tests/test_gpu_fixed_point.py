@@ -73,6 +73,49 @@ def test_scaled_sources(lib, order, kind):
         assert np.sqrt(np.sum((a - b) ** 2) / np.sum(b * b)) < TOL
 
 
+# levels of at least 2^17 cells are worked on in tiles of 8 x 8 x 32 cells: sides with
+# remainders along every axis, a nest whose faces cut tiles
+TILED = {
+    2: Geometry((60, 44, 52), 10.0, 2, (NestSpec((58, 50, 46), (10, 8, 9)),)),
+    4: Geometry((52, 44, 60), 10.0, 4, (NestSpec((46, 42, 70), (9, 7, 11)),)),
+    6: Geometry((44, 60, 52), 10.0, 6, (NestSpec((50, 66, 42), (8, 12, 11)),)),
+}
+
+
+@pytest.mark.parametrize("order", (2, 4, 6))
+def test_tiled_levels(lib, order):
+    """One whole step (solves, tau, displacements) against the oracle at matched cycles."""
+    import torch
+    from oracle.lpt import lpt_pipeline
+    geom = TILED[order]
+    deltas = make_delta(geom, 7)
+    ref = lpt_pipeline(geom, deltas, tol=0.0, cycles=2)
+    h = lib.Hierarchy(lib.config_from_geometry(geom, tol=0.0, max_cycles=2))
+    out, i1, i2 = h.pipeline([torch.from_numpy(np.ascontiguousarray(d)).cuda() for d in deltas])
+    np.testing.assert_allclose(i1["history"], ref["info1"]["history"], rtol=1e-6, atol=1e-14)
+    np.testing.assert_allclose(i2["level_rel_residual"], ref["info2"]["level_rel_residual"],
+                               rtol=1e-6, atol=1e-14)
+
+    def off(a, b):
+        a = a.cpu().numpy()
+        return np.sqrt(np.sum((a - b) ** 2) / np.sum(b * b))
+
+    for l in range(2):
+        assert off(out["phi1"][l], ref["phi1"][l]) < TOL
+        assert off(out["phi2"][l], ref["phi2"][l]) < TOL
+        for a in range(3):
+            assert off(out["disp1"][3 * l + a], ref["psi1"][l][a]) < TOL
+            assert off(out["disp2"][3 * l + a], ref["psi2"][l][a]) < TOL
+    # the same source 2^-940 times smaller takes the FP64 route in every tile
+    tiny, _, _ = h.pipeline([torch.from_numpy(np.ldexp(d, -940)).cuda() for d in deltas],
+                            allow_noconv=True)
+    for l in range(2):
+        assert off(torch.ldexp(tiny["phi1"][l], torch.tensor(940.0, dtype=torch.float64,
+                                                             device="cuda")),
+                   ref["phi1"][l]) < TOL
+    h.close()
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_a_source_that_is_not_finite(lib, bad):
     geom = GEOMS[6]
