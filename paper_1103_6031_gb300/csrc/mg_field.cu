@@ -72,23 +72,34 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// F[i][j][m] *= A(|k|) * scale, m < n2/2 + 1 (half spectrum along z).
-__global__ void __launch_bounds__(256)
+// F[i][j][m] *= A(|k|) * scale, m < n2/2 + 1 (half spectrum along z).  A block works on
+// kAmpRows rows j of one plane: the squares of its rows' and threads' frequencies are formed
+// once (their divisions, and those of a flat index, took more of the FP64-bound kernel than
+// the square root and the interpolation of a mode).
+constexpr int kAmpRows = 16, kAmpThreads = 128;
+
+__global__ void __launch_bounds__(kAmpThreads)
     k_apply_amplitude(cufftDoubleComplex* __restrict__ F, int n0, int n1, int n2, double h,
                       const double* __restrict__ amp, int nt, double dk, double scale) {
   const int n2h = n2 / 2 + 1;
-  const long long total = (long long)n0 * n1 * n2h;
   const double tp = 2.0 * 3.14159265358979323846 / h;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int m = (int)(e % n2h);
-    const long long r = e / n2h;
-    const int j = (int)(r % n1);
-    const int i = (int)(r / n1);
+  const int i = blockIdx.z, j0 = blockIdx.y * kAmpRows;
+  __shared__ double fij[kAmpRows];
+  if (threadIdx.x < kAmpRows) {
+    const int j = j0 + (int)threadIdx.x;
     const double fi = (double)(i <= n0 / 2 ? i : i - n0) / n0;
     const double fj = (double)(j <= n1 / 2 ? j : j - n1) / n1;
-    const double fm = (double)m / n2;
-    const double kmag = tp * sqrt(fi * fi + fj * fj + fm * fm);
+    fij[threadIdx.x] = fma(fi, fi, fj * fj);
+  }
+  __syncthreads();
+  const int m = blockIdx.x * kAmpThreads + threadIdx.x;
+  if (m >= n2h) return;
+  const double fm = (double)m / n2;
+  const int rows = min(kAmpRows, n1 - j0);
+  cufftDoubleComplex* e = F + ((long long)i * n1 + j0) * n2h + m;
+#pragma unroll 4
+  for (int r = 0; r < rows; ++r, e += n2h) {
+    const double kmag = tp * sqrt(fma(fm, fm, fij[r]));
     const double t = kmag / dk;
     double a = 0.0;
     if (t <= (double)(nt - 1)) {
@@ -96,11 +107,19 @@ __global__ void __launch_bounds__(256)
       if (it > nt - 2) it = nt - 2;
       a = amp[it] + (t - it) * (amp[it + 1] - amp[it]);
     }
-    if (e == 0) a = 0.0;
+    if ((i | (j0 + r) | m) == 0) a = 0.0;
     a *= scale;
-    F[e].x *= a;
-    F[e].y *= a;
+    cufftDoubleComplex v = *e;
+    v.x *= a;
+    v.y *= a;
+    *e = v;
   }
+}
+
+void launch_amplitude(cufftDoubleComplex* F, int n0, int n1, int n2, double h, const double* amp,
+                      int nt, double dk, double scale, cudaStream_t s) {
+  const dim3 grid((n2 / 2 + kAmpThreads) / kAmpThreads, (n1 + kAmpRows - 1) / kAmpRows, n0);
+  k_apply_amplitude<<<grid, kAmpThreads, 0, s>>>(F, n0, n1, n2, h, amp, nt, dk, scale);
 }
 
 int grid_for(long long work) {
@@ -274,13 +293,11 @@ mg_status convolve_grid(const int N[3], double h, const double* amp, int nt, dou
   }
   mg_status st = MG_OK;
   const double ntot = (double)N[0] * N[1] * N[2];
-  const long long spec = (long long)N[0] * N[1] * (N[2] / 2 + 1);
   if (cufftSetStream(fwd, s) != CUFFT_SUCCESS || cufftSetStream(inv, s) != CUFFT_SUCCESS ||
       cufftExecD2Z(fwd, R, F) != CUFFT_SUCCESS) {
     st = MG_ECUDA;
   } else {
-    k_apply_amplitude<<<grid_for(spec), 256, 0, s>>>(F, N[0], N[1], N[2], h, amp, nt, dk,
-                                                     1.0 / (ntot * h * sqrt(h)));
+    launch_amplitude(F, N[0], N[1], N[2], h, amp, nt, dk, 1.0 / (ntot * h * sqrt(h)), s);
     if (cudaGetLastError() != cudaSuccess || cufftExecZ2D(inv, F, R) != CUFFT_SUCCESS)
       st = MG_ECUDA;
   }
@@ -366,10 +383,8 @@ mg_status mg_field_convolve(mg_field* g, const double* noise, double* delta, voi
     g->err = "forward transform failed";
     return MG_ECUDA;
   }
-  const long long total = (long long)g->n[0] * g->n[1] * (g->n[2] / 2 + 1);
   const double scale = 1.0 / ((double)g->n[0] * g->n[1] * g->n[2]);
-  k_apply_amplitude<<<grid_for(total), 256, 0, s>>>(g->F, g->n[0], g->n[1], g->n[2], g->h,
-                                                     g->amp, g->nt, g->dk, scale);
+  launch_amplitude(g->F, g->n[0], g->n[1], g->n[2], g->h, g->amp, g->nt, g->dk, scale, s);
   if (cudaGetLastError() != cudaSuccess) {
     g->err = "amplitude kernel launch failed";
     return MG_ECUDA;
