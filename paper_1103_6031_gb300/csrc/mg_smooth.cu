@@ -119,17 +119,49 @@ __global__ void __launch_bounds__(256, 4)
   }
 }
 
-// One thread per covered parent cell: r = f - L u at its 8 children,
-// parent u := mean(u), ubar := mean(u), parent f_fas := mean(r) (L ubar added later).
+// r = f - L u at the 8 children of every covered parent cell; parent u := mean(u), ubar :=
+// mean(u), parent f_fas := mean(r) (L ubar added later).  Four threads per parent (threadIdx.y:
+// the child's x and y offset), each with the z-pair of children there: every neighbour row
+// is one 2-element load for two children (17 loads instead of 38 at order 6), and a small
+// level has four times the threads in flight of one thread per parent.  The sums run over
+// the children in residual_restrict_body's order.  Blocks of lz x 4 x (32 / lz), lz lanes
+// along z.
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
     k_residual_restrict(Grid F, const T* __restrict__ u, const T* __restrict__ f, T invh2, Grid P,
                         T* __restrict__ pu, T* __restrict__ pfas, T* __restrict__ ubar, Int3 off,
                         Int3 cn, int parent_periodic) {
-  residual_restrict_body<ORDER, T, Ldg>(F, u, f, invh2, P, pu, pfas, ubar, off, cn,
-                                        parent_periodic,
-                                        Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
-                                            (int)threadIdx.x, (int)threadIdx.y});
+  typedef typename Vec2<T>::type V2;
+  __shared__ T sm[2][8][32];  // u and r by child and parent of the block
+  const int kc = blockIdx.x * blockDim.x + threadIdx.x;
+  const int jc = blockIdx.y * blockDim.z + threadIdx.z;
+  const int ic = blockIdx.z;
+  const int child = threadIdx.y, slot = threadIdx.z * blockDim.x + threadIdx.x;
+  const bool in = kc < cn.z && jc < cn.y;
+  if (in) {
+    const long long p = gidx(F, 2 * ic + (child >> 1), 2 * jc + (child & 1), 2 * kc);
+    T n0[3 * ORDER], n1[3 * ORDER], c0, c1;
+    load_pair_neighbours<ORDER, T>(u, p, F.Zp, F.Y * F.Zp, n0, n1, c0, c1);
+    const V2 fv = __ldg(reinterpret_cast<const V2*>(f + p));
+    sm[0][2 * child][slot] = c0;
+    sm[0][2 * child + 1][slot] = c1;
+    sm[1][2 * child][slot] = add_lap_of<ORDER, T>(n0, c0, -invh2, fv.x);
+    sm[1][2 * child + 1][slot] = add_lap_of<ORDER, T>(n1, c1, -invh2, fv.y);
+  }
+  __syncthreads();
+  if (!in || child > 1) return;
+  T s = T(0);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) s += sm[child][q][slot];
+  s *= T(0.125);
+  const long long q = gidx(P, off.x + ic, off.y + jc, off.z + kc);
+  if (child == 0) {
+    pu[q] = s;
+    if (parent_periodic) write_images<T>(P, pu, off.x + ic, off.y + jc, off.z + kc, s);
+    ubar[((long long)ic * cn.y + jc) * cn.z + kc] = s;
+  } else {
+    pfas[q] = s;
+  }
 }
 
 // The same on tiles of aligned integers (mg_tile.cuh), float64: the mean of a parent's 8
@@ -311,8 +343,9 @@ cudaError_t launch_residual_restrict(int order, const Grid& F, const T* u, const
       return cudaGetLastError();
     }
   }
-  dim3 block(32, 4, 1);
-  dim3 grid = coarse_grid(cn, block);
+  const int lz = cn.z > 16 ? 32 : (cn.z > 8 ? 16 : 8);
+  const dim3 block(lz, 4, 32 / lz);
+  const dim3 grid((cn.z + lz - 1) / lz, (cn.y + 32 / lz - 1) / (32 / lz), cn.x);
   switch (order) {
     case 2: k_residual_restrict<2, T><<<grid, block, 0, s>>>(F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic); break;
     case 4: k_residual_restrict<4, T><<<grid, block, 0, s>>>(F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic); break;

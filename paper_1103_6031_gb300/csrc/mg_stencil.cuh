@@ -57,6 +57,50 @@ __device__ __forceinline__ void load_neighbours(const T* __restrict__ u, long lo
 }
 
 template <typename T>
+struct Vec2;
+template <>
+struct Vec2<double> {
+  typedef double2 type;
+};
+template <>
+struct Vec2<float> {
+  typedef float2 type;
+};
+
+// The neighbours of the z-pair at p (an even cell of its row) and the pair itself, every row
+// by 2-element loads.
+template <int ORDER, typename T, typename LD = Ldg>
+__device__ __forceinline__ void load_pair_neighbours(const T* __restrict__ u, long long p, int sy,
+                                                     int sx, T (&n0)[3 * ORDER],
+                                                     T (&n1)[3 * ORDER], T& c0, T& c1) {
+  typedef typename Vec2<T>::type V2;
+  constexpr int R = ORDER / 2, RZ = (R + 1) / 2 * 2;
+  auto ld2 = [](const T* q) { return LD::ld(reinterpret_cast<const V2*>(q)); };
+  const T* c = u + p;
+  T z[2 * RZ + 2];
+#pragma unroll
+  for (int a = 0; a <= RZ; ++a) {
+    const V2 v = ld2(c + 2 * a - RZ);
+    z[2 * a] = v.x;
+    z[2 * a + 1] = v.y;
+  }
+  c0 = z[RZ];
+  c1 = z[RZ + 1];
+#pragma unroll
+  for (int d = 1; d <= R; ++d) {
+    const V2 ym = ld2(c - d * sy), yp = ld2(c + d * sy);
+    const V2 xm = ld2(c - d * sx), xp = ld2(c + d * sx);
+    const T a[6] = {z[RZ - d], z[RZ + d], ym.x, yp.x, xm.x, xp.x};
+    const T b[6] = {z[RZ + 1 - d], z[RZ + 1 + d], ym.y, yp.y, xm.y, xp.y};
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      n0[6 * (d - 1) + q] = a[q];
+      n1[6 * (d - 1) + q] = b[q];
+    }
+  }
+}
+
+template <typename T>
 __device__ __forceinline__ T sum6(const T* o) {
   return (o[0] + o[1]) + (o[2] + o[3]) + (o[4] + o[5]);
 }
@@ -89,13 +133,11 @@ __device__ __forceinline__ T relax(const T (&nb)[3 * ORDER], T acc) {
   return acc;
 }
 
-// acc + scale h^2 L u at element p, c = u[p].  float64 on the integer pipe as in relax (2
-// FP64 instructions instead of 20; scale * FxUnit is loop-invariant) unless FX is false.
-template <int ORDER, typename T, typename LD = Ldg, bool FX = true>
-__device__ __forceinline__ T add_lap_h2(const T* __restrict__ u, long long p, int sy, int sx, T c,
-                                        T scale, T acc) {
-  T nb[3 * ORDER];
-  load_neighbours<ORDER, T, LD>(u, p, sy, sx, nb);
+// acc + scale h^2 L u from a cell's neighbours and its own value c.  float64 on the integer
+// pipe as in relax (2 FP64 instructions instead of 20; scale * FxUnit is loop-invariant)
+// unless FX is false.
+template <int ORDER, typename T, bool FX = true>
+__device__ __forceinline__ T add_lap_of(const T (&nb)[3 * ORDER], T c, T scale, T acc) {
   if constexpr (sizeof(T) == 8 && FX) {
     const unsigned key = max(neighbour_key<ORDER>(nb), fx_key(c)) | 0x1fffffu;
     const double k = scale * FxUnit<ORDER>::v;
@@ -111,6 +153,15 @@ __device__ __forceinline__ T add_lap_h2(const T* __restrict__ u, long long p, in
   return fma(scale, lu, acc);
 }
 
+// The same at element p, c = u[p].
+template <int ORDER, typename T, typename LD = Ldg, bool FX = true>
+__device__ __forceinline__ T add_lap_h2(const T* __restrict__ u, long long p, int sy, int sx, T c,
+                                        T scale, T acc) {
+  T nb[3 * ORDER];
+  load_neighbours<ORDER, T, LD>(u, p, sy, sx, nb);
+  return add_lap_of<ORDER, T, FX>(nb, c, scale, acc);
+}
+
 // On a periodic level, every ghost cell is the image of one interior cell (all
 // sides are >= g).  Along an axis of n cells with element stride st, index a has
 // an image at a + n when a < g and at a - n when a >= n - g (both when n < 2g);
@@ -122,17 +173,6 @@ struct ImgAxis {
 __device__ __forceinline__ ImgAxis img_axis(int a, int n, int g, long long st) {
   return ImgAxis{a < g ? (long long)n * st : 0, a >= n - g ? -(long long)n * st : 0};
 }
-
-template <typename T>
-struct Vec2;
-template <>
-struct Vec2<double> {
-  typedef double2 type;
-};
-template <>
-struct Vec2<float> {
-  typedef float2 type;
-};
 
 // Writes v to the images of interior cell (i, j, k): every combination of own
 // or image index per axis except own on every axis.  Straight-line predicated
