@@ -18,6 +18,7 @@
 //    only mixed derivatives read, by tensor degree-n interpolation of parent
 //    values.
 #include "mg_internal.h"
+#include "mg_launch.cuh"
 #include "mg_stencil.cuh"
 #include "mg_vbody.cuh"
 
@@ -27,6 +28,7 @@ namespace {
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_ghost_periodic(Grid G, T* __restrict__ u) {
+  grid_wait();
   ghost_periodic_body<T>(G, u, blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
 
@@ -70,6 +72,7 @@ __global__ void __launch_bounds__(kTangThreads)
     k_cf_tangential(Grid F, Grid P, const T* __restrict__ pu, Int3 off, FaceSet fs, TangTiles tt,
                     CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
                     T* __restrict__ fc_unc) {
+  grid_wait();
   constexpr int half = ORDER / 2;
   constexpr int RB = kTangB + ORDER;
   typedef typename Vec2<T>::type V2;
@@ -195,6 +198,7 @@ template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
     k_cf_flux(Grid F, T* __restrict__ u, FaceSet fs, CfW<T> w, const T* __restrict__ inter,
               const T* __restrict__ fc_unc, T fc_scale, T a0, T a1, T b0, T b1, int flux_fix) {
+  grid_wait();
   cf_flux_body<ORDER, T>(F, u, fs, w, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix,
                          blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
@@ -213,6 +217,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(128)
     k_cf_flux_fold(Grid F, double* __restrict__ u, FaceSet fs, FluxFold w,
                    const double* __restrict__ inter, const double* __restrict__ fc_unc) {
+  grid_wait();
   constexpr int half = ORDER / 2;
   const int t = blockIdx.x * 128 + threadIdx.x;
   if (t >= 4 * (int)fs.ebase[6]) return;
@@ -296,6 +301,7 @@ template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
     k_cf_edges(Grid F, T* __restrict__ u, Grid P, const T* __restrict__ pu, Int3 off,
                CfWeights w) {
+  grid_wait();
   constexpr int half = ORDER / 2;
   int i, j, k;
   if (!edge_cell(F, blockIdx.x * 128 + (int)threadIdx.x, i, j, k)) return;
@@ -325,8 +331,7 @@ cudaError_t launch_ghost_periodic(const Grid& G, T* u, cudaStream_t s) {
   const long long X = G.n0 + 2 * g, Y = G.n1 + 2 * g;
   const long long total = X * Y * 2 * g + X * 2 * g * G.n2 + 2 * g * (long long)G.n1 * G.n2;
   const int block = 256;
-  k_ghost_periodic<T><<<(unsigned)((total + block - 1) / block), block, 0, s>>>(G, u);
-  return cudaGetLastError();
+  return launch_dep(k_ghost_periodic<T>, (unsigned)((total + block - 1) / block), block, 0, s, G, u);
 }
 
 template <typename T>
@@ -348,21 +353,19 @@ cudaError_t launch_cf_tangential(int order, const Grid& F, const Grid& P, const 
           fo.bg[sd][m] = 0.25 / w.ghost_coef[sd] * w.flux[sd == 0 ? half - 1 - m : half + m];
       }
       switch (order) {
-        case 2: k_cf_tangential<2, T, true><<<grid, kTangThreads, 0, s>>>(F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc); break;
-        case 4: k_cf_tangential<4, T, true><<<grid, kTangThreads, 0, s>>>(F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc); break;
-        case 6: k_cf_tangential<6, T, true><<<grid, kTangThreads, 0, s>>>(F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc); break;
+        case 2: return launch_dep(k_cf_tangential<2, T, true>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
+        case 4: return launch_dep(k_cf_tangential<4, T, true>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
+        case 6: return launch_dep(k_cf_tangential<6, T, true>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
         default: return cudaErrorInvalidValue;
       }
-      return cudaGetLastError();
     }
   }
   switch (order) {
-    case 2: k_cf_tangential<2, T, false><<<grid, kTangThreads, 0, s>>>(F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc); break;
-    case 4: k_cf_tangential<4, T, false><<<grid, kTangThreads, 0, s>>>(F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc); break;
-    case 6: k_cf_tangential<6, T, false><<<grid, kTangThreads, 0, s>>>(F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc); break;
+    case 2: return launch_dep(k_cf_tangential<2, T, false>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
+    case 4: return launch_dep(k_cf_tangential<4, T, false>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
+    case 6: return launch_dep(k_cf_tangential<6, T, false>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_cf_flux_fold(int order, const Grid& F, double* u, const FaceSet& fs,
@@ -386,12 +389,11 @@ cudaError_t launch_cf_flux_fold(int order, const Grid& F, double* u, const FaceS
   }
   const unsigned grid = (unsigned)((4 * fs.ebase[6] + 127) / 128);
   switch (order) {
-    case 2: k_cf_flux_fold<2><<<grid, 128, 0, s>>>(F, u, fs, fo, inter, fc_unc); break;
-    case 4: k_cf_flux_fold<4><<<grid, 128, 0, s>>>(F, u, fs, fo, inter, fc_unc); break;
-    case 6: k_cf_flux_fold<6><<<grid, 128, 0, s>>>(F, u, fs, fo, inter, fc_unc); break;
+    case 2: return launch_dep(k_cf_flux_fold<2>, grid, 128, 0, s, F, u, fs, fo, inter, fc_unc);
+    case 4: return launch_dep(k_cf_flux_fold<4>, grid, 128, 0, s, F, u, fs, fo, inter, fc_unc);
+    case 6: return launch_dep(k_cf_flux_fold<6>, grid, 128, 0, s, F, u, fs, fo, inter, fc_unc);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -405,12 +407,11 @@ cudaError_t launch_cf_flux(int order, const Grid& F, T* u, const FaceSet& fs, co
   const T b0 = T(0.25 * invh * h / w.ghost_coef[0]), b1 = T(0.25 * invh * h / w.ghost_coef[1]);
   const CfW<T> wt = cf_weights_as<T>(w);
   switch (order) {
-    case 2: k_cf_flux<2, T><<<grid, block, 0, s>>>(F, u, fs, wt, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix); break;
-    case 4: k_cf_flux<4, T><<<grid, block, 0, s>>>(F, u, fs, wt, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix); break;
-    case 6: k_cf_flux<6, T><<<grid, block, 0, s>>>(F, u, fs, wt, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix); break;
+    case 2: return launch_dep(k_cf_flux<2, T>, grid, block, 0, s, F, u, fs, wt, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix);
+    case 4: return launch_dep(k_cf_flux<4, T>, grid, block, 0, s, F, u, fs, wt, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix);
+    case 6: return launch_dep(k_cf_flux<6, T>, grid, block, 0, s, F, u, fs, wt, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -419,12 +420,11 @@ cudaError_t launch_cf_edges(int order, const Grid& F, T* u, const Grid& P, const
   const int block = 128;
   const unsigned grid = (unsigned)((edge_count(F) + block - 1) / block);
   switch (order) {
-    case 2: k_cf_edges<2, T><<<grid, block, 0, s>>>(F, u, P, pu, off, w); break;
-    case 4: k_cf_edges<4, T><<<grid, block, 0, s>>>(F, u, P, pu, off, w); break;
-    case 6: k_cf_edges<6, T><<<grid, block, 0, s>>>(F, u, P, pu, off, w); break;
+    case 2: return launch_dep(k_cf_edges<2, T>, grid, block, 0, s, F, u, P, pu, off, w);
+    case 4: return launch_dep(k_cf_edges<4, T>, grid, block, 0, s, F, u, P, pu, off, w);
+    case 6: return launch_dep(k_cf_edges<6, T>, grid, block, 0, s, F, u, P, pu, off, w);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 #define MGK_GHOST_INSTANTIATE(T)                                                              \

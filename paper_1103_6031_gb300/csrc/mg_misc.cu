@@ -2,6 +2,7 @@
 // caller's dense arrays and the padded level layout, the 2LPT source and the
 // displacement gradient (Hahn & Abel 2011, Sec. 3.1, 3.2).
 #include "mg_internal.h"
+#include "mg_launch.cuh"
 #include "mg_stencil.cuh"
 #include "mg_tile.cuh"
 #include "mg_vbody.cuh"
@@ -49,6 +50,7 @@ template <typename T>
 __global__ void __launch_bounds__(kCoarseBlock)
     k_coarsest(Grid G, const T* __restrict__ f, T* __restrict__ u,
                const double* __restrict__ kern) {
+  grid_wait();
   coarsest_body<T, Ldg>(G, f, u, kern, (int)blockIdx.x, (int)threadIdx.x);
 }
 
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(kRedBlock)
     k_norm_partial(Grid G, const double* __restrict__ u, const double* __restrict__ f,
                    double invh2, double vol, Int3 clo, Int3 chi, double* __restrict__ partial,
                    float* __restrict__ r32) {
+  grid_wait();
   const int sy = G.Zp, sx = G.Y * G.Zp;
   const int i = blockIdx.y;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -124,6 +127,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(kTileThreads, 3)
     k_norm_tile(Grid G, const double* __restrict__ u, const double* __restrict__ f, double invh2,
                 double vol, Int3 clo, Int3 chi, double* __restrict__ partial, int slots) {
+  grid_wait();
   extern __shared__ __align__(16) long long norm_smem[];
   const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
   const int b = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -182,6 +186,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
 __global__ void __launch_bounds__(kRedBlock)
     k_sum_partial(Grid G, const double* __restrict__ f, double vol, Int3 clo, Int3 chi,
                   double* __restrict__ partial) {
+  grid_wait();
   const int i = blockIdx.y;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -205,6 +210,7 @@ __global__ void __launch_bounds__(kRedBlock)
 // Sums `count` consecutive (a, b) pairs in a fixed order into out[0], out[1].
 __global__ void __launch_bounds__(kRedBlock)
     k_reduce_partials(const double* __restrict__ partial, int count, double* __restrict__ out) {
+  grid_wait();
   double a = 0.0, b = 0.0;
   for (int t = threadIdx.x; t < count; t += kRedBlock) {
     a += partial[2 * t];
@@ -223,6 +229,7 @@ __global__ void __launch_bounds__(kRedBlock)
 __global__ void __launch_bounds__(kRedBlock)
     k_reduce_levels(const double* __restrict__ partial, int count, LevelRanges R,
                     double* __restrict__ out, double* __restrict__ out_levels) {
+  grid_wait();
   int lo = 0, hi = count;
   if (blockIdx.x > 0) {
     lo = R.off[blockIdx.x - 1];
@@ -251,6 +258,7 @@ inline dim3 copy_grid(const Grid& G) {
 
 __global__ void __launch_bounds__(256)
     k_pack(Grid G, const double* __restrict__ src, double* __restrict__ dst, double shift) {
+  grid_wait();
   const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
   const int i = blockIdx.z;
   if (k >= G.n2 || j >= G.n1) return;
@@ -259,6 +267,7 @@ __global__ void __launch_bounds__(256)
 
 __global__ void __launch_bounds__(256)
     k_unpack(Grid G, const double* __restrict__ src, double* __restrict__ dst, double add) {
+  grid_wait();
   const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
   const int i = blockIdx.z;
   if (k >= G.n2 || j >= G.n1) return;
@@ -269,6 +278,7 @@ __global__ void __launch_bounds__(256)
 __global__ void __launch_bounds__(256)
     k_shift_copy(Grid G, double* __restrict__ f, double* __restrict__ f2,
                  const double* __restrict__ mean_num, double inv_volume) {
+  grid_wait();
   const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
   const int i = blockIdx.z;
   if (k >= G.n2 || j >= G.n1) return;
@@ -282,6 +292,7 @@ __global__ void __launch_bounds__(256)
 // update their ghost images.  One thread per cell of a (32 x 4)-cell tile row.
 __global__ void __launch_bounds__(128)
     k_add_correction(Grid G, double* __restrict__ u, const float* __restrict__ e, int periodic) {
+  grid_wait();
   const int k = blockIdx.x * 32 + threadIdx.x;
   const int j = blockIdx.y * 4 + threadIdx.y;
   const int i = blockIdx.z;
@@ -295,11 +306,13 @@ __global__ void __launch_bounds__(128)
 // p -= sum[0] * scale over n elements (sum read on the device).
 __global__ void __launch_bounds__(256)
     k_sub_mean(double* __restrict__ p, long long n, const double* __restrict__ sum, double scale) {
+  grid_wait();
   const long long t = blockIdx.x * 256LL + threadIdx.x;
   if (t < n) p[t] -= sum[0] * scale;
 }
 
 __global__ void __launch_bounds__(256) k_fill(double* __restrict__ p, long long n, double v) {
+  grid_wait();
   const long long t = blockIdx.x * 256LL + threadIdx.x;
   if (t < n) p[t] = v;
 }
@@ -317,6 +330,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(128)
     k_first_derivs(Grid G, const double* __restrict__ phi, double* __restrict__ dy,
                    double* __restrict__ dz) {
+  grid_wait();
   constexpr int half = ORDER / 2;
   const int g = G.g;
   const int k = (int)(blockIdx.x * 32 + threadIdx.x) - g;
@@ -344,6 +358,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(128)
     k_lpt2_source(Grid G, const double* __restrict__ phi, const double* __restrict__ dy,
                   const double* __restrict__ dz, double invh2, double* __restrict__ tau) {
+  grid_wait();
   constexpr int half = ORDER / 2;
   const int k = blockIdx.x * 32 + threadIdx.x;
   const int j = blockIdx.y * 4 + threadIdx.y;
@@ -447,6 +462,7 @@ __device__ __forceinline__ bool squarable(double s) {
 template <int ORDER, typename OP>
 __global__ void __launch_bounds__(kTileThreads, 3)
     k_hessian_tile(Grid G, const double* __restrict__ phi, double invh2, double* __restrict__ out) {
+  grid_wait();
   extern __shared__ __align__(16) long long hess_smem[];
   const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
   const unsigned key = tile_load_edges<ORDER>(G, phi, i0, j0, k0, hess_smem);
@@ -496,6 +512,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(128)
     k_gradient(Grid G, const double* __restrict__ phi, double invh, double* __restrict__ dx,
                double* __restrict__ dy, double* __restrict__ dz) {
+  grid_wait();
   constexpr int half = ORDER / 2;
   const int k = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 4 + threadIdx.y, i = blockIdx.z;
   if (k >= G.n2 || j >= G.n1) return;
@@ -522,6 +539,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(kTileThreads, 3)
     k_gradient_tile(Grid G, const double* __restrict__ phi, double invh, double* __restrict__ dx,
                     double* __restrict__ dy, double* __restrict__ dz) {
+  grid_wait();
   extern __shared__ __align__(16) long long grad_smem[];
   const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
   const unsigned key = tile_load<ORDER>(G, phi, i0, j0, k0, grad_smem);
@@ -580,15 +598,13 @@ int norm_blocks(const Grid& G) { return ((G.n1 + 7) / 8) * G.n0; }
 cudaError_t launch_coarsest(const Grid& G, const double* f, double* u, const double* kern,
                             cudaStream_t s) {
   const int n = G.n0 * G.n1 * G.n2;
-  k_coarsest<double><<<n, kCoarseBlock, 0, s>>>(G, f, u, kern);
-  return cudaGetLastError();
+  return launch_dep(k_coarsest<double>, n, kCoarseBlock, 0, s, G, f, u, kern);
 }
 
 cudaError_t launch_coarsest(const Grid& G, const float* f, float* u, const double* kern,
                             cudaStream_t s) {
   const int n = G.n0 * G.n1 * G.n2;
-  k_coarsest<float><<<n, kCoarseBlock, 0, s>>>(G, f, u, kern);
-  return cudaGetLastError();
+  return launch_dep(k_coarsest<float>, n, kCoarseBlock, 0, s, G, f, u, kern);
 }
 
 cudaError_t launch_norm_partial(int order, const Grid& G, const double* u, const double* f,
@@ -599,29 +615,24 @@ cudaError_t launch_norm_partial(int order, const Grid& G, const double* u, const
   const dim3 tg = tile_grid(G);
   if (!r32 && u && tile_pays(G) && (long long)tg.x * tg.y * tg.z <= blocks) {
     switch (order) {
-      case 2: k_norm_tile<2><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(G, u, f, invh2, vol, clo, chi, partial, blocks); break;
-      case 4: k_norm_tile<4><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(G, u, f, invh2, vol, clo, chi, partial, blocks); break;
-      case 6: k_norm_tile<6><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(G, u, f, invh2, vol, clo, chi, partial, blocks); break;
+      case 2: return launch_dep(k_norm_tile<2>, tg, kTileThreads, FxTile<2>::bytes, s, G, u, f, invh2, vol, clo, chi, partial, blocks);
+      case 4: return launch_dep(k_norm_tile<4>, tg, kTileThreads, FxTile<4>::bytes, s, G, u, f, invh2, vol, clo, chi, partial, blocks);
+      case 6: return launch_dep(k_norm_tile<6>, tg, kTileThreads, FxTile<6>::bytes, s, G, u, f, invh2, vol, clo, chi, partial, blocks);
       default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
   }
   switch (order) {
     case 2:
-      if (r32) k_norm_partial<2, true><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
-      else k_norm_partial<2, false><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
-      break;
+      return r32 ? launch_dep(k_norm_partial<2, true>, grid, kRedBlock, 0, s, G, u, f, invh2, vol, clo, chi, partial, r32)
+                 : launch_dep(k_norm_partial<2, false>, grid, kRedBlock, 0, s, G, u, f, invh2, vol, clo, chi, partial, r32);
     case 4:
-      if (r32) k_norm_partial<4, true><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
-      else k_norm_partial<4, false><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
-      break;
+      return r32 ? launch_dep(k_norm_partial<4, true>, grid, kRedBlock, 0, s, G, u, f, invh2, vol, clo, chi, partial, r32)
+                 : launch_dep(k_norm_partial<4, false>, grid, kRedBlock, 0, s, G, u, f, invh2, vol, clo, chi, partial, r32);
     case 6:
-      if (r32) k_norm_partial<6, true><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
-      else k_norm_partial<6, false><<<grid, kRedBlock, 0, s>>>(G, u, f, invh2, vol, clo, chi, partial, r32);
-      break;
+      return r32 ? launch_dep(k_norm_partial<6, true>, grid, kRedBlock, 0, s, G, u, f, invh2, vol, clo, chi, partial, r32)
+                 : launch_dep(k_norm_partial<6, false>, grid, kRedBlock, 0, s, G, u, f, invh2, vol, clo, chi, partial, r32);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t prepare_norm_tile() {
@@ -636,15 +647,13 @@ cudaError_t launch_sum_partial(const Grid& G, const double* f, double vol, Int3 
                                double* partial, int blocks, cudaStream_t s) {
   const dim3 grid((G.n1 + 7) / 8, G.n0);
   if ((int)(grid.x * grid.y) != blocks) return cudaErrorInvalidValue;
-  k_sum_partial<<<grid, kRedBlock, 0, s>>>(G, f, vol, clo, chi, partial);
-  return cudaGetLastError();
+  return launch_dep(k_sum_partial, grid, kRedBlock, 0, s, G, f, vol, clo, chi, partial);
 }
 
 cudaError_t launch_reduce_partials(const double* partial, int count, int width, double* out,
                                    cudaStream_t s) {
   (void)width;
-  k_reduce_partials<<<1, kRedBlock, 0, s>>>(partial, count, out);
-  return cudaGetLastError();
+  return launch_dep(k_reduce_partials, 1, kRedBlock, 0, s, partial, count, out);
 }
 
 cudaError_t launch_reduce_levels(const double* partial, int count, const LevelRanges& R,
@@ -652,47 +661,40 @@ cudaError_t launch_reduce_levels(const double* partial, int count, const LevelRa
   if (R.n < 0 || R.n > MG_MAX_LEVELS) return cudaErrorInvalidValue;
   for (int l = 0; l < R.n; ++l)
     if (R.off[l] < 0 || R.cnt[l] < 0 || R.off[l] + R.cnt[l] > count) return cudaErrorInvalidValue;
-  k_reduce_levels<<<1 + R.n, kRedBlock, 0, s>>>(partial, count, R, out, out_levels);
-  return cudaGetLastError();
+  return launch_dep(k_reduce_levels, 1 + R.n, kRedBlock, 0, s, partial, count, R, out, out_levels);
 }
 
 cudaError_t launch_pack(const Grid& G, const double* src, double* dst, double shift,
                         cudaStream_t s) {
-  k_pack<<<copy_grid(G), dim3(kCopyZ, kCopyY), 0, s>>>(G, src, dst, shift);
-  return cudaGetLastError();
+  return launch_dep(k_pack, copy_grid(G), dim3(kCopyZ, kCopyY), 0, s, G, src, dst, shift);
 }
 
 cudaError_t launch_unpack(const Grid& G, const double* src, double* dst, cudaStream_t s,
                           double add) {
-  k_unpack<<<copy_grid(G), dim3(kCopyZ, kCopyY), 0, s>>>(G, src, dst, add);
-  return cudaGetLastError();
+  return launch_dep(k_unpack, copy_grid(G), dim3(kCopyZ, kCopyY), 0, s, G, src, dst, add);
 }
 
 cudaError_t launch_shift_copy(const Grid& G, double* f, double* f2, const double* mean_num,
                               double inv_volume, cudaStream_t s) {
-  k_shift_copy<<<copy_grid(G), dim3(kCopyZ, kCopyY), 0, s>>>(G, f, f2, mean_num, inv_volume);
-  return cudaGetLastError();
+  return launch_dep(k_shift_copy, copy_grid(G), dim3(kCopyZ, kCopyY), 0, s, G, f, f2, mean_num, inv_volume);
 }
 
 cudaError_t launch_add_correction(const Grid& G, double* u, const float* e, int periodic,
                                   cudaStream_t s) {
   dim3 block(32, 4, 1);
   dim3 grid((G.n2 + 31) / 32, (G.n1 + 3) / 4, G.n0);
-  k_add_correction<<<grid, block, 0, s>>>(G, u, e, periodic);
-  return cudaGetLastError();
+  return launch_dep(k_add_correction, grid, block, 0, s, G, u, e, periodic);
 }
 
 cudaError_t launch_sub_mean(double* p, long long n, const double* sum, double scale,
                             cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_sub_mean<<<blocks_for(n, 256), 256, 0, s>>>(p, n, sum, scale);
-  return cudaGetLastError();
+  return launch_dep(k_sub_mean, blocks_for(n, 256), 256, 0, s, p, n, sum, scale);
 }
 
 cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_fill<<<blocks_for(n, 256), 256, 0, s>>>(p, n, v);
-  return cudaGetLastError();
+  return launch_dep(k_fill, blocks_for(n, 256), 256, 0, s, p, n, v);
 }
 
 template <typename OP>
@@ -700,19 +702,17 @@ static cudaError_t launch_hessian(int order, const Grid& G, const double* phi, d
                                   double* out, cudaStream_t s) {
   const dim3 tg = tile_grid(G);
   switch (order) {
-    case 2: k_hessian_tile<2, OP><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(G, phi, invh2, out); break;
-    case 4: k_hessian_tile<4, OP><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(G, phi, invh2, out); break;
+    case 2: return launch_dep(k_hessian_tile<2, OP>, tg, kTileThreads, FxTile<2>::bytes, s, G, phi, invh2, out);
+    case 4: return launch_dep(k_hessian_tile<4, OP>, tg, kTileThreads, FxTile<4>::bytes, s, G, phi, invh2, out);
     case 6: {
       // opted in here as well: callers without a hierarchy (mg_static.cu)
       const cudaError_t e = cudaFuncSetAttribute(
           k_hessian_tile<6, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, FxTile<6>::bytes);
       if (e != cudaSuccess) return e;
-      k_hessian_tile<6, OP><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(G, phi, invh2, out);
-      break;
+      return launch_dep(k_hessian_tile<6, OP>, tg, kTileThreads, FxTile<6>::bytes, s, G, phi, invh2, out);
     }
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_lpt2_source(int order, const Grid& G, const double* phi, double invh2,
@@ -727,22 +727,19 @@ cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi,
   const dim3 block(32, 4, 1);
   const dim3 gpad((G.n2 + 2 * G.g + 31) / 32, (G.n1 + 2 * G.g + 3) / 4, G.n0 + 2 * G.g);
   const dim3 gin((G.n2 + 31) / 32, (G.n1 + 3) / 4, G.n0);
+  cudaError_t e = cudaErrorInvalidValue;
   switch (order) {
     case 2:
-      k_first_derivs<2><<<gpad, block, 0, s>>>(G, phi, dy, dz);
-      k_lpt2_source<2><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, tau);
-      break;
+      e = launch_dep(k_first_derivs<2>, gpad, block, 0, s, G, phi, dy, dz);
+      return e != cudaSuccess ? e : launch_dep(k_lpt2_source<2>, gin, block, 0, s, G, phi, dy, dz, invh2, tau);
     case 4:
-      k_first_derivs<4><<<gpad, block, 0, s>>>(G, phi, dy, dz);
-      k_lpt2_source<4><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, tau);
-      break;
+      e = launch_dep(k_first_derivs<4>, gpad, block, 0, s, G, phi, dy, dz);
+      return e != cudaSuccess ? e : launch_dep(k_lpt2_source<4>, gin, block, 0, s, G, phi, dy, dz, invh2, tau);
     case 6:
-      k_first_derivs<6><<<gpad, block, 0, s>>>(G, phi, dy, dz);
-      k_lpt2_source<6><<<gin, block, 0, s>>>(G, phi, dy, dz, invh2, tau);
-      break;
-    default: return cudaErrorInvalidValue;
+      e = launch_dep(k_first_derivs<6>, gpad, block, 0, s, G, phi, dy, dz);
+      return e != cudaSuccess ? e : launch_dep(k_lpt2_source<6>, gin, block, 0, s, G, phi, dy, dz, invh2, tau);
+    default: return e;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_lla(int order, const Grid& G, const double* phi, double invh2, double* out,
@@ -762,21 +759,19 @@ cudaError_t launch_gradient(int order, const Grid& G, const double* phi, double 
   if (tile_pays(G)) {
     const dim3 tg = tile_grid(G);
     switch (order) {
-      case 2: k_gradient_tile<2><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(G, phi, invh, dx, dy, dz); break;
-      case 4: k_gradient_tile<4><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(G, phi, invh, dx, dy, dz); break;
-      case 6: k_gradient_tile<6><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(G, phi, invh, dx, dy, dz); break;
+      case 2: return launch_dep(k_gradient_tile<2>, tg, kTileThreads, FxTile<2>::bytes, s, G, phi, invh, dx, dy, dz);
+      case 4: return launch_dep(k_gradient_tile<4>, tg, kTileThreads, FxTile<4>::bytes, s, G, phi, invh, dx, dy, dz);
+      case 6: return launch_dep(k_gradient_tile<6>, tg, kTileThreads, FxTile<6>::bytes, s, G, phi, invh, dx, dy, dz);
       default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
   }
   const dim3 b((G.n2 + 31) / 32, (G.n1 + 3) / 4, G.n0), th(32, 4);
   switch (order) {
-    case 2: k_gradient<2><<<b, th, 0, s>>>(G, phi, invh, dx, dy, dz); break;
-    case 4: k_gradient<4><<<b, th, 0, s>>>(G, phi, invh, dx, dy, dz); break;
-    case 6: k_gradient<6><<<b, th, 0, s>>>(G, phi, invh, dx, dy, dz); break;
+    case 2: return launch_dep(k_gradient<2>, b, th, 0, s, G, phi, invh, dx, dy, dz);
+    case 4: return launch_dep(k_gradient<4>, b, th, 0, s, G, phi, invh, dx, dy, dz);
+    case 6: return launch_dep(k_gradient<6>, b, th, 0, s, G, phi, invh, dx, dy, dz);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace mgk

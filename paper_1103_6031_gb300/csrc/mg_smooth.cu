@@ -9,6 +9,7 @@
 // interior cell of `uout` (colour c updated, the other colour copied), so no
 // thread ever reads a value another thread of the same launch writes.
 #include "mg_internal.h"
+#include "mg_launch.cuh"
 #include "mg_stencil.cuh"
 #include "mg_tile.cuh"
 #include "mg_vbody.cuh"
@@ -31,6 +32,7 @@ template <int ORDER, typename T>
 __global__ void __launch_bounds__(kPairX * 8, (smooth_min_blocks<ORDER, T>))
     k_smooth_half(Grid G, const T* __restrict__ uin, T* __restrict__ uout,
                   const T* __restrict__ f, T a_f, int colour, int periodic) {
+  grid_wait();
   smooth_half_body<ORDER, T, Ldg>(G, uin, uout, f, a_f, colour, periodic, (int)blockDim.y,
                                   Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
                                       (int)threadIdx.x, (int)threadIdx.y});
@@ -52,6 +54,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(256, 4)
     k_smooth_quad(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
                   const float* __restrict__ f, float a_f, int colour, int periodic) {
+  grid_wait();
   constexpr int R = ORDER / 2;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -131,6 +134,7 @@ __global__ void __launch_bounds__(128)
     k_residual_restrict(Grid F, const T* __restrict__ u, const T* __restrict__ f, T invh2, Grid P,
                         T* __restrict__ pu, T* __restrict__ pfas, T* __restrict__ ubar, Int3 off,
                         Int3 cn, int parent_periodic) {
+  grid_wait();
   typedef typename Vec2<T>::type V2;
   __shared__ T sm[2][8][32];  // u and r by child and parent of the block
   const int kc = blockIdx.x * blockDim.x + threadIdx.x;
@@ -175,6 +179,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
                              double invh2, Grid P, double* __restrict__ pu,
                              double* __restrict__ pfas, double* __restrict__ ubar, Int3 off, Int3 cn,
                              int parent_periodic) {
+  grid_wait();
   extern __shared__ __align__(16) long long tile_smem[];
   const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
   const unsigned key = tile_load<ORDER>(F, u, i0, j0, k0, tile_smem);
@@ -245,6 +250,7 @@ template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
     k_fas_source(Grid P, const T* __restrict__ pu, T* __restrict__ pfas, T invH2, Int3 off,
                  Int3 cn) {
+  grid_wait();
   fas_source_body<ORDER, T, Ldg>(P, pu, pfas, invH2, off, cn,
                                  Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
                                      (int)threadIdx.x, (int)threadIdx.y});
@@ -255,6 +261,7 @@ template <typename T>
 __global__ void __launch_bounds__(128)
     k_prolong(Grid F, T* __restrict__ u, Grid P, const T* __restrict__ pu,
               const T* __restrict__ ubar, Int3 off, Int3 cn, int periodic) {
+  grid_wait();
   prolong_body<T, Ldg>(F, u, P, pu, ubar, off, cn, periodic,
                        Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x,
                            (int)threadIdx.y});
@@ -264,6 +271,7 @@ __global__ void __launch_bounds__(128)
 template <typename T>
 __global__ void __launch_bounds__(128)
     k_restrict_u(Grid F, const T* __restrict__ u, Grid P, T* __restrict__ pu, Int3 off, Int3 cn) {
+  grid_wait();
   const int kc = blockIdx.x * blockDim.x + threadIdx.x;
   const int jc = blockIdx.y * blockDim.y + threadIdx.y;
   const int ic = blockIdx.z;
@@ -298,12 +306,11 @@ cudaError_t launch_smooth_quad(int order, const Grid& G, const float* uin, float
   dim3 block(qx, by, 1);
   dim3 grid((quads + qx - 1) / qx, (G.n1 + by - 1) / by, G.n0);
   switch (order) {
-    case 2: k_smooth_quad<2><<<grid, block, 0, s>>>(G, uin, uout, f, float(a_f), colour, periodic); break;
-    case 4: k_smooth_quad<4><<<grid, block, 0, s>>>(G, uin, uout, f, float(a_f), colour, periodic); break;
-    case 6: k_smooth_quad<6><<<grid, block, 0, s>>>(G, uin, uout, f, float(a_f), colour, periodic); break;
+    case 2: return launch_dep(k_smooth_quad<2>, grid, block, 0, s, G, uin, uout, f, float(a_f), colour, periodic);
+    case 4: return launch_dep(k_smooth_quad<4>, grid, block, 0, s, G, uin, uout, f, float(a_f), colour, periodic);
+    case 6: return launch_dep(k_smooth_quad<6>, grid, block, 0, s, G, uin, uout, f, float(a_f), colour, periodic);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -319,12 +326,11 @@ cudaError_t launch_smooth_half(int order, const Grid& G, const T* uin, T* uout, 
   const int pairs = (G.n2 + 1) / 2;
   dim3 grid((pairs + kPairX - 1) / kPairX, (G.n1 + rows - 1) / rows, G.n0);
   switch (order) {
-    case 2: k_smooth_half<2, T><<<grid, block, 0, s>>>(G, uin, uout, f, T(a_f), colour, periodic); break;
-    case 4: k_smooth_half<4, T><<<grid, block, 0, s>>>(G, uin, uout, f, T(a_f), colour, periodic); break;
-    case 6: k_smooth_half<6, T><<<grid, block, 0, s>>>(G, uin, uout, f, T(a_f), colour, periodic); break;
+    case 2: return launch_dep(k_smooth_half<2, T>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
+    case 4: return launch_dep(k_smooth_half<4, T>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
+    case 6: return launch_dep(k_smooth_half<6, T>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -335,24 +341,22 @@ cudaError_t launch_residual_restrict(int order, const Grid& F, const T* u, const
     if (tile_pays(F)) {
       const dim3 tg = tile_grid(F);
       switch (order) {
-        case 2: k_residual_restrict_tile<2><<<tg, kTileThreads, FxTile<2>::bytes, s>>>(F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic); break;
-        case 4: k_residual_restrict_tile<4><<<tg, kTileThreads, FxTile<4>::bytes, s>>>(F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic); break;
-        case 6: k_residual_restrict_tile<6><<<tg, kTileThreads, FxTile<6>::bytes, s>>>(F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic); break;
+        case 2: return launch_dep(k_residual_restrict_tile<2>, tg, kTileThreads, FxTile<2>::bytes, s, F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic);
+        case 4: return launch_dep(k_residual_restrict_tile<4>, tg, kTileThreads, FxTile<4>::bytes, s, F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic);
+        case 6: return launch_dep(k_residual_restrict_tile<6>, tg, kTileThreads, FxTile<6>::bytes, s, F, u, f, invh2, P, pu, pfas, ubar, off, cn, parent_periodic);
         default: return cudaErrorInvalidValue;
       }
-      return cudaGetLastError();
     }
   }
   const int lz = cn.z > 16 ? 32 : (cn.z > 8 ? 16 : 8);
   const dim3 block(lz, 4, 32 / lz);
   const dim3 grid((cn.z + lz - 1) / lz, (cn.y + 32 / lz - 1) / (32 / lz), cn.x);
   switch (order) {
-    case 2: k_residual_restrict<2, T><<<grid, block, 0, s>>>(F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic); break;
-    case 4: k_residual_restrict<4, T><<<grid, block, 0, s>>>(F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic); break;
-    case 6: k_residual_restrict<6, T><<<grid, block, 0, s>>>(F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic); break;
+    case 2: return launch_dep(k_residual_restrict<2, T>, grid, block, 0, s, F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic);
+    case 4: return launch_dep(k_residual_restrict<4, T>, grid, block, 0, s, F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic);
+    case 6: return launch_dep(k_residual_restrict<6, T>, grid, block, 0, s, F, u, f, T(invh2), P, pu, pfas, ubar, off, cn, parent_periodic);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -361,12 +365,11 @@ cudaError_t launch_fas_source(int order, const Grid& P, const T* pu, T* pfas, do
   dim3 block(32, 4, 1);
   dim3 grid = coarse_grid(cn, block);
   switch (order) {
-    case 2: k_fas_source<2, T><<<grid, block, 0, s>>>(P, pu, pfas, T(invH2), off, cn); break;
-    case 4: k_fas_source<4, T><<<grid, block, 0, s>>>(P, pu, pfas, T(invH2), off, cn); break;
-    case 6: k_fas_source<6, T><<<grid, block, 0, s>>>(P, pu, pfas, T(invH2), off, cn); break;
+    case 2: return launch_dep(k_fas_source<2, T>, grid, block, 0, s, P, pu, pfas, T(invH2), off, cn);
+    case 4: return launch_dep(k_fas_source<4, T>, grid, block, 0, s, P, pu, pfas, T(invH2), off, cn);
+    case 6: return launch_dep(k_fas_source<6, T>, grid, block, 0, s, P, pu, pfas, T(invH2), off, cn);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <typename T>
@@ -375,8 +378,7 @@ cudaError_t launch_prolong(const Grid& F, T* u, const Grid& P, const T* pu, cons
   dim3 block(32, 4, 1);
   const int pairs = F.n2 / 2;
   dim3 grid((pairs + 31) / 32, (F.n1 + 3) / 4, F.n0);
-  k_prolong<T><<<grid, block, 0, s>>>(F, u, P, pu, ubar, off, cn, periodic);
-  return cudaGetLastError();
+  return launch_dep(k_prolong<T>, grid, block, 0, s, F, u, P, pu, ubar, off, cn, periodic);
 }
 
 template <typename T>
@@ -384,8 +386,7 @@ cudaError_t launch_restrict_u(const Grid& F, const T* u, const Grid& P, T* pu, I
                               cudaStream_t s) {
   dim3 block(32, 4, 1);
   dim3 grid = coarse_grid(cn, block);
-  k_restrict_u<T><<<grid, block, 0, s>>>(F, u, P, pu, off, cn);
-  return cudaGetLastError();
+  return launch_dep(k_restrict_u<T>, grid, block, 0, s, F, u, P, pu, off, cn);
 }
 
 cudaError_t prepare_restrict_tile() {
