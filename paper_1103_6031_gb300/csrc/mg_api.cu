@@ -47,6 +47,10 @@ struct Bufs {
   // Periodic levels: every kernel that writes u also writes its ghost images,
   // so ghosts are refilled only after u is loaded from outside.
   bool ghosts_stale = true;
+  // Nests: the coarse-fine ghosts in u[cur] belong to its values and to the cached parent
+  // interpolants (left by a half-sweep that wrote them).  Restriction into the cells that a
+  // child covers does not touch the order layers they depend on (the validated margin).
+  bool ghosts_ready = false;
   // TMA-staged smoother: tensor maps of u[0], u[1] and ffas
   bool tma = false;
   CUtensorMap tm[2];
@@ -246,6 +250,9 @@ struct mg_hierarchy {
   int inner_now = 0;  // MG_MIXED: float32 V-cycles of the next outer iteration
   Graph* capturing = nullptr;     // graph being captured
   Graph* replayed = nullptr;      // graph whose event pairs await reading
+  // set while a batch captures this member's branch next to many others: the branches
+  // share the GPU, so that work counts and a launch's latency does not
+  bool crowded = false;
   // when set, the float32 level operations are appended here (a work list for the
   // persistent batch kernel) instead of being launched; the host-side state (buffer
   // parities, stale flags) advances exactly as for launches
@@ -618,6 +625,7 @@ mg_status tangential(mg_hierarchy* h, int l) {
   DevLevel& P = h->L[l - 1];
   Bufs<T>& b = bufs<T>(L);
   Bufs<T>& pb = bufs<T>(P);
+  b.ghosts_ready = false;
   if (recording<T>(h)) {
     POp o = pop(P_TANG);
     o.F = L.G;
@@ -655,6 +663,7 @@ mg_status ghost_fill(mg_hierarchy* h, int l, bool edges) {
     b.ghosts_stale = false;
     return MG_OK;
   }
+  if (b.ghosts_ready && !edges) return MG_OK;
   DevLevel& P = h->L[l - 1];
   Bufs<T>& pb = bufs<T>(P);
   if (recording<T>(h) && !edges) {
@@ -716,6 +725,16 @@ mg_status half_sweep(mg_hierarchy* h, int l, int colour) {
     b.cur ^= 1;
     return MG_OK;
   }
+  if (!L.periodic && !b.tma && !h->crowded && cells_of(L.G) <= kFaceFusedMaxCells) {
+    KL(MG_K_SMOOTH, (cells_of(L.G) + 1) / 2,
+       launch_smooth_faces<T>(h->cfg.order, L.G, b.u[b.cur], b.u[1 - b.cur], b.ffas, a_f, colour,
+                              !(h->cfg.flags & MG_FLAG_PAIR_SMOOTHER), L.fs, h->w, b.inter,
+                              b.fc_unc, L.geo.h, 1.0 / h->L[l - 1].geo.h, h->s));
+    b.cur ^= 1;
+    b.ghosts_ready = true;
+    return MG_OK;
+  }
+  b.ghosts_ready = false;
   if (b.tma)
     KL(MG_K_SMOOTH, (cells_of(L.G) + 1) / 2,
        launch_smooth_half_tma<T>(h->cfg.order, L.G, &b.tm[b.cur], &b.tm_f, b.u[1 - b.cur], a_f,
@@ -808,6 +827,7 @@ mg_status vcycle(mg_hierarchy* h, int l) {
                           L.cn, h->s));
   ST(vcycle<T>(h, l - 1));
   if (!L.periodic) ST(tangential<T>(h, l));
+  b.ghosts_ready = false;
   KL(MG_K_PROLONG, cells_of(L.G),
      launch_prolong<T>(L.G, b.u[b.cur], P.G, pb.u[pb.cur], b.ubar, L.off, L.cn,
                        L.periodic ? 1 : 0, h->s));
@@ -830,8 +850,15 @@ mg_status zero_state(mg_hierarchy* h, int from_level) {
       if (b.u[q]) ST(fill_zero(h, b.u[q], e));
     b.cur = 0;
     b.ghosts_stale = false;
+    b.ghosts_ready = false;
   }
   return MG_OK;
+}
+
+// At the start of a captured body: its replays may follow anything.
+template <typename T>
+void forget_ghosts(mg_hierarchy* h) {
+  for (DevLevel& L : h->L) bufs<T>(L).ghosts_ready = false;
 }
 
 // ---- float64 leaf state: sync, norms, residual -------------------------------
@@ -978,6 +1005,7 @@ mg_status run_body(mg_hierarchy* h, bool timed, Body body) {
 }
 
 mg_status fp64_cycle_body(mg_hierarchy* h) {
+  forget_ghosts<double>(h);
   ST(vcycle<double>(h, finest(h)));
   return norm_launches(h);
 }
@@ -1002,6 +1030,7 @@ mg_status zero_correction(mg_hierarchy* h) {
     DevLevel& L = h->L[l];
     L.s.cur = 0;
     L.s.ghosts_stale = false;
+    L.s.ghosts_ready = false;
     ST(zero(L.s.u[0], grid_elems(L.G)));
     if (L.geo.nest) {
       ST(zero(L.s.inter, L.fs.base[6]));
@@ -1266,6 +1295,7 @@ mg_status build_loop_graph(mg_hierarchy* h) {
   };
   if (!h->mixed) {
     ST(capture_into(h, body, nullptr, 0, &G.body[0], [&](mg_hierarchy* hh) -> mg_status {
+      forget_ghosts<double>(hh);
       ST(vcycle<double>(hh, finest(hh)));
       ST(norm_launches(hh, false, false));
       return step(hh);
@@ -1641,6 +1671,16 @@ bool batch_persistent(const mg_batch* b, const std::vector<int>& active) {
   return false;
 }
 
+// Members from which a batch's branches count as crowded (16 members of the mixed-precision
+// ensemble: 16.8 ms with separate ghost launches, 17.4 ms with fused half-sweeps).
+constexpr int kCrowdedMembers = 4;
+
+bool crowded(const std::vector<int>& active) {
+  int n = 0;
+  for (int a : active) n += a != 0;
+  return n >= kCrowdedMembers;
+}
+
 constexpr unsigned long long kPersistWaitNs = 2000000000ull;  // 2 s per dependency wait
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -1744,7 +1784,9 @@ mg_status batch_graph_persistent(mg_batch* b, const std::vector<int>& active, Ba
     const mg_stats snap = h->stats;
     const unsigned keep = h->active_mask;
     h->active_mask = 0;
+    h->crowded = crowded(active);
     rs = solve_body(h);
+    h->crowded = false;
     h->active_mask = keep;
     for (int f = 0; f < MG_K_FAMILIES; ++f) {
       g.delta[i].launches[f] = h->stats.launches[f] - snap.launches[f];
@@ -1832,7 +1874,9 @@ mg_status batch_graph(mg_batch* b, const std::vector<int>& active, BatchGraph** 
     const mg_stats snap = h->stats;
     const unsigned keep = h->active_mask;
     h->active_mask = 0;
+    h->crowded = crowded(active);
     st = solve_body(h);
+    h->crowded = false;
     h->active_mask = keep;
     for (int f = 0; f < MG_K_FAMILIES; ++f) {
       g.delta[i].launches[f] = h->stats.launches[f] - snap.launches[f];

@@ -203,63 +203,20 @@ __global__ void __launch_bounds__(128)
                          blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
 
-// The flux step of float64 solves with everything that is linear folded on the host or into
-// the tangential kernel: the ghost of layer m is G_m + sum_q nfine[m][q] v_q + shift, and
-// shift = K + sum over the 4 columns of sum_q d[side][q] v_q, where G_m and K (inter and
-// fc_unc of the folded tangential kernel) carry the parent values, and d the parent flux of
-// the covered cells minus the fine fluxes.  24 FP64 instructions per column instead of 47.
-struct FluxFold {
-  double d[2][6];
-  double nfine[3][4];
-};
-
 template <int ORDER>
 __global__ void __launch_bounds__(128)
-    k_cf_flux_fold(Grid F, double* __restrict__ u, FaceSet fs, FluxFold w,
-                   const double* __restrict__ inter, const double* __restrict__ fc_unc) {
+    k_cf_flux_fold(Grid F, double* __restrict__ u, FaceArgs<double> fa) {
   grid_wait();
-  constexpr int half = ORDER / 2;
   const int t = blockIdx.x * 128 + threadIdx.x;
-  if (t >= 4 * (int)fs.ebase[6]) return;
+  if (t >= 4 * (int)fa.fs.ebase[6]) return;
   const unsigned quad = __activemask();
-  const int e = t >> 2, col = t & 3;
-  int f = 0;
-#pragma unroll
-  for (int q = 1; q < 6; ++q)
-    if (e >= (int)fs.ebase[q]) f = q;
-  const int a = f >> 1, side = f & 1;
-  const int nt0 = fs.nt[f][0], nt1 = fs.nt[f][1];
-  const unsigned loc = e - (int)fs.ebase[f], ne1 = nt1 / 2;
-  const unsigned jc = loc / ne1, kc = loc % ne1;
-  const int tj = 2 * jc + (col >> 1), tk = 2 * kc + (col & 1);
-  const int sx = F.Y * F.Zp, sy = F.Zp;
-  const int sa = a == 0 ? sx : (a == 1 ? sy : 1);
-  const int sb = a == 0 ? sy : sx;
-  const int sc = a == 2 ? sy : 1;
-  const int na = a == 0 ? F.n0 : (a == 1 ? F.n1 : F.n2);
-  double* in0 = u + gidx(F, 0, 0, 0) + ((long long)tj * sb + tk * sc);
-  if (side) in0 += (long long)(na - 1) * sa;
-  const int step = side == 0 ? sa : -sa;
-  double v[2 * half], g[half];
-#pragma unroll
-  for (int q = 0; q < 2 * half; ++q) v[q] = in0[q * step];
-  const double* ip = inter + fs.base[f] + ((long long)tj * nt1 + tk);
-#pragma unroll
-  for (int m = 0; m < half; ++m) g[m] = __ldg(ip + (long long)m * nt0 * nt1);
-  const double k = __ldg(fc_unc + e);
-  double s = w.d[side][0] * v[0];
-#pragma unroll
-  for (int q = 1; q < 2 * half; ++q) s = fma(w.d[side][q], v[q], s);
-  s += __shfl_xor_sync(quad, s, 1);
-  s += __shfl_xor_sync(quad, s, 2);
-  s += k;
-#pragma unroll
-  for (int m = 0; m < half; ++m) {
-    double x = g[m] + s;
-#pragma unroll
-    for (int q = 0; q <= half; ++q) x = fma(w.nfine[m][q], v[q], x);
-    in0[-(m + 1) * step] = x;
-  }
+  const int e = t >> 2;
+  const int f = face_of(fa.fs, e, fa.fs.ebase);
+  const unsigned loc = (unsigned)(e - (int)fa.fs.ebase[f]), ne1 = fa.fs.nt[f][1] / 2;
+  const FaceCol c = face_col(F, f, (int)(loc / ne1), (int)(loc % ne1), t & 3);
+  double v[ORDER];
+  load_column<ORDER, double>(u, c, v);
+  fa.ghosts<ORDER>(u, c, v, quad);
 }
 
 // Edge and corner ghosts of a level in a row: the edges along x, y and z, (2 g)^2 cells at
@@ -368,13 +325,17 @@ cudaError_t launch_cf_tangential(int order, const Grid& F, const Grid& P, const 
   }
 }
 
-cudaError_t launch_cf_flux_fold(int order, const Grid& F, double* u, const FaceSet& fs,
-                                const CfWeights& w, const double* inter, const double* fc_unc,
-                                double h, double invH, cudaStream_t s) {
+template <>
+FaceArgs<double> make_face_args<double>(int order, const FaceSet& fs, const CfWeights& w,
+                                        const double* inter, const double* fc_unc, double h,
+                                        double invH) {
   const int half = order / 2;
-  FluxFold fo{};
+  FaceArgs<double> o{};
+  o.fs = fs;
+  o.inter = inter;
+  o.fc_unc = fc_unc;
   for (int m = 0; m < half; ++m)
-    for (int q = 0; q <= half; ++q) fo.nfine[m][q] = w.nfine[m][q];
+    for (int q = 0; q <= half; ++q) o.w.nfine[m][q] = w.nfine[m][q];
   for (int sd = 0; sd < 2; ++sd) {
     const double c = w.ghost_coef[sd];
     for (int q = 0; q < 2 * half; ++q) {
@@ -384,14 +345,40 @@ cudaError_t launch_cf_flux_fold(int order, const Grid& F, double* u, const FaceS
       if (q <= half)
         for (int m = 0; m < half; ++m)
           fine += w.flux[sd == 0 ? half - 1 - m : half + m] * w.nfine[m][q];
-      fo.d[sd][q] = (h / c) * (0.125 * invH) * w.flux[sp] - 0.25 / c * fine;
+      o.w.d[sd][q] = (h / c) * (0.125 * invH) * w.flux[sp] - 0.25 / c * fine;
     }
   }
+  return o;
+}
+
+template <>
+FaceArgs<float> make_face_args<float>(int order, const FaceSet& fs, const CfWeights& w,
+                                      const float* inter, const float* fc_unc, double h,
+                                      double invH) {
+  (void)order;
+  const double invh = 1.0 / h;
+  FaceArgs<float> o{};
+  o.fs = fs;
+  o.w = cf_weights_as<float>(w);
+  o.inter = inter;
+  o.fc_unc = fc_unc;
+  o.fc_scale = float(0.125 * invH);
+  o.a0 = float(h / w.ghost_coef[0]);
+  o.a1 = float(h / w.ghost_coef[1]);
+  o.b0 = float(0.25 * invh * h / w.ghost_coef[0]);
+  o.b1 = float(0.25 * invh * h / w.ghost_coef[1]);
+  return o;
+}
+
+cudaError_t launch_cf_flux_fold(int order, const Grid& F, double* u, const FaceSet& fs,
+                                const CfWeights& w, const double* inter, const double* fc_unc,
+                                double h, double invH, cudaStream_t s) {
+  const FaceArgs<double> fa = make_face_args<double>(order, fs, w, inter, fc_unc, h, invH);
   const unsigned grid = (unsigned)((4 * fs.ebase[6] + 127) / 128);
   switch (order) {
-    case 2: return launch_dep(k_cf_flux_fold<2>, grid, 128, 0, s, F, u, fs, fo, inter, fc_unc);
-    case 4: return launch_dep(k_cf_flux_fold<4>, grid, 128, 0, s, F, u, fs, fo, inter, fc_unc);
-    case 6: return launch_dep(k_cf_flux_fold<6>, grid, 128, 0, s, F, u, fs, fo, inter, fc_unc);
+    case 2: return launch_dep(k_cf_flux_fold<2>, grid, 128, 0, s, F, u, fa);
+    case 4: return launch_dep(k_cf_flux_fold<4>, grid, 128, 0, s, F, u, fa);
+    case 6: return launch_dep(k_cf_flux_fold<6>, grid, 128, 0, s, F, u, fa);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -72,6 +72,18 @@ template <typename T>
 cudaError_t launch_smooth_half(int order, const Grid& G, const T* uin, T* uout, const T* f,
                                double a_f, int colour, int periodic, int rows, bool quad,
                                cudaStream_t s);
+// Nests up to this many cells take the fused half-sweep below.  One V-cycle of a base and two
+// nests of n^3 cells, separate / fused, us: float32, order 6: n = 32 116.0 / 101.2, 48 144.3 /
+// 130.4, 64 153.2 / 151.6, 80 219.1 / 225.3, 96 292.9 / 310.2; float64, order 4: 32 172.4 /
+// 162.0, 48 220.2 / 201.0, 64 257.3 / 258.8, 80 380.7 / 392.8.
+constexpr long long kFaceFusedMaxCells = 1ll << 18;
+// The half-sweep of a nest followed by the coarse-fine ghosts of its result (float64: folded,
+// after launch_cf_tangential with fold = true); h, invH: own spacing, 1 / parent spacing.
+template <typename T>
+cudaError_t launch_smooth_faces(int order, const Grid& G, const T* uin, T* uout, const T* f,
+                                double a_f, int colour, bool quad, const FaceSet& fs,
+                                const CfWeights& w, const T* inter, const T* fc_unc, double h,
+                                double invH, cudaStream_t s);
 template <typename T>
 cudaError_t launch_residual_restrict(int order, const Grid& F, const T* u, const T* f,
                                      double invh2, const Grid& P, T* pu, T* pfas, T* ubar,

@@ -51,16 +51,11 @@ __device__ __forceinline__ float4 ld4(const float* p) {
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(256, 4)
-    k_smooth_quad(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
-                  const float* __restrict__ f, float a_f, int colour, int periodic) {
-  grid_wait();
+__device__ __forceinline__ void smooth_quad_at(const Grid& G, const float* __restrict__ uin,
+                                               float* __restrict__ uout,
+                                               const float* __restrict__ f, float a_f, int colour,
+                                               int periodic, int i, int j, int k0) {
   constexpr int R = ORDER / 2;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int i = blockIdx.z;
-  const int k0 = 4 * t;
-  if (j >= G.n1 || k0 >= G.n2) return;
   const long long sy = G.Zp;
   const long long sx = (long long)G.Y * G.Zp;
   const long long p0 = gidx(G, i, j, k0);
@@ -120,6 +115,80 @@ __global__ void __launch_bounds__(256, 4)
     write_pair_images<float>(G, uout, i, j, k0, out.x, out.y);
     write_pair_images<float>(G, uout, i, j, k0 + 2, out.z, out.w);
   }
+}
+
+template <int ORDER>
+__global__ void __launch_bounds__(256, 4)
+    k_smooth_quad(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
+                  const float* __restrict__ f, float a_f, int colour, int periodic) {
+  grid_wait();
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int k0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (j >= G.n1 || k0 >= G.n2) return;
+  smooth_quad_at<ORDER>(G, uin, uout, f, a_f, colour, periodic, blockIdx.z, j, k0);
+}
+
+// ---- half-sweep of a nest with its ghosts ----------------------------------------------
+// The half-sweep of a nest and the coarse-fine ghosts of its result, which the next
+// half-sweep or the residual reads, in one launch instead of two dependent ones.  The first
+// face_blocks blocks work on 32 fine face columns each: of the ORDER cells nearest the face
+// that a column's ghosts depend on, ORDER / 2 have the colour and are updated from uin once
+// more, one warp per depth, and one warp writes the ghosts from the block's values in shared
+// memory; the other blocks are those of the plain half-sweep.  No block reads what another
+// writes, and every value is the same chain of operations as in the separate kernels.  The
+// repeated updates cost 18 / n of a half-sweep's for order 6 and n^3 cells; the launch that
+// goes away is nearly all latency on small levels (kFaceFusedMaxCells).
+constexpr int kFacesThreads = 128;
+
+template <int ORDER, typename T, int VEC>
+__global__ void __launch_bounds__(kFacesThreads, (smooth_min_blocks<ORDER, T>) < 5 || VEC == 4 ? 8 : 10)
+    k_smooth_faces(Grid G, const T* __restrict__ uin, T* __restrict__ uout,
+                   const T* __restrict__ f, T a_f, int colour, int face_blocks, int gx, int gy,
+                   int qx, int by, FaceArgs<T> fa) {
+  grid_wait();
+  const int b = (int)blockIdx.x - face_blocks;
+  if (b >= 0) {
+    const int ty = (int)threadIdx.x / qx, tx = (int)threadIdx.x - ty * qx;
+    const int j = b / gx % gy * by + ty;
+    const int k0 = VEC * (b % gx * qx + tx);
+    if (ty >= by || j >= G.n1 || k0 >= G.n2) return;
+    if constexpr (VEC == 4)
+      smooth_quad_at<ORDER>(G, uin, uout, f, a_f, colour, 0, b / (gx * gy), j, k0);
+    else
+      smooth_pair_at<ORDER, T, Ldg>(G, uin, uout, f, a_f, colour, 0, b / (gx * gy), j, k0);
+    return;
+  }
+  __shared__ T cells[ORDER][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = (int)blockIdx.x * 32 + lane;
+  const bool in = t < 4 * (int)fa.fs.ebase[6];  // whole groups of 4, an element's columns
+  FaceCol c;
+  if (in) {
+    const int e = t >> 2;
+    const int fc = face_of(fa.fs, e, fa.fs.ebase);
+    const unsigned loc = (unsigned)(e - (int)fa.fs.ebase[fc]), ne1 = fa.fs.nt[fc][1] / 2;
+    c = face_col(G, fc, (int)(loc / ne1), (int)(loc % ne1), t & 3);
+    // the cells at depths o, o + 2, .. have the colour (index along the normal: 0 or n - 1)
+    const int na = (fc >> 1) == 0 ? G.n0 : ((fc >> 1) == 1 ? G.n1 : G.n2);
+    const int o = ((((fc & 1) ? na - 1 : 0) + c.tj + c.tk) & 1) == colour ? 0 : 1;
+    if (warp < ORDER / 2) {
+      const int q = 2 * warp + o;
+      const long long p = c.in0 + q * c.step;
+      T nb[3 * ORDER];
+      load_neighbours<ORDER, T>(uin, p, G.Zp, G.Y * G.Zp, nb);
+      cells[q][lane] = relax<ORDER, T>(nb, a_f * __ldg(f + p));
+    } else if (warp == kFacesThreads / 32 - 1) {
+#pragma unroll
+      for (int q = 0; q < ORDER / 2; ++q)
+        cells[2 * q + 1 - o][lane] = __ldg(uin + c.in0 + (2 * q + 1 - o) * c.step);
+    }
+  }
+  __syncthreads();
+  if (warp != 0 || !in) return;
+  T v[ORDER];
+#pragma unroll
+  for (int q = 0; q < ORDER; ++q) v[q] = cells[q][lane];
+  fa.template ghosts<ORDER>(uout, c, v, 0xfu << (lane & 28));
 }
 
 // r = f - L u at the 8 children of every covered parent cell; parent u := mean(u), ubar :=
@@ -333,6 +402,43 @@ cudaError_t launch_smooth_half(int order, const Grid& G, const T* uin, T* uout, 
   }
 }
 
+template <int ORDER, typename T, int VEC>
+static cudaError_t launch_faces_vec(const Grid& G, const T* uin, T* uout, const T* f, double a_f,
+                                    int colour, const FaceArgs<T>& fa, cudaStream_t s) {
+  // blocks of qx groups of a row x by rows
+  const int groups = (G.n2 + VEC - 1) / VEC;
+  const int qx = groups < 32 ? groups : 32;
+  const int by = kFacesThreads / qx < G.n1 ? kFacesThreads / qx : G.n1;
+  const int gx = (groups + qx - 1) / qx, gy = (G.n1 + by - 1) / by;
+  const int faces = (int)((4 * fa.fs.ebase[6] + 31) / 32);
+  return launch_dep(k_smooth_faces<ORDER, T, VEC>, dim3(faces + gx * gy * G.n0), kFacesThreads, 0, s,
+                    G, uin, uout, f, T(a_f), colour, faces, gx, gy, qx, by, fa);
+}
+
+template <typename T>
+cudaError_t launch_smooth_faces(int order, const Grid& G, const T* uin, T* uout, const T* f,
+                                double a_f, int colour, bool quad, const FaceSet& fs,
+                                const CfWeights& w, const T* inter, const T* fc_unc, double h,
+                                double invH, cudaStream_t s) {
+  const FaceArgs<T> fa = make_face_args<T>(order, fs, w, inter, fc_unc, h, invH);
+  if constexpr (sizeof(T) == 4) {
+    if (quad && G.n2 % 4 == 0) {
+      switch (order) {
+        case 2: return launch_faces_vec<2, T, 4>(G, uin, uout, f, a_f, colour, fa, s);
+        case 4: return launch_faces_vec<4, T, 4>(G, uin, uout, f, a_f, colour, fa, s);
+        case 6: return launch_faces_vec<6, T, 4>(G, uin, uout, f, a_f, colour, fa, s);
+        default: return cudaErrorInvalidValue;
+      }
+    }
+  }
+  switch (order) {
+    case 2: return launch_faces_vec<2, T, 2>(G, uin, uout, f, a_f, colour, fa, s);
+    case 4: return launch_faces_vec<4, T, 2>(G, uin, uout, f, a_f, colour, fa, s);
+    case 6: return launch_faces_vec<6, T, 2>(G, uin, uout, f, a_f, colour, fa, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 template <typename T>
 cudaError_t launch_residual_restrict(int order, const Grid& F, const T* u, const T* f,
                                      double invh2, const Grid& P, T* pu, T* pfas, T* ubar,
@@ -397,6 +503,10 @@ cudaError_t prepare_restrict_tile() {
 #define MGK_INSTANTIATE(T)                                                                     \
   template cudaError_t launch_smooth_half<T>(int, const Grid&, const T*, T*, const T*, double, \
                                              int, int, int, bool, cudaStream_t);               \
+  template cudaError_t launch_smooth_faces<T>(int, const Grid&, const T*, T*, const T*, double,  \
+                                              int, bool, const FaceSet&, const CfWeights&,     \
+                                              const T*, const T*, double, double,              \
+                                              cudaStream_t);                                   \
   template cudaError_t launch_residual_restrict<T>(int, const Grid&, const T*, const T*,       \
                                                    double, const Grid&, T*, T*, T*, Int3,      \
                                                    Int3, int, cudaStream_t);                   \

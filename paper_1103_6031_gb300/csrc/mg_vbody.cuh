@@ -28,14 +28,10 @@ constexpr int kVPairX = 32;
 // cell of uout (colour c updated, the other colour copied), one z-pair per thread;
 // blocks of kVPairX x rows threads.
 template <int ORDER, typename T, typename LD>
-__device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restrict__ uin,
-                                                 T* __restrict__ uout, const T* __restrict__ f,
-                                                 T a_f, int colour, int periodic, int rows, Blk b) {
-  const int t = b.bx * kVPairX + b.tx;
-  const int j = b.by * rows + b.ty;
-  const int i = b.bz;
-  const int k0 = 2 * t;
-  if (j >= G.n1 || k0 >= G.n2) return;
+__device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restrict__ uin,
+                                               T* __restrict__ uout, const T* __restrict__ f,
+                                               T a_f, int colour, int periodic, int i, int j,
+                                               int k0) {
   const int sy = G.Zp;
   const int sx = G.Y * G.Zp;
   const long long p0 = gidx(G, i, j, k0);
@@ -68,6 +64,16 @@ __device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restr
     uout[p0] = v;
     if (periodic) write_images<T>(G, uout, i, j, k0, v);
   }
+}
+
+template <int ORDER, typename T, typename LD>
+__device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restrict__ uin,
+                                                 T* __restrict__ uout, const T* __restrict__ f,
+                                                 T a_f, int colour, int periodic, int rows, Blk b) {
+  const int j = b.by * rows + b.ty;
+  const int k0 = 2 * (b.bx * kVPairX + b.tx);
+  if (j >= G.n1 || k0 >= G.n2) return;
+  smooth_pair_at<ORDER, T, LD>(G, uin, uout, f, a_f, colour, periodic, b.bz, j, k0);
 }
 
 // ---- residual + restriction: one thread per covered parent cell ---------------------
@@ -312,42 +318,56 @@ __device__ __forceinline__ void cf_tangential_body(const Grid& F, const Grid& P,
 // a_side F_c - b_side (sum of the 4 unscaled fine flux stencils), a_side = h / c_side,
 // b_side = 1 / (4 c_side) (c_side: the sum of the flux weights on the ghost side).
 // Reads and writes u with plain accesses (the ghosts it writes are not read by it).
-template <int ORDER, typename T>
-__device__ __forceinline__ void cf_flux_body(const Grid& F, T* __restrict__ u, const FaceSet& fs,
-                                             const CfW<T>& w, const T* __restrict__ inter,
-                                             const T* __restrict__ fc_unc, T fc_scale, T a0, T a1,
-                                             T b0, T b1, int flux_fix, long long t) {
-  constexpr int half = ORDER / 2;
-  if (t >= 4 * fs.ebase[6]) return;
-  const unsigned quad = __activemask();
-  const int e = (int)(t >> 2), col = (int)(t & 3);
-  const int f = face_of(fs, e, fs.ebase);
+// A fine column of face f: column col (0..3) of parent face element (jc, kc).
+struct FaceCol {
+  int f, jc, kc, col;
+  int tj, tk;      // fine tangential position
+  long long in0;   // element of the column's cell at the face
+  int step;        // element stride inwards
+};
+
+__device__ __forceinline__ FaceCol face_col(const Grid& F, int f, int jc, int kc, int col) {
+  FaceCol c;
+  c.f = f;
+  c.jc = jc;
+  c.kc = kc;
+  c.col = col;
   const int a = f >> 1, side = f & 1;
-  const int nt0 = fs.nt[f][0], nt1 = fs.nt[f][1];
-  const unsigned loc = (unsigned)(e - (int)fs.ebase[f]), ne1 = nt1 / 2;
-  const int jc = (int)(loc / ne1), kc = (int)(loc % ne1);
-  const int tj = 2 * jc + (col >> 1), tk = 2 * kc + (col & 1);
-  const long long sx = (long long)F.Y * F.Zp, sy = F.Zp;
+  c.tj = 2 * jc + (col >> 1);
+  c.tk = 2 * kc + (col & 1);
   // strides along the normal (a) and the tangential axes (b, c) of this face
-  const long long sa = a == 0 ? sx : (a == 1 ? sy : 1);
-  const long long sb = a == 0 ? sy : sx;
-  const long long sc = a == 2 ? sy : 1;
+  const int sx = F.Y * F.Zp, sy = F.Zp;
+  const int sa = a == 0 ? sx : (a == 1 ? sy : 1);
+  const int sb = a == 0 ? sy : sx;
+  const int sc = a == 2 ? sy : 1;
   const int na = a == 0 ? F.n0 : (a == 1 ? F.n1 : F.n2);
-  // element (0 along the normal, tj, tk); moving inwards is +sa (low face) or -sa (high)
-  const long long col0 = gidx(F, 0, 0, 0) + tj * sb + tk * sc;
-  const long long in0 = side == 0 ? col0 : col0 + (long long)(na - 1) * sa;
-  const long long step = side == 0 ? sa : -sa;
-  // fine interior values q = 0 .. half from the face
-  T v[half + 1];
-#pragma unroll
-  for (int q = 0; q <= half; ++q) v[q] = u[in0 + q * step];
+  // moving inwards is +sa (low face) or -sa (high)
+  c.in0 = gidx(F, 0, 0, 0) + ((long long)c.tj * sb + c.tk * sc);
+  if (side) c.in0 += (long long)(na - 1) * sa;
+  c.step = side == 0 ? sa : -sa;
+  return c;
+}
+
+// Writes the ghosts of column c into u from its ORDER cells nearest the face, v; quad: a
+// mask of converged lanes that holds the element's four.
+template <int ORDER, typename T>
+__device__ __forceinline__ void cf_flux_at(T* u, const FaceSet& fs, const CfW<T>& w,
+                                           const T* __restrict__ inter,
+                                           const T* __restrict__ fc_unc, T fc_scale, T a0, T a1,
+                                           T b0, T b1, int flux_fix, const FaceCol& fcol,
+                                           const T (&v)[ORDER], unsigned quad) {
+  constexpr int half = ORDER / 2;
+  const int f = fcol.f, side = f & 1;
+  const int nt0 = fs.nt[f][0], nt1 = fs.nt[f][1];
+  const long long e = fs.ebase[f] + (long long)fcol.jc * (nt1 / 2) + fcol.kc;
+  const int tj = fcol.tj, tk = fcol.tk;
   // parent flux: uncovered part + covered parent cells as the mean of their 8
   // children; each column holds 2 of the 8 (normal 2d, 2d+1)
   T cov = T(0);
 #pragma unroll
   for (int d = 0; d < half; ++d) {
     const int s = side == 0 ? half + d : half - 1 - d;
-    T pair = u[in0 + (2 * d) * step] + u[in0 + (2 * d + 1) * step];
+    T pair = v[2 * d] + v[2 * d + 1];
     pair += __shfl_xor_sync(quad, pair, 1);
     pair += __shfl_xor_sync(quad, pair, 2);
     cov = fma(w.flux[s], pair, cov);
@@ -379,8 +399,101 @@ __device__ __forceinline__ void cf_flux_body(const Grid& F, T* __restrict__ u, c
   T shift = T(0);
   if (flux_fix) shift = fma(-(side ? b1 : b0), ff, fc * (side ? a1 : a0));
 #pragma unroll
-  for (int m = 0; m < half; ++m) u[in0 - (m + 1) * step] = ghost[m] + shift;
+  for (int m = 0; m < half; ++m) u[fcol.in0 - (m + 1) * fcol.step] = ghost[m] + shift;
 }
+
+// The ORDER cells of a column nearest the face.
+template <int ORDER, typename T>
+__device__ __forceinline__ void load_column(const T* u, const FaceCol& c, T (&v)[ORDER]) {
+#pragma unroll
+  for (int q = 0; q < ORDER; ++q) v[q] = u[c.in0 + q * c.step];
+}
+
+template <int ORDER, typename T>
+__device__ __forceinline__ void cf_flux_body(const Grid& F, T* __restrict__ u, const FaceSet& fs,
+                                             const CfW<T>& w, const T* __restrict__ inter,
+                                             const T* __restrict__ fc_unc, T fc_scale, T a0, T a1,
+                                             T b0, T b1, int flux_fix, long long t) {
+  if (t >= 4 * fs.ebase[6]) return;
+  const unsigned quad = __activemask();
+  const int e = (int)(t >> 2);
+  const int f = face_of(fs, e, fs.ebase);
+  const unsigned loc = (unsigned)(e - (int)fs.ebase[f]), ne1 = fs.nt[f][1] / 2;
+  const FaceCol c = face_col(F, f, (int)(loc / ne1), (int)(loc % ne1), (int)(t & 3));
+  T v[ORDER];
+  load_column<ORDER, T>(u, c, v);
+  cf_flux_at<ORDER, T>(u, fs, w, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix, c, v, quad);
+}
+
+// The flux step of float64 solves with everything that is linear folded on the host or into
+// the tangential kernel: the ghost of layer m is G_m + sum_q nfine[m][q] v_q + shift, and
+// shift = K + sum over the 4 columns of sum_q d[side][q] v_q, where G_m and K (inter and
+// fc_unc of the folded tangential kernel) carry the parent values, and d the parent flux of
+// the covered cells minus the fine fluxes.  24 FP64 instructions per column instead of 47.
+struct FluxFold {
+  double d[2][6];
+  double nfine[3][4];
+};
+
+template <int ORDER>
+__device__ __forceinline__ void cf_fold_at(double* u, const FaceSet& fs, const FluxFold& w,
+                                           const double* __restrict__ inter,
+                                           const double* __restrict__ fc_unc, const FaceCol& c,
+                                           const double (&v)[ORDER], unsigned quad) {
+  constexpr int half = ORDER / 2;
+  const int side = c.f & 1;
+  const int nt0 = fs.nt[c.f][0], nt1 = fs.nt[c.f][1];
+  double g[half];
+  const double* ip = inter + fs.base[c.f] + ((long long)c.tj * nt1 + c.tk);
+#pragma unroll
+  for (int m = 0; m < half; ++m) g[m] = __ldg(ip + (long long)m * nt0 * nt1);
+  const double k = __ldg(fc_unc + fs.ebase[c.f] + (long long)c.jc * (nt1 / 2) + c.kc);
+  double s = w.d[side][0] * v[0];
+#pragma unroll
+  for (int q = 1; q < 2 * half; ++q) s = fma(w.d[side][q], v[q], s);
+  s += __shfl_xor_sync(quad, s, 1);
+  s += __shfl_xor_sync(quad, s, 2);
+  s += k;
+#pragma unroll
+  for (int m = 0; m < half; ++m) {
+    double x = g[m] + s;
+#pragma unroll
+    for (int q = 0; q <= half; ++q) x = fma(w.nfine[m][q], v[q], x);
+    u[c.in0 - (m + 1) * c.step] = x;
+  }
+}
+
+// What a kernel needs to write a nest's ghosts: float as cf_flux_at, double folded.
+template <typename T>
+struct FaceArgs;
+template <>
+struct FaceArgs<float> {
+  FaceSet fs;
+  CfW<float> w;
+  const float* inter;
+  const float* fc_unc;
+  float fc_scale, a0, a1, b0, b1;
+  template <int ORDER>
+  __device__ __forceinline__ void ghosts(float* u, const FaceCol& c, const float (&v)[ORDER],
+                                         unsigned quad) const {
+    cf_flux_at<ORDER, float>(u, fs, w, inter, fc_unc, fc_scale, a0, a1, b0, b1, 1, c, v, quad);
+  }
+};
+template <>
+struct FaceArgs<double> {
+  FaceSet fs;
+  FluxFold w;
+  const double* inter;
+  const double* fc_unc;
+  template <int ORDER>
+  __device__ __forceinline__ void ghosts(double* u, const FaceCol& c, const double (&v)[ORDER],
+                                         unsigned quad) const {
+    cf_fold_at<ORDER>(u, fs, w, inter, fc_unc, c, v, quad);
+  }
+};
+template <typename T>
+FaceArgs<T> make_face_args(int order, const FaceSet& fs, const CfWeights& w, const T* inter,
+                           const T* fc_unc, double h, double invH);
 
 // ---- coarsest level: periodic pseudo-inverse of L as a circular convolution --------
 // u(x) = sum_y K(x - y) f(y), K precomputed on the host from the DFT symbol; block x
