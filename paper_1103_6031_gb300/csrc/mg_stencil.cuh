@@ -177,16 +177,24 @@ __device__ __forceinline__ ImgAxis img_axis(int a, int n, int g, long long st) {
 // Writes v to the images of interior cell (i, j, k): every combination of own
 // or image index per axis except own on every axis.  Straight-line predicated
 // stores (the loops unroll; no local memory); the cell itself is written by the
-// caller.
+// caller.  Rows away from the x and y faces (the same for a whole warp) have z images only:
+// they take two stores instead of the 26 predicated ones, which every warp that reaches a z
+// face would execute.
 template <typename T>
 __device__ __forceinline__ void write_images(const Grid& G, T* __restrict__ u, int i, int j,
                                              int k, T v) {
   const int g = G.g;
-  if (i >= g && i < G.n0 - g && j >= g && j < G.n1 - g && k >= g && k < G.n2 - g) return;
+  const bool in_xy = i >= g && i < G.n0 - g && j >= g && j < G.n1 - g;
+  if (in_xy && k >= g && k < G.n2 - g) return;
   const long long sy = G.Zp, sx = (long long)G.Y * G.Zp;
-  const ImgAxis ax = img_axis(i, G.n0, g, sx), ay = img_axis(j, G.n1, g, sy),
-                az = img_axis(k, G.n2, g, 1);
+  const ImgAxis az = img_axis(k, G.n2, g, 1);
   T* p = u + gidx(G, i, j, k);
+  if (in_xy) {
+    if (az.lo) p[az.lo] = v;
+    if (az.hi) p[az.hi] = v;
+    return;
+  }
+  const ImgAxis ax = img_axis(i, G.n0, g, sx), ay = img_axis(j, G.n1, g, sy);
   const long long ox[3] = {0, ax.lo, ax.hi}, oy[3] = {0, ay.lo, ay.hi}, oz[3] = {0, az.lo, az.hi};
 #pragma unroll
   for (int a = 0; a < 3; ++a)
@@ -206,12 +214,20 @@ template <typename T>
 __device__ __forceinline__ void write_pair_images(const Grid& G, T* __restrict__ u, int i, int j,
                                                   int k, T va, T vb) {
   const int g = G.g;
-  if (i >= g && i < G.n0 - g && j >= g && j < G.n1 - g && k >= g && k + 1 < G.n2 - g) return;
+  const bool in_xy = i >= g && i < G.n0 - g && j >= g && j < G.n1 - g;
+  if (in_xy && k >= g && k + 1 < G.n2 - g) return;
   typedef typename Vec2<T>::type V2;
   const long long sy = G.Zp, sx = (long long)G.Y * G.Zp;
-  const ImgAxis ax = img_axis(i, G.n0, g, sx), ay = img_axis(j, G.n1, g, sy);
   const ImgAxis z0 = img_axis(k, G.n2, g, 1), z1 = img_axis(k + 1, G.n2, g, 1);
   T* p = u + gidx(G, i, j, k);
+  if (in_xy) {
+    if (z0.lo) p[z0.lo] = va;
+    if (z0.hi) p[z0.hi] = va;
+    if (z1.lo) p[1 + z1.lo] = vb;
+    if (z1.hi) p[1 + z1.hi] = vb;
+    return;
+  }
+  const ImgAxis ax = img_axis(i, G.n0, g, sx), ay = img_axis(j, G.n1, g, sy);
   const long long ox[3] = {0, ax.lo, ax.hi}, oy[3] = {0, ay.lo, ay.hi};
   V2 pv;
   pv.x = va;
