@@ -13,7 +13,10 @@
 //
 // Field: cuFFT real-to-complex transform of the noise, a kernel that multiplies
 // every mode by A(|k|) / N (linear interpolation of a table sampled at |k| = t dk,
-// 0 beyond the table and at k = 0), and the complex-to-real inverse.
+// 0 beyond the table and at k = 0), and the complex-to-real inverse.  The half spectrum is
+// along z unless n2 is odd and n0 even: real transforms of odd length cost as much as
+// complex ones, so then the real transform runs along x and complex 2D ones follow on the
+// n0/2 + 1 planes left (192x200x243: 2.56 -> 2.30 ms for both directions).
 #include <cufft.h>
 
 #include <cmath>
@@ -43,8 +46,13 @@ __device__ __forceinline__ void philox4x32_10(uint32_t (&x)[4], uint32_t k0, uin
   }
 }
 
+// (m + 1/2) / 2^53 for the 53-bit m of 27 bits of a and 26 of b, rounded to nearest: one
+// conversion of 2 m + 1 and a power of two taken off the exponent (2 m + 1 >= 1, so the
+// result is normal).
 __device__ __forceinline__ double uniform53(uint32_t a, uint32_t b) {
-  return ((double)(a >> 5) * 67108864.0 + (double)(b >> 6) + 0.5) * (1.0 / 9007199254740992.0);
+  const unsigned long long m = ((unsigned long long)(a >> 5) << 26) | (b >> 6);
+  const double d = (double)(long long)(2 * m + 1);
+  return __hiloint2double(__double2hiint(d) - (54 << 20), __double2loint(d));
 }
 
 // One Philox call per pair of elements; grid-stride over pairs.  stream is counter
@@ -72,16 +80,17 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// F[i][j][m] *= A(|k|) * scale, m < n2/2 + 1 (half spectrum along z).  A block works on
+// F[i][j][m] *= A(|k|) * scale over the half spectrum, (i, j, m) < (n0, n1, n2/2 + 1), or
+// (n0/2 + 1, n1, n2) with half_x.  A block works on
 // kAmpRows rows j of one plane: the squares of its rows' and threads' frequencies are formed
 // once (their divisions, and those of a flat index, took more of the FP64-bound kernel than
 // the square root and the interpolation of a mode).
 constexpr int kAmpRows = 16, kAmpThreads = 128;
 
 __global__ void __launch_bounds__(kAmpThreads)
-    k_apply_amplitude(cufftDoubleComplex* __restrict__ F, int n0, int n1, int n2, double h,
-                      const double* __restrict__ amp, int nt, double dk, double scale) {
-  const int n2h = n2 / 2 + 1;
+    k_apply_amplitude(cufftDoubleComplex* __restrict__ F, int n0, int n1, int n2, int half_x,
+                      double h, const double* __restrict__ amp, int nt, double dk, double scale) {
+  const int n2h = half_x ? n2 : n2 / 2 + 1;
   const double tp = 2.0 * 3.14159265358979323846 / h;
   const int i = blockIdx.z, j0 = blockIdx.y * kAmpRows;
   __shared__ double fij[kAmpRows];
@@ -94,7 +103,7 @@ __global__ void __launch_bounds__(kAmpThreads)
   __syncthreads();
   const int m = blockIdx.x * kAmpThreads + threadIdx.x;
   if (m >= n2h) return;
-  const double fm = (double)m / n2;
+  const double fm = (double)(m <= n2 / 2 ? m : m - n2) / n2;
   const int rows = min(kAmpRows, n1 - j0);
   cufftDoubleComplex* e = F + ((long long)i * n1 + j0) * n2h + m;
 #pragma unroll 4
@@ -116,10 +125,11 @@ __global__ void __launch_bounds__(kAmpThreads)
   }
 }
 
-void launch_amplitude(cufftDoubleComplex* F, int n0, int n1, int n2, double h, const double* amp,
-                      int nt, double dk, double scale, cudaStream_t s) {
-  const dim3 grid((n2 / 2 + kAmpThreads) / kAmpThreads, (n1 + kAmpRows - 1) / kAmpRows, n0);
-  k_apply_amplitude<<<grid, kAmpThreads, 0, s>>>(F, n0, n1, n2, h, amp, nt, dk, scale);
+void launch_amplitude(cufftDoubleComplex* F, int n0, int n1, int n2, bool half_x, double h,
+                      const double* amp, int nt, double dk, double scale, cudaStream_t s) {
+  const int row = half_x ? n2 : n2 / 2 + 1, planes = half_x ? n0 / 2 + 1 : n0;
+  const dim3 grid((row + kAmpThreads - 1) / kAmpThreads, (n1 + kAmpRows - 1) / kAmpRows, planes);
+  k_apply_amplitude<<<grid, kAmpThreads, 0, s>>>(F, n0, n1, n2, half_x ? 1 : 0, h, amp, nt, dk, scale);
 }
 
 int grid_for(long long work) {
@@ -297,7 +307,7 @@ mg_status convolve_grid(const int N[3], double h, const double* amp, int nt, dou
       cufftExecD2Z(fwd, R, F) != CUFFT_SUCCESS) {
     st = MG_ECUDA;
   } else {
-    launch_amplitude(F, N[0], N[1], N[2], h, amp, nt, dk, 1.0 / (ntot * h * sqrt(h)), s);
+    launch_amplitude(F, N[0], N[1], N[2], false, h, amp, nt, dk, 1.0 / (ntot * h * sqrt(h)), s);
     if (cudaGetLastError() != cudaSuccess || cufftExecZ2D(inv, F, R) != CUFFT_SUCCESS)
       st = MG_ECUDA;
   }
@@ -316,8 +326,11 @@ struct mg_field {
   int nt = 0;
   double* amp = nullptr;             // device copy of the table
   cufftDoubleComplex* F = nullptr;   // half spectrum
-  cufftHandle fwd = 0, inv = 0;
-  bool have_fwd = false, have_inv = false;
+  // half spectrum along z: 3D real transforms; along x (half_x): real transforms along x
+  // and complex 2D ones of the planes
+  bool half_x = false;
+  cufftHandle fwd = 0, inv = 0, planes = 0;
+  bool have_fwd = false, have_inv = false, have_planes = false;
   std::string err;
 };
 
@@ -347,7 +360,8 @@ mg_status mg_field_create(int n0, int n1, int n2, double h, const double* amp, i
   g->h = h;
   g->dk = dk;
   g->nt = nt;
-  const size_t nspec = (size_t)n0 * n1 * (n2 / 2 + 1);
+  g->half_x = n2 % 2 == 1 && n0 % 2 == 0;
+  const size_t nspec = g->half_x ? (size_t)(n0 / 2 + 1) * n1 * n2 : (size_t)n0 * n1 * (n2 / 2 + 1);
   mg_status st = MG_OK;
   if (cudaMalloc(&g->amp, nt * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&g->F, nspec * sizeof(cufftDoubleComplex)) != cudaSuccess) {
@@ -355,14 +369,20 @@ mg_status mg_field_create(int n0, int n1, int n2, double h, const double* amp, i
   } else if (cudaMemcpy(g->amp, amp, nt * sizeof(double), cudaMemcpyHostToDevice) !=
              cudaSuccess) {
     st = MG_ECUDA;
-  } else if (cufftPlan3d(&g->fwd, n0, n1, n2, CUFFT_D2Z) != CUFFT_SUCCESS) {
-    st = MG_ECUDA;
+  } else if (g->half_x) {
+    int nx[1] = {n0}, yz[2] = {n1, n2}, half[1] = {n0 / 2 + 1};
+    const int plane = n1 * n2;
+    g->have_fwd = cufftPlanMany(&g->fwd, 1, nx, nx, plane, 1, half, plane, 1, CUFFT_D2Z, plane) ==
+                  CUFFT_SUCCESS;
+    g->have_inv = cufftPlanMany(&g->inv, 1, nx, half, plane, 1, nx, plane, 1, CUFFT_Z2D, plane) ==
+                  CUFFT_SUCCESS;
+    g->have_planes = cufftPlanMany(&g->planes, 2, yz, nullptr, 1, 0, nullptr, 1, 0, CUFFT_Z2Z,
+                                   half[0]) == CUFFT_SUCCESS;
+    if (!g->have_fwd || !g->have_inv || !g->have_planes) st = MG_ECUDA;
   } else {
-    g->have_fwd = true;
-    if (cufftPlan3d(&g->inv, n0, n1, n2, CUFFT_Z2D) != CUFFT_SUCCESS)
-      st = MG_ECUDA;
-    else
-      g->have_inv = true;
+    g->have_fwd = cufftPlan3d(&g->fwd, n0, n1, n2, CUFFT_D2Z) == CUFFT_SUCCESS;
+    g->have_inv = cufftPlan3d(&g->inv, n0, n1, n2, CUFFT_Z2D) == CUFFT_SUCCESS;
+    if (!g->have_fwd || !g->have_inv) st = MG_ECUDA;
   }
   if (st != MG_OK) {
     mg_field_destroy(g);
@@ -375,21 +395,24 @@ mg_status mg_field_create(int n0, int n1, int n2, double h, const double* amp, i
 mg_status mg_field_convolve(mg_field* g, const double* noise, double* delta, void* cuda_stream) {
   if (!g || !noise || !delta) return MG_EINVAL;
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  if (cufftSetStream(g->fwd, s) != CUFFT_SUCCESS || cufftSetStream(g->inv, s) != CUFFT_SUCCESS) {
+  if (cufftSetStream(g->fwd, s) != CUFFT_SUCCESS || cufftSetStream(g->inv, s) != CUFFT_SUCCESS ||
+      (g->half_x && cufftSetStream(g->planes, s) != CUFFT_SUCCESS)) {
     g->err = "cufftSetStream failed";
     return MG_ECUDA;
   }
-  if (cufftExecD2Z(g->fwd, const_cast<double*>(noise), g->F) != CUFFT_SUCCESS) {
+  if (cufftExecD2Z(g->fwd, const_cast<double*>(noise), g->F) != CUFFT_SUCCESS ||
+      (g->half_x && cufftExecZ2Z(g->planes, g->F, g->F, CUFFT_FORWARD) != CUFFT_SUCCESS)) {
     g->err = "forward transform failed";
     return MG_ECUDA;
   }
   const double scale = 1.0 / ((double)g->n[0] * g->n[1] * g->n[2]);
-  launch_amplitude(g->F, g->n[0], g->n[1], g->n[2], g->h, g->amp, g->nt, g->dk, scale, s);
+  launch_amplitude(g->F, g->n[0], g->n[1], g->n[2], g->half_x, g->h, g->amp, g->nt, g->dk, scale, s);
   if (cudaGetLastError() != cudaSuccess) {
     g->err = "amplitude kernel launch failed";
     return MG_ECUDA;
   }
-  if (cufftExecZ2D(g->inv, g->F, delta) != CUFFT_SUCCESS) {
+  if ((g->half_x && cufftExecZ2Z(g->planes, g->F, g->F, CUFFT_INVERSE) != CUFFT_SUCCESS) ||
+      cufftExecZ2D(g->inv, g->F, delta) != CUFFT_SUCCESS) {
     g->err = "inverse transform failed";
     return MG_ECUDA;
   }
@@ -550,6 +573,7 @@ mg_status mg_field_destroy(mg_field* g) {
   if (!g) return MG_OK;
   if (g->have_fwd) cufftDestroy(g->fwd);
   if (g->have_inv) cufftDestroy(g->inv);
+  if (g->have_planes) cufftDestroy(g->planes);
   cudaFree(g->F);
   cudaFree(g->amp);
   delete g;
