@@ -30,6 +30,10 @@
 namespace mgk {
 
 constexpr unsigned kFxMinExp = 96;
+// Order-6 half-sweeps of more cells align 4 of the 18 neighbours on the FP64 pipe
+// (fx_align_cvt).  One V-cycle, without / with: a base and two nests of 64^3 287 / 301 us (the
+// conversions' latency), 80^3 466 / 456, 128^3 1007 / 973; a periodic 192^3 level 988 / 937.
+constexpr long long kFxCvtMinCells = 1ll << 18;
 // A value is its aligned integer times 2^(e - kFxBias), e the largest biased exponent:
 // a mantissa of 53 bits (value = mantissa 2^(e - 1075)) is shifted left by 6.
 constexpr int kFxBias = 1081;
@@ -56,6 +60,19 @@ __device__ __forceinline__ long long fx_align(double v, unsigned key) {
   unsigned s;  // the sign in every bit (prmt's sign replication: 5% of a half-sweep)
   asm("prmt.b32 %0, %1, 0, 0xbbbb;" : "=r"(s) : "r"(hi));
   return (long long)(x ^ (((unsigned long long)s << 32) | s));
+}
+
+// The same on the FP64 pipe (rounded down: at most a unit from fx_align): the exponent moved
+// by kFxBias - e, then one conversion.  That pipe is idle most of the time while neighbours
+// are aligned: 4 of 18 this way are the fastest mix (order 6, 128^3 half-sweep: none 17.2 us,
+// 2 16.8, 4 16.0, 6 19.2), on levels large enough that throughput counts (kFxCvtMinCells).  Values that the moved exponent would leave below the normal range
+// (only possible with WIDE, e > kFxBias) round to 0 or -1 all the same.
+template <bool WIDE>
+__device__ __forceinline__ long long fx_align_cvt(double v, unsigned key) {
+  const int d = kFxBias - (int)(key >> 21);
+  const int hi = __double2hiint(v);
+  if (WIDE && ((hi >> 20) & 0x7ff) + d <= 0) return hi >> 31;
+  return __double2ll_rd(__hiloint2double(hi + (d << 20), __double2loint(v)));
 }
 
 // c * 2^(e - kFxBias) by an addition to the exponent field; c a normal constant whose
@@ -99,14 +116,25 @@ __device__ __forceinline__ long long fx_weighted(const long long (&s)[3]) {
 }
 
 // The same from the neighbours (nb[6 d .. 6 d + 5] at distance d + 1); key as for fx_align.
-template <int ORDER>
-__device__ __forceinline__ long long fx_neighbours(const double (&nb)[3 * ORDER], unsigned key) {
+template <int ORDER, bool CVT, bool WIDE>
+__device__ __forceinline__ long long fx_neighbours_by(const double (&nb)[3 * ORDER], unsigned key) {
   long long s[3] = {0, 0, 0};
 #pragma unroll
   for (int d = 0; d < ORDER / 2; ++d)
 #pragma unroll
-    for (int q = 0; q < 6; ++q) s[d] += fx_align(nb[6 * d + q], key);
+    for (int q = 0; q < 6; ++q)
+      s[d] += CVT && d == 2 && q < 4 ? fx_align_cvt<WIDE>(nb[6 * d + q], key)
+                                     : fx_align(nb[6 * d + q], key);
   return fx_weighted<ORDER>(s);
+}
+
+template <int ORDER, bool CVT = false>
+__device__ __forceinline__ long long fx_neighbours(const double (&nb)[3 * ORDER], unsigned key) {
+  if constexpr (CVT && ORDER == 6) {
+    if ((int)(key >> 21) > kFxBias) return fx_neighbours_by<ORDER, true, true>(nb, key);
+    return fx_neighbours_by<ORDER, true, false>(nb, key);
+  }
+  return fx_neighbours_by<ORDER, false, false>(nb, key);
 }
 
 // The centre's term of T (weight 3 w0), c its aligned integer.

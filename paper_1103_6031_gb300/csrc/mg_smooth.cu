@@ -28,12 +28,12 @@ constexpr int kPairX = kVPairX;  // z-pairs per block row; blockDim.y = rows (1.
 template <int ORDER, typename T>
 constexpr int smooth_min_blocks = sizeof(T) == 8 && ORDER == 6 ? 4 : 5;
 
-template <int ORDER, typename T>
+template <int ORDER, typename T, bool CVT>
 __global__ void __launch_bounds__(kPairX * 8, (smooth_min_blocks<ORDER, T>))
     k_smooth_half(Grid G, const T* __restrict__ uin, T* __restrict__ uout,
                   const T* __restrict__ f, T a_f, int colour, int periodic) {
   grid_wait();
-  smooth_half_body<ORDER, T, Ldg>(G, uin, uout, f, a_f, colour, periodic, (int)blockDim.y,
+  smooth_half_body<ORDER, T, Ldg, CVT>(G, uin, uout, f, a_f, colour, periodic, (int)blockDim.y,
                                   Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
                                       (int)threadIdx.x, (int)threadIdx.y});
 }
@@ -395,9 +395,14 @@ cudaError_t launch_smooth_half(int order, const Grid& G, const T* uin, T* uout, 
   const int pairs = (G.n2 + 1) / 2;
   dim3 grid((pairs + kPairX - 1) / kPairX, (G.n1 + rows - 1) / rows, G.n0);
   switch (order) {
-    case 2: return launch_dep(k_smooth_half<2, T>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
-    case 4: return launch_dep(k_smooth_half<4, T>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
-    case 6: return launch_dep(k_smooth_half<6, T>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
+    case 2: return launch_dep(k_smooth_half<2, T, false>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
+    case 4: return launch_dep(k_smooth_half<4, T, false>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
+    case 6:
+      if constexpr (sizeof(T) == 8) {
+        if ((long long)G.n0 * G.n1 * G.n2 > kFxCvtMinCells)
+          return launch_dep(k_smooth_half<6, T, true>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
+      }
+      return launch_dep(k_smooth_half<6, T, false>, grid, block, 0, s, G, uin, uout, f, T(a_f), colour, periodic);
     default: return cudaErrorInvalidValue;
   }
 }

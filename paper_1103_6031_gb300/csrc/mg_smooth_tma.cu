@@ -118,7 +118,7 @@ __device__ __forceinline__ void tma_load_plane(void* dst, const CUtensorMap* tm,
       : "memory");
 }
 
-template <int ORDER, typename T>
+template <int ORDER, typename T, bool CVT>
 __global__ void __launch_bounds__(32 * kTY)
     k_smooth_half_tma(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tf,
                       Grid G, T* __restrict__ uout, T a_f, int colour, int periodic,
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(32 * kTY)
             nb[6 * d - 1] = comp(q[tc + d]);
           }
           const T v =
-              relax<ORDER, T>(nb, a_f * tiles[(tc % kSlots) * TL::stride + fown + upd]);
+              relax<ORDER, T, CVT>(nb, a_f * tiles[(tc % kSlots) * TL::stride + fown + upd]);
           T* o = orow + s * sx;
           const int i = i0 + s;
           const bool img = periodic && (yz_face || i < G.g || i >= G.n0 - G.g);
@@ -306,14 +306,20 @@ cudaError_t launch_order(const Grid& G, const CUtensorMap* tin, const CUtensorMa
   typedef Tile<T, ORDER / 2> TL;
   dim3 block(32, kTY, 1);
   dim3 grid((G.n2 + kTZ - 1) / kTZ, (G.n1 + kTY - 1) / kTY, (G.n0 + kLX - 1) / kLX);
-  k_smooth_half_tma<ORDER, T><<<grid, block, TL::smem, s>>>(*tin, *tf, G, uout, a_f, colour,
-                                                            periodic, err, extra_tx);
+  // the float64 sums of launch_smooth_half on a level of this size
+  constexpr bool kMayCvt = ORDER == 6 && sizeof(T) == 8;
+  if (kMayCvt && (long long)G.n0 * G.n1 * G.n2 > kFxCvtMinCells)
+    k_smooth_half_tma<ORDER, T, kMayCvt><<<grid, block, TL::smem, s>>>(
+        *tin, *tf, G, uout, a_f, colour, periodic, err, extra_tx);
+  else
+    k_smooth_half_tma<ORDER, T, false><<<grid, block, TL::smem, s>>>(
+        *tin, *tf, G, uout, a_f, colour, periodic, err, extra_tx);
   return cudaGetLastError();
 }
 
-template <int ORDER, typename T>
+template <int ORDER, typename T, bool CVT = false>
 cudaError_t set_smem_attr() {
-  return cudaFuncSetAttribute(k_smooth_half_tma<ORDER, T>,
+  return cudaFuncSetAttribute(k_smooth_half_tma<ORDER, T, CVT>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<T, ORDER / 2>::smem);
 }
 
@@ -330,6 +336,7 @@ cudaError_t prepare_smooth_tma() {
   if ((r = set_smem_attr<2, double>()) != cudaSuccess) e = r;
   if ((r = set_smem_attr<4, double>()) != cudaSuccess) e = r;
   if ((r = set_smem_attr<6, double>()) != cudaSuccess) e = r;
+  if ((r = set_smem_attr<6, double, true>()) != cudaSuccess) e = r;
   return e;
 }
 

@@ -119,13 +119,13 @@ __device__ __forceinline__ unsigned neighbour_key(const double (&nb)[3 * ORDER])
 // (mg_fixed.cuh): 3 FP64 instructions per update instead of 19.  Measured on GB300, order 6,
 // warm L2, 128^3 nest: 41.7 -> 17.6 us per half-sweep (64^3: 6.9 -> 3.9, 32^3: 3.0 -> 2.2);
 // order 4: 29.2 -> 12.8; order 2: 16.5 -> 8.7.
-template <int ORDER, typename T>
+template <int ORDER, typename T, bool CVT = false>
 __device__ __forceinline__ T relax(const T (&nb)[3 * ORDER], T acc) {
   constexpr double wc = 3.0 * Lap<ORDER>::w0;
   if constexpr (sizeof(T) == 8) {
     const unsigned key = neighbour_key<ORDER>(nb);
     if (fx_in_range(key))
-      return fma(fx_scale(-FxUnit<ORDER>::v / wc, key), (double)fx_neighbours<ORDER>(nb, key), acc);
+      return fma(fx_scale(-FxUnit<ORDER>::v / wc, key), (double)fx_neighbours<ORDER, CVT>(nb, key), acc);
   }
   acc = fma(T(-Lap<ORDER>::w1 / wc), sum6(nb), acc);
   if constexpr (ORDER >= 4) acc = fma(T(-Lap<ORDER>::w2 / wc), sum6(nb + 6), acc);

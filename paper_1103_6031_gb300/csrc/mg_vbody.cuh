@@ -27,7 +27,7 @@ constexpr int kVPairX = 32;
 // other values fixed at their pre-half-sweep values.  Reads uin, writes every interior
 // cell of uout (colour c updated, the other colour copied), one z-pair per thread;
 // blocks of kVPairX x rows threads.
-template <int ORDER, typename T, typename LD>
+template <int ORDER, typename T, typename LD, bool CVT = false>
 __device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restrict__ uin,
                                                T* __restrict__ uout, const T* __restrict__ f,
                                                T a_f, int colour, int periodic, int i, int j,
@@ -47,7 +47,7 @@ __device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restric
   // u = (h^2 f - sum_off w u_nb) / w_centre
   T nb[3 * ORDER];
   load_neighbours<ORDER, T, LD>(uin, p, sy, sx, nb);
-  const T v = relax<ORDER, T>(nb, a_f * LD::ld(f + p));
+  const T v = relax<ORDER, T, CVT>(nb, a_f * LD::ld(f + p));
   if (pair) {
     typedef typename Vec2<T>::type V2;
     V2 out;
@@ -66,14 +66,14 @@ __device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restric
   }
 }
 
-template <int ORDER, typename T, typename LD>
+template <int ORDER, typename T, typename LD, bool CVT = false>
 __device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restrict__ uin,
                                                  T* __restrict__ uout, const T* __restrict__ f,
                                                  T a_f, int colour, int periodic, int rows, Blk b) {
   const int j = b.by * rows + b.ty;
   const int k0 = 2 * (b.bx * kVPairX + b.tx);
   if (j >= G.n1 || k0 >= G.n2) return;
-  smooth_pair_at<ORDER, T, LD>(G, uin, uout, f, a_f, colour, periodic, b.bz, j, k0);
+  smooth_pair_at<ORDER, T, LD, CVT>(G, uin, uout, f, a_f, colour, periodic, b.bz, j, k0);
 }
 
 // ---- residual + restriction: one thread per covered parent cell ---------------------
