@@ -151,7 +151,8 @@ cudaError_t launch_coarsest(const Grid& G, const float* f, float* u, const doubl
 // partial sums over uncovered interior cells of level G: [2*b] = sum r^2, [2*b+1] = sum f^2
 // (times vol), r = f - L u; blocks = number of partial slots written.
 // With r32 != nullptr the residual of every interior cell is also written to r32
-// (float32, same layout) as the source of the mixed-precision correction equation.
+// (float32, same layout) as the source of the mixed-precision correction equation, and
+// [2*b+1] is written only by calls with u == nullptr (r = f), once per solve.
 cudaError_t launch_norm_partial(int order, const Grid& G, const double* u, const double* f,
                                 double invh2, double vol, Int3 clo, Int3 chi, double* partial,
                                 int blocks, float* r32, cudaStream_t s);

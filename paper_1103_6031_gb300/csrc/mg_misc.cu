@@ -81,7 +81,20 @@ constexpr int kRedBlock = 256;
 // for both.  The stencil sums run on the integer pipe (mg_fixed.cuh) except in MIXED, where
 // the last bits of r decide float32 roundings of the whole correction cycle: with them
 // changed, displacements of the deepest nest of a 5-level hierarchy moved by 1.1e-9
-// relative, so that mode keeps the FP64 operations one by one.
+// relative, so that mode keeps the FP64 operations one by one and sheds what does not touch
+// them: the source's sum is left from the solve's first call (u = nullptr, the only one to
+// form it), and r is rounded to float32 on the integer pipe (FP64-bound: 91 us per 128^3 level).
+//
+// r rounded to nearest even; results that are not normal floats by the conversion instruction.
+__device__ __forceinline__ float to_float(double r) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(r);
+  const unsigned long long m = b & 0x7fffffffffffffffull;
+  const unsigned q = (unsigned)((m + 0x0fffffffull + ((m >> 29) & 1)) >> 29);  // exponent bias 1023
+  const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+  if (e - 897u >= 253u) return (float)r;
+  return __uint_as_float((q - (896u << 23)) | ((unsigned)(b >> 32) & 0x80000000u));
+}
+
 template <int ORDER, bool MIXED>
 __global__ void __launch_bounds__(kRedBlock)
     k_norm_partial(Grid G, const double* __restrict__ u, const double* __restrict__ f,
@@ -107,16 +120,16 @@ __global__ void __launch_bounds__(kRedBlock)
       const double r = u ? add_lap_h2<ORDER, double, Ldg, !MIXED>(u, p, sy, sx, __ldg(u + p),
                                                                  -invh2, fv)
                          : fv;
-      if (MIXED) r32[p] = (float)r;
+      if (MIXED) r32[p] = to_float(r);
       rr = fma(r, r, rr);
-      ff = fma(fv, fv, ff);
+      if (!MIXED || !u) ff = fma(fv, fv, ff);
     }
   }
   block_sum2<kRedBlock>(rr, ff);
   if (threadIdx.x == 0) {
     const int b = blockIdx.y * gridDim.x + blockIdx.x;
     partial[2 * b] = rr * vol;
-    partial[2 * b + 1] = ff * vol;
+    if (!MIXED || !u) partial[2 * b + 1] = ff * vol;
   }
 }
 
