@@ -826,8 +826,14 @@ mg_status vcycle(mg_hierarchy* h, int l) {
      launch_fas_source<T>(order, P.G, pb.u[pb.cur], pb.ffas, 1.0 / (P.geo.h * P.geo.h), L.off,
                           L.cn, h->s));
   ST(vcycle<T>(h, l - 1));
-  if (!L.periodic) ST(tangential<T>(h, l));
   b.ghosts_ready = false;
+  if (!L.periodic) {
+    KL(MG_K_PROLONG, cells_of(L.G),
+       launch_cf_tangential<T>(order, L.G, P.G, pb.u[pb.cur], L.off, L.fs, h->w, L.geo.h,
+                               1.0 / P.geo.h, fold_ghosts<T>(h), b.inter, b.fc_unc, h->s,
+                               b.u[b.cur], b.ubar, L.cn));
+    return smooth<T>(h, l, h->cfg.nu2);
+  }
   KL(MG_K_PROLONG, cells_of(L.G),
      launch_prolong<T>(L.G, b.u[b.cur], P.G, pb.u[pb.cur], b.ubar, L.off, L.cn,
                        L.periodic ? 1 : 0, h->s));

@@ -68,11 +68,11 @@ struct TangFold {
 // value is the same chain of fmas either way.  FP64-bound in float64: 128^3 nest, order 6,
 // 23.2 us before (cold).
 template <int ORDER, typename T, bool FOLD>
-__global__ void __launch_bounds__(kTangThreads)
-    k_cf_tangential(Grid F, Grid P, const T* __restrict__ pu, Int3 off, FaceSet fs, TangTiles tt,
-                    CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
-                    T* __restrict__ fc_unc) {
-  grid_wait();
+__device__ __forceinline__ void tangential_tile(const Grid& F, const Grid& P,
+                                                const T* __restrict__ pu, Int3 off,
+                                                const FaceSet& fs, const TangTiles& tt,
+                                                const CfW<T>& w, const TangFold& fo, T invH,
+                                                T* __restrict__ inter, T* __restrict__ fc_unc) {
   constexpr int half = ORDER / 2;
   constexpr int RB = kTangB + ORDER;
   typedef typename Vec2<T>::type V2;
@@ -194,6 +194,35 @@ __global__ void __launch_bounds__(kTangThreads)
   }
 }
 
+template <int ORDER, typename T, bool FOLD>
+__global__ void __launch_bounds__(kTangThreads)
+    k_cf_tangential(Grid F, Grid P, const T* __restrict__ pu, Int3 off, FaceSet fs, TangTiles tt,
+                    CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
+                    T* __restrict__ fc_unc) {
+  grid_wait();
+  tangential_tile<ORDER, T, FOLD>(F, P, pu, off, fs, tt, w, fo, invH, inter, fc_unc);
+}
+
+// Tangential interpolation and prolongation of a nest, both from the parent's new values and
+// independent of each other, in one launch: the tiles of the faces first, then blocks of 32
+// z-pairs x 8 rows (gx x gy per plane).
+template <int ORDER, typename T, bool FOLD>
+__global__ void __launch_bounds__(kTangThreads)
+    k_tangential_prolong(Grid F, Grid P, const T* __restrict__ pu, Int3 off, FaceSet fs,
+                         TangTiles tt, CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
+                         T* __restrict__ fc_unc, T* __restrict__ u, const T* __restrict__ ubar,
+                         Int3 cn, int gx, int gy) {
+  grid_wait();
+  const int b = (int)blockIdx.x - tt.first[6];
+  if (b < 0) {
+    tangential_tile<ORDER, T, FOLD>(F, P, pu, off, fs, tt, w, fo, invH, inter, fc_unc);
+    return;
+  }
+  prolong_at<T, Ldg>(F, u, P, pu, ubar, off, cn, 0, b / (gx * gy),
+                     b / gx % gy * (kTangThreads / 32) + (int)(threadIdx.x >> 5),
+                     b % gx * 32 + (int)(threadIdx.x & 31));
+}
+
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
     k_cf_flux(Grid F, T* __restrict__ u, FaceSet fs, CfW<T> w, const T* __restrict__ inter,
@@ -291,36 +320,55 @@ cudaError_t launch_ghost_periodic(const Grid& G, T* u, cudaStream_t s) {
   return launch_dep(k_ghost_periodic<T>, (unsigned)((total + block - 1) / block), block, 0, s, G, u);
 }
 
+template <int ORDER, typename T, bool FOLD>
+static cudaError_t launch_tangential_as(const Grid& F, const Grid& P, const T* pu, Int3 off,
+                                        const FaceSet& fs, const CfWeights& w, double h,
+                                        double invH, T* inter, T* fc_unc, T* prolong_u,
+                                        const T* ubar, Int3 cn, cudaStream_t s) {
+  constexpr int half = ORDER / 2;
+  const CfW<T> wt = cf_weights_as<T>(w);
+  const TangTiles tt = tang_tiles(fs);
+  TangFold fo{};
+  if (FOLD) {
+    for (int m = 0; m < half; ++m)
+      for (int q = 0; q < half; ++q) fo.ncoarse[m][q] = w.ncoarse[m][q];
+    for (int sd = 0; sd < 2; ++sd) {
+      fo.a[sd] = h / w.ghost_coef[sd];
+      for (int m = 0; m < half; ++m)
+        fo.bg[sd][m] = 0.25 / w.ghost_coef[sd] * w.flux[sd == 0 ? half - 1 - m : half + m];
+    }
+  }
+  if (!prolong_u)
+    return launch_dep(k_cf_tangential<ORDER, T, FOLD>, tt.first[6], kTangThreads, 0, s, F, P, pu,
+                      off, fs, tt, wt, fo, T(invH), inter, fc_unc);
+  if constexpr (sizeof(T) == 4 || FOLD) {  // V-cycles run in float32, or in float64 folded
+    const int gx = (F.n2 / 2 + 31) / 32, gy = (F.n1 + kTangThreads / 32 - 1) / (kTangThreads / 32);
+    return launch_dep(k_tangential_prolong<ORDER, T, FOLD>, tt.first[6] + gx * gy * F.n0,
+                      kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc,
+                      prolong_u, ubar, cn, gx, gy);
+  }
+  return cudaErrorInvalidValue;
+}
+
 template <typename T>
 cudaError_t launch_cf_tangential(int order, const Grid& F, const Grid& P, const T* pu, Int3 off,
                                  const FaceSet& fs, const CfWeights& w, double h, double invH,
-                                 bool fold, T* inter, T* fc_unc, cudaStream_t s) {
-  const CfW<T> wt = cf_weights_as<T>(w);
-  const TangTiles tt = tang_tiles(fs);
-  const unsigned grid = (unsigned)tt.first[6];
-  TangFold fo{};
+                                 bool fold, T* inter, T* fc_unc, cudaStream_t s, T* prolong_u,
+                                 const T* ubar, Int3 cn) {
   if constexpr (sizeof(T) == 8) {
     if (fold) {
-      const int half = order / 2;
-      for (int m = 0; m < half; ++m)
-        for (int q = 0; q < half; ++q) fo.ncoarse[m][q] = w.ncoarse[m][q];
-      for (int sd = 0; sd < 2; ++sd) {
-        fo.a[sd] = h / w.ghost_coef[sd];
-        for (int m = 0; m < half; ++m)
-          fo.bg[sd][m] = 0.25 / w.ghost_coef[sd] * w.flux[sd == 0 ? half - 1 - m : half + m];
-      }
       switch (order) {
-        case 2: return launch_dep(k_cf_tangential<2, T, true>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
-        case 4: return launch_dep(k_cf_tangential<4, T, true>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
-        case 6: return launch_dep(k_cf_tangential<6, T, true>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
+        case 2: return launch_tangential_as<2, T, true>(F, P, pu, off, fs, w, h, invH, inter, fc_unc, prolong_u, ubar, cn, s);
+        case 4: return launch_tangential_as<4, T, true>(F, P, pu, off, fs, w, h, invH, inter, fc_unc, prolong_u, ubar, cn, s);
+        case 6: return launch_tangential_as<6, T, true>(F, P, pu, off, fs, w, h, invH, inter, fc_unc, prolong_u, ubar, cn, s);
         default: return cudaErrorInvalidValue;
       }
     }
   }
   switch (order) {
-    case 2: return launch_dep(k_cf_tangential<2, T, false>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
-    case 4: return launch_dep(k_cf_tangential<4, T, false>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
-    case 6: return launch_dep(k_cf_tangential<6, T, false>, grid, kTangThreads, 0, s, F, P, pu, off, fs, tt, wt, fo, T(invH), inter, fc_unc);
+    case 2: return launch_tangential_as<2, T, false>(F, P, pu, off, fs, w, h, invH, inter, fc_unc, prolong_u, ubar, cn, s);
+    case 4: return launch_tangential_as<4, T, false>(F, P, pu, off, fs, w, h, invH, inter, fc_unc, prolong_u, ubar, cn, s);
+    case 6: return launch_tangential_as<6, T, false>(F, P, pu, off, fs, w, h, invH, inter, fc_unc, prolong_u, ubar, cn, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -418,7 +466,8 @@ cudaError_t launch_cf_edges(int order, const Grid& F, T* u, const Grid& P, const
   template cudaError_t launch_ghost_periodic<T>(const Grid&, T*, cudaStream_t);               \
   template cudaError_t launch_cf_tangential<T>(int, const Grid&, const Grid&, const T*, Int3, \
                                                const FaceSet&, const CfWeights&, double,      \
-                                               double, bool, T*, T*, cudaStream_t);           \
+                                               double, bool, T*, T*, cudaStream_t, T*,        \
+                                               const T*, Int3);                               \
   template cudaError_t launch_cf_flux<T>(int, const Grid&, T*, const FaceSet&,                \
                                          const CfWeights&, const T*, const T*, double,        \
                                          double, double, int, cudaStream_t);                  \

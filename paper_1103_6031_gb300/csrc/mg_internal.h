@@ -124,10 +124,14 @@ cudaError_t prepare_smooth_tma();
 // ---- kernels: ghost zones (mg_ghost.cu) ----
 template <typename T>
 cudaError_t launch_ghost_periodic(const Grid& G, T* u, cudaStream_t s);
+// With prolong_u the launch also prolongates into the nest's u (launch_prolong's pu, ubar,
+// cn).
 template <typename T>
 cudaError_t launch_cf_tangential(int order, const Grid& F, const Grid& P, const T* pu, Int3 off,
                                  const FaceSet& fs, const CfWeights& w, double h, double invH,
-                                 bool fold, T* inter, T* fc_unc, cudaStream_t s);
+                                 bool fold, T* inter, T* fc_unc, cudaStream_t s,
+                                 T* prolong_u = nullptr, const T* ubar = nullptr,
+                                 Int3 cn = Int3{0, 0, 0});
 template <typename T>
 cudaError_t launch_cf_flux(int order, const Grid& F, T* u, const FaceSet& fs, const CfWeights& w,
                            const T* inter, const T* fc_unc, double h, double invh, double invH,

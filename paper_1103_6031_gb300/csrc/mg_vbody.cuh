@@ -129,12 +129,9 @@ __device__ __forceinline__ void fas_source_body(const Grid& P, const T* __restri
 
 // ---- prolongation-correction: u += inject(parent u - ubar), one thread per z-pair ----
 template <typename T, typename LD>
-__device__ __forceinline__ void prolong_body(const Grid& F, T* __restrict__ u, const Grid& P,
-                                             const T* __restrict__ pu, const T* __restrict__ ubar,
-                                             Int3 off, Int3 cn, int periodic, Blk b) {
-  const int t = b.bx * 32 + b.tx;
-  const int j = b.by * 4 + b.ty;
-  const int i = b.bz;
+__device__ __forceinline__ void prolong_at(const Grid& F, T* __restrict__ u, const Grid& P,
+                                           const T* __restrict__ pu, const T* __restrict__ ubar,
+                                           Int3 off, Int3 cn, int periodic, int i, int j, int t) {
   const int k0 = 2 * t;
   if (j >= F.n1 || k0 >= F.n2) return;
   const int ic = i >> 1, jc = j >> 1, kc = t;
@@ -150,6 +147,13 @@ __device__ __forceinline__ void prolong_body(const Grid& F, T* __restrict__ u, c
     if (k0 + 1 < F.n2) write_pair_images<T>(F, u, i, j, k0, v.x, v.y);
     else write_images<T>(F, u, i, j, k0, v.x);
   }
+}
+
+template <typename T, typename LD>
+__device__ __forceinline__ void prolong_body(const Grid& F, T* __restrict__ u, const Grid& P,
+                                             const T* __restrict__ pu, const T* __restrict__ ubar,
+                                             Int3 off, Int3 cn, int periodic, Blk b) {
+  prolong_at<T, LD>(F, u, P, pu, ubar, off, cn, periodic, b.bz, b.by * 4 + b.ty, b.bx * 32 + b.tx);
 }
 
 // ---- periodic ghost shell: element t of the shell takes its interior image ----------
