@@ -51,6 +51,10 @@ struct Bufs {
   // interpolants (left by a half-sweep that wrote them).  Restriction into the cells that a
   // child covers does not touch the order layers they depend on (the validated margin).
   bool ghosts_ready = false;
+  // The FAS source of the cells [fas_lo, fas_hi) is still to be added to ffas, by the level's
+  // next half-sweep (set by the restriction into them).
+  bool fas_pending = false;
+  Int3 fas_lo{0, 0, 0}, fas_hi{0, 0, 0};
   // TMA-staged smoother: tensor maps of u[0], u[1] and ffas
   bool tma = false;
   CUtensorMap tm[2];
@@ -709,6 +713,7 @@ mg_status half_sweep(mg_hierarchy* h, int l, int colour) {
   Bufs<T>& b = bufs<T>(L);
   ST(ghost_fill<T>(h, l, false));
   const double a_f = L.geo.h * L.geo.h / centre_weight(h->cfg.order);
+  const double invh2 = 1.0 / (L.geo.h * L.geo.h);
   if (recording<T>(h)) {
     // the plain smoother's arithmetic (bit-identical to the TMA-staged one), 32 x 4
     // threads per block
@@ -729,12 +734,24 @@ mg_status half_sweep(mg_hierarchy* h, int l, int colour) {
     KL(MG_K_SMOOTH, (cells_of(L.G) + 1) / 2,
        launch_smooth_faces<T>(h->cfg.order, L.G, b.u[b.cur], b.u[1 - b.cur], b.ffas, a_f, colour,
                               !(h->cfg.flags & MG_FLAG_PAIR_SMOOTHER), L.fs, h->w, b.inter,
-                              b.fc_unc, L.geo.h, 1.0 / h->L[l - 1].geo.h, h->s));
+                              b.fc_unc, L.geo.h, 1.0 / h->L[l - 1].geo.h, b.fas_pending, invh2,
+                              b.fas_lo, b.fas_hi, h->s));
     b.cur ^= 1;
     b.ghosts_ready = true;
+    b.fas_pending = false;
     return MG_OK;
   }
   b.ghosts_ready = false;
+  if constexpr (std::is_same<T, float>::value) {
+    if (b.fas_pending) {
+      KL(MG_K_SMOOTH, (cells_of(L.G) + 1) / 2,
+         launch_smooth_fas(h->cfg.order, L.G, b.u[b.cur], b.u[1 - b.cur], b.ffas, a_f, colour,
+                           L.periodic ? 1 : 0, invh2, b.fas_lo, b.fas_hi, h->s));
+      b.cur ^= 1;
+      b.fas_pending = false;
+      return MG_OK;
+    }
+  }
   if (b.tma)
     KL(MG_K_SMOOTH, (cells_of(L.G) + 1) / 2,
        launch_smooth_half_tma<T>(h->cfg.order, L.G, &b.tm[b.cur], &b.tm_f, b.u[1 - b.cur], a_f,
@@ -822,9 +839,18 @@ mg_status vcycle(mg_hierarchy* h, int l) {
      launch_residual_restrict<T>(order, L.G, b.u[b.cur], b.ffas, 1.0 / (L.geo.h * L.geo.h), P.G,
                                  pb.u[pb.cur], pb.ffas, b.ubar, L.off, L.cn,
                                  P.periodic ? 1 : 0, h->s));
-  KL(MG_K_FAS, cells_of(L.cn),
-     launch_fas_source<T>(order, P.G, pb.u[pb.cur], pb.ffas, 1.0 / (P.geo.h * P.geo.h), L.off,
-                          L.cn, h->s));
+  // float32: left to the parent's first half-sweep where there is one that can take it (a
+  // V-cycle of a base and two nests of 48^3 131.7 -> 123.9 us, of 128^3 402 -> 388).  float64
+  // gains nothing: the second cell's sums cost what the launch did (48^3 225 -> 231, 128^3 960).
+  if (sizeof(T) == 4 && l - 1 > 0 && h->cfg.nu1 > 0 && !pb.tma) {
+    pb.fas_pending = true;
+    pb.fas_lo = L.off;
+    pb.fas_hi = Int3{L.off.x + L.cn.x, L.off.y + L.cn.y, L.off.z + L.cn.z};
+  } else {
+    KL(MG_K_FAS, cells_of(L.cn),
+       launch_fas_source<T>(order, P.G, pb.u[pb.cur], pb.ffas, 1.0 / (P.geo.h * P.geo.h), L.off,
+                            L.cn, h->s));
+  }
   ST(vcycle<T>(h, l - 1));
   b.ghosts_ready = false;
   if (!L.periodic) {

@@ -79,11 +79,16 @@ cudaError_t launch_smooth_half(int order, const Grid& G, const T* uin, T* uout, 
 constexpr long long kFaceFusedMaxCells = 1ll << 18;
 // The half-sweep of a nest followed by the coarse-fine ghosts of its result (float64: folded,
 // after launch_cf_tangential with fold = true); h, invH: own spacing, 1 / parent spacing.
+// fas (float32): f of the cells [lo, hi) gains invh2 h^2 L u first (launch_fas_source).
 template <typename T>
-cudaError_t launch_smooth_faces(int order, const Grid& G, const T* uin, T* uout, const T* f,
-                                double a_f, int colour, bool quad, const FaceSet& fs,
-                                const CfWeights& w, const T* inter, const T* fc_unc, double h,
-                                double invH, cudaStream_t s);
+cudaError_t launch_smooth_faces(int order, const Grid& G, const T* uin, T* uout, T* f, double a_f,
+                                int colour, bool quad, const FaceSet& fs, const CfWeights& w,
+                                const T* inter, const T* fc_unc, double h, double invH, bool fas,
+                                double invh2, Int3 lo, Int3 hi, cudaStream_t s);
+// launch_fas_source on the cells [lo, hi), then the half-sweep; rows of even length.
+cudaError_t launch_smooth_fas(int order, const Grid& G, const float* uin, float* uout, float* f,
+                              double a_f, int colour, int periodic, double invh2, Int3 lo, Int3 hi,
+                              cudaStream_t s);
 template <typename T>
 cudaError_t launch_residual_restrict(int order, const Grid& F, const T* u, const T* f,
                                      double invh2, const Grid& P, T* pu, T* pfas, T* ubar,

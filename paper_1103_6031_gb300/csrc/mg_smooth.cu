@@ -38,6 +38,21 @@ __global__ void __launch_bounds__(kPairX * 8, (smooth_min_blocks<ORDER, T>))
                                       (int)threadIdx.x, (int)threadIdx.y});
 }
 
+// The first half-sweep of a level after a restriction into it, with the FAS source of the
+// restricted cells (smooth_fas_pair_at): one launch instead of two.
+template <int ORDER>
+__global__ void __launch_bounds__(128, 8)
+    k_smooth_fas(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
+                 float* __restrict__ f, float a_f, float invh2, FasBox box, int colour,
+                 int periodic) {
+  grid_wait();
+  const int j = blockIdx.y * 4 + threadIdx.y;
+  const int k0 = 2 * (blockIdx.x * 32 + threadIdx.x);
+  if (j >= G.n1 || k0 >= G.n2) return;
+  smooth_fas_pair_at<ORDER, float, Ldg>(G, uin, uout, f, a_f, invh2, box, colour, periodic,
+                                        blockIdx.z, j, k0);
+}
+
 // float32 rows whose length is a multiple of 4: one z-quad per thread (elements k0 ..
 // k0 + 3, 16-byte aligned: the first interior element of a row sits at index 4 and the
 // row pitch is a multiple of 8), updating the quad's two cells of colour c.  Every
@@ -140,11 +155,14 @@ __global__ void __launch_bounds__(256, 4)
 // goes away is nearly all latency on small levels (kFaceFusedMaxCells).
 constexpr int kFacesThreads = 128;
 
-template <int ORDER, typename T, int VEC>
-__global__ void __launch_bounds__(kFacesThreads, (smooth_min_blocks<ORDER, T>) < 5 || VEC == 4 ? 8 : 10)
-    k_smooth_faces(Grid G, const T* __restrict__ uin, T* __restrict__ uout,
-                   const T* __restrict__ f, T a_f, int colour, int face_blocks, int gx, int gy,
-                   int qx, int by, FaceArgs<T> fa) {
+// FAS (VEC = 2): the plain part is smooth_fas_pair_at, whose cells with a new f lie deeper
+// than the face columns.
+template <int ORDER, typename T, int VEC, bool FAS>
+__global__ void __launch_bounds__(kFacesThreads,
+                                  FAS ? 5 : ((smooth_min_blocks<ORDER, T>) < 5 || VEC == 4 ? 8 : 10))
+    k_smooth_faces(Grid G, const T* __restrict__ uin, T* __restrict__ uout, T* f, T a_f, int colour,
+                   int face_blocks, int gx, int gy, int qx, int by, T invh2, FasBox box,
+                   FaceArgs<T> fa) {
   grid_wait();
   const int b = (int)blockIdx.x - face_blocks;
   if (b >= 0) {
@@ -152,7 +170,10 @@ __global__ void __launch_bounds__(kFacesThreads, (smooth_min_blocks<ORDER, T>) <
     const int j = b / gx % gy * by + ty;
     const int k0 = VEC * (b % gx * qx + tx);
     if (ty >= by || j >= G.n1 || k0 >= G.n2) return;
-    if constexpr (VEC == 4)
+    if constexpr (FAS)
+      smooth_fas_pair_at<ORDER, T, Ldg>(G, uin, uout, f, a_f, invh2, box, colour, 0,
+                                               b / (gx * gy), j, k0);
+    else if constexpr (VEC == 4)
       smooth_quad_at<ORDER>(G, uin, uout, f, a_f, colour, 0, b / (gx * gy), j, k0);
     else
       smooth_pair_at<ORDER, T, Ldg>(G, uin, uout, f, a_f, colour, 0, b / (gx * gy), j, k0);
@@ -176,7 +197,7 @@ __global__ void __launch_bounds__(kFacesThreads, (smooth_min_blocks<ORDER, T>) <
       const long long p = c.in0 + q * c.step;
       T nb[3 * ORDER];
       load_neighbours<ORDER, T>(uin, p, G.Zp, G.Y * G.Zp, nb);
-      cells[q][lane] = relax<ORDER, T>(nb, a_f * __ldg(f + p));
+      cells[q][lane] = relax<ORDER, T>(nb, a_f * f[p]);
     } else if (warp == kFacesThreads / 32 - 1) {
 #pragma unroll
       for (int q = 0; q < ORDER / 2; ++q)
@@ -407,39 +428,64 @@ cudaError_t launch_smooth_half(int order, const Grid& G, const T* uin, T* uout, 
   }
 }
 
-template <int ORDER, typename T, int VEC>
-static cudaError_t launch_faces_vec(const Grid& G, const T* uin, T* uout, const T* f, double a_f,
-                                    int colour, const FaceArgs<T>& fa, cudaStream_t s) {
+template <int ORDER, typename T, int VEC, bool FAS = false>
+static cudaError_t launch_faces_vec(const Grid& G, const T* uin, T* uout, T* f, double a_f,
+                                    int colour, double invh2, const FasBox& box,
+                                    const FaceArgs<T>& fa, cudaStream_t s) {
   // blocks of qx groups of a row x by rows
   const int groups = (G.n2 + VEC - 1) / VEC;
   const int qx = groups < 32 ? groups : 32;
   const int by = kFacesThreads / qx < G.n1 ? kFacesThreads / qx : G.n1;
   const int gx = (groups + qx - 1) / qx, gy = (G.n1 + by - 1) / by;
   const int faces = (int)((4 * fa.fs.ebase[6] + 31) / 32);
-  return launch_dep(k_smooth_faces<ORDER, T, VEC>, dim3(faces + gx * gy * G.n0), kFacesThreads, 0, s,
-                    G, uin, uout, f, T(a_f), colour, faces, gx, gy, qx, by, fa);
+  return launch_dep(k_smooth_faces<ORDER, T, VEC, FAS>, dim3(faces + gx * gy * G.n0), kFacesThreads,
+                    0, s, G, uin, uout, f, T(a_f), colour, faces, gx, gy, qx, by, T(invh2), box, fa);
 }
 
 template <typename T>
-cudaError_t launch_smooth_faces(int order, const Grid& G, const T* uin, T* uout, const T* f,
-                                double a_f, int colour, bool quad, const FaceSet& fs,
-                                const CfWeights& w, const T* inter, const T* fc_unc, double h,
-                                double invH, cudaStream_t s) {
+cudaError_t launch_smooth_faces(int order, const Grid& G, const T* uin, T* uout, T* f, double a_f,
+                                int colour, bool quad, const FaceSet& fs, const CfWeights& w,
+                                const T* inter, const T* fc_unc, double h, double invH, bool fas,
+                                double invh2, Int3 lo, Int3 hi, cudaStream_t s) {
   const FaceArgs<T> fa = make_face_args<T>(order, fs, w, inter, fc_unc, h, invH);
+  const FasBox box{lo, hi};
   if constexpr (sizeof(T) == 4) {
+    if (fas) {
+      switch (order) {
+        case 2: return launch_faces_vec<2, T, 2, true>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+        case 4: return launch_faces_vec<4, T, 2, true>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+        case 6: return launch_faces_vec<6, T, 2, true>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+        default: return cudaErrorInvalidValue;
+      }
+    }
     if (quad && G.n2 % 4 == 0) {
       switch (order) {
-        case 2: return launch_faces_vec<2, T, 4>(G, uin, uout, f, a_f, colour, fa, s);
-        case 4: return launch_faces_vec<4, T, 4>(G, uin, uout, f, a_f, colour, fa, s);
-        case 6: return launch_faces_vec<6, T, 4>(G, uin, uout, f, a_f, colour, fa, s);
+        case 2: return launch_faces_vec<2, T, 4>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+        case 4: return launch_faces_vec<4, T, 4>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+        case 6: return launch_faces_vec<6, T, 4>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
         default: return cudaErrorInvalidValue;
       }
     }
   }
   switch (order) {
-    case 2: return launch_faces_vec<2, T, 2>(G, uin, uout, f, a_f, colour, fa, s);
-    case 4: return launch_faces_vec<4, T, 2>(G, uin, uout, f, a_f, colour, fa, s);
-    case 6: return launch_faces_vec<6, T, 2>(G, uin, uout, f, a_f, colour, fa, s);
+    case 2: return launch_faces_vec<2, T, 2>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+    case 4: return launch_faces_vec<4, T, 2>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+    case 6: return launch_faces_vec<6, T, 2>(G, uin, uout, f, a_f, colour, invh2, box, fa, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_smooth_fas(int order, const Grid& G, const float* uin, float* uout, float* f,
+                              double a_f, int colour, int periodic, double invh2, Int3 lo, Int3 hi,
+                              cudaStream_t s) {
+  if (G.n2 % 2) return cudaErrorInvalidValue;
+  const dim3 block(32, 4, 1);
+  const dim3 grid((G.n2 / 2 + 31) / 32, (G.n1 + 3) / 4, G.n0);
+  const FasBox box{lo, hi};
+  switch (order) {
+    case 2: return launch_dep(k_smooth_fas<2>, grid, block, 0, s, G, uin, uout, f, float(a_f), float(invh2), box, colour, periodic);
+    case 4: return launch_dep(k_smooth_fas<4>, grid, block, 0, s, G, uin, uout, f, float(a_f), float(invh2), box, colour, periodic);
+    case 6: return launch_dep(k_smooth_fas<6>, grid, block, 0, s, G, uin, uout, f, float(a_f), float(invh2), box, colour, periodic);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -508,10 +554,10 @@ cudaError_t prepare_restrict_tile() {
 #define MGK_INSTANTIATE(T)                                                                     \
   template cudaError_t launch_smooth_half<T>(int, const Grid&, const T*, T*, const T*, double, \
                                              int, int, int, bool, cudaStream_t);               \
-  template cudaError_t launch_smooth_faces<T>(int, const Grid&, const T*, T*, const T*, double,  \
-                                              int, bool, const FaceSet&, const CfWeights&,     \
-                                              const T*, const T*, double, double,              \
-                                              cudaStream_t);                                   \
+  template cudaError_t launch_smooth_faces<T>(int, const Grid&, const T*, T*, T*, double, int, \
+                                              bool, const FaceSet&, const CfWeights&,          \
+                                              const T*, const T*, double, double, bool,        \
+                                              double, Int3, Int3, cudaStream_t);               \
   template cudaError_t launch_residual_restrict<T>(int, const Grid&, const T*, const T*,       \
                                                    double, const Grid&, T*, T*, T*, Int3,      \
                                                    Int3, int, cudaStream_t);                   \

@@ -66,6 +66,40 @@ __device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restric
   }
 }
 
+// FAS source of the cells [lo, hi) of a level and the level's first half-sweep after it: f of
+// those cells (the restricted residual) gains L u of the restricted solution, whose neighbours
+// the half-sweep reads anyway, before the pair's cell of the colour is updated.  Rows of even
+// length (levels with a parent).
+struct FasBox {
+  Int3 lo, hi;
+};
+
+template <int ORDER, typename T, typename LD>
+__device__ __forceinline__ void smooth_fas_pair_at(const Grid& G, const T* __restrict__ uin,
+                                                   T* __restrict__ uout, T* __restrict__ f,
+                                                   T a_f, T invh2, const FasBox& box, int colour,
+                                                   int periodic, int i, int j, int k0) {
+  typedef typename Vec2<T>::type V2;
+  const long long p = gidx(G, i, j, k0);
+  T n0[3 * ORDER], n1[3 * ORDER], c0, c1;
+  load_pair_neighbours<ORDER, T, LD>(uin, p, G.Zp, G.Y * G.Zp, n0, n1, c0, c1);
+  V2 fv = *reinterpret_cast<const V2*>(f + p);
+  if (i >= box.lo.x && i < box.hi.x && j >= box.lo.y && j < box.hi.y) {
+    const bool in0 = k0 >= box.lo.z && k0 < box.hi.z;
+    const bool in1 = k0 + 1 >= box.lo.z && k0 + 1 < box.hi.z;
+    if (in0) fv.x = add_lap_of<ORDER, T>(n0, c0, invh2, fv.x);
+    if (in1) fv.y = add_lap_of<ORDER, T>(n1, c1, invh2, fv.y);
+    if (in0 || in1) *reinterpret_cast<V2*>(f + p) = fv;
+  }
+  V2 out;
+  out.x = c0;
+  out.y = c1;
+  if (((i + j + k0) & 1) == colour) out.x = relax<ORDER, T>(n0, a_f * fv.x);
+  else out.y = relax<ORDER, T>(n1, a_f * fv.y);
+  *reinterpret_cast<V2*>(uout + p) = out;
+  if (periodic) write_pair_images<T>(G, uout, i, j, k0, out.x, out.y);
+}
+
 template <int ORDER, typename T, typename LD, bool CVT = false>
 __device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restrict__ uin,
                                                  T* __restrict__ uout, const T* __restrict__ f,
