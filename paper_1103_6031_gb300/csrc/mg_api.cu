@@ -265,6 +265,10 @@ struct mg_hierarchy {
   std::string err;
   void* arena = nullptr;
   size_t arena_bytes = 0;
+  // the pieces of the arena that start as zeros (carve)
+  double* zero_d = nullptr;
+  float* zero_f = nullptr;
+  long long zero_d_count = 0, zero_f_count = 0;
   double* partial = nullptr;
   int partial_slots = 0;
   // [0..1] norm sums, [2..3] source sum, [4] wait flag, [8 + 2 l, 9 + 2 l] the norm
@@ -428,6 +432,40 @@ size_t carve(const mg_config* cfg, const Plan& p, mg_hierarchy* h, char* arena) 
   long long max_leaf = 0;
   long long max_leaf_padded = 0;
   const size_t nl = p.geo.size();
+  // What a solve or an outer iteration starts by zeroing lies in one piece each: float64 u
+  // (MG_FP64: both buffers of every level; MG_MIXED: the leaf levels'), and in MG_MIXED the
+  // float32 correction with its nests' parent interpolants and fluxes.
+  struct LevelArrays {
+    double *u0 = nullptr, *u1 = nullptr;
+    float *s0 = nullptr, *sin = nullptr, *sfu = nullptr;
+  };
+  std::vector<LevelArrays> arr(nl);
+  auto elems = [&](size_t l) {
+    return (size_t)grid_elems(make_grid(p.geo[l].n[0], p.geo[l].n[1], p.geo[l].n[2], g));
+  };
+  const size_t d0 = c.used;
+  for (size_t l = 0; l < nl; ++l) {
+    if (mixed && (int)l < p.base) continue;
+    arr[l].u0 = c.take<double>(elems(l));
+    if (!mixed) arr[l].u1 = c.take<double>(elems(l));
+  }
+  const size_t d1 = c.used;
+  for (size_t l = 0; l < nl && mixed; ++l) {
+    const LevelGeom& lg = p.geo[l];
+    FaceSet fs;
+    make_faceset(make_grid(lg.n[0], lg.n[1], lg.n[2], g), g, &fs);
+    arr[l].s0 = c.take<float>(elems(l));
+    if (lg.nest) {
+      arr[l].sin = c.take<float>((size_t)fs.base[6]);
+      arr[l].sfu = c.take<float>((size_t)fs.ebase[6]);
+    }
+  }
+  if (h) {
+    h->zero_d = reinterpret_cast<double*>(arena + d0);
+    h->zero_d_count = (long long)((d1 - d0) / sizeof(double));
+    h->zero_f = reinterpret_cast<float*>(arena + d1);
+    h->zero_f_count = (long long)((c.used - d1) / sizeof(float));
+  }
   for (size_t l = 0; l < nl; ++l) {
     const LevelGeom& lg = p.geo[l];
     const Grid G = make_grid(lg.n[0], lg.n[1], lg.n[2], g);
@@ -438,41 +476,35 @@ size_t carve(const mg_config* cfg, const Plan& p, mg_hierarchy* h, char* arena) 
     make_faceset(G, g, &fs);
     DevLevel* L = h ? &h->L[l] : nullptr;
     if (!mixed) {
-      double* u0 = c.take<double>(e);
-      double* u1 = c.take<double>(e);
       double* ff = c.take<double>(e);
       double* ub = l > 0 ? c.take<double>(ncov) : nullptr;
       double* in = lg.nest ? c.take<double>((size_t)fs.base[6]) : nullptr;
       double* fu = lg.nest ? c.take<double>((size_t)fs.ebase[6]) : nullptr;
       if (L) {
-        L->d.u[0] = u0;
-        L->d.u[1] = u1;
+        L->d.u[0] = arr[l].u0;
+        L->d.u[1] = arr[l].u1;
         L->d.ffas = ff;
         L->d.ubar = ub;
         L->d.inter = in;
         L->d.fc_unc = fu;
       }
     } else {
-      float* u0 = c.take<float>(e);
       float* u1 = c.take<float>(e);
       float* ff = c.take<float>(e);
       float* ub = l > 0 ? c.take<float>(ncov) : nullptr;
-      float* in = lg.nest ? c.take<float>((size_t)fs.base[6]) : nullptr;
-      float* fu = lg.nest ? c.take<float>((size_t)fs.ebase[6]) : nullptr;
       if (L) {
-        L->s.u[0] = u0;
+        L->s.u[0] = arr[l].s0;
         L->s.u[1] = u1;
         L->s.ffas = ff;
         L->s.ubar = ub;
-        L->s.inter = in;
-        L->s.fc_unc = fu;
+        L->s.inter = arr[l].sin;
+        L->s.fc_unc = arr[l].sfu;
       }
       if (leaf) {
-        double* u0d = c.take<double>(e);
         double* ind = lg.nest ? c.take<double>((size_t)fs.base[6]) : nullptr;
         double* fud = lg.nest ? c.take<double>((size_t)fs.ebase[6]) : nullptr;
         if (L) {
-          L->d.u[0] = u0d;
+          L->d.u[0] = arr[l].u0;
           L->d.u[1] = nullptr;
           L->d.inter = ind;
           L->d.fc_unc = fud;
@@ -867,22 +899,13 @@ mg_status vcycle(mg_hierarchy* h, int l) {
   return MG_OK;
 }
 
-mg_status fill_zero(mg_hierarchy* h, double* p, long long e) {
-  KL(MG_K_COPY, e, launch_fill(p, e, 0.0, h->s));
-  return MG_OK;
-}
-
-template <typename T>
-mg_status zero_state(mg_hierarchy* h, int from_level) {
-  for (int l = from_level; l <= finest(h); ++l) {
-    DevLevel& L = h->L[l];
-    Bufs<T>& b = bufs<T>(L);
-    const long long e = grid_elems(L.G);
-    for (int q = 0; q < 2; ++q)
-      if (b.u[q]) ST(fill_zero(h, b.u[q], e));
-    b.cur = 0;
-    b.ghosts_stale = false;
-    b.ghosts_ready = false;
+// The float64 u of every level that has one: zero, in one launch.
+mg_status zero_state(mg_hierarchy* h) {
+  KL(MG_K_COPY, h->zero_d_count, launch_fill(h->zero_d, h->zero_d_count, 0.0, h->s));
+  for (DevLevel& L : h->L) {
+    L.d.cur = 0;
+    L.d.ghosts_stale = false;
+    L.d.ghosts_ready = false;
   }
   return MG_OK;
 }
@@ -1047,28 +1070,19 @@ mg_status fp64_cycle_body(mg_hierarchy* h) {
 // the other buffer before it is read), and a zero parent gives zero
 // tangential intermediate values and parent fluxes on every nest.
 mg_status zero_correction(mg_hierarchy* h) {
-  auto zero = [&](float* p, long long n) -> mg_status {
-    if (h->rec) {
-      POp o = pop(P_ZERO);
-      o.out0 = p;
-      o.n = n;
-      rec_push(h, o, ceil_div(n, kZeroPerBlock));
-      return MG_OK;
-    }
-    CK(cudaMemsetAsync(p, 0, (size_t)n * sizeof(float), h->s));
-    return MG_OK;
-  };
-  for (int l = 0; l <= finest(h); ++l) {
-    DevLevel& L = h->L[l];
+  for (DevLevel& L : h->L) {
     L.s.cur = 0;
     L.s.ghosts_stale = false;
     L.s.ghosts_ready = false;
-    ST(zero(L.s.u[0], grid_elems(L.G)));
-    if (L.geo.nest) {
-      ST(zero(L.s.inter, L.fs.base[6]));
-      ST(zero(L.s.fc_unc, L.fs.ebase[6]));
-    }
   }
+  if (h->rec) {
+    POp o = pop(P_ZERO);
+    o.out0 = h->zero_f;
+    o.n = h->zero_f_count;
+    rec_push(h, o, ceil_div(h->zero_f_count, kZeroPerBlock));
+    return MG_OK;
+  }
+  CK(cudaMemsetAsync(h->zero_f, 0, (size_t)h->zero_f_count * sizeof(float), h->s));
   return MG_OK;
 }
 
@@ -1145,7 +1159,7 @@ struct SolveState {
 // and, in MG_MIXED, the first residual (the source itself: u = 0).
 mg_status solve_begin(mg_hierarchy* h) {
   ST(remove_source_mean(h));
-  ST(zero_state<double>(h, h->mixed ? h->base : 0));
+  ST(zero_state(h));
   for (int l = h->base + 1; l <= finest(h); ++l) ST(tangential<double>(h, l));
   if (h->mixed) ST(norm_launches(h, true));
   return MG_OK;
@@ -1433,51 +1447,24 @@ mg_status solve_prepared(mg_hierarchy* h, mg_info* info) {
   return solve_end(h, st, info);
 }
 
-cudaMemcpy3DParms dense_padded_parms(const DevLevel& L, double* padded, double* dense,
-                                     bool to_padded) {
-  cudaMemcpy3DParms p;
-  std::memset(&p, 0, sizeof(p));
-  const Grid& G = L.G;
-  cudaPitchedPtr pp = make_cudaPitchedPtr(padded, (size_t)G.Zp * sizeof(double),
-                                          (size_t)G.Zp * sizeof(double), (size_t)G.Y);
-  cudaPitchedPtr dp = make_cudaPitchedPtr(dense, (size_t)G.n2 * sizeof(double),
-                                          (size_t)G.n2 * sizeof(double), (size_t)G.n1);
-  cudaPos ppos = make_cudaPos((size_t)G.za * sizeof(double), (size_t)G.g, (size_t)G.g);
-  if (to_padded) {
-    p.srcPtr = dp;
-    p.dstPtr = pp;
-    p.dstPos = ppos;
-  } else {
-    p.srcPtr = pp;
-    p.srcPos = ppos;
-    p.dstPtr = dp;
-  }
-  p.extent = make_cudaExtent((size_t)G.n2 * sizeof(double), (size_t)G.n1, (size_t)G.n0);
-  p.kind = cudaMemcpyDefault;
-  return p;
-}
-
+// src (dense, on the device or, with host, in host memory) into the padded array.  Host
+// arrays go through the level's stage in one contiguous copy: the copy engine moves rows
+// of a pitched copy one by one.
 mg_status load_leaf(mg_hierarchy* h, int l, const double* src, double* padded, bool host) {
   DevLevel& L = h->L[l];
   if (host) {
-    cudaMemcpy3DParms p = dense_padded_parms(L, padded, const_cast<double*>(src), true);
-    CK(cudaMemcpy3DAsync(&p, h->s));
-  } else {
-    KL(MG_K_COPY, cells_of(L.G), launch_pack(L.G, src, padded, 0.0, h->s));
+    double* land = h->stage + L.stage_off;
+    CK(cudaMemcpyAsync(land, src, cells_of(L.G) * sizeof(double), cudaMemcpyDefault, h->s));
+    src = land;
   }
+  KL(MG_K_COPY, cells_of(L.G), launch_pack(L.G, src, padded, 0.0, h->s));
   return MG_OK;
 }
 
-// add (device buffers only): dst = interior + add
-mg_status store_leaf(mg_hierarchy* h, int l, const double* padded, double* dst, bool host,
-                     double add = 0.0) {
+// dst (dense, device) = interior + add
+mg_status store_leaf(mg_hierarchy* h, int l, const double* padded, double* dst, double add = 0.0) {
   DevLevel& L = h->L[l];
-  if (host) {
-    cudaMemcpy3DParms p = dense_padded_parms(L, const_cast<double*>(padded), dst, false);
-    CK(cudaMemcpy3DAsync(&p, h->s));
-  } else {
-    KL(MG_K_COPY, cells_of(L.G), launch_unpack(L.G, padded, dst, h->s, add));
-  }
+  KL(MG_K_COPY, cells_of(L.G), launch_unpack(L.G, padded, dst, h->s, add));
   return MG_OK;
 }
 
@@ -1526,81 +1513,6 @@ mg_status hybrid_into(mg_hierarchy* h, const double* f_dense, double* const psi[
   return MG_OK;
 }
 
-// -G phi of the potential in the float64 u; outputs dense, 3 per leaf level.  With
-// hybrid (and MG_FLAG_HYBRID), the finest level's psi also gets the hybrid
-// correction of the source in f (the source of the potential just solved for).
-mg_status gradient_out(mg_hierarchy* h, double* const disp[], bool host, bool hybrid = false) {
-  for (int l = h->base; l <= finest(h); ++l) {
-    DevLevel& L = h->L[l];
-    const int i = l - h->base;
-    ST(ghost_fill<double>(h, l, false));
-    double* dx = disp[3 * i];
-    double* dy = disp[3 * i + 1];
-    double* dz = disp[3 * i + 2];
-    const long long n = (long long)L.G.n0 * L.G.n1 * L.G.n2;
-    const bool hyb = hybrid && l == finest(h) && (h->cfg.flags & MG_FLAG_HYBRID);
-    if (hyb && !h->hybrid_f) CK(cudaMalloc(&h->hybrid_f, n * sizeof(double)));
-    if (hyb) ST(store_leaf(h, l, L.f, h->hybrid_f, false));
-    if (host) {
-      if (!dx && !dy && !dz) continue;
-      KL(MG_K_LPT, n,
-         launch_gradient(h->cfg.order, L.G, phi_of(L), 1.0 / L.geo.h, h->scratch,
-                         h->scratch + n, h->scratch + 2 * n, h->s));
-      if (hyb) {
-        double* const psi[3] = {h->scratch, h->scratch + n, h->scratch + 2 * n};
-        ST(hybrid_into(h, h->hybrid_f, psi));
-      }
-      for (int a = 0; a < 3; ++a)
-        if (disp[3 * i + a])
-          CK(cudaMemcpyAsync(disp[3 * i + a], h->scratch + a * n, n * sizeof(double),
-                             cudaMemcpyDeviceToHost, h->s));
-    } else {
-      if (!dx || !dy || !dz) return fail(h, MG_EINVAL, "displacement output pointer is NULL");
-      KL(MG_K_LPT, n, launch_gradient(h->cfg.order, L.G, phi_of(L), 1.0 / L.geo.h, dx, dy, dz, h->s));
-      if (hyb) {
-        double* const psi[3] = {dx, dy, dz};
-        ST(hybrid_into(h, h->hybrid_f, psi));
-      }
-    }
-  }
-  return MG_OK;
-}
-
-// Host-buffer pipelines: phi and the displacements of the solve just finished go
-// into the stage (dense, on the device) and their copies to the caller's host
-// buffers are queued on the copy stream, where they run while the work stream goes
-// on with tau and the second solve (the host link, ~190 GB/s, would otherwise add
-// the copies to the step).
-mg_status stage_outputs(mg_hierarchy* h, double* const phi[], double* const disp[]) {
-  if (!phi && !disp) return MG_OK;
-  std::vector<double*> dd;
-  for (int l = h->base; l <= finest(h); ++l) {
-    DevLevel& L = h->L[l];
-    const long long n = cells_of(L.G);
-    double* base = h->stage + L.stage_off;
-    if (phi && phi[l - h->base]) ST(store_leaf(h, l, phi_of(L), base, false));
-    for (int a = 1; a <= 3; ++a) dd.push_back(base + a * n);
-  }
-  if (disp) ST(gradient_out(h, dd.data(), false, true));
-  CK(cudaEventRecord(h->ev_staged, h->s));
-  CK(cudaStreamWaitEvent(h->cs, h->ev_staged, 0));
-  h->copies_pending = true;
-  for (int l = h->base; l <= finest(h); ++l) {
-    DevLevel& L = h->L[l];
-    const int i = l - h->base;
-    const long long n = cells_of(L.G);
-    const double* base = h->stage + L.stage_off;
-    if (phi && phi[i])
-      CK(cudaMemcpyAsync(phi[i], base, n * sizeof(double), cudaMemcpyDeviceToHost, h->cs));
-    for (int a = 0; disp && a < 3; ++a)
-      if (disp[3 * i + a])
-        CK(cudaMemcpyAsync(disp[3 * i + a], base + (a + 1) * n, n * sizeof(double),
-                           cudaMemcpyDeviceToHost, h->cs));
-  }
-  CK(cudaEventRecord(h->ev_copied, h->cs));
-  return MG_OK;
-}
-
 // Orders the work stream after the staged copies: before the stage is written
 // again and before the caller is told that the results are in host memory.
 mg_status join_copies(mg_hierarchy* h) {
@@ -1611,6 +1523,72 @@ mg_status join_copies(mg_hierarchy* h) {
     cudaStreamSynchronize(h->cs);  // no copy may outlive the call
     return fail_cuda(h, e, "cudaStreamWaitEvent(copies)");
   }
+  return MG_OK;
+}
+
+// -G phi of leaf level l of the potential in the float64 u (dense, device).  With hybrid (and
+// MG_FLAG_HYBRID), the finest level's psi also gets the hybrid correction of the source in f
+// (the source of the potential just solved for).
+mg_status gradient_level(mg_hierarchy* h, int l, double* dx, double* dy, double* dz, bool hybrid) {
+  DevLevel& L = h->L[l];
+  ST(ghost_fill<double>(h, l, false));
+  const long long n = cells_of(L.G);
+  const bool hyb = hybrid && l == finest(h) && (h->cfg.flags & MG_FLAG_HYBRID);
+  if (hyb && !h->hybrid_f) CK(cudaMalloc(&h->hybrid_f, n * sizeof(double)));
+  if (hyb) ST(store_leaf(h, l, L.f, h->hybrid_f));
+  if (!dx || !dy || !dz) return fail(h, MG_EINVAL, "displacement output pointer is NULL");
+  KL(MG_K_LPT, n, launch_gradient(h->cfg.order, L.G, phi_of(L), 1.0 / L.geo.h, dx, dy, dz, h->s));
+  if (hyb) {
+    double* const psi[3] = {dx, dy, dz};
+    ST(hybrid_into(h, h->hybrid_f, psi));
+  }
+  return MG_OK;
+}
+
+// The same of every leaf level, 3 outputs each.
+mg_status gradient_out(mg_hierarchy* h, double* const disp[], bool hybrid = false) {
+  for (int l = h->base; l <= finest(h); ++l) {
+    double* const* d = disp + 3 * (l - h->base);
+    ST(gradient_level(h, l, d[0], d[1], d[2], hybrid));
+  }
+  return MG_OK;
+}
+
+// Host-buffer pipelines: phi and the displacements of the solve just finished go into the
+// stage (dense, on the device), and each level's copies to the caller's host buffers are
+// queued on the copy stream as soon as that level is staged.  They run while the work stream
+// goes on with the next level, tau and the second solve (the host link moves ~190 GB/s).
+mg_status stage_outputs(mg_hierarchy* h, double* const phi[], double* const disp[]) {
+  if (!phi && !disp) return MG_OK;
+  ST(join_copies(h));  // the stage may still be read by the first solve's copies
+  for (int l = h->base; l <= finest(h); ++l) {
+    DevLevel& L = h->L[l];
+    const int i = l - h->base;
+    const long long n = cells_of(L.G);
+    double* base = h->stage + L.stage_off;
+    double* const none[3] = {nullptr, nullptr, nullptr};
+    double* const* d = disp ? disp + 3 * i : none;
+    double* out[4] = {phi ? phi[i] : nullptr, d[0], d[1], d[2]};
+    if (out[0]) ST(store_leaf(h, l, phi_of(L), base));
+    if (d[0] || d[1] || d[2]) ST(gradient_level(h, l, base + n, base + 2 * n, base + 3 * n, true));
+    CK(cudaEventRecord(h->ev_staged, h->s));
+    CK(cudaStreamWaitEvent(h->cs, h->ev_staged, 0));
+    h->copies_pending = true;
+    for (int a = 0; a < 4; ++a)
+      if (out[a])
+        CK(cudaMemcpyAsync(out[a], base + a * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->cs));
+    CK(cudaEventRecord(h->ev_copied, h->cs));
+  }
+  return MG_OK;
+}
+
+// The results of the solve just finished into the caller's arrays (any may be NULL).
+mg_status put_outputs(mg_hierarchy* h, double* const phi[], double* const disp[], bool host) {
+  if (host) return stage_outputs(h, phi, disp);
+  if (phi)
+    for (int l = h->base; l <= finest(h); ++l)
+      if (phi[l - h->base]) ST(store_leaf(h, l, phi_of(h->L[l]), phi[l - h->base]));
+  if (disp) ST(gradient_out(h, disp, true));
   return MG_OK;
 }
 
@@ -2033,15 +2011,7 @@ mg_status batch_pipeline(mg_batch* b, bool host, const double* const* const delt
   if (st1 != MG_OK && st1 != MG_ENOCONV) return st1;
   for (size_t i = 0; i < n; ++i) {
     mg_hierarchy* h = b->m[i];
-    mg_status r = MG_OK;
-    if (host) {
-      r = stage_outputs(h, phi1 ? phi1[i] : nullptr, disp1 ? disp1[i] : nullptr);
-    } else {
-      if (phi1 && phi1[i])
-        for (int l = h->base; l <= finest(h) && r == MG_OK; ++l)
-          if (phi1[i][l - h->base]) r = store_leaf(h, l, phi_of(h->L[l]), phi1[i][l - h->base], host);
-      if (r == MG_OK && disp1 && disp1[i]) r = gradient_out(h, disp1[i], host, true);
-    }
+    mg_status r = put_outputs(h, phi1 ? phi1[i] : nullptr, disp1 ? disp1[i] : nullptr, host);
     if (r == MG_OK) r = tau_into_f(h);
     if (r != MG_OK) return member_status(b, (int)i, r);
   }
@@ -2049,11 +2019,7 @@ mg_status batch_pipeline(mg_batch* b, bool host, const double* const* const delt
   if (st2 != MG_OK && st2 != MG_ENOCONV) return st2;
   for (size_t i = 0; i < n; ++i) {
     mg_hierarchy* h = b->m[i];
-    mg_status r = MG_OK;
-    if (phi2 && phi2[i])
-      for (int l = h->base; l <= finest(h) && r == MG_OK; ++l)
-        if (phi2[i][l - h->base]) r = store_leaf(h, l, phi_of(h->L[l]), phi2[i][l - h->base], host);
-    if (r == MG_OK && disp2 && disp2[i]) r = gradient_out(h, disp2[i], host, true);
+    const mg_status r = put_outputs(h, phi2 ? phi2[i] : nullptr, disp2 ? disp2[i] : nullptr, host);
     if (r != MG_OK) return member_status(b, (int)i, r);
   }
   for (size_t i = 0; i < n; ++i) {
@@ -2089,23 +2055,13 @@ mg_status pipeline_device_loops(mg_hierarchy* h, bool host, const double* const 
   ST(loop_launch(h));
   CK(cudaMemcpyAsync(h->loop_host1, h->loop_dev, sizeof(LoopState), cudaMemcpyDeviceToHost, h->s));
   if (h->mixed) ST(gauge_zero_base_mean(h));
-  if (host) {
-    ST(stage_outputs(h, phi1, disp1));
-  } else {
-    if (phi1)
-      for (int l = h->base; l <= finest(h); ++l)
-        if (phi1[l - h->base]) ST(store_leaf(h, l, phi_of(h->L[l]), phi1[l - h->base], false));
-    if (disp1) ST(gradient_out(h, disp1, false, true));
-  }
+  ST(put_outputs(h, phi1, disp1, host));
   ST(tau_into_f(h));
   ST(solve_begin(h));
   ST(solve_begin_read(h, st2));
   ST(loop_launch(h));
   if (h->mixed) ST(gauge_zero_base_mean(h));
-  if (phi2)
-    for (int l = h->base; l <= finest(h); ++l)
-      if (phi2[l - h->base]) ST(store_leaf(h, l, phi_of(h->L[l]), phi2[l - h->base], host));
-  if (disp2) ST(gradient_out(h, disp2, host, true));
+  ST(put_outputs(h, phi2, disp2, host));
   CK(cudaStreamSynchronize(h->s));
   ST(loop_read(h, st1, h->loop_host1));
   const mg_status r1 = finish_info(h, st1.local, st1.rel, st1.at_floor, info1);
@@ -2161,16 +2117,6 @@ mg_status job_begin_solve(PipelineJob* j) {
   return job_record(j);
 }
 
-mg_status job_store(PipelineJob* j, const std::vector<double*>& phi,
-                    const std::vector<double*>& disp) {
-  mg_hierarchy* h = j->h;
-  if (!phi.empty())
-    for (int l = h->base; l <= finest(h); ++l)
-      ST(store_leaf(h, l, phi_of(h->L[l]), phi[l - h->base], true));
-  if (!disp.empty()) ST(gradient_out(h, const_cast<double* const*>(disp.data()), true, true));
-  return MG_OK;
-}
-
 // The iteration queued last has finished: read it and queue what comes next.
 mg_status job_advance(PipelineJob* j) {
   mg_hierarchy* h = j->h;
@@ -2194,7 +2140,8 @@ mg_status job_advance(PipelineJob* j) {
     j->phase = 2;
     return job_begin_solve(j);
   }
-  ST(job_store(j, j->phi2, j->disp2));
+  ST(stage_outputs(h, j->phi2.empty() ? nullptr : j->phi2.data(),
+                   j->disp2.empty() ? nullptr : j->disp2.data()));
   ST(join_copies(h));
   j->phase = 3;
   return job_record(j);
@@ -2634,7 +2581,7 @@ mg_status mg_solve_1lpt(mg_hierarchy* h, const double* const delta[], double* co
     const mg_status st = solve_prepared(h, info);
     if (st != MG_OK && st != MG_ENOCONV) return st;
     for (int l = h->base; l <= finest(h); ++l)
-      ST(store_leaf(h, l, phi_of(h->L[l]), phi[l - h->base], false));
+      ST(store_leaf(h, l, phi_of(h->L[l]), phi[l - h->base]));
     CK(cudaStreamSynchronize(h->s));
     return st;
   });
@@ -2648,7 +2595,7 @@ mg_status mg_lpt2_source(mg_hierarchy* h, const double* const phi1[], double* co
   return on_streams(h, [&]() -> mg_status {
     ST(load_potential(h, phi1, false));
     ST(tau_into_f(h));
-    for (int l = h->base; l <= finest(h); ++l) ST(store_leaf(h, l, h->L[l].f, tau[l - h->base], false));
+    for (int l = h->base; l <= finest(h); ++l) ST(store_leaf(h, l, h->L[l].f, tau[l - h->base]));
     CK(cudaStreamSynchronize(h->s));
     return MG_OK;
   });
@@ -2666,7 +2613,7 @@ mg_status mg_solve_2lpt(mg_hierarchy* h, const double* const phi1[], double* con
     const mg_status st = solve_prepared(h, info);
     if (st != MG_OK && st != MG_ENOCONV) return st;
     for (int l = h->base; l <= finest(h); ++l)
-      ST(store_leaf(h, l, phi_of(h->L[l]), phi2[l - h->base], false));
+      ST(store_leaf(h, l, phi_of(h->L[l]), phi2[l - h->base]));
     CK(cudaStreamSynchronize(h->s));
     return st;
   });
@@ -2679,7 +2626,7 @@ mg_status mg_displacements(mg_hierarchy* h, const double* const phi[], double* c
     return fail(h, MG_EINVAL, "phi/disp must hold 1 and 3 non-NULL pointers per level");
   return on_streams(h, [&]() -> mg_status {
     ST(load_potential(h, phi, false));
-    ST(gradient_out(h, disp, false));
+    ST(gradient_out(h, disp));
     CK(cudaStreamSynchronize(h->s));
     return MG_OK;
   });
@@ -2734,7 +2681,7 @@ mg_status mg_lla_density(mg_hierarchy* h, const double* const phi1[], const doub
     // unit composite mean: remove the volume-weighted leaf mean, then add 1 on output
     ST(remove_source_mean(h));
     for (int l = h->base; l <= finest(h); ++l)
-      ST(store_leaf(h, l, h->L[l].f, rho[l - h->base], false, 1.0));
+      ST(store_leaf(h, l, h->L[l].f, rho[l - h->base], 1.0));
     CK(cudaStreamSynchronize(h->s));
     return MG_OK;
   });
@@ -2768,21 +2715,11 @@ mg_status mg_lpt_pipeline(mg_hierarchy* h, int host_buffers, const double* const
         ST(load_leaf(h, l, delta[l - h->base], h->L[l].f, host));
       mg_status st1 = solve_prepared(h, info1);
       if (st1 != MG_OK && st1 != MG_ENOCONV) return st1;
-      if (host) {
-        ST(stage_outputs(h, phi1, disp1));
-      } else {
-        if (phi1)
-          for (int l = h->base; l <= finest(h); ++l)
-            if (phi1[l - h->base]) ST(store_leaf(h, l, phi_of(h->L[l]), phi1[l - h->base], host));
-        if (disp1) ST(gradient_out(h, disp1, host, true));
-      }
+      ST(put_outputs(h, phi1, disp1, host));
       ST(tau_into_f(h));
       mg_status st2 = solve_prepared(h, info2);
       if (st2 != MG_OK && st2 != MG_ENOCONV) return st2;
-      if (phi2)
-        for (int l = h->base; l <= finest(h); ++l)
-          if (phi2[l - h->base]) ST(store_leaf(h, l, phi_of(h->L[l]), phi2[l - h->base], host));
-      if (disp2) ST(gradient_out(h, disp2, host, true));
+      ST(put_outputs(h, phi2, disp2, host));
       return st1 != MG_OK ? st1 : st2;
     };
     const mg_status st = steps();
