@@ -100,6 +100,7 @@ __device__ __forceinline__ void tangential_tile(const Grid& F, const Grid& P,
   const T* org = pu + gidx(P, coord(0, p0a, pb, pc), coord(1, p0a, pb, pc), coord(2, p0a, pb, pc));
   const int sm = side == 0 ? -sa : sa;
   const int rows = nb + ORDER;
+  grid_wait();
   for (int q = threadIdx.x; q < half * RB * kTangC; q += kTangThreads) {
     const int kc = q % kTangC, r = q / kTangC % RB, m = q / (kTangC * RB);
     if (kc >= nc || r >= rows) continue;
@@ -199,7 +200,6 @@ __global__ void __launch_bounds__(kTangThreads)
     k_cf_tangential(Grid F, Grid P, const T* __restrict__ pu, Int3 off, FaceSet fs, TangTiles tt,
                     CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
                     T* __restrict__ fc_unc) {
-  grid_wait();
   tangential_tile<ORDER, T, FOLD>(F, P, pu, off, fs, tt, w, fo, invH, inter, fc_unc);
 }
 
@@ -212,12 +212,12 @@ __global__ void __launch_bounds__(kTangThreads)
                          TangTiles tt, CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
                          T* __restrict__ fc_unc, T* __restrict__ u, const T* __restrict__ ubar,
                          Int3 cn, int gx, int gy) {
-  grid_wait();
   const int b = (int)blockIdx.x - tt.first[6];
   if (b < 0) {
     tangential_tile<ORDER, T, FOLD>(F, P, pu, off, fs, tt, w, fo, invH, inter, fc_unc);
     return;
   }
+  grid_wait();
   prolong_at<T, Ldg>(F, u, P, pu, ubar, off, cn, 0, b / (gx * gy),
                      b / gx % gy * (kTangThreads / 32) + (int)(threadIdx.x >> 5),
                      b % gx * 32 + (int)(threadIdx.x & 31));
@@ -227,15 +227,22 @@ template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
     k_cf_flux(Grid F, T* __restrict__ u, FaceSet fs, CfW<T> w, const T* __restrict__ inter,
               const T* __restrict__ fc_unc, T fc_scale, T a0, T a1, T b0, T b1, int flux_fix) {
+  const int t = blockIdx.x * 128 + threadIdx.x;
+  if (t >= 4 * (int)fs.ebase[6]) return;
+  const unsigned quad = __activemask();
+  const int e = t >> 2;
+  const int f = face_of(fs, e, fs.ebase);
+  const unsigned loc = (unsigned)(e - (int)fs.ebase[f]), ne1 = fs.nt[f][1] / 2;
+  const FaceCol c = face_col(F, f, (int)(loc / ne1), (int)(loc % ne1), t & 3);
   grid_wait();
-  cf_flux_body<ORDER, T>(F, u, fs, w, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix,
-                         blockIdx.x * (long long)blockDim.x + threadIdx.x);
+  T v[ORDER];
+  load_column<ORDER, T>(u, c, v);
+  cf_flux_at<ORDER, T>(u, fs, w, inter, fc_unc, fc_scale, a0, a1, b0, b1, flux_fix, c, v, quad);
 }
 
 template <int ORDER>
 __global__ void __launch_bounds__(128)
     k_cf_flux_fold(Grid F, double* __restrict__ u, FaceArgs<double> fa) {
-  grid_wait();
   const int t = blockIdx.x * 128 + threadIdx.x;
   if (t >= 4 * (int)fa.fs.ebase[6]) return;
   const unsigned quad = __activemask();
@@ -243,6 +250,7 @@ __global__ void __launch_bounds__(128)
   const int f = face_of(fa.fs, e, fa.fs.ebase);
   const unsigned loc = (unsigned)(e - (int)fa.fs.ebase[f]), ne1 = fa.fs.nt[f][1] / 2;
   const FaceCol c = face_col(F, f, (int)(loc / ne1), (int)(loc % ne1), t & 3);
+  grid_wait();
   double v[ORDER];
   load_column<ORDER, double>(u, c, v);
   fa.ghosts<ORDER>(u, c, v, quad);

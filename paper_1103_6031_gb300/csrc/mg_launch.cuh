@@ -12,7 +12,8 @@
 namespace mgk {
 
 // Waits until the kernels this one depends on have finished and their writes are visible.
-// Every kernel launched with launch_dep calls it before it touches memory.
+// Every thread of a kernel launched with launch_dep that touches memory calls it before it
+// does; what comes earlier (indices, bounds) overlaps the predecessor.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... P, typename... A>

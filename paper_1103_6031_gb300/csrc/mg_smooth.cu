@@ -32,10 +32,11 @@ template <int ORDER, typename T, bool CVT>
 __global__ void __launch_bounds__(kPairX * 8, (smooth_min_blocks<ORDER, T>))
     k_smooth_half(Grid G, const T* __restrict__ uin, T* __restrict__ uout,
                   const T* __restrict__ f, T a_f, int colour, int periodic) {
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int k0 = 2 * (blockIdx.x * kPairX + threadIdx.x);
+  if (j >= G.n1 || k0 >= G.n2) return;
   grid_wait();
-  smooth_half_body<ORDER, T, Ldg, CVT>(G, uin, uout, f, a_f, colour, periodic, (int)blockDim.y,
-                                  Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
-                                      (int)threadIdx.x, (int)threadIdx.y});
+  smooth_pair_at<ORDER, T, Ldg, CVT>(G, uin, uout, f, a_f, colour, periodic, blockIdx.z, j, k0);
 }
 
 // The first half-sweep of a level after a restriction into it, with the FAS source of the
@@ -45,10 +46,10 @@ __global__ void __launch_bounds__(128, 8)
     k_smooth_fas(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
                  float* __restrict__ f, float a_f, float invh2, FasBox box, int colour,
                  int periodic) {
-  grid_wait();
   const int j = blockIdx.y * 4 + threadIdx.y;
   const int k0 = 2 * (blockIdx.x * 32 + threadIdx.x);
   if (j >= G.n1 || k0 >= G.n2) return;
+  grid_wait();
   smooth_fas_pair_at<ORDER, float, Ldg>(G, uin, uout, f, a_f, invh2, box, colour, periodic,
                                         blockIdx.z, j, k0);
 }
@@ -136,10 +137,10 @@ template <int ORDER>
 __global__ void __launch_bounds__(256, 4)
     k_smooth_quad(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
                   const float* __restrict__ f, float a_f, int colour, int periodic) {
-  grid_wait();
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (j >= G.n1 || k0 >= G.n2) return;
+  grid_wait();
   smooth_quad_at<ORDER>(G, uin, uout, f, a_f, colour, periodic, blockIdx.z, j, k0);
 }
 
@@ -163,13 +164,13 @@ __global__ void __launch_bounds__(kFacesThreads,
     k_smooth_faces(Grid G, const T* __restrict__ uin, T* __restrict__ uout, T* f, T a_f, int colour,
                    int face_blocks, int gx, int gy, int qx, int by, T invh2, FasBox box,
                    FaceArgs<T> fa) {
-  grid_wait();
   const int b = (int)blockIdx.x - face_blocks;
   if (b >= 0) {
     const int ty = (int)threadIdx.x / qx, tx = (int)threadIdx.x - ty * qx;
     const int j = b / gx % gy * by + ty;
     const int k0 = VEC * (b % gx * qx + tx);
     if (ty >= by || j >= G.n1 || k0 >= G.n2) return;
+    grid_wait();
     if constexpr (FAS)
       smooth_fas_pair_at<ORDER, T, Ldg>(G, uin, uout, f, a_f, invh2, box, colour, 0,
                                                b / (gx * gy), j, k0);
@@ -192,6 +193,7 @@ __global__ void __launch_bounds__(kFacesThreads,
     // the cells at depths o, o + 2, .. have the colour (index along the normal: 0 or n - 1)
     const int na = (fc >> 1) == 0 ? G.n0 : ((fc >> 1) == 1 ? G.n1 : G.n2);
     const int o = ((((fc & 1) ? na - 1 : 0) + c.tj + c.tk) & 1) == colour ? 0 : 1;
+    grid_wait();
     if (warp < ORDER / 2) {
       const int q = 2 * warp + o;
       const long long p = c.in0 + q * c.step;
@@ -224,7 +226,6 @@ __global__ void __launch_bounds__(128)
     k_residual_restrict(Grid F, const T* __restrict__ u, const T* __restrict__ f, T invh2, Grid P,
                         T* __restrict__ pu, T* __restrict__ pfas, T* __restrict__ ubar, Int3 off,
                         Int3 cn, int parent_periodic) {
-  grid_wait();
   typedef typename Vec2<T>::type V2;
   __shared__ T sm[2][8][32];  // u and r by child and parent of the block
   const int kc = blockIdx.x * blockDim.x + threadIdx.x;
@@ -232,6 +233,7 @@ __global__ void __launch_bounds__(128)
   const int ic = blockIdx.z;
   const int child = threadIdx.y, slot = threadIdx.z * blockDim.x + threadIdx.x;
   const bool in = kc < cn.z && jc < cn.y;
+  grid_wait();
   if (in) {
     const long long p = gidx(F, 2 * ic + (child >> 1), 2 * jc + (child & 1), 2 * kc);
     T n0[3 * ORDER], n1[3 * ORDER], c0, c1;
