@@ -2593,6 +2593,14 @@ mg_status mg_lpt2_source(mg_hierarchy* h, const double* const phi1[], double* co
   if (!check_ptrs((const void* const*)phi1, nleaf) || !check_ptrs((const void* const*)tau, nleaf))
     return fail(h, MG_EINVAL, "phi1/tau must hold one non-NULL pointer per level");
   return on_streams(h, [&]() -> mg_status {
+    DevLevel& B = h->L[h->base];
+    if (nleaf == 1 && !h->mixed && lpt2_source_dense_usable(B.G, phi1[0], tau[0])) {
+      KL(MG_K_LPT, cells_of(B.G),
+         launch_lpt2_source_dense(h->cfg.order, B.G, phi1[0], 1.0 / (B.geo.h * B.geo.h), tau[0],
+                                  h->s));
+      CK(cudaStreamSynchronize(h->s));
+      return MG_OK;
+    }
     ST(load_potential(h, phi1, false));
     ST(tau_into_f(h));
     for (int l = h->base; l <= finest(h); ++l) ST(store_leaf(h, l, h->L[l].f, tau[l - h->base]));

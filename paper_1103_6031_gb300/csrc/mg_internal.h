@@ -195,6 +195,11 @@ cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t s);
 // tau from phi (ghosts, including edges, filled)
 cudaError_t launch_lpt2_source(int order, const Grid& G, const double* phi, double invh2,
                                double* tau, cudaStream_t s);
+// the same from a dense phi of a periodic level to a dense tau (no ghosts needed), where
+// lpt2_source_dense_usable: even rows, phi 16-byte aligned, the arrays apart
+bool lpt2_source_dense_usable(const Grid& G, const double* phi, const double* tau);
+cudaError_t launch_lpt2_source_dense(int order, const Grid& G, const double* phi, double invh2,
+                                     double* tau, cudaStream_t s);
 // the same in FP64 arithmetic; work holds 2 * grid_elems(G) float64
 cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi, double invh2,
                                     double* tau, double* work, cudaStream_t s);

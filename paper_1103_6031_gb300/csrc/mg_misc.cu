@@ -1,6 +1,8 @@
 // Coarsest-level solve, convergence norms, composite mean, packing between the
 // caller's dense arrays and the padded level layout, the 2LPT source and the
 // displacement gradient (Hahn & Abel 2011, Sec. 3.1, 3.2).
+#include <type_traits>
+
 #include "mg_internal.h"
 #include "mg_launch.cuh"
 #include "mg_stencil.cuh"
@@ -405,29 +407,31 @@ __global__ void __launch_bounds__(128)
 
 // Finite-difference Hessian at element p in FP64 arithmetic: d[a] = phi_aa h^2, m = (phi_xy,
 // phi_xz, phi_yz) h^2 with phi_ab = G_a (G_b phi).
-template <int ORDER>
-__device__ __forceinline__ void fd_hessian(const Grid& G, const double* __restrict__ phi,
-                                           long long p, double (&d)[3], double (&m)[3]) {
+template <int ORDER, typename Src>
+__device__ __forceinline__ void fd_hessian(const Src& src, int i, int j, int k, double (&d)[3],
+                                           double (&m)[3]) {
   constexpr int half = ORDER / 2;
-  const int st[3] = {G.Y * G.Zp, G.Zp, 1};
-  const double c = __ldg(phi + p);
+  // the cell at offset s along axis a and t along axis b
+  auto at = [&](int a, int s, int b, int t) {
+    return __ldg(src.at(i + (a == 0 ? s : 0) + (b == 0 ? t : 0), j + (a == 1 ? s : 0) + (b == 1 ? t : 0),
+                        k + (a == 2 ? s : 0) + (b == 2 ? t : 0)));
+  };
+  const double c = at(0, 0, 0, 0);
 #pragma unroll 1
   for (int a = 0; a < 3; ++a) {
     double acc = Lap<ORDER>::w0 * c;
     for (int s = 1; s <= half; ++s)
-      acc = fma(lap_w<ORDER>(s), __ldg(phi + p + s * st[a]) + __ldg(phi + p - s * st[a]), acc);
+      acc = fma(lap_w<ORDER>(s), at(a, s, a, 0) + at(a, -s, a, 0), acc);
     d[a] = acc;
   }
 #pragma unroll 1
   for (int q = 0; q < 3; ++q) {
-    const int sa = st[q == 2 ? 1 : 0], sb = st[q == 0 ? 1 : 2];
+    const int a = q == 2 ? 1 : 0, b = q == 0 ? 1 : 2;
     double acc = 0.0;
     for (int s = -half; s <= half; ++s) {
       if (s == 0) continue;
       double g = 0.0;
-      for (int t = 1; t <= half; ++t)
-        g = fma(grad_w<ORDER>(t),
-                __ldg(phi + p + s * sa + t * sb) - __ldg(phi + p + s * sa - t * sb), g);
+      for (int t = 1; t <= half; ++t) g = fma(grad_w<ORDER>(t), at(a, s, b, t) - at(a, s, b, -t), g);
       acc = fma(grad_w<ORDER>(s), g, acc);
     }
     m[q] = acc;
@@ -456,8 +460,8 @@ struct LlaOp {
   __device__ __forceinline__ double operator()(const double (&d)[3], const double (&m_)[3]) const {
     const double a = fma(-s2, d[0], 1.0), b = fma(-s2, d[1], 1.0), c = fma(-s2, d[2], 1.0);
     const double m[3] = {s1 * m_[0], s1 * m_[1], s1 * m_[2]};
-    const double det = a * b * c - a * m[2] * m[2] - b * m[1] * m[1] - c * m[0] * m[0] -
-                       2.0 * m[0] * m[1] * m[2];
+    const double w = fma(2.0, m[0] * m[2], b * m[1]);
+    const double det = fma(a, fma(b, c, -(m[2] * m[2])), -fma(m[1], w, c * m[0] * m[0]));
     return 1.0 / det - 1.0;
   }
 };
@@ -471,18 +475,22 @@ __device__ __forceinline__ bool squarable(double s) {
 // OP of the Hessian of phi (ghosts and edge ghosts filled), one launch and no work arrays:
 // a tile of aligned integers with its edges (mg_tile.cuh), first derivatives and their
 // derivatives as integer sums; FP64 instructions are left only for the 6 conversions and OP
-// (14 per cell for tau, 65 when every sum ran on the FP64 pipe).
-template <int ORDER, typename OP>
+// (14 per cell for tau, 65 when every sum ran on the FP64 pipe).  DENSE: phi and out are
+// dense arrays of a periodic level, read and written without a padded copy (256^3, order 6:
+// the copies and the ghost fill were 128 of 845 us).
+template <int ORDER, typename OP, bool DENSE>
 __global__ void __launch_bounds__(kTileThreads, 3)
     k_hessian_tile(Grid G, const double* __restrict__ phi, double invh2, double* __restrict__ out) {
   grid_wait();
   extern __shared__ __align__(16) long long hess_smem[];
   const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
-  const unsigned key = tile_load_edges<ORDER>(G, phi, i0, j0, k0, hess_smem);
+  typedef typename std::conditional<DENSE, DensePeriodicSource, PaddedSource>::type Src;
+  const Src src(G, phi);
+  const unsigned key = tile_load_edges<ORDER>(G, src, i0, j0, k0, hess_smem);
   const int j = j0 + (threadIdx.x >> 5), k = k0 + (threadIdx.x & 31);
   if (j >= G.n1 || k >= G.n2) return;
-  const long long p = gidx(G, i0, j, k);
-  const int sx = G.Y * G.Zp;
+  const long long p = DENSE ? ((long long)i0 * G.n1 + j) * G.n2 + k : gidx(G, i0, j, k);
+  const int sx = DENSE ? G.n1 * G.n2 : G.Y * G.Zp;
   const int nx = min(kTileX, G.n0 - i0);
   const double k2 = invh2 * FxUnit<ORDER>::v;
   const double k1 = invh2 * (FxGradUnit<ORDER>::v * FxGradUnit<ORDER>::v);
@@ -502,7 +510,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
 #pragma unroll 1
   for (int x = 0; x < nx; ++x) {
     double d[3], m[3];
-    fd_hessian<ORDER>(G, phi, p + x * sx, d, m);
+    fd_hessian<ORDER>(src, i0 + x, j, k, d, m);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       d[a] *= invh2;
@@ -710,19 +718,20 @@ cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t s) {
   return launch_dep(k_fill, blocks_for(n, 256), 256, 0, s, p, n, v);
 }
 
-template <typename OP>
+template <typename OP, bool DENSE>
 static cudaError_t launch_hessian(int order, const Grid& G, const double* phi, double invh2,
                                   double* out, cudaStream_t s) {
   const dim3 tg = tile_grid(G);
   switch (order) {
-    case 2: return launch_dep(k_hessian_tile<2, OP>, tg, kTileThreads, FxTile<2>::bytes, s, G, phi, invh2, out);
-    case 4: return launch_dep(k_hessian_tile<4, OP>, tg, kTileThreads, FxTile<4>::bytes, s, G, phi, invh2, out);
+    case 2: return launch_dep(k_hessian_tile<2, OP, DENSE>, tg, kTileThreads, FxTile<2>::bytes, s, G, phi, invh2, out);
+    case 4: return launch_dep(k_hessian_tile<4, OP, DENSE>, tg, kTileThreads, FxTile<4>::bytes, s, G, phi, invh2, out);
     case 6: {
       // opted in here as well: callers without a hierarchy (mg_static.cu)
-      const cudaError_t e = cudaFuncSetAttribute(
-          k_hessian_tile<6, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize, FxTile<6>::bytes);
+      const cudaError_t e =
+          cudaFuncSetAttribute(k_hessian_tile<6, OP, DENSE>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, FxTile<6>::bytes);
       if (e != cudaSuccess) return e;
-      return launch_dep(k_hessian_tile<6, OP>, tg, kTileThreads, FxTile<6>::bytes, s, G, phi, invh2, out);
+      return launch_dep(k_hessian_tile<6, OP, DENSE>, tg, kTileThreads, FxTile<6>::bytes, s, G, phi, invh2, out);
     }
     default: return cudaErrorInvalidValue;
   }
@@ -730,7 +739,18 @@ static cudaError_t launch_hessian(int order, const Grid& G, const double* phi, d
 
 cudaError_t launch_lpt2_source(int order, const Grid& G, const double* phi, double invh2,
                                double* tau, cudaStream_t s) {
-  return launch_hessian<TauOp>(order, G, phi, invh2, tau, s);
+  return launch_hessian<TauOp, false>(order, G, phi, invh2, tau, s);
+}
+
+bool lpt2_source_dense_usable(const Grid& G, const double* phi, const double* tau) {
+  const size_t a = reinterpret_cast<size_t>(phi), b = reinterpret_cast<size_t>(tau);
+  const size_t bytes = (size_t)G.n0 * G.n1 * G.n2 * sizeof(double);
+  return G.n2 % 2 == 0 && a % 16 == 0 && (a + bytes <= b || b + bytes <= a);
+}
+
+cudaError_t launch_lpt2_source_dense(int order, const Grid& G, const double* phi, double invh2,
+                                     double* tau, cudaStream_t s) {
+  return launch_hessian<TauOp, true>(order, G, phi, invh2, tau, s);
 }
 
 cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi, double invh2,
@@ -757,7 +777,7 @@ cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi,
 
 cudaError_t launch_lla(int order, const Grid& G, const double* phi, double invh2, double* out,
                        cudaStream_t s) {
-  return launch_hessian<LlaOp>(order, G, phi, invh2, out, s);
+  return launch_hessian<LlaOp, false>(order, G, phi, invh2, out, s);
 }
 
 cudaError_t launch_axpby(long long n, double a1, const double* x1, double a2, const double* x2,

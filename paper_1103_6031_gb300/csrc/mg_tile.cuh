@@ -235,17 +235,40 @@ __device__ __forceinline__ void tile_gradients(const long long* S, F do_pair) {
   }
 }
 
+// A level as a kernel reads it: padded, with its ghosts filled, or a dense periodic array
+// whose ghosts are the cells one period away (sides at least the halo, even rows).  at(i, j, k):
+// address of cell (i, j, k), of a pair for even k.
+struct PaddedSource {
+  const double* cell0;
+  int sx, sy;
+  __device__ __forceinline__ PaddedSource(const Grid& G, const double* u)
+      : cell0(u + gidx(G, 0, 0, 0)), sx(G.Y * G.Zp), sy(G.Zp) {}
+  __device__ __forceinline__ const double* at(int i, int j, int k) const {
+    return cell0 + ((long long)i * sx + j * sy + k);
+  }
+};
+struct DensePeriodicSource {
+  const double* cell0;
+  int n0, n1, n2;
+  __device__ __forceinline__ DensePeriodicSource(const Grid& G, const double* u)
+      : cell0(u), n0(G.n0), n1(G.n1), n2(G.n2) {}
+  static __device__ __forceinline__ int wrap(int a, int n) {
+    return a < 0 ? a + n : (a >= n ? a - n : a);
+  }
+  __device__ __forceinline__ const double* at(int i, int j, int k) const {
+    return cell0 + ((long long)wrap(i, n0) * n1 + wrap(j, n1)) * n2 + wrap(k, n2);
+  }
+};
+
 // The tile with the edges between two faces as well (mixed derivatives), in two passes:
 // the values into shared memory with their largest exponent, then every value aligned in
 // place.  Cells outside along more than two axes count as 0.
-template <int ORDER>
-__device__ __forceinline__ unsigned tile_load_edges(const Grid& G, const double* __restrict__ u,
-                                                    int i0, int j0, int k0, long long* S) {
+template <int ORDER, typename Src>
+__device__ __forceinline__ unsigned tile_load_edges(const Grid& G, const Src& src, int i0, int j0,
+                                                    int k0, long long* S) {
   typedef FxTile<ORDER> L;
   constexpr int R = L::R, RZ = L::RZ, ZP = L::SZ / 2;
   const int ex = min(kTileX, G.n0 - i0), ey = min(kTileY, G.n1 - j0), ez = min(kTileZ, G.n2 - k0);
-  const int sy = G.Zp, sx = G.Y * G.Zp;
-  const double* base = u + gidx(G, i0, j0, k0);
   double2* D = reinterpret_cast<double2*>(S);
   unsigned m = 0;
 #pragma unroll 4
@@ -259,7 +282,7 @@ __device__ __forceinline__ unsigned tile_load_edges(const Grid& G, const double*
       const bool a = (z >= 0 && z < ez) || (all && z >= -R && z < ez + R);
       const bool b = (z + 1 >= 0 && z + 1 < ez) || (all && z + 1 >= -R && z + 1 < ez + R);
       if (a || b) {
-        v = __ldg(reinterpret_cast<const double2*>(base + (x * sx + y * sy + z)));
+        v = __ldg(reinterpret_cast<const double2*>(src.at(i0 + x, j0 + y, k0 + z)));
         if (!a) v.x = 0.0;
         if (!b) v.y = 0.0;
       }

@@ -116,6 +116,39 @@ def test_tiled_levels(lib, order):
     h.close()
 
 
+@pytest.mark.parametrize("shape", [(4, 4, 4), (20, 36, 34), (12, 8, 70), (20, 24, 35), (3, 5, 6)])
+@pytest.mark.parametrize("order", (2, 4, 6))
+def test_tau_of_one_periodic_level(lib, order, shape):
+    """tau of a single periodic level is read and written dense where its rows are even, phi
+    is 16-byte aligned and the arrays are apart, and through padded copies otherwise; both
+    match the oracle, also where every tile takes the FP64 route."""
+    import torch
+    from oracle.hierarchy import Hierarchy as OracleHierarchy
+    from oracle.lpt import lpt2_source as oracle_tau
+    geom = Geometry(shape, 7.0, order, ())
+    x = np.random.Generator(np.random.PCG64(2)).standard_normal(shape)
+    want = oracle_tau(OracleHierarchy(geom), [x])[0]
+    h = lib.Hierarchy(lib.config_from_geometry(geom))
+
+    def off(a, b):
+        a = a.cpu().numpy()
+        return np.sqrt(np.sum((a - b) ** 2) / np.sum(b * b))
+
+    phi = torch.from_numpy(x).cuda()
+    assert off(h.lpt2_source([phi])[0], want) < TOL
+    shifted = torch.empty(phi.numel() + 1, dtype=torch.float64, device="cuda")[1:].view(shape)
+    shifted.copy_(phi)
+    assert off(h.lpt2_source([shifted])[0], want) < TOL
+    tiny = torch.from_numpy(np.ldexp(x, -480)).cuda()
+    assert off(torch.ldexp(h.lpt2_source([tiny])[0],
+                           torch.tensor(960.0, dtype=torch.float64, device="cuda")), want) < TOL
+    # in place
+    from paper_1103_6031_gb300.mg import _ptrs
+    assert h.lib.mg_lpt2_source(h.h, _ptrs([phi]), _ptrs([phi])) == 0
+    assert off(phi, want) < TOL
+    h.close()
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_a_source_that_is_not_finite(lib, bad):
     geom = GEOMS[6]
