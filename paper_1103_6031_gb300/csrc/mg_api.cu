@@ -942,8 +942,8 @@ LevelRanges leaf_ranges(const mg_hierarchy* h) {
 }
 
 // Leaf residual norm after syncing covered cells, queued on the stream (no
-// host synchronisation, so it can be captured); ends with the copy of 4
-// doubles to pinned host memory.  In MG_MIXED the residual is also stored
+// host synchronisation, so it can be captured); the record also goes to pinned
+// host memory.  In MG_MIXED the residual is also stored
 // (float32) as the correction source.
 mg_status norm_launches(mg_hierarchy* h, bool zero_u = false, bool copy_out = true) {
   if (!zero_u) ST(sync_covered(h));
@@ -958,10 +958,8 @@ mg_status norm_launches(mg_hierarchy* h, bool zero_u = false, bool copy_out = tr
                            h->mixed ? L.s.ffas : nullptr, h->s));
   }
   KL(MG_K_NORM, h->partial_slots,
-     launch_reduce_levels(h->partial, h->partial_slots, leaf_ranges(h), h->red, h->red + 8, h->s));
-  if (copy_out)
-    CK(cudaMemcpyAsync(h->host_red, h->red, kRedDoubles * sizeof(double), cudaMemcpyDeviceToHost,
-                       h->s));
+     launch_reduce_levels(h->partial, h->partial_slots, leaf_ranges(h), h->red, h->red + 8,
+                          copy_out ? h->host_red : nullptr, h->s));
   return MG_OK;
 }
 

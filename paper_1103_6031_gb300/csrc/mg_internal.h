@@ -182,8 +182,9 @@ struct LevelRanges {
 };
 // out[0..1] = the sums of all `count` pairs (the same order as launch_reduce_partials);
 // out_levels[2 l .. 2 l + 1] = the sums of leaf level l's pairs.
+// host (may be NULL): pinned host memory that gets the same, and out[2..4], at the same offsets.
 cudaError_t launch_reduce_levels(const double* partial, int count, const LevelRanges& R,
-                                 double* out, double* out_levels, cudaStream_t s);
+                                 double* out, double* out_levels, double* host, cudaStream_t s);
 cudaError_t launch_pack(const Grid& G, const double* src, double* dst, double shift,
                         cudaStream_t s);
 // dense dst = padded interior of src + add

@@ -240,10 +240,13 @@ __global__ void __launch_bounds__(kRedBlock)
 
 // Block 0: exactly k_reduce_partials over all `count` pairs into out[0], out[1].
 // Block 1 + l: the pairs of leaf level l alone, [R.off[l], R.off[l] + R.cnt[l]), into
-// out_levels[2 l], out_levels[2 l + 1] (the per-level residual and source sums).
+// out_levels[2 l], out_levels[2 l + 1] (the per-level residual and source sums).  With host
+// (pinned host memory, laid out like the record that starts at out) the record's entries go
+// there as well, so that no copy follows: out[2..4], left by earlier kernels, by block 0.
 __global__ void __launch_bounds__(kRedBlock)
     k_reduce_levels(const double* __restrict__ partial, int count, LevelRanges R,
-                    double* __restrict__ out, double* __restrict__ out_levels) {
+                    double* __restrict__ out, double* __restrict__ out_levels,
+                    double* __restrict__ host) {
   grid_wait();
   int lo = 0, hi = count;
   if (blockIdx.x > 0) {
@@ -260,6 +263,13 @@ __global__ void __launch_bounds__(kRedBlock)
     double* o = blockIdx.x == 0 ? out : out_levels + 2 * (blockIdx.x - 1);
     o[0] = a;
     o[1] = b;
+    if (host) {
+      double* ho = host + (o - out);
+      ho[0] = a;
+      ho[1] = b;
+      if (blockIdx.x == 0)
+        for (int q = 2; q < 5; ++q) host[q] = out[q];
+    }
   }
 }
 
@@ -678,11 +688,11 @@ cudaError_t launch_reduce_partials(const double* partial, int count, int width, 
 }
 
 cudaError_t launch_reduce_levels(const double* partial, int count, const LevelRanges& R,
-                                 double* out, double* out_levels, cudaStream_t s) {
+                                 double* out, double* out_levels, double* host, cudaStream_t s) {
   if (R.n < 0 || R.n > MG_MAX_LEVELS) return cudaErrorInvalidValue;
   for (int l = 0; l < R.n; ++l)
     if (R.off[l] < 0 || R.cnt[l] < 0 || R.off[l] + R.cnt[l] > count) return cudaErrorInvalidValue;
-  return launch_dep(k_reduce_levels, 1 + R.n, kRedBlock, 0, s, partial, count, R, out, out_levels);
+  return launch_dep(k_reduce_levels, 1 + R.n, kRedBlock, 0, s, partial, count, R, out, out_levels, host);
 }
 
 cudaError_t launch_pack(const Grid& G, const double* src, double* dst, double shift,
