@@ -611,7 +611,8 @@ int finest(const mg_hierarchy* h) { return (int)h->L.size() - 1; }
 // cells.  Measured in CUDA graphs on GB300: it beats the plain kernel by ~25% on a
 // 256^3 float32 nest, ties at 128^3 and loses below (each block marches through 8
 // planes in sequence, so small grids have too few blocks), and loses on periodic
-// levels (ghost-image stores); the float64 smoother is bound by the FP64 pipe.
+// levels (ghost-image stores); the float64 smoother is bound by instruction issue, which
+// staged planes do not lower.
 constexpr long long kTmaMinCells = 1ll << 23;
 
 template <typename T>

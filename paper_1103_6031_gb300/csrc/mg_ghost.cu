@@ -1,7 +1,8 @@
 // Ghost zones (Hahn & Abel 2011, Sec. 3.2 periodic boundaries; Sec. 3.3
 // coarse-fine boundaries).
 //
-// Coarse-fine faces of a nest, in three kernels:
+// Coarse-fine faces of a nest, in three steps (large nests and float64 leave the flux step
+// its own launch; small ones run it with the half-sweep, k_smooth_faces in mg_smooth.cu):
 //  * k_cf_tangential (once per parent state): for each face, each of the n/2
 //    parent layers outside it and each fine tangential position, the degree-n
 //    tensor Lagrange interpolant of the parent values parallel to the face
@@ -13,7 +14,8 @@
 //    the parent flux with covered parent cells taken as the mean of their
 //    current 8 children (two-way interface); the mean of the 4 fine fluxes;
 //    and the difference added uniformly to the ghosts of each column so that
-//    the fine fluxes average to the parent flux.
+//    the fine fluxes average to the parent flux.  MG_FP64 folds everything linear into
+//    per-layer weights and the interpolants (k_cf_flux_fold).
 //  * k_cf_edges (before the 2LPT source only): edge and corner ghosts, which
 //    only mixed derivatives read, by tensor degree-n interpolation of parent
 //    values.
@@ -66,7 +68,7 @@ struct TangFold {
 // a row serves the up to ORDER + 1 elements whose patch it is in, so an element of order 6
 // costs 53 operations per layer (126 when every element reduces its own 7 rows).  Every
 // value is the same chain of fmas either way.  FP64-bound in float64: 128^3 nest, order 6,
-// 23.2 us before (cold).
+// cold, 23.2 us with an element per thread, 16.1 so, 19.5 with the folded coarse parts.
 template <int ORDER, typename T, bool FOLD>
 __device__ __forceinline__ void tangential_tile(const Grid& F, const Grid& P,
                                                 const T* __restrict__ pu, Int3 off,

@@ -1,9 +1,9 @@
 // Issue rate of the FP64 pipe, measured on the device in use.
 //
-// The float64 stencil kernels of this library need more FP64 instructions per
-// HBM byte than the GPU's FP64 pipe can issue at its copy bandwidth, so their
-// roofline is the FP64 issue rate, not HBM.  This probe measures that rate the
-// way the stencils use the pipe: every thread runs 8 independent chains of
+// A float64 stencil of this library summed with FP64 instructions needs more of them per
+// HBM byte than the GPU's FP64 pipe can issue at its copy bandwidth, which is why MG_FP64 sums
+// on the integer pipe (mg_fixed.cuh); the FP64 instructions that remain are compared with
+// this rate.  The probe measures it the way the stencils use the pipe: every thread runs 8 independent chains of
 // fused multiply-adds (enough independent work per warp to cover the pipe's
 // latency), on a grid of 8 blocks of 256 threads per SM, timed with CUDA events.
 //

@@ -7,7 +7,9 @@
 // the 7-point stencil; for 13/19 points same-colour cells at distance 2 couple
 // and this fixes their order).  The kernel reads buffer `uin` and writes every
 // interior cell of `uout` (colour c updated, the other colour copied), so no
-// thread ever reads a value another thread of the same launch writes.
+// thread ever reads a value another thread of the same launch writes.  k_smooth_faces is the
+// half-sweep of a small nest with the coarse-fine ghosts of its result, k_smooth_fas the
+// float32 half-sweep after a restriction with the FAS source.
 #include "mg_internal.h"
 #include "mg_launch.cuh"
 #include "mg_stencil.cuh"

@@ -1,11 +1,12 @@
 // Bodies of the kernels of one float32/float64 V-cycle (Hahn & Abel 2011, Sec. 3.2
-// steps 2-9; Sec. 3.3), written once and run two ways: by their own stream kernels
-// (one launch per level operation, block and thread indices from the hardware) and
-// by the persistent batch kernel (mg_persist.cu), which runs any block of any level
-// operation of any hierarchy as a work item of a 128-thread block.  Every body gets
+// steps 2-9; Sec. 3.3), run two ways: by stream kernels (block and thread indices from the
+// hardware) and by the persistent batch kernel (mg_persist.cu), which runs any block of any
+// level operation of any hierarchy as a work item of a 128-thread block.  Every body gets
 // its block and thread indices as arguments and loads through a policy (Ldg in the
-// stream kernels, Weak in the persistent kernel); the arithmetic is the same code,
-// so both ways give bit-identical results.
+// stream kernels, Weak in the persistent kernel).  residual_restrict_body and
+// cf_tangential_body serve the persistent kernel only: the stream kernels share a parent's
+// or a tile's work between threads, with the operations of every value in the same order, so
+// both ways give bit-identical results in float32, which is all the persistent kernel runs.
 #pragma once
 
 #include "mg_internal.h"
