@@ -2661,6 +2661,26 @@ mg_status mg_lla_density(mg_hierarchy* h, const double* const phi1[], const doub
   if (!std::isfinite(a1) || !std::isfinite(a2))
     return fail(h, MG_EINVAL, "a1 and a2 must be finite");
   return on_streams(h, [&]() -> mg_status {
+    // One periodic level with even rows: Phi stays dense in the scratch array (apart from rho,
+    // which may be phi1 or phi2) and the mean comes off rho in place.  Same tiles and same
+    // order of every sum as through the padded arrays, so the same bits; without the pack, the
+    // ghost fill and one of two output passes: 128x192x160, order 4, 348 -> 331 us.
+    if (nleaf == 1 && h->L[h->base].G.n2 % 2 == 0) {
+      DevLevel& L = h->L[h->base];
+      const long long n = cells_of(L.G);
+      const Grid flat{L.G.n0, L.G.n1, L.G.n2, 0, 0, L.G.n1, L.G.n2, L.G.n0};
+      KL(MG_K_COPY, n, launch_axpby(n, a1, phi1[0], a2, phi2 ? phi2[0] : nullptr, h->scratch, h->s));
+      KL(MG_K_LPT, n,
+         launch_lla_dense(h->cfg.order, L.G, h->scratch, 1.0 / (L.geo.h * L.geo.h), rho[0], h->s));
+      KL(MG_K_NORM, n,
+         launch_sum_partial(flat, rho[0], L.geo.h * L.geo.h * L.geo.h, L.child_lo, L.child_hi,
+                            h->partial + 2 * L.partial_off, L.nblocks, h->s));
+      KL(MG_K_NORM, h->partial_slots,
+         launch_reduce_partials(h->partial, h->partial_slots, 2, h->red + 2, h->s));
+      KL(MG_K_COPY, n, launch_sub_mean(rho[0], n, h->red + 2, 1.0 / h->volume, h->s, 1.0));
+      CK(cudaStreamSynchronize(h->s));
+      return MG_OK;
+    }
     // Phi = a1 phi1 + a2 phi2 into the float64 u of every leaf level
     for (int l = h->base; l <= finest(h); ++l) {
       DevLevel& L = h->L[l];

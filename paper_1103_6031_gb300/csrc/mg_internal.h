@@ -169,7 +169,8 @@ cudaError_t launch_add_correction(const Grid& G, double* u, const float* e, int 
                                   cudaStream_t s);
 // p[0..n) -= sum[0] * scale, with sum on the device
 cudaError_t launch_sub_mean(double* p, long long n, const double* sum, double scale,
-                            cudaStream_t s);
+                            cudaStream_t s,
+                            double add = 0.0);
 cudaError_t launch_sum_partial(const Grid& G, const double* f, double vol, Int3 clo, Int3 chi,
                                double* partial, int blocks, cudaStream_t s);
 cudaError_t launch_reduce_partials(const double* partial, int count, int width, double* out,
@@ -208,6 +209,9 @@ cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi,
 // edges filled)
 cudaError_t launch_lla(int order, const Grid& G, const double* phi, double invh2, double* out,
                        cudaStream_t s);
+// the same from a dense, 16-byte aligned phi of a periodic level with even rows to a dense out
+cudaError_t launch_lla_dense(int order, const Grid& G, const double* phi, double invh2,
+                             double* out, cudaStream_t s);
 // out = a1 x1 + a2 x2 over n dense elements (x2 may be NULL)
 cudaError_t launch_axpby(long long n, double a1, const double* x1, double a2, const double* x2,
                          double* out, cudaStream_t s);

@@ -328,12 +328,15 @@ __global__ void __launch_bounds__(128)
   if (periodic) write_images<double>(G, u, i, j, k, v);
 }
 
-// p -= sum[0] * scale over n elements (sum read on the device).
+// p = p - sum[0] * scale (+ add) over n elements (sum read on the device).
 __global__ void __launch_bounds__(256)
-    k_sub_mean(double* __restrict__ p, long long n, const double* __restrict__ sum, double scale) {
+    k_sub_mean(double* __restrict__ p, long long n, const double* __restrict__ sum, double scale,
+               double add) {
   grid_wait();
   const long long t = blockIdx.x * 256LL + threadIdx.x;
-  if (t < n) p[t] -= sum[0] * scale;
+  if (t >= n) return;
+  const double v = p[t] - sum[0] * scale;
+  p[t] = add != 0.0 ? v + add : v;
 }
 
 __global__ void __launch_bounds__(256) k_fill(double* __restrict__ p, long long n, double v) {
@@ -718,9 +721,9 @@ cudaError_t launch_add_correction(const Grid& G, double* u, const float* e, int 
 }
 
 cudaError_t launch_sub_mean(double* p, long long n, const double* sum, double scale,
-                            cudaStream_t s) {
+                            cudaStream_t s, double add) {
   if (n <= 0) return cudaSuccess;
-  return launch_dep(k_sub_mean, blocks_for(n, 256), 256, 0, s, p, n, sum, scale);
+  return launch_dep(k_sub_mean, blocks_for(n, 256), 256, 0, s, p, n, sum, scale, add);
 }
 
 cudaError_t launch_fill(double* p, long long n, double v, cudaStream_t s) {
@@ -788,6 +791,11 @@ cudaError_t launch_lpt2_source_fp64(int order, const Grid& G, const double* phi,
 cudaError_t launch_lla(int order, const Grid& G, const double* phi, double invh2, double* out,
                        cudaStream_t s) {
   return launch_hessian<LlaOp, false>(order, G, phi, invh2, out, s);
+}
+
+cudaError_t launch_lla_dense(int order, const Grid& G, const double* phi, double invh2,
+                             double* out, cudaStream_t s) {
+  return launch_hessian<LlaOp, true>(order, G, phi, invh2, out, s);
 }
 
 cudaError_t launch_axpby(long long n, double a1, const double* x1, double a2, const double* x2,

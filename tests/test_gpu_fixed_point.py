@@ -149,6 +149,39 @@ def test_tau_of_one_periodic_level(lib, order, shape):
     h.close()
 
 
+@pytest.mark.parametrize("shape", [(4, 4, 4), (20, 36, 34), (12, 8, 70), (20, 24, 35), (3, 5, 6)])
+@pytest.mark.parametrize("order", (2, 4, 6))
+def test_local_density_of_one_periodic_level(lib, order, shape):
+    """The local density of a single periodic level goes through dense arrays where its rows
+    are even and through padded ones otherwise; both match the oracle, with an output that is
+    one of the inputs or starts on an odd element too."""
+    import torch
+    from oracle.hierarchy import Hierarchy as OracleHierarchy
+    from oracle.lpt import lla_density as oracle_lla
+    from paper_1103_6031_gb300.mg import _ptrs
+    geom = Geometry(shape, 7.0, order, ())
+    rng = np.random.Generator(np.random.PCG64(4))
+    x, y = rng.standard_normal(shape), rng.standard_normal(shape)
+    # second derivatives of 0.1 at most: no shell crossing
+    hh = (7.0 / shape[0]) ** 2
+    a1, a2 = 0.1 * hh / (40 * np.abs(x).max()), 0.04 * hh / (40 * np.abs(y).max())
+    want = oracle_lla(OracleHierarchy(geom), [x], [y], a1, a2)[0]
+    h = lib.Hierarchy(lib.config_from_geometry(geom))
+
+    def off(a):
+        a = a.cpu().numpy()
+        return np.sqrt(np.sum((a - want) ** 2) / np.sum((want - 1.0) ** 2))
+
+    p, q = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+    # rho - 1 is about 1e-3, stored next to 1 (2^-53)
+    assert off(h.lla_density([p], [q], a1, a2)[0]) < TOL
+    odd = torch.empty(p.numel() + 1, dtype=torch.float64, device="cuda")[1:].view(shape)
+    for out in (odd, p):
+        assert h.lib.mg_lla_density(h.h, _ptrs([p]), _ptrs([q]), a1, a2, _ptrs([out])) == 0
+        assert off(out) < TOL
+    h.close()
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_a_source_that_is_not_finite(lib, bad):
     geom = GEOMS[6]
