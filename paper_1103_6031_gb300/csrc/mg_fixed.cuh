@@ -106,9 +106,15 @@ struct FxUnit<6> {
   static constexpr double v = 256.0 / 180.0;
 };
 
+// The integer formulas below are written over the integer type I, so that a host program can
+// run them on a type that records the size of every intermediate.  In units of 2^59, above
+// which no aligned value lies, the largest intermediates at orders 2 / 4 / 6 are: Laplacian
+// 12 / 12 / 12.75, second difference 4 / 4.13 / 4.34, first derivative 2 / 2.25 / 6, first
+// derivative of first derivatives 4 / 5.07 / 10.32.  64 bits hold 16.
+
 // The neighbours' part of T from their sums at distance 1, 2, 3.
-template <int ORDER>
-__device__ __forceinline__ long long fx_weighted(const long long (&s)[3]) {
+template <int ORDER, typename I>
+__host__ __device__ __forceinline__ I fx_weighted(const I (&s)[3]) {
   if (ORDER == 2) return s[0];
   if (ORDER == 4) return s[0] - (s[1] >> 4);
   // 270/256 = 1 + 1/16 - 1/128, 27/256 = 1/8 - 1/64 - 1/256, 2/256 = 1/128
@@ -138,34 +144,36 @@ __device__ __forceinline__ long long fx_neighbours(const double (&nb)[3 * ORDER]
 }
 
 // The centre's term of T (weight 3 w0), c its aligned integer.
-template <int ORDER>
-__device__ __forceinline__ long long fx_centre(long long c) {
+template <int ORDER, typename I>
+__host__ __device__ __forceinline__ I fx_centre(I c) {
   if (ORDER == 2) return -6 * c;
   if (ORDER == 4) return -6 * c + (c >> 2) + (c >> 3);  // 90/16 = 6 - 1/4 - 1/8
   return -6 * c + (c >> 2) + (c >> 7);                  // 1470/256 = 6 - 1/4 - 1/128
 }
 
 // One axis: h^2 u'' = T FxUnit 2^(e - kFxBias) from the sums u(+d) + u(-d) and the centre.
-template <int ORDER>
-__device__ __forceinline__ long long fx_second(const long long (&s)[3], long long c) {
+template <int ORDER, typename I>
+__host__ __device__ __forceinline__ I fx_second(const I (&s)[3], I c) {
   if (ORDER == 2) return s[0] - 2 * c;
   if (ORDER == 4) return fx_weighted<4>(s) - 2 * c + (c >> 3);  // 30/16 = 2 - 1/8
   return fx_weighted<6>(s) - 2 * c + (c >> 4) + (c >> 6) + (c >> 7);  // 490/256 = 2 - 22/256
 }
 
 // One axis: h u' = T FxGradUnit 2^(e - kFxBias) from the differences u(+d) - u(-d); order 6:
-// T = (45 d1 - 9 d2 + d3) / 64, order 4: (8 d1 - d2) / 8.  |T| <= 2 max |u|, so that the
-// operator can be applied to its own result.
+// T = (45 d1 - 9 d2 + d3) / 64, order 4: (8 d1 - d2) / 8.  |T| <= 2, 9/4, 110/64 max |u|.  The
+// operator is applied to its own result for mixed derivatives, whose differences reach 3.44
+// max |u| at order 6: every term is shifted before its factor could carry the sum past 64
+// bits (45/64 = 1 - 1/4 - 1/32 - 1/64).
 template <int ORDER>
 struct FxGradUnit {
   static constexpr double v = ORDER == 2 ? 0.5 : (ORDER == 4 ? 8.0 / 12.0 : 64.0 / 60.0);
 };
 
-template <int ORDER>
-__device__ __forceinline__ long long fx_first(const long long (&d)[3]) {
+template <int ORDER, typename I>
+__host__ __device__ __forceinline__ I fx_first(const I (&d)[3]) {
   if (ORDER == 2) return d[0];
   if (ORDER == 4) return d[0] - (d[1] >> 3);
-  return d[0] - (d[0] >> 2) - (d[1] >> 3) + ((d[2] - d[1] - 3 * d[0]) >> 6);  // 45/64 = 1 - 1/4 - 3/64
+  return d[0] - (d[0] >> 2) - (d[0] >> 5) - (d[1] >> 3) + ((d[2] - d[1] - d[0]) >> 6);
 }
 
 }  // namespace mgk
