@@ -15,10 +15,11 @@
 // weights by a few such units, the conversion rounds to 53 bits.  A sum in FP64
 // arithmetic rounds at every addition, each time by up to 2^-53 of its partial sum, so
 // the result here is the more accurate one unless a whole stencil cancels below 2^-6 of
-// its largest value, where both are at the rounding level of the values themselves.  The
-// alignment depends only on the cell's own neighbours (no level-wide scale, no state), and
-// the integer sums do not depend on the order: every kernel that uses these functions on
-// the same values gives the same bits.
+// its largest value, where both are at the rounding level of the values themselves.  In the
+// kernels that work cell by cell the alignment depends only on the cell's own neighbours (no
+// level-wide scale, no state) and the integer sums do not depend on the order: these kernels
+// give the same bits on the same values.  The tile kernels (mg_tile.cuh) align to the largest
+// value of a block of cells instead and leave blocks of too wide a range to FP64.
 //
 // Range: the largest neighbour must be finite and at least 2^-926 in magnitude (biased
 // exponent kFxMinExp); otherwise (all zero, denormal, infinite, NaN) the caller uses FP64

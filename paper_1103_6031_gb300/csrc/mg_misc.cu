@@ -156,12 +156,17 @@ __global__ void __launch_bounds__(kTileThreads, 3)
                        min(j0 + kTileY, G.n1) <= chi.y && k0 >= clo.z &&
                        min(k0 + kTileZ, G.n2) <= chi.z;
   if (!covered) {
-    const unsigned key = tile_load<ORDER>(G, u, i0, j0, k0, norm_smem);
     const TilePos t = tile_pos();
     const int i = i0 + 4 * t.xh, j = j0 + t.y, k = k0 + 2 * t.zz;
     const long long p = gidx(G, i, j, k);
     const int sx = G.Y * G.Zp;
     const double kr = -invh2 * FxUnit<ORDER>::v;
+    double2 fv[4];  // under way while the tile is filled
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      fv[q] = i + q < G.n0 && j < G.n1 && k < G.n2
+                  ? __ldg(reinterpret_cast<const double2*>(f + p + q * sx)) : make_double2(0.0, 0.0);
+    const unsigned key = tile_load<ORDER>(G, u, i0, j0, k0, norm_smem);
     const bool fx = fx_in_range(key) && fx_scalable(kr, key);
     const double ks = fx_scale(kr, key);
     auto leaf = [&](int q, int dk) {
@@ -175,11 +180,8 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     };
     if (fx) {
       tile_laplacians<ORDER>(norm_smem, [&](int q, longlong2 T, longlong2) {
-        const bool l0 = leaf(q, 0), l1 = leaf(q, 1);
-        if (!(l0 || l1)) return;
-        const double2 fv = __ldg(reinterpret_cast<const double2*>(f + p + q * sx));
-        if (l0) add(fma(ks, (double)T.x, fv.x), fv.x);
-        if (l1) add(fma(ks, (double)T.y, fv.y), fv.y);
+        if (leaf(q, 0)) add(fma(ks, (double)T.x, fv[q].x), fv[q].x);
+        if (leaf(q, 1)) add(fma(ks, (double)T.y, fv[q].y), fv[q].y);
       });
     } else {
 #pragma unroll 1

@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(128)
 }
 
 // The same on tiles of aligned integers (mg_tile.cuh), float64: the mean of a parent's 8
-// children and of their T are integer sums (T shifted by 3 first, so that the sum cannot
-// overflow: 2^-56 of the tile's largest value), leaving about 12 FP64 instructions per
+// children and of their T are integer sums (every T shifted by 3 first, so that the sum cannot
+// overflow: up to 8 more units lost of a mean's 20, mg_tile.cuh), leaving about 12 FP64 instructions per
 // parent cell, 7 of them the sum of f.  A thread holds 2 x 1 x 2 children of two parents;
 // the row above or below is in the other half of its warp.
 template <int ORDER>

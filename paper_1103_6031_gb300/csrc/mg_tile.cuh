@@ -8,6 +8,13 @@
 // instructions per cell; 63 KB of shared memory at order 6 let three blocks share an SM,
 // so that one block's loads overlap the others' sums.  A half-sweep, which needs only
 // every second cell's sum, gains nothing from it (17.8 against 17.6 us at 128^3).
+//
+// Accuracy: a unit is 2^-58 to 2^-59 of the BLOCK's largest value (halo included), not of the
+// cell's own neighbours'.  A tile is summed as integers only if every cell's star holds a value
+// of at least 2^52 units or nothing but zeros (tile_too_wide); the rounding of a difference, at
+// most 30 units, then stays below 2^-47 of the largest value in the cell's own star, and is far
+// smaller where that is the block's largest too.  Other tiles (a strong cell among weak ones, a
+// steep tail) are left to FP64 arithmetic.
 #pragma once
 
 #include "mg_fixed.cuh"
@@ -59,6 +66,31 @@ __device__ __forceinline__ TilePos tile_pos() {
   return TilePos{t & 15, (t >> 4) & 7, t >> 7};
 }
 
+// A level as a kernel reads it: padded, with its ghosts filled, or a dense periodic array
+// whose ghosts are the cells one period away (sides at least the halo, even rows).  at(i, j, k):
+// address of cell (i, j, k), of a pair for even k.
+struct PaddedSource {
+  const double* cell0;
+  int sx, sy;
+  __device__ __forceinline__ PaddedSource(const Grid& G, const double* u)
+      : cell0(u + gidx(G, 0, 0, 0)), sx(G.Y * G.Zp), sy(G.Zp) {}
+  __device__ __forceinline__ const double* at(int i, int j, int k) const {
+    return cell0 + ((long long)i * sx + j * sy + k);
+  }
+};
+struct DensePeriodicSource {
+  const double* cell0;
+  int n0, n1, n2;
+  __device__ __forceinline__ DensePeriodicSource(const Grid& G, const double* u)
+      : cell0(u), n0(G.n0), n1(G.n1), n2(G.n2) {}
+  static __device__ __forceinline__ int wrap(int a, int n) {
+    return a < 0 ? a + n : (a >= n ? a - n : a);
+  }
+  __device__ __forceinline__ const double* at(int i, int j, int k) const {
+    return cell0 + ((long long)wrap(i, n0) * n1 + wrap(j, n1)) * n2 + wrap(k, n2);
+  }
+};
+
 __device__ __forceinline__ unsigned block_max(unsigned m) {
   __shared__ unsigned red[kTileThreads / 32];
   m = __reduce_max_sync(~0u, m);
@@ -69,10 +101,90 @@ __device__ __forceinline__ unsigned block_max(unsigned m) {
   return m;
 }
 
+// Exponents a cell's star may lie below the block's largest: the bits that an aligned value has
+// beyond a mantissa's 53.  Tiles of a smooth field pass, also where it is zero on a surface:
+// its star reaches ORDER / 2 cells to either side, a tile 32.
+constexpr int kTileRange = 6;
+
+// Of a thread's cells (tile_pos: a z-pair in 4 planes, a and b their keys or magnitudes) those
+// whose stars may be too low, as bits 2 q + dk: neither the cell nor its neighbours among the
+// thread's lie above lim.  in(q): which cells of the pair exist.  Of the tiles of a potential 2%
+// have such cells, 35% cells that are low themselves.
+template <int ORDER, typename In>
+__device__ __forceinline__ unsigned low_cells(const unsigned (&a)[4], const unsigned (&b)[4],
+                                              unsigned lim, In in) {
+  constexpr int R = ORDER / 2;
+  // the least of the windows' largest: every x neighbourhood within the 4 planes holds one
+  constexpr int W = R < 3 ? R + 1 : 4;
+  unsigned least = ~0u;
+#pragma unroll
+  for (int q = 0; q + W <= 4; q += 4 - W > 0 ? 4 - W : 4) {
+    unsigned ma = 0, mb = 0;
+#pragma unroll
+    for (int n = q; n < q + W; ++n) {
+      ma = max(ma, a[n]);
+      mb = max(mb, b[n]);
+    }
+    least = min(least, min(ma, mb));
+  }
+  if (least > lim) return 0;
+  unsigned low = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    unsigned ma = b[q], mb = a[q];
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+      if (n - q <= R && q - n <= R) {
+        ma = max(ma, a[n]);
+        mb = max(mb, b[n]);
+      }
+    low |= (((ma <= lim ? 1u : 0u) | (mb <= lim ? 2u : 0u)) & in(q)) << (2 * q);
+  }
+  return low;
+}
+
+// Ends the filling of a tile: its key, or 0 (out of range: FP64 arithmetic) where the star of a
+// cell holds only values more than 2^kTileRange below the block's largest, and not only zeros (a
+// star that the alignment leaves nothing of is looked up in src, the tile at (i0, j0, k0)).
+// low: the thread's cells to look at (low_cells).  The same answer in every thread.  What the
+// question costs, without / with, order 6: the first-cycle restrictions of a 192 x 160 x 224 level
+// and the next 36.9 / 40.9 us, its norm 83.8 / 82.6 (with f loaded ahead), tau of 256^3 705 / 721,
+// a whole step 0.5 to 2%; asked after the sums, the restriction takes 38.9, the norm 85.8, tau 737.
+template <int ORDER, typename Src>
+__device__ __forceinline__ unsigned tile_key(unsigned key, const long long* S, const Src& src,
+                                             int i0, int j0, int k0, unsigned low) {
+  typedef FxTile<ORDER> L;
+  constexpr long long kWeak = 1ll << (58 - kTileRange);
+  auto mag = [](long long v) { return v ^ (v >> 63); };
+  if (__builtin_expect(!__syncthreads_or(low), 1)) return key;
+  const TilePos t = tile_pos();
+  bool wide = false;
+#pragma unroll 1
+  for (; low; low &= low - 1) {
+    const int bit = __ffs(low) - 1;
+    const int x = 4 * t.xh + (bit >> 1), y = t.y, z = 2 * t.zz + (bit & 1);
+    const long long* c = S + L::at(x, y, z);
+    long long m = mag(c[0]);
+#pragma unroll 1
+    for (int d = 1; d <= L::R; ++d)
+      m |= mag(c[d]) | mag(c[-d]) | mag(c[d * L::py]) | mag(c[-d * L::py]) | mag(c[d * L::px]) |
+           mag(c[-d * L::px]);
+    if (m >= kWeak) continue;
+    wide |= m != 0;
+    if (m == 0)
+#pragma unroll 1
+      for (int d = -L::R; d <= L::R; ++d)
+        wide |= __ldg(src.at(i0 + x + d, j0 + y, k0 + z)) != 0.0 ||
+                __ldg(src.at(i0 + x, j0 + y + d, k0 + z)) != 0.0 ||
+                __ldg(src.at(i0 + x, j0 + y, k0 + z + d)) != 0.0;
+  }
+  return __syncthreads_or(wide) ? 0u : key;
+}
+
 // Loads the tile at cell (i0, j0, k0) of u with its star halo into S, aligned to the
 // returned key (low bits set).  Values outside the stencils' reach (beyond the ghosts,
-// row padding, edge and corner ghosts) count as 0.  If the key is out of range
-// (fx_in_range), S is not written.
+// row padding, edge and corner ghosts) count as 0.  If the returned key is out of range
+// (fx_in_range; 0 for a tile of too wide a range), S is not to be used.
 template <int ORDER>
 __device__ __forceinline__ unsigned tile_load(const Grid& G, const double* __restrict__ u, int i0,
                                               int j0, int k0, long long* S) {
@@ -151,8 +263,19 @@ __device__ __forceinline__ unsigned tile_load(const Grid& G, const double* __res
     }
     if (zact) put(zx, zy, zo, vz);
   }
-  __syncthreads();
-  return m;
+  unsigned low = 0;
+  if (fx_in_range(m)) {
+    unsigned a[4], b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      a[q] = fx_key(c[q].x);
+      b[q] = fx_key(c[q].y);
+    }
+    low = low_cells<ORDER>(a, b, m - ((kTileRange + 1u) << 21), [&](int q) {
+      return 4 * t.xh + q < ex && t.y < ey ? (in0 ? 1u : 0u) | (in1 ? 2u : 0u) : 0u;
+    });
+  }
+  return tile_key<ORDER>(m, S, PaddedSource(G, u), i0, j0, k0, low);
 }
 
 // T (mg_fixed.cuh: h^2 L u = T FxUnit 2^(e - kFxBias)) of the thread's 8 cells and their
@@ -237,31 +360,6 @@ __device__ __forceinline__ void tile_gradients(const long long* S, F do_pair) {
   }
 }
 
-// A level as a kernel reads it: padded, with its ghosts filled, or a dense periodic array
-// whose ghosts are the cells one period away (sides at least the halo, even rows).  at(i, j, k):
-// address of cell (i, j, k), of a pair for even k.
-struct PaddedSource {
-  const double* cell0;
-  int sx, sy;
-  __device__ __forceinline__ PaddedSource(const Grid& G, const double* u)
-      : cell0(u + gidx(G, 0, 0, 0)), sx(G.Y * G.Zp), sy(G.Zp) {}
-  __device__ __forceinline__ const double* at(int i, int j, int k) const {
-    return cell0 + ((long long)i * sx + j * sy + k);
-  }
-};
-struct DensePeriodicSource {
-  const double* cell0;
-  int n0, n1, n2;
-  __device__ __forceinline__ DensePeriodicSource(const Grid& G, const double* u)
-      : cell0(u), n0(G.n0), n1(G.n1), n2(G.n2) {}
-  static __device__ __forceinline__ int wrap(int a, int n) {
-    return a < 0 ? a + n : (a >= n ? a - n : a);
-  }
-  __device__ __forceinline__ const double* at(int i, int j, int k) const {
-    return cell0 + ((long long)wrap(i, n0) * n1 + wrap(j, n1)) * n2 + wrap(k, n2);
-  }
-};
-
 // The tile with the edges between two faces as well (mixed derivatives), in two passes:
 // the values into shared memory with their largest exponent, then every value aligned in
 // place.  Cells outside along more than two axes count as 0.
@@ -302,7 +400,23 @@ __device__ __forceinline__ unsigned tile_load_edges(const Grid& G, const Src& sr
     }
   }
   __syncthreads();
-  return m;
+  unsigned low = 0;
+  if (fx_in_range(m)) {
+    const TilePos t = tile_pos();
+    unsigned a[4], b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const longlong2 v =
+          *reinterpret_cast<const longlong2*>(S + L::at(4 * t.xh + q, t.y, 2 * t.zz));
+      a[q] = (unsigned)((int)(v.x >> 32) ^ (int)(v.x >> 63));
+      b[q] = (unsigned)((int)(v.y >> 32) ^ (int)(v.y >> 63));
+    }
+    low = low_cells<ORDER>(a, b, (1u << (26 - kTileRange)) - 1u, [&](int q) {
+      return 4 * t.xh + q < ex && t.y < ey
+                 ? (2 * t.zz < ez ? 1u : 0u) | (2 * t.zz + 1 < ez ? 2u : 0u) : 0u;
+    });
+  }
+  return tile_key<ORDER>(m, S, src, i0, j0, k0, low);
 }
 
 // The finite-difference Hessian of a column of 8 cells per thread (z = lane, y = warp) as
