@@ -29,7 +29,7 @@ namespace mgk {
 namespace {
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_ghost_periodic(Grid G, T* __restrict__ u) {
+__global__ void __launch_bounds__(256) k_ghost_periodic(Grid G, T* u) {
   grid_wait();
   ghost_periodic_body<T>(G, u, blockIdx.x * (long long)blockDim.x + threadIdx.x);
 }
@@ -71,10 +71,10 @@ struct TangFold {
 // cold, 23.2 us with an element per thread, 16.1 so, 19.5 with the folded coarse parts.
 template <int ORDER, typename T, bool FOLD>
 __device__ __forceinline__ void tangential_tile(const Grid& F, const Grid& P,
-                                                const T* __restrict__ pu, Int3 off,
+                                                const T* pu, Int3 off,
                                                 const FaceSet& fs, const TangTiles& tt,
                                                 const CfW<T>& w, const TangFold& fo, T invH,
-                                                T* __restrict__ inter, T* __restrict__ fc_unc) {
+                                                T* inter, T* fc_unc) {
   constexpr int half = ORDER / 2;
   constexpr int RB = kTangB + ORDER;
   typedef typename Vec2<T>::type V2;
@@ -110,7 +110,7 @@ __device__ __forceinline__ void tangential_tile(const Grid& F, const Grid& P,
     T r0 = T(0), r1 = T(0);
 #pragma unroll
     for (int cc = 0; cc <= ORDER; ++cc) {
-      const T x = __ldg(v + cc * sc);
+      const T x = v[cc * sc];
       r0 = fma(w.tang[0][cc], x, r0);
       r1 = fma(w.tang[1][cc], x, r1);
     }
@@ -153,10 +153,10 @@ __device__ __forceinline__ void tangential_tile(const Grid& F, const Grid& P,
       const T* v = org + (jc * sb + kc * sc);
       if (side == 0) {
 #pragma unroll
-        for (int s = 0; s < half; ++s) fc = fma(w.flux[s], __ldg(v + (half - 1 - s) * sm), fc);
+        for (int s = 0; s < half; ++s) fc = fma(w.flux[s], v[(half - 1 - s) * sm], fc);
       } else {
 #pragma unroll
-        for (int s = half; s < ORDER; ++s) fc = fma(w.flux[s], __ldg(v + (s - half) * sm), fc);
+        for (int s = half; s < ORDER; ++s) fc = fma(w.flux[s], v[(s - half) * sm], fc);
       }
       fc *= invH;
     }
@@ -199,9 +199,9 @@ __device__ __forceinline__ void tangential_tile(const Grid& F, const Grid& P,
 
 template <int ORDER, typename T, bool FOLD>
 __global__ void __launch_bounds__(kTangThreads)
-    k_cf_tangential(Grid F, Grid P, const T* __restrict__ pu, Int3 off, FaceSet fs, TangTiles tt,
-                    CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
-                    T* __restrict__ fc_unc) {
+    k_cf_tangential(Grid F, Grid P, const T* pu, Int3 off, FaceSet fs, TangTiles tt,
+                    CfW<T> w, TangFold fo, T invH, T* inter,
+                    T* fc_unc) {
   tangential_tile<ORDER, T, FOLD>(F, P, pu, off, fs, tt, w, fo, invH, inter, fc_unc);
 }
 
@@ -210,9 +210,9 @@ __global__ void __launch_bounds__(kTangThreads)
 // z-pairs x 8 rows (gx x gy per plane).
 template <int ORDER, typename T, bool FOLD>
 __global__ void __launch_bounds__(kTangThreads)
-    k_tangential_prolong(Grid F, Grid P, const T* __restrict__ pu, Int3 off, FaceSet fs,
-                         TangTiles tt, CfW<T> w, TangFold fo, T invH, T* __restrict__ inter,
-                         T* __restrict__ fc_unc, T* __restrict__ u, const T* __restrict__ ubar,
+    k_tangential_prolong(Grid F, Grid P, const T* pu, Int3 off, FaceSet fs,
+                         TangTiles tt, CfW<T> w, TangFold fo, T invH, T* inter,
+                         T* fc_unc, T* u, const T* ubar,
                          Int3 cn, int gx, int gy) {
   const int b = (int)blockIdx.x - tt.first[6];
   if (b < 0) {
@@ -220,15 +220,15 @@ __global__ void __launch_bounds__(kTangThreads)
     return;
   }
   grid_wait();
-  prolong_at<T, Ldg>(F, u, P, pu, ubar, off, cn, 0, b / (gx * gy),
+  prolong_at<T>(F, u, P, pu, ubar, off, cn, 0, b / (gx * gy),
                      b / gx % gy * (kTangThreads / 32) + (int)(threadIdx.x >> 5),
                      b % gx * 32 + (int)(threadIdx.x & 31));
 }
 
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
-    k_cf_flux(Grid F, T* __restrict__ u, FaceSet fs, CfW<T> w, const T* __restrict__ inter,
-              const T* __restrict__ fc_unc, T fc_scale, T a0, T a1, T b0, T b1, int flux_fix) {
+    k_cf_flux(Grid F, T* u, FaceSet fs, CfW<T> w, const T* inter,
+              const T* fc_unc, T fc_scale, T a0, T a1, T b0, T b1, int flux_fix) {
   const int t = blockIdx.x * 128 + threadIdx.x;
   if (t >= 4 * (int)fs.ebase[6]) return;
   const unsigned quad = __activemask();
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(128)
 
 template <int ORDER>
 __global__ void __launch_bounds__(128)
-    k_cf_flux_fold(Grid F, double* __restrict__ u, FaceArgs<double> fa) {
+    k_cf_flux_fold(Grid F, double* u, FaceArgs<double> fa) {
   const int t = blockIdx.x * 128 + threadIdx.x;
   if (t >= 4 * (int)fa.fs.ebase[6]) return;
   const unsigned quad = __activemask();
@@ -295,7 +295,7 @@ __device__ __forceinline__ bool edge_cell(const Grid& F, int t, int& i, int& j, 
 
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
-    k_cf_edges(Grid F, T* __restrict__ u, Grid P, const T* __restrict__ pu, Int3 off,
+    k_cf_edges(Grid F, T* u, Grid P, const T* pu, Int3 off,
                CfWeights w) {
   grid_wait();
   constexpr int half = ORDER / 2;
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(128)
     for (int bq = 0; bq <= ORDER; ++bq) {
       T row = T(0);
       for (int cq = 0; cq <= ORDER; ++cq)
-        row = fma(T(wk[cq]), __ldg(pu + gidx(P, pi + a - half, pj + bq - half, pk + cq - half)), row);
+        row = fma(T(wk[cq]), pu[gidx(P, pi + a - half, pj + bq - half, pk + cq - half)], row);
       pa = fma(T(wj[bq]), row, pa);
     }
     acc = fma(T(wi[a]), pa, acc);

@@ -50,10 +50,10 @@ constexpr int kCoarseBlock = kCoarseThreads;
 
 template <typename T>
 __global__ void __launch_bounds__(kCoarseBlock)
-    k_coarsest(Grid G, const T* __restrict__ f, T* __restrict__ u,
-               const double* __restrict__ kern) {
+    k_coarsest(Grid G, const T* f, T* u,
+               const double* kern) {
   grid_wait();
-  coarsest_body<T, Ldg>(G, f, u, kern, (int)blockIdx.x, (int)threadIdx.x);
+  coarsest_body<T>(G, f, u, kern, (int)blockIdx.x, (int)threadIdx.x);
 }
 
 template <int BLOCK>
@@ -99,7 +99,7 @@ __device__ __forceinline__ float to_float(double r) {
 
 template <int ORDER, bool MIXED>
 __global__ void __launch_bounds__(kRedBlock)
-    k_norm_partial(Grid G, const double* __restrict__ u, const double* __restrict__ f,
+    k_norm_partial(Grid G, const double* u, const double* f,
                    double invh2, double vol, Int3 clo, Int3 chi, double* __restrict__ partial,
                    float* __restrict__ r32) {
   grid_wait();
@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(kRedBlock)
       const bool cov = row_cov && k >= clo.z && k < chi.z;
       if (cov) continue;
       const long long p = row + k;
-      const double fv = __ldg(f + p);
-      const double r = u ? add_lap_h2<ORDER, double, Ldg, !MIXED>(u, p, sy, sx, __ldg(u + p),
+      const double fv = f[p];
+      const double r = u ? add_lap_h2<ORDER, double, !MIXED>(u, p, sy, sx, u[p],
                                                                  -invh2, fv)
                          : fv;
       if (MIXED) r32[p] = to_float(r);
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kRedBlock)
 // the first block zeros the slots that k_norm_partial would use beyond.
 template <int ORDER>
 __global__ void __launch_bounds__(kTileThreads, 3)
-    k_norm_tile(Grid G, const double* __restrict__ u, const double* __restrict__ f, double invh2,
+    k_norm_tile(Grid G, const double* u, const double* f, double invh2,
                 double vol, Int3 clo, Int3 chi, double* __restrict__ partial, int slots) {
   grid_wait();
   extern __shared__ __align__(16) long long norm_smem[];
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       fv[q] = i + q < G.n0 && j < G.n1 && k < G.n2
-                  ? __ldg(reinterpret_cast<const double2*>(f + p + q * sx)) : make_double2(0.0, 0.0);
+                  ? *reinterpret_cast<const double2*>(f + p + q * sx) : make_double2(0.0, 0.0);
     const unsigned key = tile_load<ORDER>(G, u, i0, j0, k0, norm_smem);
     const bool fx = fx_in_range(key) && fx_scalable(kr, key);
     const double ks = fx_scale(kr, key);
@@ -188,8 +188,8 @@ __global__ void __launch_bounds__(kTileThreads, 3)
       for (int q = 0; q < 8; ++q) {
         if (!leaf(q >> 1, q & 1)) continue;
         const long long e = p + (q >> 1) * sx + (q & 1);
-        const double fv = __ldg(f + e);
-        add(add_lap_h2<ORDER, double, Ldg, false>(u, e, G.Zp, sx, __ldg(u + e), -invh2, fv), fv);
+        const double fv = f[e];
+        add(add_lap_h2<ORDER, double, false>(u, e, G.Zp, sx, u[e], -invh2, fv), fv);
       }
     }
   }
@@ -201,8 +201,8 @@ __global__ void __launch_bounds__(kTileThreads, 3)
 }
 
 __global__ void __launch_bounds__(kRedBlock)
-    k_sum_partial(Grid G, const double* __restrict__ f, double vol, Int3 clo, Int3 chi,
-                  double* __restrict__ partial) {
+    k_sum_partial(Grid G, const double* f, double vol, Int3 clo, Int3 chi,
+                  double* partial) {
   grid_wait();
   const int i = blockIdx.y;
   const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kRedBlock)
     const long long row = gidx(G, i, j, 0);
     for (int k = lane; k < G.n2; k += 32) {
       if (row_cov && k >= clo.z && k < chi.z) continue;
-      s += __ldg(f + row + k);
+      s += f[row + k];
     }
   }
   block_sum2<kRedBlock>(s, unused);
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kRedBlock)
 
 // Sums `count` consecutive (a, b) pairs in a fixed order into out[0], out[1].
 __global__ void __launch_bounds__(kRedBlock)
-    k_reduce_partials(const double* __restrict__ partial, int count, double* __restrict__ out) {
+    k_reduce_partials(const double* partial, int count, double* out) {
   grid_wait();
   double a = 0.0, b = 0.0;
   for (int t = threadIdx.x; t < count; t += kRedBlock) {
@@ -246,9 +246,9 @@ __global__ void __launch_bounds__(kRedBlock)
 // (pinned host memory, laid out like the record that starts at out) the record's entries go
 // there as well, so that no copy follows: out[2..4], left by earlier kernels, by block 0.
 __global__ void __launch_bounds__(kRedBlock)
-    k_reduce_levels(const double* __restrict__ partial, int count, LevelRanges R,
-                    double* __restrict__ out, double* __restrict__ out_levels,
-                    double* __restrict__ host) {
+    k_reduce_levels(const double* partial, int count, LevelRanges R,
+                    double* out, double* out_levels,
+                    double* host) {
   grid_wait();
   int lo = 0, hi = count;
   if (blockIdx.x > 0) {
@@ -284,27 +284,27 @@ inline dim3 copy_grid(const Grid& G) {
 }
 
 __global__ void __launch_bounds__(256)
-    k_pack(Grid G, const double* __restrict__ src, double* __restrict__ dst, double shift) {
+    k_pack(Grid G, const double* src, double* __restrict__ dst, double shift) {
   grid_wait();
   const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
   const int i = blockIdx.z;
   if (k >= G.n2 || j >= G.n1) return;
-  dst[gidx(G, i, j, k)] = __ldg(src + ((long long)i * G.n1 + j) * G.n2 + k) - shift;
+  dst[gidx(G, i, j, k)] = src[((long long)i * G.n1 + j) * G.n2 + k] - shift;
 }
 
 __global__ void __launch_bounds__(256)
-    k_unpack(Grid G, const double* __restrict__ src, double* __restrict__ dst, double add) {
+    k_unpack(Grid G, const double* src, double* __restrict__ dst, double add) {
   grid_wait();
   const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
   const int i = blockIdx.z;
   if (k >= G.n2 || j >= G.n1) return;
-  dst[((long long)i * G.n1 + j) * G.n2 + k] = __ldg(src + gidx(G, i, j, k)) + add;
+  dst[((long long)i * G.n1 + j) * G.n2 + k] = src[gidx(G, i, j, k)] + add;
 }
 
 // f -= mean, f2 = f on the interior; mean = *mean_num * inv_volume (device-side).
 __global__ void __launch_bounds__(256)
-    k_shift_copy(Grid G, double* __restrict__ f, double* __restrict__ f2,
-                 const double* __restrict__ mean_num, double inv_volume) {
+    k_shift_copy(Grid G, double* f, double* f2,
+                 const double* mean_num, double inv_volume) {
   grid_wait();
   const int k = blockIdx.x * kCopyZ + threadIdx.x, j = blockIdx.y * kCopyY + threadIdx.y;
   const int i = blockIdx.z;
@@ -318,21 +318,21 @@ __global__ void __launch_bounds__(256)
 // u += e on the interior (float64 += float32 correction); periodic levels also
 // update their ghost images.  One thread per cell of a (32 x 4)-cell tile row.
 __global__ void __launch_bounds__(128)
-    k_add_correction(Grid G, double* __restrict__ u, const float* __restrict__ e, int periodic) {
+    k_add_correction(Grid G, double* u, const float* e, int periodic) {
   grid_wait();
   const int k = blockIdx.x * 32 + threadIdx.x;
   const int j = blockIdx.y * 4 + threadIdx.y;
   const int i = blockIdx.z;
   if (k >= G.n2 || j >= G.n1) return;
   const long long p = gidx(G, i, j, k);
-  const double v = u[p] + (double)__ldg(e + p);
+  const double v = u[p] + (double)e[p];
   u[p] = v;
   if (periodic) write_images<double>(G, u, i, j, k, v);
 }
 
 // p = p - sum[0] * scale (+ add) over n elements (sum read on the device).
 __global__ void __launch_bounds__(256)
-    k_sub_mean(double* __restrict__ p, long long n, const double* __restrict__ sum, double scale,
+    k_sub_mean(double* p, long long n, const double* sum, double scale,
                double add) {
   grid_wait();
   const long long t = blockIdx.x * 256LL + threadIdx.x;
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(256)
   p[t] = add != 0.0 ? v + add : v;
 }
 
-__global__ void __launch_bounds__(256) k_fill(double* __restrict__ p, long long n, double v) {
+__global__ void __launch_bounds__(256) k_fill(double* p, long long n, double v) {
   grid_wait();
   const long long t = blockIdx.x * 256LL + threadIdx.x;
   if (t < n) p[t] = v;
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(256) k_fill(double* __restrict__ p, long long 
 // axes).
 template <int ORDER>
 __global__ void __launch_bounds__(128)
-    k_first_derivs(Grid G, const double* __restrict__ phi, double* __restrict__ dy,
+    k_first_derivs(Grid G, const double* phi, double* __restrict__ dy,
                    double* __restrict__ dz) {
   grid_wait();
   constexpr int half = ORDER / 2;
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(128)
     double acc = 0.0;
 #pragma unroll
     for (int s = 1; s <= half; ++s)
-      acc = fma(grad_w<ORDER>(s), __ldg(phi + p + s * st[b]) - __ldg(phi + p - s * st[b]), acc);
+      acc = fma(grad_w<ORDER>(s), phi[p + s * st[b]] - phi[p - s * st[b]], acc);
     out[b][p] = acc;
   }
 }
@@ -386,8 +386,8 @@ __global__ void __launch_bounds__(128)
 // G_x D_y, phi_xz = G_x D_z, phi_yz = G_y D_z.
 template <int ORDER>
 __global__ void __launch_bounds__(128)
-    k_lpt2_source(Grid G, const double* __restrict__ phi, const double* __restrict__ dy,
-                  const double* __restrict__ dz, double invh2, double* __restrict__ tau) {
+    k_lpt2_source(Grid G, const double* phi, const double* dy,
+                  const double* dz, double invh2, double* __restrict__ tau) {
   grid_wait();
   constexpr int half = ORDER / 2;
   const int k = blockIdx.x * 32 + threadIdx.x;
@@ -397,13 +397,13 @@ __global__ void __launch_bounds__(128)
   const long long p = gidx(G, i, j, k);
   const int st[3] = {G.Y * G.Zp, G.Zp, 1};
   double d[3], m[3];
-  const double c = __ldg(phi + p);
+  const double c = phi[p];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     double acc = Lap<ORDER>::w0 * c;
 #pragma unroll
     for (int s = 1; s <= half; ++s)
-      acc = fma(lap_w<ORDER>(s), __ldg(phi + p + s * st[a]) + __ldg(phi + p - s * st[a]), acc);
+      acc = fma(lap_w<ORDER>(s), phi[p + s * st[a]] + phi[p - s * st[a]], acc);
     d[a] = acc * invh2;
   }
   const double* src[3] = {dy, dz, dz};
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(128)
     double acc = 0.0;
 #pragma unroll
     for (int s = 1; s <= half; ++s)
-      acc = fma(grad_w<ORDER>(s), __ldg(src[q] + p + s * st[ax[q]]) - __ldg(src[q] + p - s * st[ax[q]]),
+      acc = fma(grad_w<ORDER>(s), src[q][p + s * st[ax[q]]] - src[q][p - s * st[ax[q]]],
                 acc);
     m[q] = acc * invh2;
   }
@@ -428,8 +428,8 @@ __device__ __forceinline__ void fd_hessian(const Src& src, int i, int j, int k, 
   constexpr int half = ORDER / 2;
   // the cell at offset s along axis a and t along axis b
   auto at = [&](int a, int s, int b, int t) {
-    return __ldg(src.at(i + (a == 0 ? s : 0) + (b == 0 ? t : 0), j + (a == 1 ? s : 0) + (b == 1 ? t : 0),
-                        k + (a == 2 ? s : 0) + (b == 2 ? t : 0)));
+    return *src.at(i + (a == 0 ? s : 0) + (b == 0 ? t : 0), j + (a == 1 ? s : 0) + (b == 1 ? t : 0),
+                        k + (a == 2 ? s : 0) + (b == 2 ? t : 0));
   };
   const double c = at(0, 0, 0, 0);
 #pragma unroll 1
@@ -495,7 +495,7 @@ __device__ __forceinline__ bool squarable(double s) {
 // the copies and the ghost fill were 128 of 845 us).
 template <int ORDER, typename OP, bool DENSE>
 __global__ void __launch_bounds__(kTileThreads, 3)
-    k_hessian_tile(Grid G, const double* __restrict__ phi, double invh2, double* __restrict__ out) {
+    k_hessian_tile(Grid G, const double* phi, double invh2, double* __restrict__ out) {
   grid_wait();
   extern __shared__ __align__(16) long long hess_smem[];
   const int i0 = blockIdx.z * kTileX, j0 = blockIdx.y * kTileY, k0 = blockIdx.x * kTileZ;
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(256)
 
 template <int ORDER>
 __global__ void __launch_bounds__(128)
-    k_gradient(Grid G, const double* __restrict__ phi, double invh, double* __restrict__ dx,
+    k_gradient(Grid G, const double* phi, double invh, double* __restrict__ dx,
                double* __restrict__ dy, double* __restrict__ dz) {
   grid_wait();
   constexpr int half = ORDER / 2;
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(128)
     double acc = 0.0;
 #pragma unroll
     for (int s = 1; s <= half; ++s)
-      acc = fma(grad_w<ORDER>(s), __ldg(phi + p + s * st[a]) - __ldg(phi + p - s * st[a]), acc);
+      acc = fma(grad_w<ORDER>(s), phi[p + s * st[a]] - phi[p - s * st[a]], acc);
     out[a] = -acc * invh;
   }
   dx[t] = out[0];
@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(128)
 // of 21.
 template <int ORDER>
 __global__ void __launch_bounds__(kTileThreads, 3)
-    k_gradient_tile(Grid G, const double* __restrict__ phi, double invh, double* __restrict__ dx,
+    k_gradient_tile(Grid G, const double* phi, double invh, double* __restrict__ dx,
                     double* __restrict__ dy, double* __restrict__ dz) {
   grid_wait();
   extern __shared__ __align__(16) long long grad_smem[];
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     for (int a = 0; a < 3; ++a) {
       double acc = 0.0;
       for (int d = 1; d <= ORDER / 2; ++d)
-        acc = fma(grad_w<ORDER>(d), __ldg(c + d * st[a]) - __ldg(c - d * st[a]), acc);
+        acc = fma(grad_w<ORDER>(d), c[d * st[a]] - c[-d * st[a]], acc);
       out[a][o + (q >> 1) * ox + (q & 1)] = -acc * invh;
     }
   }

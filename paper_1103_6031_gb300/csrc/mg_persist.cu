@@ -54,7 +54,7 @@ __device__ __forceinline__ void run_block(const POp& op, const CfW<float>& w, in
     }
     case P_SMOOTH: {
       const Blk b{blk % op.gx, (blk / op.gx) % op.gy, blk / (op.gx * op.gy), tid & 31, tid >> 5};
-      smooth_half_body<ORDER, float, Weak>(op.F, op.in0, op.out0, op.in1, op.s[0], op.colour,
+      smooth_half_body<ORDER, float>(op.F, op.in0, op.out0, op.in1, op.s[0], op.colour,
                                            op.periodic, kPersistThreads / kVPairX, b);
       break;
     }
@@ -68,26 +68,26 @@ __device__ __forceinline__ void run_block(const POp& op, const CfW<float>& w, in
       break;
     case P_RESTRICT: {
       const Blk b{blk % op.gx, (blk / op.gx) % op.gy, blk / (op.gx * op.gy), tid & 31, tid >> 5};
-      residual_restrict_body<ORDER, float, Weak>(op.F, op.in0, op.in1, op.s[0], op.P, op.out0,
+      residual_restrict_body<ORDER, float>(op.F, op.in0, op.in1, op.s[0], op.P, op.out0,
                                                  op.out1, op.out2, op.off, op.cn, op.periodic, b);
       break;
     }
     case P_FAS: {
       const Blk b{blk % op.gx, (blk / op.gx) % op.gy, blk / (op.gx * op.gy), tid & 31, tid >> 5};
-      fas_source_body<ORDER, float, Weak>(op.P, op.in0, op.out0, op.s[0], op.off, op.cn, b);
+      fas_source_body<ORDER, float>(op.P, op.in0, op.out0, op.s[0], op.off, op.cn, b);
       break;
     }
     case P_COARSEST:
-      coarsest_body<float, Weak>(op.F, op.in0, op.out0, op.kern, blk, tid);
+      coarsest_body<float>(op.F, op.in0, op.out0, op.kern, blk, tid);
       break;
     case P_TANG:
-      cf_tangential_body<ORDER, float, Weak>(op.F, op.P, op.in0, op.off, op.fs, w, op.s[0],
+      cf_tangential_body<ORDER, float>(op.F, op.P, op.in0, op.off, op.fs, w, op.s[0],
                                              op.out0, op.out1,
                                              (long long)blk * kPersistThreads + tid);
       break;
     case P_PROLONG: {
       const Blk b{blk % op.gx, (blk / op.gx) % op.gy, blk / (op.gx * op.gy), tid & 31, tid >> 5};
-      prolong_body<float, Weak>(op.F, op.out0, op.P, op.in0, op.in1, op.off, op.cn, op.periodic, b);
+      prolong_body<float>(op.F, op.out0, op.P, op.in0, op.in1, op.off, op.cn, op.periodic, b);
       break;
     }
     default:

@@ -32,27 +32,27 @@ constexpr int smooth_min_blocks = sizeof(T) == 8 && ORDER == 6 ? 4 : 5;
 
 template <int ORDER, typename T, bool CVT>
 __global__ void __launch_bounds__(kPairX * 8, (smooth_min_blocks<ORDER, T>))
-    k_smooth_half(Grid G, const T* __restrict__ uin, T* __restrict__ uout,
-                  const T* __restrict__ f, T a_f, int colour, int periodic) {
+    k_smooth_half(Grid G, const T* uin, T* __restrict__ uout,
+                  const T* f, T a_f, int colour, int periodic) {
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = 2 * (blockIdx.x * kPairX + threadIdx.x);
   if (j >= G.n1 || k0 >= G.n2) return;
   grid_wait();
-  smooth_pair_at<ORDER, T, Ldg, CVT>(G, uin, uout, f, a_f, colour, periodic, blockIdx.z, j, k0);
+  smooth_pair_at<ORDER, T, CVT>(G, uin, uout, f, a_f, colour, periodic, blockIdx.z, j, k0);
 }
 
 // The first half-sweep of a level after a restriction into it, with the FAS source of the
 // restricted cells (smooth_fas_pair_at): one launch instead of two.
 template <int ORDER>
 __global__ void __launch_bounds__(128, 8)
-    k_smooth_fas(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
-                 float* __restrict__ f, float a_f, float invh2, FasBox box, int colour,
+    k_smooth_fas(Grid G, const float* uin, float* __restrict__ uout,
+                 float* f, float a_f, float invh2, FasBox box, int colour,
                  int periodic) {
   const int j = blockIdx.y * 4 + threadIdx.y;
   const int k0 = 2 * (blockIdx.x * 32 + threadIdx.x);
   if (j >= G.n1 || k0 >= G.n2) return;
   grid_wait();
-  smooth_fas_pair_at<ORDER, float, Ldg>(G, uin, uout, f, a_f, invh2, box, colour, periodic,
+  smooth_fas_pair_at<ORDER, float>(G, uin, uout, f, a_f, invh2, box, colour, periodic,
                                         blockIdx.z, j, k0);
 }
 
@@ -65,13 +65,13 @@ __global__ void __launch_bounds__(128, 8)
 // offset (0 or 1) is a run-time value shared by a row: it picks operands by select,
 // never by a dynamic index into a register array.
 __device__ __forceinline__ float4 ld4(const float* p) {
-  return __ldg(reinterpret_cast<const float4*>(p));
+  return *reinterpret_cast<const float4*>(p);
 }
 
 template <int ORDER>
-__device__ __forceinline__ void smooth_quad_at(const Grid& G, const float* __restrict__ uin,
-                                               float* __restrict__ uout,
-                                               const float* __restrict__ f, float a_f, int colour,
+__device__ __forceinline__ void smooth_quad_at(const Grid& G, const float* uin,
+                                               float* uout,
+                                               const float* f, float a_f, int colour,
                                                int periodic, int i, int j, int k0) {
   constexpr int R = ORDER / 2;
   const long long sy = G.Zp;
@@ -137,8 +137,8 @@ __device__ __forceinline__ void smooth_quad_at(const Grid& G, const float* __res
 
 template <int ORDER>
 __global__ void __launch_bounds__(256, 4)
-    k_smooth_quad(Grid G, const float* __restrict__ uin, float* __restrict__ uout,
-                  const float* __restrict__ f, float a_f, int colour, int periodic) {
+    k_smooth_quad(Grid G, const float* uin, float* __restrict__ uout,
+                  const float* f, float a_f, int colour, int periodic) {
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (j >= G.n1 || k0 >= G.n2) return;
@@ -163,7 +163,7 @@ constexpr int kFacesThreads = 128;
 template <int ORDER, typename T, int VEC, bool FAS>
 __global__ void __launch_bounds__(kFacesThreads,
                                   FAS ? 5 : ((smooth_min_blocks<ORDER, T>) < 5 || VEC == 4 ? 8 : 10))
-    k_smooth_faces(Grid G, const T* __restrict__ uin, T* __restrict__ uout, T* f, T a_f, int colour,
+    k_smooth_faces(Grid G, const T* uin, T* uout, T* f, T a_f, int colour,
                    int face_blocks, int gx, int gy, int qx, int by, T invh2, FasBox box,
                    FaceArgs<T> fa) {
   const int b = (int)blockIdx.x - face_blocks;
@@ -174,12 +174,12 @@ __global__ void __launch_bounds__(kFacesThreads,
     if (ty >= by || j >= G.n1 || k0 >= G.n2) return;
     grid_wait();
     if constexpr (FAS)
-      smooth_fas_pair_at<ORDER, T, Ldg>(G, uin, uout, f, a_f, invh2, box, colour, 0,
+      smooth_fas_pair_at<ORDER, T>(G, uin, uout, f, a_f, invh2, box, colour, 0,
                                                b / (gx * gy), j, k0);
     else if constexpr (VEC == 4)
       smooth_quad_at<ORDER>(G, uin, uout, f, a_f, colour, 0, b / (gx * gy), j, k0);
     else
-      smooth_pair_at<ORDER, T, Ldg>(G, uin, uout, f, a_f, colour, 0, b / (gx * gy), j, k0);
+      smooth_pair_at<ORDER, T>(G, uin, uout, f, a_f, colour, 0, b / (gx * gy), j, k0);
     return;
   }
   __shared__ T cells[ORDER][32];
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kFacesThreads,
     } else if (warp == kFacesThreads / 32 - 1) {
 #pragma unroll
       for (int q = 0; q < ORDER / 2; ++q)
-        cells[2 * q + 1 - o][lane] = __ldg(uin + c.in0 + (2 * q + 1 - o) * c.step);
+        cells[2 * q + 1 - o][lane] = uin[c.in0 + (2 * q + 1 - o) * c.step];
     }
   }
   __syncthreads();
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kFacesThreads,
 // along z.
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
-    k_residual_restrict(Grid F, const T* __restrict__ u, const T* __restrict__ f, T invh2, Grid P,
+    k_residual_restrict(Grid F, const T* u, const T* f, T invh2, Grid P,
                         T* __restrict__ pu, T* __restrict__ pfas, T* __restrict__ ubar, Int3 off,
                         Int3 cn, int parent_periodic) {
   typedef typename Vec2<T>::type V2;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(128)
     const long long p = gidx(F, 2 * ic + (child >> 1), 2 * jc + (child & 1), 2 * kc);
     T n0[3 * ORDER], n1[3 * ORDER], c0, c1;
     load_pair_neighbours<ORDER, T>(u, p, F.Zp, F.Y * F.Zp, n0, n1, c0, c1);
-    const V2 fv = __ldg(reinterpret_cast<const V2*>(f + p));
+    const V2 fv = *reinterpret_cast<const V2*>(f + p);
     sm[0][2 * child][slot] = c0;
     sm[0][2 * child + 1][slot] = c1;
     sm[1][2 * child][slot] = add_lap_of<ORDER, T>(n0, c0, -invh2, fv.x);
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(128)
 // the row above or below is in the other half of its warp.
 template <int ORDER>
 __global__ void __launch_bounds__(kTileThreads, 3)
-    k_residual_restrict_tile(Grid F, const double* __restrict__ u, const double* __restrict__ f,
+    k_residual_restrict_tile(Grid F, const double* u, const double* f,
                              double invh2, Grid P, double* __restrict__ pu,
                              double* __restrict__ pfas, double* __restrict__ ubar, Int3 off, Int3 cn,
                              int parent_periodic) {
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     if (!(row && i + q < F.n0)) continue;
-    const double2 fv = __ldg(reinterpret_cast<const double2*>(f + p + q * sx));
+    const double2 fv = *reinterpret_cast<const double2*>(f + p + q * sx);
     mr[q >> 1] += fv.x + fv.y;
   }
   if (fx_in_range(key) && fx_scalable(kr, key)) {
@@ -309,9 +309,9 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     for (int q = 0; q < 4; ++q) {
       if (!(row && i + q < F.n0)) continue;
       for (int dk = 0; dk < 2; ++dk) {
-        const double c = __ldg(u + p + q * sx + dk);
+        const double c = u[p + q * sx + dk];
         const double r =
-            add_lap_h2<ORDER, double, Ldg, false>(u, p + q * sx + dk, F.Zp, sx, c, -invh2, 0.0);
+            add_lap_h2<ORDER, double, false>(u, p + q * sx + dk, F.Zp, sx, c, -invh2, 0.0);
         if (q < 2) {
           mu[0] += c;
           mr[0] += r;
@@ -342,10 +342,10 @@ __global__ void __launch_bounds__(kTileThreads, 3)
 // Covered parent cells: f_fas += L u (u = restricted fine solution there).
 template <int ORDER, typename T>
 __global__ void __launch_bounds__(128)
-    k_fas_source(Grid P, const T* __restrict__ pu, T* __restrict__ pfas, T invH2, Int3 off,
+    k_fas_source(Grid P, const T* pu, T* pfas, T invH2, Int3 off,
                  Int3 cn) {
   grid_wait();
-  fas_source_body<ORDER, T, Ldg>(P, pu, pfas, invH2, off, cn,
+  fas_source_body<ORDER, T>(P, pu, pfas, invH2, off, cn,
                                  Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z,
                                      (int)threadIdx.x, (int)threadIdx.y});
 }
@@ -353,10 +353,10 @@ __global__ void __launch_bounds__(128)
 // u += inject(parent u - ubar) on the fine interior; one thread per z-pair.
 template <typename T>
 __global__ void __launch_bounds__(128)
-    k_prolong(Grid F, T* __restrict__ u, Grid P, const T* __restrict__ pu,
-              const T* __restrict__ ubar, Int3 off, Int3 cn, int periodic) {
+    k_prolong(Grid F, T* u, Grid P, const T* pu,
+              const T* ubar, Int3 off, Int3 cn, int periodic) {
   grid_wait();
-  prolong_body<T, Ldg>(F, u, P, pu, ubar, off, cn, periodic,
+  prolong_body<T>(F, u, P, pu, ubar, off, cn, periodic,
                        Blk{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x,
                            (int)threadIdx.y});
 }
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(128)
 // parent u := mean of children (covered region), one thread per parent cell.
 template <typename T>
 __global__ void __launch_bounds__(128)
-    k_restrict_u(Grid F, const T* __restrict__ u, Grid P, T* __restrict__ pu, Int3 off, Int3 cn) {
+    k_restrict_u(Grid F, const T* u, Grid P, T* __restrict__ pu, Int3 off, Int3 cn) {
   grid_wait();
   const int kc = blockIdx.x * blockDim.x + threadIdx.x;
   const int jc = blockIdx.y * blockDim.y + threadIdx.y;

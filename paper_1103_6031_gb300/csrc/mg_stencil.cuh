@@ -25,34 +25,21 @@ struct Lap<6> {
                           w3 = 2.0 / 180.0;
 };
 
-// Load policies.  Ldg: the read-only data path, for kernels whose inputs no thread of
-// the launch writes.  Weak: plain loads, for the persistent kernel, whose work items
-// read what earlier items of the same launch wrote (ordered by release/acquire
-// flags, which the read-only path does not observe).
-struct Ldg {
-  template <typename T>
-  static __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
-};
-struct Weak {
-  template <typename T>
-  static __device__ __forceinline__ T ld(const T* p) { return *p; }
-};
-
 // The 6 neighbours at each distance 1 .. ORDER / 2 of element p: nb[6 (d - 1)] ..: -z, +z,
 // -y, +y, -x, +x.
-template <int ORDER, typename T, typename LD = Ldg>
-__device__ __forceinline__ void load_neighbours(const T* __restrict__ u, long long p, int sy,
+template <int ORDER, typename T>
+__device__ __forceinline__ void load_neighbours(const T* u, long long p, int sy,
                                                 int sx, T (&nb)[3 * ORDER]) {
   const T* c = u + p;
 #pragma unroll
   for (int d = 1; d <= ORDER / 2; ++d) {
     T* o = nb + 6 * (d - 1);
-    o[0] = LD::ld(c - d);
-    o[1] = LD::ld(c + d);
-    o[2] = LD::ld(c - d * sy);
-    o[3] = LD::ld(c + d * sy);
-    o[4] = LD::ld(c - d * sx);
-    o[5] = LD::ld(c + d * sx);
+    o[0] = c[-d];
+    o[1] = c[d];
+    o[2] = *(c - d * sy);
+    o[3] = c[d * sy];
+    o[4] = *(c - d * sx);
+    o[5] = c[d * sx];
   }
 }
 
@@ -69,13 +56,13 @@ struct Vec2<float> {
 
 // The neighbours of the z-pair at p (an even cell of its row) and the pair itself, every row
 // by 2-element loads.
-template <int ORDER, typename T, typename LD = Ldg>
-__device__ __forceinline__ void load_pair_neighbours(const T* __restrict__ u, long long p, int sy,
+template <int ORDER, typename T>
+__device__ __forceinline__ void load_pair_neighbours(const T* u, long long p, int sy,
                                                      int sx, T (&n0)[3 * ORDER],
                                                      T (&n1)[3 * ORDER], T& c0, T& c1) {
   typedef typename Vec2<T>::type V2;
   constexpr int R = ORDER / 2, RZ = (R + 1) / 2 * 2;
-  auto ld2 = [](const T* q) { return LD::ld(reinterpret_cast<const V2*>(q)); };
+  auto ld2 = [](const T* q) { return *reinterpret_cast<const V2*>(q); };
   const T* c = u + p;
   T z[2 * RZ + 2];
 #pragma unroll
@@ -154,11 +141,11 @@ __device__ __forceinline__ T add_lap_of(const T (&nb)[3 * ORDER], T c, T scale, 
 }
 
 // The same at element p, c = u[p].
-template <int ORDER, typename T, typename LD = Ldg, bool FX = true>
-__device__ __forceinline__ T add_lap_h2(const T* __restrict__ u, long long p, int sy, int sx, T c,
+template <int ORDER, typename T, bool FX = true>
+__device__ __forceinline__ T add_lap_h2(const T* u, long long p, int sy, int sx, T c,
                                         T scale, T acc) {
   T nb[3 * ORDER];
-  load_neighbours<ORDER, T, LD>(u, p, sy, sx, nb);
+  load_neighbours<ORDER, T>(u, p, sy, sx, nb);
   return add_lap_of<ORDER, T, FX>(nb, c, scale, acc);
 }
 
@@ -181,7 +168,7 @@ __device__ __forceinline__ ImgAxis img_axis(int a, int n, int g, long long st) {
 // they take two stores instead of the 26 predicated ones, which every warp that reaches a z
 // face would execute.
 template <typename T>
-__device__ __forceinline__ void write_images(const Grid& G, T* __restrict__ u, int i, int j,
+__device__ __forceinline__ void write_images(const Grid& G, T* u, int i, int j,
                                              int k, T v) {
   const int g = G.g;
   const bool in_xy = i >= g && i < G.n0 - g && j >= g && j < G.n1 - g;
@@ -211,7 +198,7 @@ __device__ __forceinline__ void write_images(const Grid& G, T* __restrict__ u, i
 // of the row pitch, so the alignment of the pair is kept), the z images of each
 // cell scalar, at the cell's own row and at every x/y image row.
 template <typename T>
-__device__ __forceinline__ void write_pair_images(const Grid& G, T* __restrict__ u, int i, int j,
+__device__ __forceinline__ void write_pair_images(const Grid& G, T* u, int i, int j,
                                                   int k, T va, T vb) {
   const int g = G.g;
   const bool in_xy = i >= g && i < G.n0 - g && j >= g && j < G.n1 - g;

@@ -11,7 +11,7 @@
 //
 // Accuracy: a unit is 2^-58 to 2^-59 of the BLOCK's largest value (halo included), not of the
 // cell's own neighbours'.  A tile is summed as integers only if every cell's star holds a value
-// of at least 2^52 units or nothing but zeros (tile_too_wide); the rounding of a difference, at
+// of at least 2^52 units or nothing but zeros (tile_key); the rounding of a difference, at
 // most 30 units, then stays below 2^-47 of the largest value in the cell's own star, and is far
 // smaller where that is the block's largest too.  Other tiles (a strong cell among weak ones, a
 // steep tail) are left to FP64 arithmetic.
@@ -174,9 +174,9 @@ __device__ __forceinline__ unsigned tile_key(unsigned key, const long long* S, c
     if (m == 0)
 #pragma unroll 1
       for (int d = -L::R; d <= L::R; ++d)
-        wide |= __ldg(src.at(i0 + x + d, j0 + y, k0 + z)) != 0.0 ||
-                __ldg(src.at(i0 + x, j0 + y + d, k0 + z)) != 0.0 ||
-                __ldg(src.at(i0 + x, j0 + y, k0 + z + d)) != 0.0;
+        wide |= *src.at(i0 + x + d, j0 + y, k0 + z) != 0.0 ||
+                *src.at(i0 + x, j0 + y + d, k0 + z) != 0.0 ||
+                *src.at(i0 + x, j0 + y, k0 + z + d) != 0.0;
   }
   return __syncthreads_or(wide) ? 0u : key;
 }
@@ -186,7 +186,7 @@ __device__ __forceinline__ unsigned tile_key(unsigned key, const long long* S, c
 // row padding, edge and corner ghosts) count as 0.  If the returned key is out of range
 // (fx_in_range; 0 for a tile of too wide a range), S is not to be used.
 template <int ORDER>
-__device__ __forceinline__ unsigned tile_load(const Grid& G, const double* __restrict__ u, int i0,
+__device__ __forceinline__ unsigned tile_load(const Grid& G, const double* u, int i0,
                                               int j0, int k0, long long* S) {
   typedef FxTile<ORDER> L;
   constexpr int R = L::R, RZ = L::RZ;
@@ -200,7 +200,7 @@ __device__ __forceinline__ unsigned tile_load(const Grid& G, const double* __res
   auto pair = [&](int x, int y, bool a, bool b) {
     double2 v = make_double2(0.0, 0.0);
     if (a || b) {
-      v = __ldg(reinterpret_cast<const double2*>(base + (x * sx + y * sy + z)));
+      v = *reinterpret_cast<const double2*>(base + (x * sx + y * sy + z));
       if (!a) v.x = 0.0;
       if (!b) v.y = 0.0;
     }
@@ -235,7 +235,7 @@ __device__ __forceinline__ unsigned tile_load(const Grid& G, const double* __res
   if (zact && zx < ex && zy < ey) {
     const bool a = zo >= -R && zo < ez + R, b = zo + 1 < ez + R;
     if (a || b) {
-      vz = __ldg(reinterpret_cast<const double2*>(base + (zx * sx + zy * sy + zo)));
+      vz = *reinterpret_cast<const double2*>(base + (zx * sx + zy * sy + zo));
       if (!a) vz.x = 0.0;
       if (!b) vz.y = 0.0;
     }
@@ -382,7 +382,7 @@ __device__ __forceinline__ unsigned tile_load_edges(const Grid& G, const Src& sr
       const bool a = (z >= 0 && z < ez) || (all && z >= -R && z < ez + R);
       const bool b = (z + 1 >= 0 && z + 1 < ez) || (all && z + 1 >= -R && z + 1 < ez + R);
       if (a || b) {
-        v = __ldg(reinterpret_cast<const double2*>(src.at(i0 + x, j0 + y, k0 + z)));
+        v = *reinterpret_cast<const double2*>(src.at(i0 + x, j0 + y, k0 + z));
         if (!a) v.x = 0.0;
         if (!b) v.y = 0.0;
       }

@@ -2,8 +2,9 @@
 // steps 2-9; Sec. 3.3), run two ways: by stream kernels (block and thread indices from the
 // hardware) and by the persistent batch kernel (mg_persist.cu), which runs any block of any
 // level operation of any hierarchy as a work item of a 128-thread block.  Every body gets
-// its block and thread indices as arguments and loads through a policy (Ldg in the
-// stream kernels, Weak in the persistent kernel).  residual_restrict_body and
+// its block and thread indices as arguments and reads by plain loads: in the persistent kernel
+// earlier items of the same launch wrote the data (ordered by release/acquire flags), in the
+// stream kernels the predecessor that grid_wait waits for (mg_launch.cuh).  residual_restrict_body and
 // cf_tangential_body serve the persistent kernel only: the stream kernels share a parent's
 // or a tile's work between threads, with the operations of every value in the same order, so
 // both ways give bit-identical results in float32, which is all the persistent kernel runs.
@@ -28,9 +29,9 @@ constexpr int kVPairX = 32;
 // other values fixed at their pre-half-sweep values.  Reads uin, writes every interior
 // cell of uout (colour c updated, the other colour copied), one z-pair per thread;
 // blocks of kVPairX x rows threads.
-template <int ORDER, typename T, typename LD, bool CVT = false>
-__device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restrict__ uin,
-                                               T* __restrict__ uout, const T* __restrict__ f,
+template <int ORDER, typename T, bool CVT = false>
+__device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* uin,
+                                               T* uout, const T* f,
                                                T a_f, int colour, int periodic, int i, int j,
                                                int k0) {
   const int sy = G.Zp;
@@ -39,7 +40,7 @@ __device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restric
   const int upd = (((i + j + k0) & 1) == colour) ? 0 : 1;
   const bool pair = (k0 + 1) < G.n2;
   if (!pair && upd == 1) {
-    const T c = LD::ld(uin + p0);
+    const T c = uin[p0];
     uout[p0] = c;
     if (periodic) write_images<T>(G, uout, i, j, k0, c);
     return;
@@ -47,18 +48,14 @@ __device__ __forceinline__ void smooth_pair_at(const Grid& G, const T* __restric
   const long long p = p0 + upd;
   // u = (h^2 f - sum_off w u_nb) / w_centre
   T nb[3 * ORDER];
-  load_neighbours<ORDER, T, LD>(uin, p, sy, sx, nb);
-  const T v = relax<ORDER, T, CVT>(nb, a_f * LD::ld(f + p));
+  load_neighbours<ORDER, T>(uin, p, sy, sx, nb);
+  const T other = upd == 0 ? nb[1] : nb[0];  // the pair's cell of the other colour
+  const T v = relax<ORDER, T, CVT>(nb, a_f * f[p]);
   if (pair) {
     typedef typename Vec2<T>::type V2;
     V2 out;
-    if (upd == 0) {
-      out.x = v;
-      out.y = LD::ld(uin + p0 + 1);
-    } else {
-      out.x = LD::ld(uin + p0);
-      out.y = v;
-    }
+    out.x = upd == 0 ? v : other;
+    out.y = upd == 0 ? other : v;
     *reinterpret_cast<V2*>(uout + p0) = out;
     if (periodic) write_pair_images<T>(G, uout, i, j, k0, out.x, out.y);
   } else {
@@ -75,15 +72,15 @@ struct FasBox {
   Int3 lo, hi;
 };
 
-template <int ORDER, typename T, typename LD>
-__device__ __forceinline__ void smooth_fas_pair_at(const Grid& G, const T* __restrict__ uin,
-                                                   T* __restrict__ uout, T* __restrict__ f,
+template <int ORDER, typename T>
+__device__ __forceinline__ void smooth_fas_pair_at(const Grid& G, const T* uin,
+                                                   T* uout, T* f,
                                                    T a_f, T invh2, const FasBox& box, int colour,
                                                    int periodic, int i, int j, int k0) {
   typedef typename Vec2<T>::type V2;
   const long long p = gidx(G, i, j, k0);
   T n0[3 * ORDER], n1[3 * ORDER], c0, c1;
-  load_pair_neighbours<ORDER, T, LD>(uin, p, G.Zp, G.Y * G.Zp, n0, n1, c0, c1);
+  load_pair_neighbours<ORDER, T>(uin, p, G.Zp, G.Y * G.Zp, n0, n1, c0, c1);
   V2 fv = *reinterpret_cast<const V2*>(f + p);
   if (i >= box.lo.x && i < box.hi.x && j >= box.lo.y && j < box.hi.y) {
     const bool in0 = k0 >= box.lo.z && k0 < box.hi.z;
@@ -101,24 +98,24 @@ __device__ __forceinline__ void smooth_fas_pair_at(const Grid& G, const T* __res
   if (periodic) write_pair_images<T>(G, uout, i, j, k0, out.x, out.y);
 }
 
-template <int ORDER, typename T, typename LD, bool CVT = false>
-__device__ __forceinline__ void smooth_half_body(const Grid& G, const T* __restrict__ uin,
-                                                 T* __restrict__ uout, const T* __restrict__ f,
+template <int ORDER, typename T, bool CVT = false>
+__device__ __forceinline__ void smooth_half_body(const Grid& G, const T* uin,
+                                                 T* uout, const T* f,
                                                  T a_f, int colour, int periodic, int rows, Blk b) {
   const int j = b.by * rows + b.ty;
   const int k0 = 2 * (b.bx * kVPairX + b.tx);
   if (j >= G.n1 || k0 >= G.n2) return;
-  smooth_pair_at<ORDER, T, LD, CVT>(G, uin, uout, f, a_f, colour, periodic, b.bz, j, k0);
+  smooth_pair_at<ORDER, T, CVT>(G, uin, uout, f, a_f, colour, periodic, b.bz, j, k0);
 }
 
 // ---- residual + restriction: one thread per covered parent cell ---------------------
 // r = f - L u at its 8 children; parent u := mean(u), ubar := mean(u), parent
 // f_fas := mean(r) (L ubar is added by fas_source).  Blocks of 32 x 4 threads.
-template <int ORDER, typename T, typename LD>
-__device__ __forceinline__ void residual_restrict_body(const Grid& F, const T* __restrict__ u,
-                                                       const T* __restrict__ f, T invh2,
-                                                       const Grid& P, T* __restrict__ pu,
-                                                       T* __restrict__ pfas, T* __restrict__ ubar,
+template <int ORDER, typename T>
+__device__ __forceinline__ void residual_restrict_body(const Grid& F, const T* u,
+                                                       const T* f, T invh2,
+                                                       const Grid& P, T* pu,
+                                                       T* pfas, T* ubar,
                                                        Int3 off, Int3 cn, int parent_periodic,
                                                        Blk b) {
   const int kc = b.bx * 32 + b.tx;
@@ -135,9 +132,9 @@ __device__ __forceinline__ void residual_restrict_body(const Grid& F, const T* _
 #pragma unroll
       for (int dk = 0; dk < 2; ++dk) {
         const long long p = gidx(F, 2 * ic + di, 2 * jc + dj, 2 * kc + dk);
-        const T c = LD::ld(u + p);
+        const T c = u[p];
         su += c;
-        sr += add_lap_h2<ORDER, T, LD>(u, p, sy, sx, c, -invh2, LD::ld(f + p));
+        sr += add_lap_h2<ORDER, T>(u, p, sy, sx, c, -invh2, f[p]);
       }
     }
   }
@@ -150,28 +147,28 @@ __device__ __forceinline__ void residual_restrict_body(const Grid& F, const T* _
 }
 
 // ---- FAS source: covered parent cells f_fas += L u (u = restricted fine solution) ----
-template <int ORDER, typename T, typename LD>
-__device__ __forceinline__ void fas_source_body(const Grid& P, const T* __restrict__ pu,
-                                                T* __restrict__ pfas, T invH2, Int3 off, Int3 cn,
+template <int ORDER, typename T>
+__device__ __forceinline__ void fas_source_body(const Grid& P, const T* pu,
+                                                T* pfas, T invH2, Int3 off, Int3 cn,
                                                 Blk b) {
   const int kc = b.bx * 32 + b.tx;
   const int jc = b.by * 4 + b.ty;
   const int ic = b.bz;
   if (kc >= cn.z || jc >= cn.y) return;
   const long long q = gidx(P, off.x + ic, off.y + jc, off.z + kc);
-  pfas[q] = add_lap_h2<ORDER, T, LD>(pu, q, P.Zp, P.Y * P.Zp, LD::ld(pu + q), invH2, pfas[q]);
+  pfas[q] = add_lap_h2<ORDER, T>(pu, q, P.Zp, P.Y * P.Zp, pu[q], invH2, pfas[q]);
 }
 
 // ---- prolongation-correction: u += inject(parent u - ubar), one thread per z-pair ----
-template <typename T, typename LD>
-__device__ __forceinline__ void prolong_at(const Grid& F, T* __restrict__ u, const Grid& P,
-                                           const T* __restrict__ pu, const T* __restrict__ ubar,
+template <typename T>
+__device__ __forceinline__ void prolong_at(const Grid& F, T* u, const Grid& P,
+                                           const T* pu, const T* ubar,
                                            Int3 off, Int3 cn, int periodic, int i, int j, int t) {
   const int k0 = 2 * t;
   if (j >= F.n1 || k0 >= F.n2) return;
   const int ic = i >> 1, jc = j >> 1, kc = t;
-  const T d = LD::ld(pu + gidx(P, off.x + ic, off.y + jc, off.z + kc)) -
-              LD::ld(ubar + ((long long)ic * cn.y + jc) * cn.z + kc);
+  const T d = pu[gidx(P, off.x + ic, off.y + jc, off.z + kc)] -
+              ubar[((long long)ic * cn.y + jc) * cn.z + kc];
   const long long p = gidx(F, i, j, k0);
   typedef typename Vec2<T>::type V2;
   V2 v = *reinterpret_cast<const V2*>(u + p);
@@ -184,18 +181,18 @@ __device__ __forceinline__ void prolong_at(const Grid& F, T* __restrict__ u, con
   }
 }
 
-template <typename T, typename LD>
-__device__ __forceinline__ void prolong_body(const Grid& F, T* __restrict__ u, const Grid& P,
-                                             const T* __restrict__ pu, const T* __restrict__ ubar,
+template <typename T>
+__device__ __forceinline__ void prolong_body(const Grid& F, T* u, const Grid& P,
+                                             const T* pu, const T* ubar,
                                              Int3 off, Int3 cn, int periodic, Blk b) {
-  prolong_at<T, LD>(F, u, P, pu, ubar, off, cn, periodic, b.bz, b.by * 4 + b.ty, b.bx * 32 + b.tx);
+  prolong_at<T>(F, u, P, pu, ubar, off, cn, periodic, b.bz, b.by * 4 + b.ty, b.bx * 32 + b.tx);
 }
 
 // ---- periodic ghost shell: element t of the shell takes its interior image ----------
 // (ghost_shell_count(G) elements, mg_internal.h)
 
 template <typename T>
-__device__ __forceinline__ void ghost_periodic_body(const Grid& G, T* __restrict__ u, long long t) {
+__device__ __forceinline__ void ghost_periodic_body(const Grid& G, T* u, long long t) {
   const long long g = G.g;
   const long long X = G.n0 + 2 * g, Y = G.n1 + 2 * g;
   const long long cntA = X * Y * 2 * g;
@@ -275,11 +272,11 @@ __device__ __forceinline__ int face_of(const FaceSet& fs, long long t, const lon
 // layer m: the 4 fine positions over it (tj = 2 jc + pj, tk = 2 kc + pk) interpolate
 // the same (n+1) x (n+1) patch of parent values, so each row of the patch is reduced
 // along c once per parity pk, then along b once per parity pj.
-template <int ORDER, typename T, typename LD>
+template <int ORDER, typename T>
 __device__ __forceinline__ void cf_tangential_body(const Grid& F, const Grid& P,
-                                                   const T* __restrict__ pu, Int3 off,
+                                                   const T* pu, Int3 off,
                                                    const FaceSet& fs, const CfW<T>& w, T invH,
-                                                   T* __restrict__ inter, T* __restrict__ fc_unc,
+                                                   T* inter, T* fc_unc,
                                                    long long t) {
   constexpr int half = ORDER / 2;
   if (t >= half * fs.ebase[6]) return;
@@ -314,7 +311,7 @@ __device__ __forceinline__ void cf_tangential_body(const Grid& F, const Grid& P,
     T r0 = T(0), r1 = T(0);
 #pragma unroll
     for (int cc = 0; cc <= ORDER; ++cc) {
-      const T v = LD::ld(pu + p0 + bb * sb + cc * sc);
+      const T v = pu[p0 + bb * sb + cc * sc];
       r0 = fma(w.tang[0][cc], v, r0);
       r1 = fma(w.tang[1][cc], v, r1);
     }
@@ -344,7 +341,7 @@ __device__ __forceinline__ void cf_tangential_body(const Grid& F, const Grid& P,
     const long long q0 = p0 + half * sb + half * sc + (long long)(pface - half - pn) * sa;
     T fc = T(0);
     const int s0 = side == 0 ? 0 : half, s1 = side == 0 ? half : ORDER;
-    for (int s = s0; s < s1; ++s) fc = fma(w.flux[s], LD::ld(pu + q0 + s * sa), fc);
+    for (int s = s0; s < s1; ++s) fc = fma(w.flux[s], pu[q0 + s * sa], fc);
     fc_unc[fs.ebase[f] + (long long)jc * ne1 + kc] = fc * invH;
   }
 }
@@ -391,8 +388,8 @@ __device__ __forceinline__ FaceCol face_col(const Grid& F, int f, int jc, int kc
 // mask of converged lanes that holds the element's four.
 template <int ORDER, typename T>
 __device__ __forceinline__ void cf_flux_at(T* u, const FaceSet& fs, const CfW<T>& w,
-                                           const T* __restrict__ inter,
-                                           const T* __restrict__ fc_unc, T fc_scale, T a0, T a1,
+                                           const T* inter,
+                                           const T* fc_unc, T fc_scale, T a0, T a1,
                                            T b0, T b1, int flux_fix, const FaceCol& fcol,
                                            const T (&v)[ORDER], unsigned quad) {
   constexpr int half = ORDER / 2;
@@ -449,9 +446,9 @@ __device__ __forceinline__ void load_column(const T* u, const FaceCol& c, T (&v)
 }
 
 template <int ORDER, typename T>
-__device__ __forceinline__ void cf_flux_body(const Grid& F, T* __restrict__ u, const FaceSet& fs,
-                                             const CfW<T>& w, const T* __restrict__ inter,
-                                             const T* __restrict__ fc_unc, T fc_scale, T a0, T a1,
+__device__ __forceinline__ void cf_flux_body(const Grid& F, T* u, const FaceSet& fs,
+                                             const CfW<T>& w, const T* inter,
+                                             const T* fc_unc, T fc_scale, T a0, T a1,
                                              T b0, T b1, int flux_fix, long long t) {
   if (t >= 4 * fs.ebase[6]) return;
   const unsigned quad = __activemask();
@@ -476,8 +473,8 @@ struct FluxFold {
 
 template <int ORDER>
 __device__ __forceinline__ void cf_fold_at(double* u, const FaceSet& fs, const FluxFold& w,
-                                           const double* __restrict__ inter,
-                                           const double* __restrict__ fc_unc, const FaceCol& c,
+                                           const double* inter,
+                                           const double* fc_unc, const FaceCol& c,
                                            const double (&v)[ORDER], unsigned quad) {
   constexpr int half = ORDER / 2;
   const int side = c.f & 1;
@@ -485,8 +482,8 @@ __device__ __forceinline__ void cf_fold_at(double* u, const FaceSet& fs, const F
   double g[half];
   const double* ip = inter + fs.base[c.f] + ((long long)c.tj * nt1 + c.tk);
 #pragma unroll
-  for (int m = 0; m < half; ++m) g[m] = __ldg(ip + (long long)m * nt0 * nt1);
-  const double k = __ldg(fc_unc + fs.ebase[c.f] + (long long)c.jc * (nt1 / 2) + c.kc);
+  for (int m = 0; m < half; ++m) g[m] = ip[(long long)m * nt0 * nt1];
+  const double k = fc_unc[fs.ebase[c.f] + (long long)c.jc * (nt1 / 2) + c.kc];
   double s = w.d[side][0] * v[0];
 #pragma unroll
   for (int q = 1; q < 2 * half; ++q) s = fma(w.d[side][q], v[q], s);
@@ -541,9 +538,9 @@ FaceArgs<T> make_face_args(int order, const FaceSet& fs, const CfWeights& w, con
 // Every thread of the block must call it (block-wide reduction).
 constexpr int kCoarseThreads = 128;
 
-template <typename T, typename LD>
-__device__ __forceinline__ void coarsest_body(const Grid& G, const T* __restrict__ f,
-                                              T* __restrict__ u, const double* __restrict__ kern,
+template <typename T>
+__device__ __forceinline__ void coarsest_body(const Grid& G, const T* f,
+                                              T* u, const double* kern,
                                               int x, int tid) {
   const int n12 = G.n1 * G.n2;
   const int n = G.n0 * n12;
@@ -555,7 +552,7 @@ __device__ __forceinline__ void coarsest_body(const Grid& G, const T* __restrict
     di += di < 0 ? G.n0 : 0;
     dj += dj < 0 ? G.n1 : 0;
     dk += dk < 0 ? G.n2 : 0;
-    acc = fma(__ldg(kern + (di * G.n1 + dj) * G.n2 + dk), (double)LD::ld(f + gidx(G, yi, yj, yk)), acc);
+    acc = fma(__ldg(kern + (di * G.n1 + dj) * G.n2 + dk), (double)f[gidx(G, yi, yj, yk)], acc);
   }
   __shared__ double red[kCoarseThreads];
   red[tid] = acc;
