@@ -92,7 +92,10 @@ __global__ void __launch_bounds__(kAmpThreads)
                       double h, const double* __restrict__ amp, int nt, double dk, double scale) {
   const int n2h = half_x ? n2 : n2 / 2 + 1;
   const double tp = 2.0 * 3.14159265358979323846 / h;
-  const int i = blockIdx.z, j0 = blockIdx.y * kAmpRows;
+  // blocks in one dimension, along m first: a side may pass the 65535 of the other dimensions
+  const unsigned bm = (n2h + kAmpThreads - 1) / kAmpThreads, bj = (n1 + kAmpRows - 1) / kAmpRows;
+  const unsigned row = blockIdx.x / bm;
+  const int i = row / bj, j0 = row % bj * kAmpRows;
   __shared__ double fij[kAmpRows];
   if (threadIdx.x < kAmpRows) {
     const int j = j0 + (int)threadIdx.x;
@@ -101,7 +104,7 @@ __global__ void __launch_bounds__(kAmpThreads)
     fij[threadIdx.x] = fma(fi, fi, fj * fj);
   }
   __syncthreads();
-  const int m = blockIdx.x * kAmpThreads + threadIdx.x;
+  const int m = (blockIdx.x - row * bm) * kAmpThreads + threadIdx.x;
   if (m >= n2h) return;
   const double fm = (double)(m <= n2 / 2 ? m : m - n2) / n2;
   const int rows = min(kAmpRows, n1 - j0);
@@ -128,7 +131,8 @@ __global__ void __launch_bounds__(kAmpThreads)
 void launch_amplitude(cufftDoubleComplex* F, int n0, int n1, int n2, bool half_x, double h,
                       const double* amp, int nt, double dk, double scale, cudaStream_t s) {
   const int row = half_x ? n2 : n2 / 2 + 1, planes = half_x ? n0 / 2 + 1 : n0;
-  const dim3 grid((row + kAmpThreads - 1) / kAmpThreads, (n1 + kAmpRows - 1) / kAmpRows, planes);
+  const unsigned grid = (unsigned)((row + kAmpThreads - 1) / kAmpThreads) *
+                        ((n1 + kAmpRows - 1) / kAmpRows) * planes;
   k_apply_amplitude<<<grid, kAmpThreads, 0, s>>>(F, n0, n1, n2, half_x ? 1 : 0, h, amp, nt, dk, scale);
 }
 

@@ -96,8 +96,10 @@ __global__ void __launch_bounds__(256)
                       int N0, int N1, int N2, const AxisSymbol* __restrict__ tab, double scale,
                       int comp) {
   const int N2h = N2 / 2 + 1;
-  const int j = blockIdx.y, i = blockIdx.z;
-  const int m = blockIdx.x * 256 + threadIdx.x;
+  // blocks in one dimension, along m first: a side may pass the 65535 of the other dimensions
+  const unsigned bm = (N2h + 255) / 256, row = blockIdx.x / bm;
+  const int i = row / N1, j = row % N1;
+  const int m = (blockIdx.x - row * bm) * 256 + threadIdx.x;
   if (m >= N2h) return;
   const AxisSymbol a[3] = {tab[i], tab[N0 + j], tab[N0 + N1 + m]};
   const int idx[3] = {i, j, m}, N[3] = {N0, N1, N2};
@@ -250,7 +252,7 @@ cudaError_t hybrid_apply(HybridFFT* hy, const double* f, double* const psi[3], c
   if (cufftExecZ2Z(hy->lines, hy->F, hy->F, CUFFT_FORWARD) != CUFFT_SUCCESS)
     return cudaErrorUnknown;
   const double scale = hy->h / ((double)N0 * N1 * N2);
-  const dim3 grid((N2h + 255) / 256, N1, N0);
+  const unsigned grid = (unsigned)((N2h + 255) / 256) * N1 * N0;
   for (int c = 0; c < 3; ++c) {
     k_hybrid_multiply<<<grid, 256, 0, s>>>(hy->F, hy->W, N0, N1, N2, hy->tab, scale, c);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
