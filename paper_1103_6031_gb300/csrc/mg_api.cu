@@ -276,8 +276,7 @@ struct mg_hierarchy {
   double* red = nullptr;
   double* host_red = nullptr;  // pinned copy of red
   unsigned* wait_err = nullptr;  // device flag: a bounded wait in a kernel ran out
-  double* scratch = nullptr;   // 3 dense arrays of the largest leaf level
-  long long scratch_elems = 0;
+  double* scratch = nullptr;   // local density: Phi of a leaf level (dense, the largest's size)
   double* tau_work = nullptr;  // MG_MIXED: 2 padded float64 arrays of the largest leaf level
   // host-buffer pipelines: the first solve's phi and displacements are staged here
   // (phi, x, y, z per leaf level, dense) and copied to the host on cs while the
@@ -532,7 +531,7 @@ size_t carve(const mg_config* cfg, const Plan& p, mg_hierarchy* h, char* arena) 
   }
   double* partial = c.take<double>((size_t)slots * 2);
   double* red = c.take<double>(kRedDoubles);
-  double* scratch = c.take<double>((size_t)3 * max_leaf);
+  double* scratch = c.take<double>((size_t)max_leaf);
   double* tau_work = mixed ? c.take<double>((size_t)2 * max_leaf_padded) : nullptr;
   double* stage = c.take<double>((size_t)4 * leaf_total);
   if (h) {
@@ -543,7 +542,6 @@ size_t carve(const mg_config* cfg, const Plan& p, mg_hierarchy* h, char* arena) 
     h->red = red;
     h->wait_err = reinterpret_cast<unsigned*>(red + 4);
     h->scratch = scratch;
-    h->scratch_elems = max_leaf;
   }
   return c.used;
 }
