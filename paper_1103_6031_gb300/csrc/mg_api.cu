@@ -1678,9 +1678,12 @@ bool batch_persistent(const mg_batch* b, const std::vector<int>& active) {
   return false;
 }
 
-// Members from which a batch's branches count as crowded (16 members of the mixed-precision
-// ensemble: 16.8 ms with separate ghost launches, 17.4 ms with fused half-sweeps).
-constexpr int kCrowdedMembers = 4;
+// Members from which a batch's branches count as crowded.  Members of the mixed-precision and of
+// the float64 ensemble, ms with separate ghost launches / with fused half-sweeps: 2 members 3.24 /
+// 3.08 and 4.65 / 4.30, 3 3.70 / 3.54 and 5.30 / 5.16, 4 4.19 / 3.97 and 5.66 / 5.46, 6 9.00 / 9.07
+// and 13.48 / 13.69, 8 9.58 / 9.69 and 14.56 / 14.89, 12 11.9 / 12.2 and 19.1 / 19.5, 16 15.9 / 16.6
+// and 27.1 / 27.9.
+constexpr int kCrowdedMembers = 6;
 
 bool crowded(const std::vector<int>& active) {
   int n = 0;

@@ -74,8 +74,9 @@ cudaError_t launch_smooth_half(int order, const Grid& G, const T* uin, T* uout, 
                                cudaStream_t s);
 // Nests up to this many cells take the fused half-sweep below.  One V-cycle of a base and two
 // nests of n^3 cells, separate / fused, us: float32, order 6: n = 32 116.0 / 101.2, 48 144.3 /
-// 130.4, 64 153.2 / 151.6, 80 219.1 / 225.3, 96 292.9 / 310.2; float64, order 4: 32 172.4 /
-// 162.0, 48 220.2 / 201.0, 64 257.3 / 258.8, 80 380.7 / 392.8.
+// 130.4, 64 153.2 / 151.6, 80 219.1 / 225.3, 96 292.9 / 310.2; float64, order 6: 32 182.8 / 173.1,
+// 48 234.5 / 222.2, 64 305.8 / 300.6, 80 453.3 / 488.3, 96 590.2 / 636.1; order 4: 32 155.2 / 142.2,
+// 48 199.0 / 184.8, 64 263.8 / 255.9, 80 394.1 / 414.4, 96 520.2 / 532.0.
 constexpr long long kFaceFusedMaxCells = 1ll << 18;
 // The half-sweep of a nest followed by the coarse-fine ghosts of its result (float64: folded,
 // after launch_cf_tangential with fold = true); h, invH: own spacing, 1 / parent spacing.
