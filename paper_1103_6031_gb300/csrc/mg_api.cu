@@ -269,6 +269,8 @@ struct mg_hierarchy {
   double* zero_d = nullptr;
   float* zero_f = nullptr;
   long long zero_d_count = 0, zero_f_count = 0;
+  // block sums of norms and means.  MG_MIXED: reserved from a solve's first norm to its last, which
+  // leaves the source's sums in the odd entries for the later ones (k_norm_partial)
   double* partial = nullptr;
   int partial_slots = 0;
   // [0..1] norm sums, [2..3] source sum, [4] wait flag, [8 + 2 l, 9 + 2 l] the norm

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kTileThreads, 3)
     const long long p = gidx(G, i, j, k);
     const int sx = G.Y * G.Zp;
     const double kr = -invh2 * FxUnit<ORDER>::v;
-    double2 fv[4];  // under way while the tile is filled
+    double2 fv[4];  // under way while the tile is filled (86.3 us after it, 82.5 so)
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       fv[q] = i + q < G.n0 && j < G.n1 && k < G.n2

@@ -11,10 +11,10 @@
 //
 // Accuracy: a unit is 2^-58 to 2^-59 of the BLOCK's largest value (halo included), not of the
 // cell's own neighbours'.  A tile is summed as integers only if every cell's star holds a value
-// of at least 2^52 units or nothing but zeros (tile_key); the rounding of a difference, at
-// most 30 units, then stays below 2^-47 of the largest value in the cell's own star, and is far
-// smaller where that is the block's largest too.  Other tiles (a strong cell among weak ones, a
-// steep tail) are left to FP64 arithmetic.
+// of at least 2^52 units (2^51 at order 2) or nothing but zeros (tile_key); the rounding of a
+// difference, at most 30 units (12), then stays below 2^-47 of the largest value in the cell's own
+// star, and is far smaller where that is the block's largest too.  Other tiles (a strong cell
+// among weak ones, a steep tail) are left to FP64 arithmetic.
 #pragma once
 
 #include "mg_fixed.cuh"
@@ -103,22 +103,22 @@ __device__ __forceinline__ unsigned block_max(unsigned m) {
 
 // Exponents a cell's star may lie below the block's largest: the bits that an aligned value has
 // beyond a mantissa's 53.  Tiles of a smooth field pass, also where it is zero on a surface:
-// its star reaches ORDER / 2 cells to either side, a tile 32.
-constexpr int kTileRange = 6;
+// its star reaches ORDER / 2 cells to either side, a tile 32.  At order 2, whose unweighted sums
+// lose half as many units, one more: 6 rejects 0.2 to 0.9% of the tiles of a potential (none at
+// orders 4 and 6), and on a small level one tile in FP64 arithmetic is what the launch waits for
+// (solve to 1e-10 of 64^3 886 us with 6, 842 with 7).
+template <int ORDER>
+constexpr int kTileRange = ORDER == 2 ? 7 : 6;
 
-// Of a thread's cells (tile_pos: a z-pair in 4 planes, a and b their keys or magnitudes) those
-// whose stars may be too low, as bits 2 q + dk: neither the cell nor its neighbours among the
-// thread's lie above lim.  in(q): which cells of the pair exist.  Of the tiles of a potential 2%
-// have such cells, 35% cells that are low themselves.
-template <int ORDER, typename In>
-__device__ __forceinline__ unsigned low_cells(const unsigned (&a)[4], const unsigned (&b)[4],
-                                              unsigned lim, In in) {
-  constexpr int R = ORDER / 2;
-  // the least of the windows' largest: every x neighbourhood within the 4 planes holds one
-  constexpr int W = R < 3 ? R + 1 : 4;
+// Whether the star of one of a thread's cells (tile_pos: a z-pair in 4 planes; a and b their keys or
+// magnitudes) can be low: the least of the largest values of windows along x of which every star
+// holds one.
+template <int ORDER>
+__device__ __forceinline__ unsigned least_window(const unsigned (&a)[4], const unsigned (&b)[4]) {
+  constexpr int W = ORDER / 2 < 3 ? ORDER / 2 + 1 : 4, STEP = W < 4 ? 4 - W : 1;
   unsigned least = ~0u;
 #pragma unroll
-  for (int q = 0; q + W <= 4; q += 4 - W > 0 ? 4 - W : 4) {
+  for (int q = 0; q + W <= 4; q += STEP) {
     unsigned ma = 0, mb = 0;
 #pragma unroll
     for (int n = q; n < q + W; ++n) {
@@ -127,42 +127,32 @@ __device__ __forceinline__ unsigned low_cells(const unsigned (&a)[4], const unsi
     }
     least = min(least, min(ma, mb));
   }
-  if (least > lim) return 0;
-  unsigned low = 0;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    unsigned ma = b[q], mb = a[q];
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-      if (n - q <= R && q - n <= R) {
-        ma = max(ma, a[n]);
-        mb = max(mb, b[n]);
-      }
-    low |= (((ma <= lim ? 1u : 0u) | (mb <= lim ? 2u : 0u)) & in(q)) << (2 * q);
-  }
-  return low;
+  return least;
 }
 
-// Ends the filling of a tile: its key, or 0 (out of range: FP64 arithmetic) where the star of a
-// cell holds only values more than 2^kTileRange below the block's largest, and not only zeros (a
-// star that the alignment leaves nothing of is looked up in src, the tile at (i0, j0, k0)).
-// low: the thread's cells to look at (low_cells).  The same answer in every thread.  What the
-// question costs, without / with, order 6: the first-cycle restrictions of a 192 x 160 x 224 level
-// and the next 36.9 / 40.9 us, its norm 83.8 / 82.6 (with f loaded ahead), tau of 256^3 705 / 721,
-// a whole step 0.5 to 2%; asked after the sums, the restriction takes 38.9, the norm 85.8, tau 737.
+// Ends the filling of a tile of ex x ey x ez cells at (i0, j0, k0) of src: its key, or 0 (out of
+// range: FP64 arithmetic) where the star of a cell holds only values more than kTileRange exponents
+// below the block's largest, and not only zeros (a star that the alignment leaves nothing of is
+// looked up in src).  low: a star of the thread's cells can be (least_window).  The same answer in
+// every thread.  Few tiles of a potential have to look: 4.4% in the steps of 192 x 160 x 224 and
+// 3.4% of two levels of 128^3, 0.02% of which then go to FP64.  What the question costs, without /
+// with, order 6, 192 x 160 x 224: the first cycle's restriction 50.1 / 52.8 us, the norm 83.8 /
+// 82.9 (with f loaded ahead); tau of 256^3 705 / 721 us.  Asked after the sums it costs the norm 2
+// and tau 4% more; with every cell of the thread told apart beforehand, the restriction 56.0.
 template <int ORDER, typename Src>
 __device__ __forceinline__ unsigned tile_key(unsigned key, const long long* S, const Src& src,
-                                             int i0, int j0, int k0, unsigned low) {
+                                             int i0, int j0, int k0, int ex, int ey, int ez,
+                                             bool low) {
   typedef FxTile<ORDER> L;
-  constexpr long long kWeak = 1ll << (58 - kTileRange);
+  constexpr long long kWeak = 1ll << (58 - kTileRange<ORDER>);
   auto mag = [](long long v) { return v ^ (v >> 63); };
   if (__builtin_expect(!__syncthreads_or(low), 1)) return key;
-  const TilePos t = tile_pos();
   bool wide = false;
 #pragma unroll 1
-  for (; low; low &= low - 1) {
-    const int bit = __ffs(low) - 1;
-    const int x = 4 * t.xh + (bit >> 1), y = t.y, z = 2 * t.zz + (bit & 1);
+  for (int e = low ? 0 : 8; e < 8; ++e) {
+    const TilePos t = tile_pos();
+    const int x = 4 * t.xh + (e >> 1), y = t.y, z = 2 * t.zz + (e & 1);
+    if (x >= ex || y >= ey || z >= ez) continue;
     const long long* c = S + L::at(x, y, z);
     long long m = mag(c[0]);
 #pragma unroll 1
@@ -263,19 +253,15 @@ __device__ __forceinline__ unsigned tile_load(const Grid& G, const double* u, in
     }
     if (zact) put(zx, zy, zo, vz);
   }
-  unsigned low = 0;
-  if (fx_in_range(m)) {
-    unsigned a[4], b[4];
+  unsigned a[4], b[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      a[q] = fx_key(c[q].x);
-      b[q] = fx_key(c[q].y);
-    }
-    low = low_cells<ORDER>(a, b, m - ((kTileRange + 1u) << 21), [&](int q) {
-      return 4 * t.xh + q < ex && t.y < ey ? (in0 ? 1u : 0u) | (in1 ? 2u : 0u) : 0u;
-    });
+  for (int q = 0; q < 4; ++q) {
+    a[q] = fx_key(c[q].x);
+    b[q] = fx_key(c[q].y);
   }
-  return tile_key<ORDER>(m, S, PaddedSource(G, u), i0, j0, k0, low);
+  const bool low =
+      fx_in_range(m) && least_window<ORDER>(a, b) <= m - ((kTileRange<ORDER> + 1u) << 21);
+  return tile_key<ORDER>(m, S, PaddedSource(G, u), i0, j0, k0, ex, ey, ez, low);
 }
 
 // T (mg_fixed.cuh: h^2 L u = T FxUnit 2^(e - kFxBias)) of the thread's 8 cells and their
@@ -400,23 +386,17 @@ __device__ __forceinline__ unsigned tile_load_edges(const Grid& G, const Src& sr
     }
   }
   __syncthreads();
-  unsigned low = 0;
-  if (fx_in_range(m)) {
-    const TilePos t = tile_pos();
-    unsigned a[4], b[4];
+  if (!fx_in_range(m)) return m;
+  const TilePos t = tile_pos();
+  unsigned a[4], b[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const longlong2 v =
-          *reinterpret_cast<const longlong2*>(S + L::at(4 * t.xh + q, t.y, 2 * t.zz));
-      a[q] = (unsigned)((int)(v.x >> 32) ^ (int)(v.x >> 63));
-      b[q] = (unsigned)((int)(v.y >> 32) ^ (int)(v.y >> 63));
-    }
-    low = low_cells<ORDER>(a, b, (1u << (26 - kTileRange)) - 1u, [&](int q) {
-      return 4 * t.xh + q < ex && t.y < ey
-                 ? (2 * t.zz < ez ? 1u : 0u) | (2 * t.zz + 1 < ez ? 2u : 0u) : 0u;
-    });
+  for (int q = 0; q < 4; ++q) {
+    const longlong2 v = *reinterpret_cast<const longlong2*>(S + L::at(4 * t.xh + q, t.y, 2 * t.zz));
+    a[q] = (unsigned)((int)(v.x >> 32) ^ (int)(v.x >> 63));
+    b[q] = (unsigned)((int)(v.y >> 32) ^ (int)(v.y >> 63));
   }
-  return tile_key<ORDER>(m, S, src, i0, j0, k0, low);
+  const bool low = least_window<ORDER>(a, b) < 1u << (26 - kTileRange<ORDER>);
+  return tile_key<ORDER>(m, S, src, i0, j0, k0, ex, ey, ez, low);
 }
 
 // The finite-difference Hessian of a column of 8 cells per thread (z = lane, y = warp) as
