@@ -465,8 +465,9 @@ typedef struct mg_field mg_field;  /* opaque: FFT plans and spectrum of one grid
  * 2..4096).  The amplitude A(|k|) is the linear interpolation of amp[0..nt) (host,
  * nt >= 2, finite), sampled at |k| = t dk; A = 0 beyond (nt - 1) dk and at k = 0.
  * For the density of Sec. 2.1 with numpy-style unnormalised transforms, A = sqrt(P(k)
- * / h^3).  Allocates the half spectrum (16 n0 n1 (n2/2+1) bytes) and two cuFFT plans
- * on the current device.  Errors: MG_EINVAL, MG_ENOMEM, MG_ECUDA. */
+ * / h^3).  Allocates the half spectrum and cuFFT plans on the current device: along z
+ * (16 n0 n1 (n2/2+1) bytes, two plans), or along x if n2 is odd and n0 even
+ * (16 (n0/2+1) n1 n2 bytes, three plans).  Errors: MG_EINVAL, MG_ENOMEM, MG_ECUDA. */
 mg_status mg_field_create(int n0, int n1, int n2, double h, const double* amp, int nt,
                           double dk, mg_field** out);
 

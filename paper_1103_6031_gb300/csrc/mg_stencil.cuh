@@ -105,7 +105,8 @@ __device__ __forceinline__ unsigned neighbour_key(const double (&nb)[3 * ORDER])
 // acc = (h^2 / w_centre) f.  float64 sums the neighbours on the integer pipe
 // (mg_fixed.cuh): 3 FP64 instructions per update instead of 19.  Measured on GB300, order 6,
 // warm L2, 128^3 nest: 41.7 -> 17.6 us per half-sweep, 16.0 with CVT (64^3: 6.9 -> 3.9,
-// 32^3: 3.0 -> 2.2); order 4: 29.2 -> 12.8; order 2: 16.5 -> 8.7.
+// 32^3: 3.0 -> 2.2); order 4: 29.2 -> 12.8; order 2: 16.5 -> 8.7.  Plain instead of read-only
+// loads (mg_launch.cuh) have added 2 to 4% since.
 template <int ORDER, typename T, bool CVT = false>
 __device__ __forceinline__ T relax(const T (&nb)[3 * ORDER], T acc) {
   constexpr double wc = 3.0 * Lap<ORDER>::w0;
